@@ -18,6 +18,7 @@
 #include "sd2_format.hpp"
 #include "sd2_format_mma.hpp"
 #include "sd2_kernels.cuh"
+#include "sd2_cell_kernel.cuh"
 #include "sd2_mma_kernel.cuh"
 #include "sd2_glue.cuh"
 
@@ -33,10 +34,23 @@ struct sd2_handle_s {
     // GAP4 geometry
     int S, B, T, max_tile_bytes, V;
     int paired;   // GAP4: rows 2i, 2i+1 share a tile (header field `pairing`)
+    // GAP4: the same weights as cells (sd2_cells.hpp), for panels of rows (d_image NULL: none)
+    uint8_t* d_image;
+    const unsigned char* d_cells;
+    int64_t image_bytes, cell_bytes;   // device bytes; what a launch reads of them
+    int cell_T, cell_D, max_cell;
     // GAP4_MMA: fp32 partial sums [64][rows padded to 128] followed by one arrival count per row panel,
     // all zero between launches (the CTA that completes a panel writes Y and clears them)
     float* d_partial;
     int64_t partial_bytes;
+};
+
+// What a program over cells needs from shared memory.
+struct CellNeeds {
+    int pitch[2] = {0, 0};     // bytes of a staged activation row, by parity of the stage: the largest
+    int max_cell = 0;
+    int parts = 0;             // most contributions to a tile
+    int tiles_max = 0;         // most tiles of any stage
 };
 
 struct sd2_drafter_s {
@@ -57,6 +71,14 @@ struct sd2_drafter_s {
     int K_max, max_tile;       // what decides the shared-memory split
     int free_tiles;            // every stage has enough tiles per CTA for free tile assignment
     int xs_need[4];            // bytes of staged activations at panel widths 1, 2, 4, 8
+    // the same blocks as a program over cells, with barrier words, production counts and tagged words of its own
+    // (a word of either program must never show a tag of the other); NULL: a handle has no cells
+    CStage* d_cstages;
+    unsigned int* d_cbar;
+    uint32_t* d_ctags;
+    int64_t ctags_bytes;
+    int n_cstages;
+    CellNeeds cell_needs;
 };
 
 namespace {
@@ -134,6 +156,14 @@ cudaError_t set_smem_attr()
     return cudaFuncSetAttribute(stream_kernel<NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - kFoldStaticBytes);
 }
 
+template <int MAXS, int NR>
+cudaError_t set_cell_attr()
+{
+    cudaError_t e = cudaFuncSetAttribute(cell_kernel<MAXS, NR, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(cell_kernel<MAXS, NR, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+}
+
 // Once per device: SM count, shared-memory opt-in, the error word and the barrier pool.
 sd2_status ensure_device(int* dev_out)
 {
@@ -147,7 +177,8 @@ sd2_status ensure_device(int* dev_out)
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev) != cudaSuccess) { cudaGetLastError(); return SD2_ERR_CUDA; }
         if (set_smem_attr<1>() != cudaSuccess || set_smem_attr<2>() != cudaSuccess || set_smem_attr<4>() != cudaSuccess ||
-            set_smem_attr<8>() != cudaSuccess ||
+            set_smem_attr<8>() != cudaSuccess || set_cell_attr<1, 8>() != cudaSuccess || set_cell_attr<1, 16>() != cudaSuccess ||
+            set_cell_attr<kMaxStagesInline, 8>() != cudaSuccess || set_cell_attr<kMaxStagesInline, 16>() != cudaSuccess ||
             cudaFuncSetAttribute(mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
             cudaFuncSetAttribute(lm_head_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess) {
             cudaGetLastError();
@@ -243,6 +274,7 @@ sd2_status upload(const uint8_t* blob, int64_t bytes, const BlobHeader& hd, sd2_
     h->max_tile_bytes = (int)hd.max_tile_bytes;
     h->V = (int)hd.overlap;
     h->paired = (int)hd.pairing;
+    h->d_image = nullptr;
     h->d_partial = nullptr;
     h->partial_bytes = 0;
     if (h->format == SD2_FORMAT_GAP4_MMA) {
@@ -258,6 +290,37 @@ sd2_status upload(const uint8_t* blob, int64_t bytes, const BlobHeader& hd, sd2_
         g_live.insert(h);
     }
     *out = h;
+    return SD2_OK;
+}
+
+// Gives a fresh GAP4 handle its cells.  On failure the handle is freed.
+sd2_status add_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask)
+{
+    CellImage im;
+    sd2_status st = SD2_OK;
+    try {
+        im = pack_cells(W, mask, h->M, h->K);
+        st = from_pack(im.status);
+    } catch (const std::bad_alloc&) {
+        st = SD2_ERR_ALLOC;
+    }
+    void* d = nullptr;
+    if (st == SD2_OK && dev_malloc(&d, im.bytes) != cudaSuccess) { cudaGetLastError(); st = SD2_ERR_ALLOC; }
+    if (st == SD2_OK && cudaMemcpy(d, im.data, im.bytes, cudaMemcpyHostToDevice) != cudaSuccess) { cudaGetLastError(); st = SD2_ERR_CUDA; }
+    std::free(im.data);
+    if (st != SD2_OK) {
+        if (d) cudaFree(d);
+        sd2_free(h);
+        return st;
+    }
+    const CellGeom g = cell_geometry(h->M, h->K);
+    h->d_image = (uint8_t*)d;
+    h->d_cells = h->d_image + im.sec1_off;
+    h->image_bytes = (int64_t)im.bytes;
+    h->cell_bytes = (g.T * g.D + 1) * 4 + (int64_t)(im.bytes - im.sec1_off);
+    h->cell_T = (int)g.T;
+    h->cell_D = g.D;
+    h->max_cell = im.max_cell;
     return SD2_OK;
 }
 
@@ -523,6 +586,175 @@ sd2_status run_program(SArgs& a, int dev, int64_t N, const ProgramNeeds& needs, 
     return run_panels(a, N, needs.xs_need, needs.K_max, needs.max_tile, grid, s);
 }
 
+// ------------------------------------------------------------------ programs over cells
+
+struct CellPlan {
+    int part_bytes, xbuf_bytes[2], slot_bytes, n_slots;
+};
+
+constexpr int kCellFixedBytes = (int)((sizeof(CellShared) + 127) & ~127) + kRingGuardBytes;
+
+// Shared memory of a launch of n rows.  false: not even two cells per warp fit beside the staged rows.
+bool plan_cells(int n, const CellNeeds& needs, bool tagged, CellPlan* p)
+{
+    p->part_bytes = (needs.parts * n * 32 + 127) & ~127;
+    p->slot_bytes = (needs.max_cell + 31) & ~31;
+    const int x0 = (n * needs.pitch[0] + 127) & ~127, x1 = (n * needs.pitch[1] + 127) & ~127;
+    const int rest = kSmemMax - kCellFixedBytes - kPartSlots * p->part_bytes;
+    const int per_slot = kCellWarps * p->slot_bytes;
+    // With two buffers a warp fetches the next stage's activations while others still compute.  Only tagged programs have
+    // no barrier there anyway, and the ring comes first.
+    const bool two = tagged && needs.pitch[1] > 0 && rest - x0 - x1 >= 3 * per_slot;
+    p->xbuf_bytes[0] = two ? x0 : (x0 > x1 ? x0 : x1);
+    p->xbuf_bytes[1] = two ? x1 : 0;
+    const int ring = rest - p->xbuf_bytes[0] - p->xbuf_bytes[1];
+    p->n_slots = ring / per_slot;
+    if (p->n_slots > kCellSlots) p->n_slots = kCellSlots;
+    return ring > 0 && p->n_slots >= 2;
+}
+
+// Most rows a launch of the program can take (at most 16); 0 if none.
+int widest_cell_panel(const CellNeeds& needs, bool tagged)
+{
+    CellPlan p;
+    for (int n = kPanelRows; n >= 1; --n)
+        if (plan_cells(n, needs, tagged, &p)) return n;
+    return 0;
+}
+
+template <int MAXS, int NR>
+sd2_status launch_cells(const CArgs<MAXS>& a, int grid, int smem, cudaStream_t s)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3(kCellThreads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = a.n_stages > 1 ? 1 : 0;
+    const cudaError_t e = a.fold_any ? cudaLaunchKernelEx(&cfg, cell_kernel<MAXS, NR, true>, a) : cudaLaunchKernelEx(&cfg, cell_kernel<MAXS, NR, false>, a);
+    if (e != cudaSuccess) { cudaGetLastError(); return SD2_ERR_CUDA; }
+    return SD2_OK;
+}
+
+void set_stage_grid(CStage& st, int grid)
+{
+    st.tiles_div = st.V / grid;
+    st.tiles_rem = st.V % grid;
+}
+
+// Stages of a program over cells while it is put together.
+struct CellBuilder {
+    CStage* stages;
+    CellNeeds needs;
+    int n = 0, grid, rot = 0;
+    CellBuilder(CStage* s, int g) : stages(s), grid(g) {}
+
+    // One stage of `count` handles of equal K.  pair: hs[0] and hs[1] are gate and up.
+    CStage& add(const sd2_handle* hs, int count, const uint16_t* x, void* const* Y, bool y_force_bf16, bool pair = false)
+    {
+        CStage& st = stages[n];
+        std::memset(&st, 0, sizeof st);
+        st.count = count;
+        st.K = (int)hs[0]->K;
+        st.D = hs[0]->cell_D;
+        st.x = x;
+        st.pair = pair ? 1 : 0;
+        for (int i = 0; i < count; ++i) {
+            CMat& m = st.mat[i];
+            m.off = (const uint32_t*)hs[i]->d_image;
+            m.cells = hs[i]->d_cells;
+            m.y = Y[i];
+            m.M = (int)hs[i]->M;
+            m.T = hs[i]->cell_T;
+            m.y_f32 = (!y_force_bf16 && hs[i]->y_dtype == SD2_DTYPE_F32) ? 1 : 0;
+            if (!pair || i == 0) st.V += m.T;
+            if (hs[i]->max_cell > needs.max_cell) needs.max_cell = hs[i]->max_cell;
+        }
+        const int pitch = 2 * st.D * kCellCols + 64, parts = st.D < kCellWarps ? st.D : kCellWarps;
+        if (pitch > needs.pitch[n & 1]) needs.pitch[n & 1] = pitch;
+        if (parts > needs.parts) needs.parts = parts;
+        if (st.V > needs.tiles_max) needs.tiles_max = st.V;
+        st.rot = rot;
+        rot = (int)(((int64_t)rot + st.V) % grid);
+        set_stage_grid(st, grid);
+        ++n;
+        return st;
+    }
+};
+
+// Launches a program over all N rows, in panels of equal size (rows are independent).
+sd2_status run_cell_panels(CArgs<kMaxStagesInline>& a, int64_t N, const CellNeeds& needs, int grid, cudaStream_t s)
+{
+    const int cap = widest_cell_panel(needs, a.tagged != 0);
+    if (cap == 0) return SD2_ERR_UNSUPPORTED;
+    const int64_t panels = (N + cap - 1) / cap;
+    const int64_t rows = (N + panels - 1) / panels;
+    CArgs<1> one;
+    if (a.n_stages == 1) {
+        one.inl[0] = a.inl[0];
+        one.fold[0] = a.fold[0];
+    }
+    for (int64_t n0 = 0; n0 < N; n0 += rows) {
+        a.N = (int)((N - n0) < rows ? (N - n0) : rows);
+        a.n0 = (int)n0;
+        CellPlan p;
+        if (!plan_cells(a.N, needs, a.tagged != 0, &p)) return SD2_ERR_UNSUPPORTED;
+        a.part_bytes = p.part_bytes;
+        a.xbuf_bytes[0] = p.xbuf_bytes[0];
+        a.xbuf_bytes[1] = p.xbuf_bytes[1];
+        a.slot_bytes = p.slot_bytes;
+        a.n_slots = p.n_slots;
+        const int smem = kCellFixedBytes + kPartSlots * p.part_bytes + p.xbuf_bytes[0] + p.xbuf_bytes[1] + kCellWarps * p.n_slots * p.slot_bytes;
+        sd2_status st;
+        if (a.n_stages == 1) {
+            static_cast<CArgsBase&>(one) = a;
+            st = a.N > 8 ? launch_cells<1, 16>(one, grid, smem, s) : launch_cells<1, 8>(one, grid, smem, s);
+        } else {
+            st = a.N > 8 ? launch_cells<kMaxStagesInline, 16>(a, grid, smem, s) : launch_cells<kMaxStagesInline, 8>(a, grid, smem, s);
+        }
+        if (st != SD2_OK) return st;
+    }
+    return SD2_OK;
+}
+
+// Runs a program of inline stages.
+sd2_status run_cell_program(CArgs<kMaxStagesInline>& a, const CellBuilder& b, int dev, int64_t N, cudaStream_t s)
+{
+    a.n_stages = b.n;
+    const bool coop = a.n_stages > 1;
+    int grid = g_dev[dev].sms;
+    if (!coop && b.needs.tiles_max < grid) {
+        grid = b.needs.tiles_max;
+        set_stage_grid(a.inl[0], grid);
+    }
+    a.err = g_dev[dev].err_word;
+    a.wait_cycles = wait_budget(dev);
+    if (!a.gbar && coop) a.gbar = g_dev[dev].barriers + (size_t)(g_next_barrier.fetch_add(1) % kBarrierPool) * kBarrierStrideWords;
+    return run_cell_panels(a, N, b.needs, grid, s);
+}
+
+// Whether a call of N rows over these GAP4 handles takes their cells.
+#ifndef SD2_CELLS_MIN
+#define SD2_CELLS_MIN 4
+#endif
+bool use_cells(const sd2_handle* hs, int count, int64_t N)
+{
+    if (N < SD2_CELLS_MIN) return false;
+    CellNeeds needs;
+    for (int i = 0; i < count; ++i) {
+        if (!hs[i]->d_image) return false;
+        const int pitch = 2 * hs[i]->cell_D * kCellCols + 64;
+        if (pitch > needs.pitch[0]) needs.pitch[0] = pitch;
+        if (hs[i]->max_cell > needs.max_cell) needs.max_cell = hs[i]->max_cell;
+    }
+    needs.parts = kCellWarps;
+    return widest_cell_panel(needs, false) > 0;
+}
+
 // Shared by sd2_spmm and sd2_spmm_fused (and by block steps that mix formats).
 // cuTensorMapEncodeTiled through the runtime (no link against the driver library).  NULL: not available.
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -651,6 +883,15 @@ sd2_status run_group(const sd2_handle* hs, int count, const uint16_t* x, const u
             if (si != SD2_OK) return si;
         }
         return SD2_OK;
+    }
+    if (use_cells(hs, count, N)) {
+        CArgs<kMaxStagesInline> a = {};
+        CellBuilder b(a.inl, g_dev[dev].sms);
+        CStage& sg = b.add(hs, count, x, Y, y_force_bf16);
+        sg.g = g;
+        sg.u = u;
+        sg.t_out = t_out;
+        return run_cell_program(a, b, dev, N, s);
     }
     SArgs a;
     std::memset(&a, 0, sizeof a);
@@ -787,6 +1028,36 @@ int append_block_stages(SStage* stages, const sd2_handle* h, const uint16_t* x, 
     return n;   // at most 7
 }
 
+// Tagged 32-bit copies (value << 16 | tag) of a block's activations in a program over cells.
+struct CellTags {
+    const uint32_t* x_t;                  // the block's input as tagged words, or NULL (plain bf16 input)
+    uint32_t *q_t, *hdn_t, *t_t, *out_t;  // out_t NULL: the block's output is not handed on
+};
+
+// Appends the four stages of one block (h[0..6] = q,k,v,o,gate,up,down) to a program over cells.  t = silu(g) * u is
+// formed where g and u are produced.
+void append_block_cells(CellBuilder& b, const sd2_handle* h, const uint16_t* x, uint16_t* q, uint16_t* k, uint16_t* v, uint16_t* hdn,
+                        uint16_t* g, uint16_t* u, uint16_t* t, void* y, bool y_force_bf16, const CellTags* tg = nullptr)
+{
+    void* y_qkv[3] = {q, k, v};
+    void* y_o[1] = {hdn};
+    void* y_gu[2] = {g, u};
+    void* y_d[1] = {y};
+    CStage& s0 = b.add(h + 0, 3, tg && tg->x_t ? (const uint16_t*)tg->x_t : x, y_qkv, true);
+    CStage& s1 = b.add(h + 3, 1, tg ? (const uint16_t*)tg->q_t : q, y_o, true);
+    CStage& s2 = b.add(h + 4, 2, tg ? (const uint16_t*)tg->hdn_t : hdn, y_gu, true, true);
+    CStage& s3 = b.add(h + 6, 1, tg ? (const uint16_t*)tg->t_t : t, y_d, y_force_bf16);
+    s2.t_out = t;
+    if (tg) {
+        s0.tagged_in = tg->x_t ? 1 : 0;
+        s0.mat[0].yt = tg->q_t;
+        s1.tagged_in = s2.tagged_in = s3.tagged_in = 1;
+        s1.mat[0].yt = tg->hdn_t;
+        s2.tt = tg->t_t;
+        s3.mat[0].yt = tg->out_t;
+    }
+}
+
 // Builds the paired stack of a block's gate and up (row 2i = gate row i, row 2i+1 = up row i)
 // from the decoded contents of the two handles.  *out stays NULL where the shape has no paired
 // form (fewer than two rows per tile); the caller then keeps the two weights apart.
@@ -907,13 +1178,17 @@ sd2_status sd2_compress(const void* weight_bf16, const uint8_t* mask, int64_t M,
     uint8_t* blob = nullptr;
     int64_t bytes = 0;
     if (st == SD2_OK) st = pack_any(W, mask, M, K, opt, &blob, &bytes);
+    if (st == SD2_OK) {
+        BlobHeader hd;
+        std::memcpy(&hd, blob, sizeof hd);
+        sd2_handle h = nullptr;
+        st = upload(blob, bytes, hd, &h);
+        std::free(blob);
+        if (st == SD2_OK && h->format == SD2_FORMAT_GAP4) st = add_cells(h, W, mask);
+        if (st == SD2_OK) *out = h;
+    }
     std::free(w_tmp);
     std::free(m_tmp);
-    if (st != SD2_OK) return st;
-    BlobHeader hd;
-    std::memcpy(&hd, blob, sizeof hd);
-    st = upload(blob, bytes, hd, out);
-    std::free(blob);
     return st;
 }
 
@@ -923,14 +1198,22 @@ sd2_status sd2_load_blob(const void* blob, int64_t blob_bytes, sd2_handle* out)
     BlobHeader hd;
     if (check_header((const uint8_t*)blob, blob_bytes, hd, true) != 0) return SD2_ERR_CORRUPT;
     // full structural validation before anything reaches a kernel
+    uint16_t* dense = nullptr;
+    if (hd.format == (uint32_t)kFormatGap4 && !(dense = (uint16_t*)lib_malloc((size_t)(hd.M * hd.K) * 2))) return SD2_ERR_ALLOC;
     int rc;
     try {
-        rc = unpack_any(hd, (const uint8_t*)blob, nullptr);
+        rc = unpack_any(hd, (const uint8_t*)blob, dense);
     } catch (const std::bad_alloc&) {
+        std::free(dense);
         return SD2_ERR_ALLOC;
     }
-    if (rc != 0) return SD2_ERR_CORRUPT;
-    return upload((const uint8_t*)blob, blob_bytes, hd, out);
+    sd2_handle h = nullptr;
+    sd2_status st = rc != 0 ? SD2_ERR_CORRUPT : upload((const uint8_t*)blob, blob_bytes, hd, &h);
+    // for the cells what decoded to +0 or -0 was masked out, or was a kept zero, which adds nothing
+    if (st == SD2_OK && dense) st = add_cells(h, dense, nullptr);
+    std::free(dense);
+    if (st == SD2_OK) *out = h;
+    return st;
 }
 
 sd2_status sd2_decompress(sd2_handle h, void* dense_bf16_out)
@@ -972,6 +1255,7 @@ sd2_status sd2_free(sd2_handle h)
     }
     sd2_status st = SD2_OK;
     if (cudaFree(h->d_blob) != cudaSuccess) { cudaGetLastError(); st = SD2_ERR_CUDA; }
+    if (h->d_image && cudaFree(h->d_image) != cudaSuccess) { cudaGetLastError(); st = SD2_ERR_CUDA; }
     if (h->d_partial && cudaFree(h->d_partial) != cudaSuccess) { cudaGetLastError(); st = SD2_ERR_CUDA; }
     delete h;
     return st;
@@ -996,6 +1280,8 @@ sd2_status sd2_stream_check(void* cuda_stream)
                 if (d->device == dev) {   // barrier words, production counts and every tagged word start over
                     cudaMemset(d->d_gbar, 0, kDrafterWordsBytes);
                     if (d->d_tags) cudaMemset(d->d_tags, 0, (size_t)d->tags_bytes);
+                    if (d->d_cbar) cudaMemset(d->d_cbar, 0, kDrafterWordsBytes);
+                    if (d->d_ctags) cudaMemset(d->d_ctags, 0, (size_t)d->ctags_bytes);
                 }
             for (sd2_handle h : g_live)
                 if (h->device == dev && h->d_partial) cudaMemset(h->d_partial, 0, (size_t)h->partial_bytes);
@@ -1204,6 +1490,40 @@ sd2_status sd2_decoder_block_step(const sd2_handle* h, const void* norm_attn, co
         for (int i = 0; i < 7; ++i)
             if (h[i]->device != dev) return SD2_ERR_INVALID_ARG;
         const int grid = g_dev[dev].sms;
+        if (use_cells(h, 7, N)) {
+            {
+                CArgs<kMaxStagesInline> a = {};
+                CellBuilder b(a.inl, grid);
+                void* yqkv[3] = {q, k, v};
+                b.add(h, 3, (const uint16_t*)x, yqkv, true);
+                a.fold[0].norm_w = (const uint16_t*)norm_attn;
+                a.fold[0].eps = eps;
+                a.fold_any = 1;
+                Range r_("q|k|v");
+                if ((st = run_cell_program(a, b, dev, N, s)) != SD2_OK) return st;
+            }
+            if ((st = sd2_rope_attention(q, k, v, k_cache, v_cache, att, N, heads_q, heads_kv, hd, pos, T_max, theta, s)) != SD2_OK) return st;
+            {
+                CArgs<kMaxStagesInline> a = {};
+                CellBuilder b(a.inl, grid);
+                void* yo[1] = {hdn};
+                void* ygu[2] = {g, u};
+                void* yd[1] = {dn};
+                b.add(h + 3, 1, att, yo, true);
+                SFold& f = a.fold[b.n];
+                f.res = (const uint16_t*)x;
+                f.norm_w = (const uint16_t*)norm_ffn;
+                f.eps = eps;
+                f.sum_out = x1;
+                f.norm_out = xn;
+                a.fold_any = 1;
+                b.add(h + 4, 2, hdn, ygu, true, true).t_out = t;
+                b.add(h + 6, 1, t, yd, true);
+                Range r_("o, gate|up, down");
+                if ((st = run_cell_program(a, b, dev, N, s)) != SD2_OK) return st;
+            }
+            return sd2_add(x1, dn, y, N * d.hidden, s);
+        }
         {
             SArgs a;
             std::memset(&a, 0, sizeof a);
@@ -1364,6 +1684,12 @@ sd2_status sd2_block_step(const sd2_handle* h, const void* x, void* y, int64_t N
         if (st != SD2_OK) return st;
         for (int i = 0; i < 7; ++i)
             if (h[i]->device != dev) return SD2_ERR_INVALID_ARG;
+        if (use_cells(h, 7, N)) {
+            CArgs<kMaxStagesInline> a = {};
+            CellBuilder b(a.inl, g_dev[dev].sms);
+            append_block_cells(b, h, (const uint16_t*)x, q, k, v, hdn, g, u, t, y, false);
+            return run_cell_program(a, b, dev, N, s);
+        }
         SArgs a;
         std::memset(&a, 0, sizeof a);
         ProgramNeeds needs;
@@ -1428,6 +1754,14 @@ sd2_status sd2_block_step_static(const sd2_handle* h, const void* x, void* y, in
     // the barrier words must start at zero whatever the last call left behind
     if (cudaMemsetAsync(base, 0, 256, s) != cudaSuccess) { cudaGetLastError(); return SD2_ERR_CUDA; }
     char* ws = (char*)base + 256;
+    if (use_cells(h, 7, N)) {
+        CArgs<kMaxStagesInline> a = {};
+        CellBuilder b(a.inl, g_dev[dev].sms);
+        append_block_cells(b, h, (const uint16_t*)x, (uint16_t*)(ws + off[0]), (uint16_t*)(ws + off[1]), (uint16_t*)(ws + off[2]),
+                           (uint16_t*)(ws + off[3]), (uint16_t*)(ws + off[4]), (uint16_t*)(ws + off[5]), (uint16_t*)(ws + off[6]), y, false);
+        a.gbar = (unsigned int*)base;
+        return run_cell_program(a, b, dev, N, s);
+    }
     SArgs a;
     std::memset(&a, 0, sizeof a);
     ProgramNeeds needs;
@@ -1472,6 +1806,11 @@ sd2_status sd2_drafter_create(const sd2_handle* h, int32_t L, int64_t n_max, sd2
     d->d_ws = nullptr;
     d->d_stages = nullptr;
     d->d_gbar = nullptr;
+    d->d_cstages = nullptr;
+    d->d_cbar = nullptr;
+    d->d_ctags = nullptr;
+    d->ctags_bytes = 0;
+    d->n_cstages = 0;
     // workspace: per block q,k,v,hdn,g,u,t and the block's bf16 output (the next block's input)
     d->ws_off.assign((size_t)L * 8 + 1, 0);
     int64_t o = 0;
@@ -1547,17 +1886,59 @@ sd2_status sd2_drafter_create(const sd2_handle* h, int32_t L, int64_t n_max, sd2
              cudaMemcpy(d->d_stages, stages.data(), sizeof(SStage) * (size_t)n, cudaMemcpyHostToDevice) == cudaSuccess &&
              dev_malloc((void**)&d->d_gbar, kDrafterWordsBytes) == cudaSuccess && cudaMemset(d->d_gbar, 0, kDrafterWordsBytes) == cudaSuccess;
     }
-    if (ok && widest_panel(needs.xs_need, needs.K_max, needs.max_tile) == 0) {
+    bool cells = tagged;
+    for (const sd2_handle hh : d->handles)
+        if (!hh->d_image) cells = false;
+    if (ok && cells && n_max >= SD2_CELLS_MIN) {
+        // the same blocks over cells, for steps of several rows
+        std::vector<CStage> cstages((size_t)L * 4);
+        std::vector<int64_t> ct((size_t)L * 4 + 1, 0);
+        int64_t to = 0;
+        for (int b = 0; b < L; ++b) {
+            const BlockDims& bd = dims[(size_t)b];
+            const int64_t w[4] = {bd.q_out, h[7 * b + 3]->M, bd.inter, bd.out};
+            for (int i = 0; i < 4; ++i) {
+                ct[(size_t)b * 4 + i] = to;
+                to = a256(to + 4 * n_max * w[i]);
+            }
+        }
+        d->ctags_bytes = to;
+        ok = dev_malloc((void**)&d->d_ctags, (size_t)to) == cudaSuccess && cudaMemset(d->d_ctags, 0, (size_t)to) == cudaSuccess;
+        CellBuilder bld(cstages.data(), g_dev[dev].sms);
+        for (int b = 0; b < L && ok; ++b) {
+            uint8_t *base = d->d_ws, *tb = (uint8_t*)d->d_ctags;
+            const int64_t* wo = &d->ws_off[(size_t)b * 8];
+            const int64_t* tw = &ct[(size_t)b * 4];
+            CellTags tg;
+            tg.x_t = b == 0 ? nullptr : (const uint32_t*)(tb + ct[(size_t)(b - 1) * 4 + 3]);
+            tg.q_t = (uint32_t*)(tb + tw[0]);
+            tg.hdn_t = (uint32_t*)(tb + tw[1]);
+            tg.t_t = (uint32_t*)(tb + tw[2]);
+            tg.out_t = b + 1 < L ? (uint32_t*)(tb + tw[3]) : nullptr;
+            append_block_cells(bld, h + 7 * b, nullptr, (uint16_t*)(base + wo[0]), (uint16_t*)(base + wo[1]), (uint16_t*)(base + wo[2]),
+                               (uint16_t*)(base + wo[3]), (uint16_t*)(base + wo[4]), (uint16_t*)(base + wo[5]), (uint16_t*)(base + wo[6]),
+                               base + wo[7], b + 1 < L, &tg);
+        }
+        d->n_cstages = bld.n;
+        d->cell_needs = bld.needs;
+        ok = ok && dev_malloc((void**)&d->d_cstages, sizeof(CStage) * (size_t)bld.n) == cudaSuccess &&
+             cudaMemcpy(d->d_cstages, cstages.data(), sizeof(CStage) * (size_t)bld.n, cudaMemcpyHostToDevice) == cudaSuccess &&
+             dev_malloc((void**)&d->d_cbar, kDrafterWordsBytes) == cudaSuccess && cudaMemset(d->d_cbar, 0, kDrafterWordsBytes) == cudaSuccess;
+    }
+    auto drop = [&]() {
+        cudaGetLastError();
         for (sd2_handle p : d->owned) sd2_free(p);
         cudaFree(d->d_ws); cudaFree(d->d_stages); cudaFree(d->d_gbar); cudaFree(d->d_tags);
+        cudaFree(d->d_cstages); cudaFree(d->d_cbar); cudaFree(d->d_ctags);
+        cudaGetLastError();
+    };
+    if (ok && widest_panel(needs.xs_need, needs.K_max, needs.max_tile) == 0) {
+        drop();
         delete d;
         return SD2_ERR_UNSUPPORTED;
     }
     if (!ok) {
-        cudaGetLastError();
-        for (sd2_handle p : d->owned) sd2_free(p);
-        cudaFree(d->d_ws); cudaFree(d->d_stages); cudaFree(d->d_gbar); cudaFree(d->d_tags);
-        cudaGetLastError();
+        drop();
         delete d;
         return SD2_ERR_ALLOC;
     }
@@ -1573,6 +1954,13 @@ sd2_status sd2_drafter_create(const sd2_handle* h, int32_t L, int64_t n_max, sd2
     return SD2_OK;
 }
 
+namespace {
+bool drafter_uses_cells(sd2_drafter d, int64_t N)
+{
+    return N >= SD2_CELLS_MIN && d->d_cstages && widest_cell_panel(d->cell_needs, true) > 0;
+}
+}  // namespace
+
 sd2_status sd2_drafter_step(sd2_drafter d, const void* x, void* y, int64_t N, void* cuda_stream)
 {
     Range range_("sd2_drafter_step");
@@ -1583,6 +1971,19 @@ sd2_status sd2_drafter_step(sd2_drafter d, const void* x, void* y, int64_t N, vo
     sd2_status st = ensure_device(&dev);
     if (st != SD2_OK) return st;
     if (dev != d->device) return SD2_ERR_INVALID_ARG;
+    if (drafter_uses_cells(d, N)) {
+        CArgs<kMaxStagesInline> c = {};
+        c.ext = d->d_cstages;
+        c.n_stages = d->n_cstages;
+        c.x_in = (const uint16_t*)x;
+        c.y_out = y;
+        c.gbar = d->d_cbar;
+        c.err = g_dev[dev].err_word;
+        c.wait_cycles = wait_budget(dev);
+        c.tagged = 1;
+        c.rowseq = d->d_cbar + 64;
+        return run_cell_panels(c, N, d->cell_needs, g_dev[dev].sms, (cudaStream_t)cuda_stream);
+    }
     SArgs a;
     std::memset(&a, 0, sizeof a);
     a.ext = d->d_stages;
@@ -1610,13 +2011,15 @@ sd2_status sd2_drafter_query(sd2_drafter d, int64_t N, int64_t* out)
 {
     if (!live(d) || !out) return SD2_ERR_INVALID_ARG;
     if (N < 1 || N > d->n_max) return SD2_ERR_SHAPE;
-    const int cap = widest_panel(d->xs_need, d->K_max, d->max_tile);
+    const bool cells = drafter_uses_cells(d, N);
+    const int cap = cells ? widest_cell_panel(d->cell_needs, true) : widest_panel(d->xs_need, d->K_max, d->max_tile);
     if (cap == 0) return SD2_ERR_UNSUPPORTED;
     int64_t streamed = 0, owned = 0, kept = 0;
     // what a step streams: every handle once, except that a block's gate and up are read from the
     // drafter's own paired stack where it has one
     std::vector<char> paired((size_t)d->L, 0);
     for (sd2_handle p : d->owned) { streamed += p->compressed_bytes; owned += p->blob_bytes; }
+    owned += d->ctags_bytes + (int64_t)sizeof(CStage) * d->n_cstages + (d->d_cbar ? kDrafterWordsBytes : 0);
     size_t oi = 0;
     for (int b = 0; b < d->L; ++b) {
         // (owned stacks were built in block order, one per block that could be paired)
@@ -1628,6 +2031,10 @@ sd2_status sd2_drafter_query(sd2_drafter d, int64_t N, int64_t* out)
             kept += h->nnz;
             if (!(has_pair && (i == 4 || i == 5))) streamed += h->compressed_bytes;
         }
+    }
+    if (cells) {
+        streamed = 0;
+        for (const sd2_handle h : d->handles) streamed += h->cell_bytes;
     }
     out[0] = (N + cap - 1) / cap;                                  // launches per step of N rows
     out[1] = cap;                                                  // rows of the widest panel
@@ -1658,6 +2065,9 @@ sd2_status sd2_drafter_free(sd2_drafter d)
     if (cudaFree(d->d_stages) != cudaSuccess) st = SD2_ERR_CUDA;
     if (cudaFree(d->d_gbar) != cudaSuccess) st = SD2_ERR_CUDA;
     if (d->d_tags && cudaFree(d->d_tags) != cudaSuccess) st = SD2_ERR_CUDA;
+    if (d->d_cstages && cudaFree(d->d_cstages) != cudaSuccess) st = SD2_ERR_CUDA;
+    if (d->d_cbar && cudaFree(d->d_cbar) != cudaSuccess) st = SD2_ERR_CUDA;
+    if (d->d_ctags && cudaFree(d->d_ctags) != cudaSuccess) st = SD2_ERR_CUDA;
     for (sd2_handle p : d->owned)
         if (sd2_free(p) != SD2_OK) st = SD2_ERR_CUDA;
     cudaGetLastError();
