@@ -38,7 +38,7 @@ struct sd2_handle_s {
     uint8_t* d_image;
     const unsigned char* d_cells;
     int64_t image_bytes, cell_bytes;   // device bytes; what a launch reads of them
-    int cell_T, cell_D, max_cell;
+    int cell_T, cell_D, max_chunk;
     // GAP4_MMA: fp32 partial sums [64][rows padded to 128] followed by one arrival count per row panel,
     // all zero between launches (the CTA that completes a panel writes Y and clears them)
     float* d_partial;
@@ -47,9 +47,9 @@ struct sd2_handle_s {
 
 // What a program over cells needs from shared memory.
 struct CellNeeds {
-    int pitch[2] = {0, 0};     // bytes of a staged activation row, by parity of the stage: the largest
-    int max_cell = 0;
-    int parts = 0;             // most contributions to a tile
+    int pitch = 0;             // bytes of a staged activation row: the largest
+    int max_chunk = 0;
+    int parts = 0;             // most contributions of a CTA to a tile
     int tiles_max = 0;         // most tiles of any stage
 };
 
@@ -71,12 +71,9 @@ struct sd2_drafter_s {
     int K_max, max_tile;       // what decides the shared-memory split
     int free_tiles;            // every stage has enough tiles per CTA for free tile assignment
     int xs_need[4];            // bytes of staged activations at panel widths 1, 2, 4, 8
-    // the same blocks as a program over cells, with barrier words, production counts and tagged words of its own
-    // (a word of either program must never show a tag of the other); NULL: a handle has no cells
+    // the same blocks as a program over cells, with barrier words of its own; NULL: a handle has no cells
     CStage* d_cstages;
     unsigned int* d_cbar;
-    uint32_t* d_ctags;
-    int64_t ctags_bytes;
     int n_cstages;
     CellNeeds cell_needs;
 };
@@ -320,7 +317,7 @@ sd2_status add_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask)
     h->cell_bytes = (g.T * g.D + 1) * 4 + (int64_t)(im.bytes - im.sec1_off);
     h->cell_T = (int)g.T;
     h->cell_D = g.D;
-    h->max_cell = im.max_cell;
+    h->max_chunk = im.max_chunk;
     return SD2_OK;
 }
 
@@ -589,38 +586,36 @@ sd2_status run_program(SArgs& a, int dev, int64_t N, const ProgramNeeds& needs, 
 // ------------------------------------------------------------------ programs over cells
 
 struct CellPlan {
-    int part_bytes, xbuf_bytes[2], slot_bytes, n_slots;
+    int part_bytes, n_parts, xbuf_bytes, chunk_bytes, n_slots;
 };
 
 constexpr int kCellFixedBytes = (int)((sizeof(CellShared) + 127) & ~127) + kRingGuardBytes;
 
-// Shared memory of a launch of n rows.  false: not even two cells per warp fit beside the staged rows.
-bool plan_cells(int n, const CellNeeds& needs, bool tagged, CellPlan* p)
+// Shared memory of a launch of n rows.  false: not even two chunks per group fit beside the staged rows.
+bool plan_cells(int n, const CellNeeds& needs, CellPlan* p)
 {
     p->part_bytes = (needs.parts * n * 32 + 127) & ~127;
-    p->slot_bytes = (needs.max_cell + 31) & ~31;
-    const int x0 = (n * needs.pitch[0] + 127) & ~127, x1 = (n * needs.pitch[1] + 127) & ~127;
-    const int rest = kSmemMax - kCellFixedBytes - kPartSlots * p->part_bytes;
-    const int per_slot = kCellWarps * p->slot_bytes;
-    // With two buffers a warp fetches the next stage's activations while others still compute.  Only tagged programs have
-    // no barrier there anyway, and the ring comes first.
-    const bool two = tagged && needs.pitch[1] > 0 && rest - x0 - x1 >= 3 * per_slot;
-    p->xbuf_bytes[0] = two ? x0 : (x0 > x1 ? x0 : x1);
-    p->xbuf_bytes[1] = two ? x1 : 0;
-    const int ring = rest - p->xbuf_bytes[0] - p->xbuf_bytes[1];
-    p->n_slots = ring / per_slot;
-    if (p->n_slots > kCellSlots) p->n_slots = kCellSlots;
-    return ring > 0 && p->n_slots >= 2;
+    p->chunk_bytes = (needs.max_chunk + 127) & ~127;
+    p->xbuf_bytes = (n * needs.pitch + 127) & ~127;
+    for (p->n_parts = kPartSlots; p->n_parts >= 2; p->n_parts >>= 1) {
+        const int ring = kSmemMax - kCellFixedBytes - p->n_parts * p->part_bytes - p->xbuf_bytes;
+        p->n_slots = ring > 0 ? ring / (kCellGroups * p->chunk_bytes) : 0;
+        if (p->n_slots > kGroupSlots) p->n_slots = kGroupSlots;
+        if (p->n_slots >= 2) return true;
+    }
+    return false;
 }
 
 // Most rows a launch of the program can take (at most 16); 0 if none.
-int widest_cell_panel(const CellNeeds& needs, bool tagged)
+int widest_cell_panel(const CellNeeds& needs)
 {
     CellPlan p;
     for (int n = kPanelRows; n >= 1; --n)
-        if (plan_cells(n, needs, tagged, &p)) return n;
+        if (plan_cells(n, needs, &p)) return n;
     return 0;
 }
+
+int cell_pitch(int D) { return 2 * share_cells(D, 0) * kCellCols + 64; }
 
 template <int MAXS, int NR>
 sd2_status launch_cells(const CArgs<MAXS>& a, int grid, int smem, cudaStream_t s)
@@ -630,28 +625,31 @@ sd2_status launch_cells(const CArgs<MAXS>& a, int grid, int smem, cudaStream_t s
     cfg.blockDim = dim3(kCellThreads);
     cfg.dynamicSmemBytes = (size_t)smem;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeCooperative;
+    attr[1].val.cooperative = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = a.n_stages > 1 ? 1 : 0;
+    cfg.numAttrs = a.n_stages > 1 ? 2 : 1;
     const cudaError_t e = a.fold_any ? cudaLaunchKernelEx(&cfg, cell_kernel<MAXS, NR, true>, a) : cudaLaunchKernelEx(&cfg, cell_kernel<MAXS, NR, false>, a);
     if (e != cudaSuccess) { cudaGetLastError(); return SD2_ERR_CUDA; }
     return SD2_OK;
 }
 
-void set_stage_grid(CStage& st, int grid)
+void set_stage_clusters(CStage& st, int clusters)
 {
-    st.tiles_div = st.V / grid;
-    st.tiles_rem = st.V % grid;
+    st.tiles_div = st.V / clusters;
+    st.tiles_rem = st.V % clusters;
 }
 
 // Stages of a program over cells while it is put together.
 struct CellBuilder {
     CStage* stages;
     CellNeeds needs;
-    int n = 0, grid, rot = 0;
-    CellBuilder(CStage* s, int g) : stages(s), grid(g) {}
+    int n = 0, clusters, rot = 0;
+    CellBuilder(CStage* s, int sms) : stages(s), clusters(sms / 2) {}
 
     // One stage of `count` handles of equal K.  pair: hs[0] and hs[1] are gate and up.
     CStage& add(const sd2_handle* hs, int count, const uint16_t* x, void* const* Y, bool y_force_bf16, bool pair = false)
@@ -672,15 +670,15 @@ struct CellBuilder {
             m.T = hs[i]->cell_T;
             m.y_f32 = (!y_force_bf16 && hs[i]->y_dtype == SD2_DTYPE_F32) ? 1 : 0;
             if (!pair || i == 0) st.V += m.T;
-            if (hs[i]->max_cell > needs.max_cell) needs.max_cell = hs[i]->max_cell;
+            if (hs[i]->max_chunk > needs.max_chunk) needs.max_chunk = hs[i]->max_chunk;
         }
-        const int pitch = 2 * st.D * kCellCols + 64, parts = st.D < kCellWarps ? st.D : kCellWarps;
-        if (pitch > needs.pitch[n & 1]) needs.pitch[n & 1] = pitch;
+        const int pitch = cell_pitch(st.D), share = share_cells(st.D, 0), parts = share < kCellWarps ? share : kCellWarps;
+        if (pitch > needs.pitch) needs.pitch = pitch;
         if (parts > needs.parts) needs.parts = parts;
         if (st.V > needs.tiles_max) needs.tiles_max = st.V;
         st.rot = rot;
-        rot = (int)(((int64_t)rot + st.V) % grid);
-        set_stage_grid(st, grid);
+        rot = (int)(((int64_t)rot + st.V) % clusters);
+        set_stage_clusters(st, clusters);
         ++n;
         return st;
     }
@@ -689,7 +687,7 @@ struct CellBuilder {
 // Launches a program over all N rows, in panels of equal size (rows are independent).
 sd2_status run_cell_panels(CArgs<kMaxStagesInline>& a, int64_t N, const CellNeeds& needs, int grid, cudaStream_t s)
 {
-    const int cap = widest_cell_panel(needs, a.tagged != 0);
+    const int cap = widest_cell_panel(needs);
     if (cap == 0) return SD2_ERR_UNSUPPORTED;
     const int64_t panels = (N + cap - 1) / cap;
     const int64_t rows = (N + panels - 1) / panels;
@@ -702,13 +700,13 @@ sd2_status run_cell_panels(CArgs<kMaxStagesInline>& a, int64_t N, const CellNeed
         a.N = (int)((N - n0) < rows ? (N - n0) : rows);
         a.n0 = (int)n0;
         CellPlan p;
-        if (!plan_cells(a.N, needs, a.tagged != 0, &p)) return SD2_ERR_UNSUPPORTED;
+        if (!plan_cells(a.N, needs, &p)) return SD2_ERR_UNSUPPORTED;
         a.part_bytes = p.part_bytes;
-        a.xbuf_bytes[0] = p.xbuf_bytes[0];
-        a.xbuf_bytes[1] = p.xbuf_bytes[1];
-        a.slot_bytes = p.slot_bytes;
+        a.part_mask = p.n_parts - 1;
+        a.xbuf_bytes = p.xbuf_bytes;
+        a.chunk_bytes = p.chunk_bytes;
         a.n_slots = p.n_slots;
-        const int smem = kCellFixedBytes + kPartSlots * p.part_bytes + p.xbuf_bytes[0] + p.xbuf_bytes[1] + kCellWarps * p.n_slots * p.slot_bytes;
+        const int smem = kCellFixedBytes + p.n_parts * p.part_bytes + p.xbuf_bytes + kCellGroups * p.n_slots * p.chunk_bytes;
         sd2_status st;
         if (a.n_stages == 1) {
             static_cast<CArgsBase&>(one) = a;
@@ -726,11 +724,12 @@ sd2_status run_cell_program(CArgs<kMaxStagesInline>& a, const CellBuilder& b, in
 {
     a.n_stages = b.n;
     const bool coop = a.n_stages > 1;
-    int grid = g_dev[dev].sms;
-    if (!coop && b.needs.tiles_max < grid) {
-        grid = b.needs.tiles_max;
-        set_stage_grid(a.inl[0], grid);
+    int clusters = b.clusters;
+    if (!coop && b.needs.tiles_max < clusters) {
+        clusters = b.needs.tiles_max;
+        set_stage_clusters(a.inl[0], clusters);
     }
+    const int grid = 2 * clusters;
     a.err = g_dev[dev].err_word;
     a.wait_cycles = wait_budget(dev);
     if (!a.gbar && coop) a.gbar = g_dev[dev].barriers + (size_t)(g_next_barrier.fetch_add(1) % kBarrierPool) * kBarrierStrideWords;
@@ -747,12 +746,12 @@ bool use_cells(const sd2_handle* hs, int count, int64_t N)
     CellNeeds needs;
     for (int i = 0; i < count; ++i) {
         if (!hs[i]->d_image) return false;
-        const int pitch = 2 * hs[i]->cell_D * kCellCols + 64;
-        if (pitch > needs.pitch[0]) needs.pitch[0] = pitch;
-        if (hs[i]->max_cell > needs.max_cell) needs.max_cell = hs[i]->max_cell;
+        const int pitch = cell_pitch(hs[i]->cell_D);
+        if (pitch > needs.pitch) needs.pitch = pitch;
+        if (hs[i]->max_chunk > needs.max_chunk) needs.max_chunk = hs[i]->max_chunk;
     }
     needs.parts = kCellWarps;
-    return widest_cell_panel(needs, false) > 0;
+    return widest_cell_panel(needs) > 0;
 }
 
 // Shared by sd2_spmm and sd2_spmm_fused (and by block steps that mix formats).
@@ -1028,34 +1027,19 @@ int append_block_stages(SStage* stages, const sd2_handle* h, const uint16_t* x, 
     return n;   // at most 7
 }
 
-// Tagged 32-bit copies (value << 16 | tag) of a block's activations in a program over cells.
-struct CellTags {
-    const uint32_t* x_t;                  // the block's input as tagged words, or NULL (plain bf16 input)
-    uint32_t *q_t, *hdn_t, *t_t, *out_t;  // out_t NULL: the block's output is not handed on
-};
-
 // Appends the four stages of one block (h[0..6] = q,k,v,o,gate,up,down) to a program over cells.  t = silu(g) * u is
 // formed where g and u are produced.
 void append_block_cells(CellBuilder& b, const sd2_handle* h, const uint16_t* x, uint16_t* q, uint16_t* k, uint16_t* v, uint16_t* hdn,
-                        uint16_t* g, uint16_t* u, uint16_t* t, void* y, bool y_force_bf16, const CellTags* tg = nullptr)
+                        uint16_t* g, uint16_t* u, uint16_t* t, void* y, bool y_force_bf16)
 {
     void* y_qkv[3] = {q, k, v};
     void* y_o[1] = {hdn};
     void* y_gu[2] = {g, u};
     void* y_d[1] = {y};
-    CStage& s0 = b.add(h + 0, 3, tg && tg->x_t ? (const uint16_t*)tg->x_t : x, y_qkv, true);
-    CStage& s1 = b.add(h + 3, 1, tg ? (const uint16_t*)tg->q_t : q, y_o, true);
-    CStage& s2 = b.add(h + 4, 2, tg ? (const uint16_t*)tg->hdn_t : hdn, y_gu, true, true);
-    CStage& s3 = b.add(h + 6, 1, tg ? (const uint16_t*)tg->t_t : t, y_d, y_force_bf16);
-    s2.t_out = t;
-    if (tg) {
-        s0.tagged_in = tg->x_t ? 1 : 0;
-        s0.mat[0].yt = tg->q_t;
-        s1.tagged_in = s2.tagged_in = s3.tagged_in = 1;
-        s1.mat[0].yt = tg->hdn_t;
-        s2.tt = tg->t_t;
-        s3.mat[0].yt = tg->out_t;
-    }
+    b.add(h + 0, 3, x, y_qkv, true);
+    b.add(h + 3, 1, q, y_o, true);
+    b.add(h + 4, 2, hdn, y_gu, true, true).t_out = t;
+    b.add(h + 6, 1, t, y_d, y_force_bf16);
 }
 
 // Builds the paired stack of a block's gate and up (row 2i = gate row i, row 2i+1 = up row i)
@@ -1281,7 +1265,6 @@ sd2_status sd2_stream_check(void* cuda_stream)
                     cudaMemset(d->d_gbar, 0, kDrafterWordsBytes);
                     if (d->d_tags) cudaMemset(d->d_tags, 0, (size_t)d->tags_bytes);
                     if (d->d_cbar) cudaMemset(d->d_cbar, 0, kDrafterWordsBytes);
-                    if (d->d_ctags) cudaMemset(d->d_ctags, 0, (size_t)d->ctags_bytes);
                 }
             for (sd2_handle h : g_live)
                 if (h->device == dev && h->d_partial) cudaMemset(h->d_partial, 0, (size_t)h->partial_bytes);
@@ -1808,8 +1791,6 @@ sd2_status sd2_drafter_create(const sd2_handle* h, int32_t L, int64_t n_max, sd2
     d->d_gbar = nullptr;
     d->d_cstages = nullptr;
     d->d_cbar = nullptr;
-    d->d_ctags = nullptr;
-    d->ctags_bytes = 0;
     d->n_cstages = 0;
     // workspace: per block q,k,v,hdn,g,u,t and the block's bf16 output (the next block's input)
     d->ws_off.assign((size_t)L * 8 + 1, 0);
@@ -1886,42 +1867,24 @@ sd2_status sd2_drafter_create(const sd2_handle* h, int32_t L, int64_t n_max, sd2
              cudaMemcpy(d->d_stages, stages.data(), sizeof(SStage) * (size_t)n, cudaMemcpyHostToDevice) == cudaSuccess &&
              dev_malloc((void**)&d->d_gbar, kDrafterWordsBytes) == cudaSuccess && cudaMemset(d->d_gbar, 0, kDrafterWordsBytes) == cudaSuccess;
     }
-    bool cells = tagged;
+    bool cells = true;
     for (const sd2_handle hh : d->handles)
         if (!hh->d_image) cells = false;
     if (ok && cells && n_max >= SD2_CELLS_MIN) {
         // the same blocks over cells, for steps of several rows
         std::vector<CStage> cstages((size_t)L * 4);
-        std::vector<int64_t> ct((size_t)L * 4 + 1, 0);
-        int64_t to = 0;
-        for (int b = 0; b < L; ++b) {
-            const BlockDims& bd = dims[(size_t)b];
-            const int64_t w[4] = {bd.q_out, h[7 * b + 3]->M, bd.inter, bd.out};
-            for (int i = 0; i < 4; ++i) {
-                ct[(size_t)b * 4 + i] = to;
-                to = a256(to + 4 * n_max * w[i]);
-            }
-        }
-        d->ctags_bytes = to;
-        ok = dev_malloc((void**)&d->d_ctags, (size_t)to) == cudaSuccess && cudaMemset(d->d_ctags, 0, (size_t)to) == cudaSuccess;
         CellBuilder bld(cstages.data(), g_dev[dev].sms);
-        for (int b = 0; b < L && ok; ++b) {
-            uint8_t *base = d->d_ws, *tb = (uint8_t*)d->d_ctags;
+        for (int b = 0; b < L; ++b) {
+            uint8_t* base = d->d_ws;
             const int64_t* wo = &d->ws_off[(size_t)b * 8];
-            const int64_t* tw = &ct[(size_t)b * 4];
-            CellTags tg;
-            tg.x_t = b == 0 ? nullptr : (const uint32_t*)(tb + ct[(size_t)(b - 1) * 4 + 3]);
-            tg.q_t = (uint32_t*)(tb + tw[0]);
-            tg.hdn_t = (uint32_t*)(tb + tw[1]);
-            tg.t_t = (uint32_t*)(tb + tw[2]);
-            tg.out_t = b + 1 < L ? (uint32_t*)(tb + tw[3]) : nullptr;
-            append_block_cells(bld, h + 7 * b, nullptr, (uint16_t*)(base + wo[0]), (uint16_t*)(base + wo[1]), (uint16_t*)(base + wo[2]),
+            const uint16_t* xin = b == 0 ? nullptr : (const uint16_t*)(base + d->ws_off[(size_t)(b - 1) * 8 + 7]);
+            append_block_cells(bld, h + 7 * b, xin, (uint16_t*)(base + wo[0]), (uint16_t*)(base + wo[1]), (uint16_t*)(base + wo[2]),
                                (uint16_t*)(base + wo[3]), (uint16_t*)(base + wo[4]), (uint16_t*)(base + wo[5]), (uint16_t*)(base + wo[6]),
-                               base + wo[7], b + 1 < L, &tg);
+                               base + wo[7], b + 1 < L);
         }
         d->n_cstages = bld.n;
         d->cell_needs = bld.needs;
-        ok = ok && dev_malloc((void**)&d->d_cstages, sizeof(CStage) * (size_t)bld.n) == cudaSuccess &&
+        ok = dev_malloc((void**)&d->d_cstages, sizeof(CStage) * (size_t)bld.n) == cudaSuccess &&
              cudaMemcpy(d->d_cstages, cstages.data(), sizeof(CStage) * (size_t)bld.n, cudaMemcpyHostToDevice) == cudaSuccess &&
              dev_malloc((void**)&d->d_cbar, kDrafterWordsBytes) == cudaSuccess && cudaMemset(d->d_cbar, 0, kDrafterWordsBytes) == cudaSuccess;
     }
@@ -1929,7 +1892,7 @@ sd2_status sd2_drafter_create(const sd2_handle* h, int32_t L, int64_t n_max, sd2
         cudaGetLastError();
         for (sd2_handle p : d->owned) sd2_free(p);
         cudaFree(d->d_ws); cudaFree(d->d_stages); cudaFree(d->d_gbar); cudaFree(d->d_tags);
-        cudaFree(d->d_cstages); cudaFree(d->d_cbar); cudaFree(d->d_ctags);
+        cudaFree(d->d_cstages); cudaFree(d->d_cbar);
         cudaGetLastError();
     };
     if (ok && widest_panel(needs.xs_need, needs.K_max, needs.max_tile) == 0) {
@@ -1957,7 +1920,7 @@ sd2_status sd2_drafter_create(const sd2_handle* h, int32_t L, int64_t n_max, sd2
 namespace {
 bool drafter_uses_cells(sd2_drafter d, int64_t N)
 {
-    return N >= SD2_CELLS_MIN && d->d_cstages && widest_cell_panel(d->cell_needs, true) > 0;
+    return N >= SD2_CELLS_MIN && d->d_cstages && widest_cell_panel(d->cell_needs) > 0;
 }
 }  // namespace
 
@@ -1980,9 +1943,7 @@ sd2_status sd2_drafter_step(sd2_drafter d, const void* x, void* y, int64_t N, vo
         c.gbar = d->d_cbar;
         c.err = g_dev[dev].err_word;
         c.wait_cycles = wait_budget(dev);
-        c.tagged = 1;
-        c.rowseq = d->d_cbar + 64;
-        return run_cell_panels(c, N, d->cell_needs, g_dev[dev].sms, (cudaStream_t)cuda_stream);
+        return run_cell_panels(c, N, d->cell_needs, 2 * (g_dev[dev].sms / 2), (cudaStream_t)cuda_stream);
     }
     SArgs a;
     std::memset(&a, 0, sizeof a);
@@ -2012,14 +1973,14 @@ sd2_status sd2_drafter_query(sd2_drafter d, int64_t N, int64_t* out)
     if (!live(d) || !out) return SD2_ERR_INVALID_ARG;
     if (N < 1 || N > d->n_max) return SD2_ERR_SHAPE;
     const bool cells = drafter_uses_cells(d, N);
-    const int cap = cells ? widest_cell_panel(d->cell_needs, true) : widest_panel(d->xs_need, d->K_max, d->max_tile);
+    const int cap = cells ? widest_cell_panel(d->cell_needs) : widest_panel(d->xs_need, d->K_max, d->max_tile);
     if (cap == 0) return SD2_ERR_UNSUPPORTED;
     int64_t streamed = 0, owned = 0, kept = 0;
     // what a step streams: every handle once, except that a block's gate and up are read from the
     // drafter's own paired stack where it has one
     std::vector<char> paired((size_t)d->L, 0);
     for (sd2_handle p : d->owned) { streamed += p->compressed_bytes; owned += p->blob_bytes; }
-    owned += d->ctags_bytes + (int64_t)sizeof(CStage) * d->n_cstages + (d->d_cbar ? kDrafterWordsBytes : 0);
+    owned += (int64_t)sizeof(CStage) * d->n_cstages + (d->d_cbar ? kDrafterWordsBytes : 0);
     size_t oi = 0;
     for (int b = 0; b < d->L; ++b) {
         // (owned stacks were built in block order, one per block that could be paired)
@@ -2067,7 +2028,6 @@ sd2_status sd2_drafter_free(sd2_drafter d)
     if (d->d_tags && cudaFree(d->d_tags) != cudaSuccess) st = SD2_ERR_CUDA;
     if (d->d_cstages && cudaFree(d->d_cstages) != cudaSuccess) st = SD2_ERR_CUDA;
     if (d->d_cbar && cudaFree(d->d_cbar) != cudaSuccess) st = SD2_ERR_CUDA;
-    if (d->d_ctags && cudaFree(d->d_ctags) != cudaSuccess) st = SD2_ERR_CUDA;
     for (sd2_handle p : d->owned)
         if (sd2_free(p) != SD2_OK) st = SD2_ERR_CUDA;
     cudaGetLastError();

@@ -1,29 +1,32 @@
 // The streaming kernel over cells (sd2_cells.hpp): programs of dependent stages for panels of up to 16 activation rows.
 //
-// One persistent CTA per SM runs a *program* of stages.  A stage is one launch's worth of work: up to four weights
-// that read the same activations (q|k|v, or one weight), or a gate and an up projection whose results meet in
-// t = silu(g) * u.  Consecutive stages depend on each other.  The hand-off is the one of sd2_kernels.cuh: a grid-wide
-// barrier (programs over a caller's workspace) or tagged words (drafters).
+// A launch runs a *program* of stages with one persistent CTA per SM.  A stage is up to four weights that read the same
+// activations (q|k|v, or one weight), or a gate and an up projection whose results meet in t = silu(g) * u.
+// Consecutive stages depend on each other; a grid-wide barrier separates them.  (Tagged words, the hand-off of
+// sd2_kernels.cuh, double the bytes every CTA has to fetch, which is what a panel of rows cannot afford.)
 //
-// Warps of a CTA: 15 consumers, 1 producer (four per scheduler, 128 registers each).
+// CTAs work in clusters of two.  A cluster owns a run of 8-row tiles; each of its CTAs multiplies one half of the
+// columns, so it stages half of the activations only (they are the largest thing in shared memory, and every CTA
+// fetches them through L2), and sends its sums of every other tile to the CTA that finishes that tile.
 //
-//   producer   one bulk asynchronous copy per cell (about 2.7 KB at 50 % density), one lane per consumer warp: lane w fills
-//              the few ring slots that warp w alone empties, and the copies of a round are issued by one instruction.
-//              Nothing waits for a stage boundary: while the consumers wait for the previous stage's outputs, the next
-//              stages' weights land.
-//   consumers  the cells of the CTA's tiles, numbered through, go to the 15 warps in turn.  A warp expands a cell in
-//              registers and multiplies it with mma.m16n8k16: the activation rows are the A operand (16 rows), eight
-//              weight rows the B operand, so the expanded weights never pass through shared memory.  At the end of a
-//              tile a warp leaves its 8 x N partial sums in shared memory; the warp that brings the last of a tile's
-//              contributions adds them up in one fixed order (so a row's result depends neither on the launch nor on
-//              N), rounds and stores.
+// Warps of a CTA:
+//   15 consumers, in three groups of five.  A chunk of five cells goes to a group, a cell to each of its warps.  A warp
+//              expands its cell in registers and multiplies it with mma.m16n8k16: the activation rows are the A operand
+//              (16 rows), eight weight rows the B operand, so the expanded weights never pass through shared memory.  At
+//              the end of a tile a warp leaves its 8 x N partial sums in shared memory; the warp that brings the last
+//              of a tile's contributions adds them up in one fixed order (so a row's result depends neither on the
+//              launch nor on N), and sends or stores them.
+//   1 producer: one bulk asynchronous copy per chunk (13 KB at 50 % density) into the group's own ring slots.  Copies of
+//              single cells (2.7 KB) took 147 cycles each to start, 18 bytes per clock; HBM brings 23.  Nothing waits for a
+//              stage boundary: while the previous stage finishes, the next stages' weights land.
+//   1 service warp: waits for the grid barrier, starts the bulk copies of the stage's activation rows, and fetches the
+//              next stage's descriptor.
 //
 // What bounds it: the expansion, about 75 permute / logic instructions per warp and 1024 slots, which an SM retires at
-// two per clock (measured): 27 slots per clock and SM at most, against 17 that arrive from HBM at 50 % density.  The
-// activations are staged as plain rows and nothing is gathered, so the work per slot does not grow with N.
+// two per clock (measured): 27 slots per clock and SM at most, against 17 that arrive from HBM at 50 % density.
 //
-// Every wait (ring barriers, tag polls, counters, grid barrier) is bounded by a cycle budget: when it runs out the CTA
-// raises the error word and winds down instead of hanging.
+// Every wait (ring barriers, counters, grid barrier) is bounded by a cycle budget: when it runs out the CTA raises the
+// error word and winds down instead of hanging.
 
 #pragma once
 
@@ -33,10 +36,13 @@
 namespace sd2 {
 
 constexpr int kCellWarps = 15;
+constexpr int kCellGroups = 3;
+static_assert(kCellWarps == kCellGroups * kChunkCells, "a group has a warp for every cell of a chunk");
 constexpr int kCellConsumers = kCellWarps * 32;
-constexpr int kCellThreads = kCellConsumers + 32;
-constexpr int kCellSlots = 8;               // cells in flight per consumer warp, at most
-constexpr int kPartSlots = 4;               // tiles whose partial sums may be incomplete
+constexpr int kCellThreads = kCellConsumers + 64;
+constexpr int kGroupSlots = 4;              // chunks in flight per group, at most
+constexpr int kPartSlots = 4;               // tiles whose partial sums may be incomplete, at most
+constexpr int kRecvSlots = 4;               // sums from the other CTA that wait to be used
 constexpr int kPairSlots = 8;               // gate tiles whose results wait for the up tile's
 constexpr int kPanelRows = 16;              // activation rows of a launch, at most
 constexpr int kRingGuardBytes = 256;        // the two words read past a cell's last row may lie behind the ring
@@ -44,8 +50,7 @@ constexpr int kRingGuardBytes = 256;        // the two words read past a cell's 
 struct CMat {
     const uint32_t* off;           // [T * D + 1], 32-byte units into `cells`
     const unsigned char* cells;
-    void* y;                       // [N * M] (may be NULL when yt is set, or in a gate|up stage)
-    uint32_t* yt;                  // [N * M] tagged words for the next stage, or NULL
+    void* y;                       // [N * M] (may be NULL in a gate|up stage)
     int M;
     int T;
     int y_f32;                     // 1: fp32 output, 0: bf16
@@ -54,21 +59,18 @@ struct CMat {
 
 struct CStage {
     CMat mat[kMaxFused];
-    const uint16_t* x;     // [N * K] bf16 (or tagged words), or NULL: the activation is bf16(silu(g) * u)
+    const uint16_t* x;     // [N * K] bf16, or NULL: the activation is bf16(silu(g) * u)
     const uint16_t* g;
     const uint16_t* u;
-    uint16_t* t_out;       // gate|up stage, or x == NULL: plain copy of t (may be NULL)
-    uint32_t* tt;          // gate|up stage of a tagged program: tagged t
+    uint16_t* t_out;       // gate|up stage, or x == NULL: t (may be NULL)
     int K;
     int D;                 // cells per tile
-    int tiles_div;         // V / grid size: the CTA with stage-local number c runs tiles_div + (c < tiles_rem) tiles (pairs)
+    int tiles_div;         // V / clusters: the cluster with stage-local number c runs tiles_div + (c < tiles_rem) tiles (pairs)
     int tiles_rem;
-    int rot;               // the stage's first tile goes to CTA `rot`, so that uneven stages even out over a program
-    int tagged_in;         // x points at tagged 32-bit words
-    int pair;              // mat[0] is gate, mat[1] up (equal shapes): tile i of both go to one CTA, one after the other
-    int V;                 // tiles of all weights; tile pairs in a gate|up stage
+    int rot;               // the stage's first tile goes to cluster `rot`, so that uneven stages even out over a program
+    int pair;              // mat[0] is gate, mat[1] up (equal shapes)
     int count;             // weights
-    int reserved;
+    int V;                 // tiles of all weights; tile pairs in a gate|up stage
 };
 static_assert(sizeof(CStage) % 8 == 0, "stage descriptors are arrays of 8-byte fields");
 
@@ -77,16 +79,14 @@ struct CArgsBase {
     const uint16_t* x_in;           // replaces stage 0's x when not NULL
     void* y_out;                    // replaces the last stage's mat[0].y when not NULL
     unsigned int* gbar;             // grid barrier: [0] arrivals, [32] exits (two cache lines)
-    unsigned int* rowseq;           // tagged programs: per activation row, how often it has been produced
     int* err;                       // device error word
     long long wait_cycles;          // budget of every bounded wait
     int n_stages;
     int N;                          // activation rows of this launch
     int n0;                         // first activation row: every X / Y pointer is advanced by n0 rows
-    int tagged;                     // 1: stages hand activations over as tagged words, no grid barrier
-    int part_bytes;                 // shared memory: one tile's partial sums (kPartSlots of them), staged activations
-    int xbuf_bytes[2];              // (two buffers, or one where xbuf_bytes[1] == 0), ring
-    int slot_bytes, n_slots;        // a cell's slot, slots per consumer warp
+    int part_bytes, part_mask;      // shared memory: one tile's partial sums, number of such slots - 1 (a power of two)
+    int xbuf_bytes;                 // staged activations
+    int chunk_bytes, n_slots;       // a ring slot, slots per group
     int fold_any;                   // host side: launch the FOLD instance
 };
 
@@ -98,67 +98,122 @@ struct CArgs : CArgsBase {
 };
 
 struct CellShared {
-    unsigned long long full[kCellWarps][kCellSlots];    // a cell landed
-    unsigned long long empty[kCellWarps][kCellSlots];   // ... and has been consumed
-    int rows[kCellWarps][kCellSlots];                   // H of the cell in the slot
+    unsigned long long full[kCellGroups][kGroupSlots];    // a chunk landed
+    unsigned long long empty[kCellGroups][kGroupSlots];   // ... and has been consumed
+    unsigned long long xfull;                           // the stage's activations have landed, its descriptor is there
+    unsigned long long left;                            // all consumers have left the stage: its descriptor and rows are free
+    unsigned long long csync;                           // all consumers have come this far
+    uint32_t cell[kCellGroups][kGroupSlots][kChunkCells]; // of each cell of the chunk: byte offset << 8 | H
     unsigned int arrived[kPartSlots];                   // contributions to the tile in the slot so far
     unsigned int finished[kPartSlots];                  // 1 + number of the last tile that was finished in the slot
+    unsigned int recv_seq[kRecvSlots];                  // 1 + number of the last sums the other CTA has put into recv[]
+    unsigned int credit[kRecvSlots];                    // 1 + number of the last sums the other CTA has taken out of its recv[]
     unsigned int gate_done[kPairSlots];                 // 1 + number of the last gate tile whose results are in gate[]
     uint16_t gate[kPairSlots][kPanelRows][kTileRows];   // bf16 results of gate tiles
-    unsigned int stage_tiles;                           // grid-barrier programs: tiles of the stage finished so far
+    float2 recv[kRecvSlots][kPanelRows][kTileRows / 2];
+    unsigned int stage_tiles;                           // tiles of the stage finished so far by this CTA
     int abort_flag;                                     // any warp: a bounded wait ran out
-    int stage_dead[2];                                  // thread 0 only: copy of abort_flag taken before a stage's barrier
-    unsigned int tag_base[kPanelRows];                  // tagged programs: (production count of row n0 + n & 0xFF) << 8
     float red[2][kCellWarps];                           // FOLD: per-warp partial sums of squares of two rows
     CStage stage[2];                                    // descriptors of the current and the next stage
 };
 
 // The lanes of a warp come back from wait_phase one by one, with answers of their own.  This one brings the warp back
-// together and with one answer: mma.sync, bar.sync and the like need it whole.
+// together and with one answer: mma.sync and other warp-wide instructions need it whole.
 __device__ __forceinline__ bool wait_phase_warp(uint32_t bar, uint32_t parity, const WaitCtx& w)
 {
     const bool ok = wait_phase(bar, parity, w);
     return __all_sync(0xFFFFFFFFu, ok);
 }
 
+__device__ __forceinline__ unsigned int ld_acquire_shared(const unsigned int* p)
+{
+    unsigned int v;
+    asm volatile("ld.acquire.cluster.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
+    return v;
+}
+
 // Until the shared counter at p has reached `want` (one warp, together).
 __device__ __forceinline__ bool wait_count(const unsigned int* p, unsigned int want, const WaitCtx& w)
 {
     bool ok = true;
-    if ((int)(*(const volatile unsigned int*)p - want) < 0) {
+    if ((int)(ld_acquire_shared(p) - want) < 0) {
         const long long t0 = clock64();
         uint32_t it = 0;
-        while ((int)(*(const volatile unsigned int*)p - want) < 0) {
+        while ((int)(ld_acquire_shared(p) - want) < 0) {
             if ((++it & 15u) == 0u) {
                 if (*w.abort_flag) { ok = false; break; }
                 if (clock64() - t0 > w.budget) { *w.abort_flag = 1; ok = false; break; }
             }
         }
     }
-    ok = __all_sync(0xFFFFFFFFu, ok);
-    __threadfence_block();
-    return ok;
+    return __all_sync(0xFFFFFFFFu, ok);
 }
 
-// Until `target` arrivals have been counted (or the wait budget is out).
-__device__ __forceinline__ void grid_wait(const unsigned int* gbar, unsigned int target, const WaitCtx& w)
+// Until `target` arrivals have been counted.  false: the wait budget is out.
+__device__ __forceinline__ bool grid_wait(const unsigned int* gbar, unsigned int target, const WaitCtx& w)
 {
     const long long t0 = clock64();
     uint32_t it = 0;
     while ((int)(ld_acquire_gpu(gbar) - target) < 0) {
         if ((++it & 15u) == 0u) {
-            if (*w.abort_flag) break;
-            if (clock64() - t0 > w.budget) { *w.abort_flag = 1; break; }
+            if (*w.abort_flag) return false;
+            if (clock64() - t0 > w.budget) { *w.abort_flag = 1; return false; }
         }
     }
-    __threadfence();
+    return true;
 }
 
-__device__ __forceinline__ void consumer_sync()
+// the same shared-memory address in CTA `rank` of the cluster
+__device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t rank)
 {
-    __syncwarp();
-    named_bar_sync(1, kCellConsumers);
+    uint32_t a;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+    return a;
 }
+__device__ __forceinline__ void st_cluster_f2(uint32_t a, float2 v)
+{
+    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ void st_release_cluster(uint32_t a, unsigned int v)
+{
+    asm volatile("st.release.cluster.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+}
+
+// The runs of consecutive tiles of one weight that a cluster works through in a stage, in order.
+struct TileRuns {
+    int v, end, half, stop;      // next tile (pair), last + 1; gate|up: which of the two, end of the current group
+    __device__ __forceinline__ TileRuns(int cluster, int clusters, int rot, int div, int rem)
+    {
+        const int c = cluster - rot + (cluster < rot ? clusters : 0);
+        v = c * div + (c < rem ? c : rem);
+        end = v + div + (c < rem ? 1 : 0);
+        half = 0;
+        stop = 0;
+    }
+    // mat: weight, t0: its first tile, nt: tiles.  false: that was all.
+    __device__ __forceinline__ bool next(int pair, int count, int T0, int T1, int T2, int& mat, int& t0, int& nt)
+    {
+        if (v >= end) return false;
+        if (pair) {
+            if (half == 0) stop = min(v + kPairSlots, end);
+            mat = half;
+            t0 = v;
+            nt = stop - v;
+            if (half) v = stop;
+            half ^= 1;
+            return true;
+        }
+        int base = 0, T = T0;
+        mat = 0;
+        if (count > 1 && v >= T0) { base = T0; T = T1; mat = 1; }
+        if (count > 2 && v >= T0 + T1) { base = T0 + T1; T = T2; mat = 2; }
+        if (count > 3 && v >= T0 + T1 + T2) { base = T0 + T1 + T2; T = end - base; mat = 3; }
+        t0 = v - base;
+        nt = min(end, base + T) - v;
+        v += nt;
+        return true;
+    }
+};
 
 // ---- expanding a cell -----------------------------------------------------------------
 
@@ -242,7 +297,8 @@ __device__ __forceinline__ void half_cell(const unsigned char* smem, uint32_t m,
 struct XRows {
     unsigned char* buf;      // staged rows: bf16, row n at n * pitch bytes, zero from column K to the last cell's end
     int pitch;
-    int K, N;
+    int K, N;                // columns staged here
+    int ld;                  // columns of a whole row in global memory
 };
 
 // Walks the groups (n, k) of a panel of rows, `kq` groups to a row, in steps of the consumer threads.
@@ -263,213 +319,152 @@ struct PanelWalk {
     }
 };
 
-constexpr int kStageBatch = 4;   // loads a thread keeps in flight while staging
+constexpr int kStageBatch = 8;   // loads a thread keeps in flight while staging
 
-__device__ __forceinline__ bool tags_ok(const uint4& v, uint32_t tag)
+// Rows that a bulk copy cannot bring: unaligned ones, and bf16(silu(g) * u) where x is NULL (t_out then gets t).
+__device__ __noinline__ void stage_rows(const XRows& r, const uint16_t* x, const uint16_t* g, const uint16_t* u, uint16_t* t_out, int ctid)
 {
-    return ((((v.x ^ tag) | (v.y ^ tag) | (v.z ^ tag) | (v.w ^ tag)) & 0xFFFFu) == 0u);
-}
-__device__ __forceinline__ uint4 ld_relaxed_v4(const uint32_t* p)
-{
-    uint4 v;
-    asm volatile("ld.relaxed.gpu.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p) : "memory");
-    return v;
-}
-
-// Rows of tagged words -> bf16 rows, waiting for each word's tag.
-__device__ __noinline__ void stage_tagged(const XRows& r, const uint32_t* x, uint32_t tag, const unsigned int* tagb, const WaitCtx& w, int ctid)
-{
-    if ((r.K & 3) == 0 && (((uintptr_t)x) & 15) == 0) {
-        PanelWalk at((uint32_t)r.K >> 2, (uint32_t)ctid);
-        while (at.n < (uint32_t)r.N) {
-            uint4 v[kStageBatch];
-            PanelWalk ahead = at;
-#pragma unroll
-            for (int b = 0; b < kStageBatch; ++b, ahead.next())
-                if (ahead.n < (uint32_t)r.N) v[b] = ld_relaxed_v4(x + 4 * ((size_t)ahead.n * at.kq + ahead.k));
-#pragma unroll
-            for (int b = 0; b < kStageBatch; ++b, at.next()) {
-                if (at.n >= (uint32_t)r.N) break;
-                const uint32_t want = tag | tagb[at.n];
-                if (!tags_ok(v[b], want)) {
-                    const long long t0 = clock64();
-                    uint32_t it = 0;
-                    do {
-                        v[b] = ld_relaxed_v4(x + 4 * ((size_t)at.n * at.kq + at.k));
-                        if ((++it & 7u) == 0u) {
-                            if (*w.abort_flag) break;
-                            if (clock64() - t0 > w.budget) { *w.abort_flag = 1; break; }
-                        }
-                    } while (!tags_ok(v[b], want));
-                }
-                *(uint2*)(r.buf + at.n * (uint32_t)r.pitch + 8u * at.k) =
-                    make_uint2(__byte_perm(v[b].x, v[b].y, 0x7632), __byte_perm(v[b].z, v[b].w, 0x7632));
-            }
-        }
-        return;
-    }
-    for (PanelWalk at((uint32_t)r.K, (uint32_t)ctid); at.n < (uint32_t)r.N; at.next()) {
-        const uint32_t v = poll_tagged1(x + (size_t)at.n * r.K + at.k, tag | tagb[at.n], w);
-        *(uint16_t*)(r.buf + at.n * (uint32_t)r.pitch + 2u * at.k) = (uint16_t)(v >> 16);
-    }
-}
-
-// Plain bf16 rows, or bf16(silu(g) * u) where x is NULL (CTA 0 then stores t as well).
-__device__ __noinline__ void stage_plain(const XRows& r, const uint16_t* x, const uint16_t* g, const uint16_t* u, uint16_t* t_out, int ctid)
-{
-    const bool pub = !x && t_out && blockIdx.x == 0;
-    if ((r.K & 7) == 0 && ((((uintptr_t)x) | ((uintptr_t)g) | ((uintptr_t)u) | ((uintptr_t)t_out)) & 15) == 0) {
-        PanelWalk at((uint32_t)r.K >> 3, (uint32_t)ctid);
-        while (at.n < (uint32_t)r.N) {
-            uint4 v[kStageBatch];
-            PanelWalk ahead = at;
-#pragma unroll
-            for (int b = 0; b < kStageBatch; ++b, ahead.next()) {
-                if (ahead.n >= (uint32_t)r.N) break;
-                const size_t i = (size_t)ahead.n * at.kq + ahead.k;
-                if (x) {
-                    v[b] = __ldcg((const uint4*)x + i);
-                } else {
-                    const uint4 gv = __ldcg((const uint4*)g + i), uv = __ldcg((const uint4*)u + i);
-                    v[b] = make_uint4(silu_mul_pair(gv.x, uv.x), silu_mul_pair(gv.y, uv.y), silu_mul_pair(gv.z, uv.z), silu_mul_pair(gv.w, uv.w));
-                    if (pub) ((uint4*)t_out)[i] = v[b];
-                }
-            }
-#pragma unroll
-            for (int b = 0; b < kStageBatch; ++b, at.next()) {
-                if (at.n >= (uint32_t)r.N) break;
-                *(uint4*)(r.buf + at.n * (uint32_t)r.pitch + 16u * at.k) = v[b];
-            }
-        }
-        return;
-    }
     PanelWalk at((uint32_t)r.K, (uint32_t)ctid);
     while (at.n < (uint32_t)r.N) {
-        uint16_t v[2 * kStageBatch];
+        uint16_t v[kStageBatch];
         PanelWalk ahead = at;
 #pragma unroll
-        for (int b = 0; b < 2 * kStageBatch; ++b, ahead.next()) {
+        for (int b = 0; b < kStageBatch; ++b, ahead.next()) {
             if (ahead.n >= (uint32_t)r.N) break;
-            const size_t i = (size_t)ahead.n * r.K + ahead.k;
+            const size_t i = (size_t)ahead.n * r.ld + ahead.k;
             v[b] = x ? __ldcg(x + i) : silu_mul_bits(__ldcg(g + i), __ldcg(u + i));
-            if (pub) t_out[i] = v[b];
+            if (t_out) t_out[i] = v[b];
         }
 #pragma unroll
-        for (int b = 0; b < 2 * kStageBatch; ++b, at.next()) {
+        for (int b = 0; b < kStageBatch; ++b, at.next()) {
             if (at.n >= (uint32_t)r.N) break;
             *(uint16_t*)(r.buf + at.n * (uint32_t)r.pitch + 2u * at.k) = v[b];
         }
     }
 }
 
-// rows[n] = rmsnorm(rows[n] [+ res]) * norm_w on the staged rows, two at a time
-__device__ __noinline__ void fold_norm(const XRows& r, const SFold& f, int row0, float (*red)[kCellWarps], int ctid)
+// All consumer warps have come this far (an mbarrier and not bar.sync: the wait is bounded like every other).
+struct ConsumerSync {
+    uint32_t bar, phase;
+    __device__ __forceinline__ bool operator()(const WaitCtx& w, int lane)
+    {
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar);
+        const bool ok = wait_phase_warp(bar, phase, w);
+        phase ^= 1u;
+        return ok;
+    }
+};
+
+// rows[n] = rmsnorm(rows[n] [+ res]) * norm_w on the staged columns, two rows at a time.  The sum of squares is over the
+// whole row: the columns that the other CTA of the cluster stages are read from global memory.  xg: the rows in global
+// memory, from the first column on; c0: first staged column.
+__device__ __noinline__ bool fold_norm(const XRows& r, const SFold& f, const uint16_t* xg, int row0, int c0, bool pub, float (*red)[kCellWarps],
+                                       ConsumerSync& sync, const WaitCtx& wc, int ctid)
 {
-    const bool pub = blockIdx.x == 0;
+    const int lane = ctid & 31;
     for (int n0 = 0; n0 < r.N; n0 += 2) {
-        consumer_sync();     // the rows are staged; red is free
+        if (!sync(wc, lane)) return false;     // the rows are staged; red is free
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int n = n0 + q;
             if (n >= r.N) continue;
             uint16_t* xl = (uint16_t*)(r.buf + (size_t)n * r.pitch);
-            const size_t go = (size_t)(row0 + n) * r.K;
+            const size_t go = (size_t)(row0 + n) * r.ld, gx = (size_t)n * r.ld;
             float ss = 0.f;
-            for (int i = ctid; i < r.K; i += kCellConsumers) {
-                float v = bf16_to_f32(xl[i]);
+            for (int i = ctid; i < r.ld; i += kCellConsumers) {
+                const int j = i - c0;
+                const bool own = j >= 0 && j < r.K;
+                float v = bf16_to_f32(own ? xl[j] : __ldcg(xg + gx + i));
                 if (f.res) {
                     const uint16_t sb = f32_to_bf16_rne(v + bf16_to_f32(__ldcg(f.res + go + i)));
-                    xl[i] = sb;
-                    if (pub && f.sum_out) f.sum_out[go + i] = sb;
+                    if (own) {
+                        xl[j] = sb;
+                        if (pub && f.sum_out) f.sum_out[go + i] = sb;
+                    }
                     v = bf16_to_f32(sb);
                 }
                 ss += v * v;
             }
             __syncwarp();
             ss = warp_sum(ss);
-            if ((ctid & 31) == 0) red[q][ctid >> 5] = ss;
+            if (lane == 0) red[q][ctid >> 5] = ss;
         }
-        consumer_sync();
+        if (!sync(wc, lane)) return false;
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int n = n0 + q;
             if (n >= r.N) continue;
             uint16_t* xl = (uint16_t*)(r.buf + (size_t)n * r.pitch);
-            const size_t go = (size_t)(row0 + n) * r.K;
+            const size_t go = (size_t)(row0 + n) * r.ld;
             float tot = 0.f;
 #pragma unroll
             for (int w = 0; w < kCellWarps; ++w) tot += red[q][w];
-            const float rs = rsqrtf(tot / (float)r.K + f.eps);
-            for (int i = ctid; i < r.K; i += kCellConsumers) {
-                const uint16_t o = f32_to_bf16_rne(bf16_to_f32(xl[i]) * rs * bf16_to_f32(__ldg(f.norm_w + i)));
-                xl[i] = o;
+            const float rs = rsqrtf(tot / (float)r.ld + f.eps);
+            // (a column is normalised by the thread that added its residual)
+            for (int i = ctid; i < r.ld; i += kCellConsumers) {
+                const int j = i - c0;
+                if (j < 0 || j >= r.K) continue;
+                const uint16_t o = f32_to_bf16_rne(bf16_to_f32(xl[j]) * rs * bf16_to_f32(__ldg(f.norm_w + i)));
+                xl[j] = o;
                 if (pub && f.norm_out) f.norm_out[go + i] = o;
             }
         }
     }
+    return true;
 }
 
 // ---- finishing a tile ---------------------------------------------------------------------
 
-struct TileOut {
-    int n0, N, tagged;
-    uint32_t tag;            // stage part
+struct TileJob {
+    int n0, N;
     void* y_out;             // replaces mat[0].y (last stage), or NULL
+    int mat, t0;             // weight and first tile of the run
+    int j;                   // tile of the run
+    unsigned int ord;        // number of the tile among those this CTA contributes to
+    unsigned int seq;        // ... among those that are sent to the CTA that finishes it
+    unsigned int pair;       // gate|up: number of the pair in the program
+    int C;                   // contributions of this CTA
+    int owner, rank;         // who finishes the tile (j & 1, or 0 where only that CTA has cells), this CTA
+    int alone;               // the other CTA has no cells
 };
 
-// Stores rows 2 t and 2 t + 1 (values r) of tile v of a stage for panel row n.
-__device__ __forceinline__ void store_tile(const CStage& st, int v, int n, int t2, const float (&r)[2], const TileOut& o, const unsigned int* tagb)
+// Rows 2 t and 2 t + 1 (values r) of tile v of weight md for panel row n.
+__device__ __forceinline__ void store_tile(const CMat& md, void* yp, int v, int n, int t2, const float (&r)[2])
 {
-    int mi = 0;
-    for (int m = 0; m + 1 < st.count; ++m)
-        if (mi == m && v >= st.mat[m].T) { v -= st.mat[m].T; mi = m + 1; }
-    const CMat& md = st.mat[mi];
-    void* yp = (o.y_out && mi == 0) ? o.y_out : md.y;
-    uint32_t* yt = o.tagged ? md.yt : nullptr;
     const size_t M = (size_t)md.M;
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
         const size_t row = (size_t)v * kTileRows + t2 + j;
         if (row >= M) break;
-        const size_t at = (size_t)(o.n0 + n) * M + row;
-        if (yt) {
-            const uint32_t bits = f32_to_bf16_rne(r[j]);
-            st_relaxed_u32(yt + at, (bits << 16) | o.tag | tagb[n]);
-            if (yp) ((uint16_t*)yp)[at] = (uint16_t)bits;
-        } else if (md.y_f32) {
-            ((float*)yp)[at] = r[j];
-        } else {
-            ((uint16_t*)yp)[at] = f32_to_bf16_rne(r[j]);
-        }
+        const size_t at = (size_t)n * M + row;
+        if (md.y_f32) ((float*)yp)[at] = r[j];
+        else ((uint16_t*)yp)[at] = f32_to_bf16_rne(r[j]);
     }
 }
 
-// The same for a gate|up stage: g, u as plain bf16 (where asked for), t = silu(g) * u plain and tagged.
-__device__ __forceinline__ void store_pair(const CStage& st, int v, int n, int t2, const uint16_t* g, const float (&r)[2], const TileOut& o,
-                                           const unsigned int* tagb)
+// The same for an up tile: g, u as plain bf16 (where asked for) and t = silu(g) * u.
+__device__ __forceinline__ void store_pair(const CStage& st, int v, int n, int t2, const uint16_t* g, const float (&r)[2])
 {
     const size_t M = (size_t)st.mat[0].M;
     uint16_t *gp = (uint16_t*)st.mat[0].y, *up = (uint16_t*)st.mat[1].y, *tp = st.t_out;
-    uint32_t* tt = o.tagged ? st.tt : nullptr;
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
         const size_t row = (size_t)v * kTileRows + t2 + j;
         if (row >= M) break;
-        const size_t at = (size_t)(o.n0 + n) * M + row;
-        const uint16_t gb = g[j], ub = f32_to_bf16_rne(r[j]), tv = silu_mul_bits(gb, ub);
-        if (tt) st_relaxed_u32(tt + at, ((uint32_t)tv << 16) | o.tag | tagb[n]);
-        if (tp) tp[at] = tv;
+        const size_t at = (size_t)n * M + row;
+        const uint16_t gb = g[j], ub = f32_to_bf16_rne(r[j]);
+        if (tp) tp[at] = silu_mul_bits(gb, ub);
         if (gp) gp[at] = gb;
         if (up) up[at] = ub;
     }
 }
 
-// The warp that brought a tile's last contribution: adds the C contributions up (four running sums, then one tree: an
-// order that depends neither on N nor on the CTA), and stores.  tl: number of the tile (gate and up apart) in the CTA's
-// share of the stage, ord: in the CTA's share of the program.
+// The warp that brought this CTA's last contribution to a tile: adds the contributions up (four running sums, then one
+// tree: an order that depends neither on N nor on the CTA), then sends the sums to the CTA that finishes the tile, or
+// adds what the other CTA has sent and stores.
 template <int NR>
-__device__ __noinline__ bool finish_tile(CellShared* sh, const CStage& st, const unsigned char* part, int C, int tl, unsigned int ord,
-                                         int first, int G, const TileOut& o, const WaitCtx& wc, int lane)
+__device__ __noinline__ bool finish_tile(CellShared* sh, const CStage& st, const unsigned char* part, const TileJob& o, const WaitCtx& wc, int lane)
 {
     const int t2 = (lane & 3) * 2;
     const uint32_t part_row = (uint32_t)o.N * 32u;               // bytes of one contribution: N x 8 fp32
@@ -483,7 +478,7 @@ __device__ __noinline__ bool finish_tile(CellShared* sh, const CStage& st, const
         for (int k = 0; k < 4; ++k) acc[k] = make_float2(0.f, 0.f);
 #pragma unroll
         for (int c = 0; c < kCellWarps; ++c)
-            if (c < C) {
+            if (c < o.C) {
                 const float2 v = *(const float2*)(p + (uint32_t)c * part_row);
                 acc[c & 3].x += v.x;
                 acc[c & 3].y += v.y;
@@ -491,19 +486,45 @@ __device__ __noinline__ bool finish_tile(CellShared* sh, const CStage& st, const
         r[q][0] = (acc[0].x + acc[1].x) + (acc[2].x + acc[3].x);
         r[q][1] = (acc[0].y + acc[1].y) + (acc[2].y + acc[3].y);
     }
-    if (!st.pair) {
+    const uint32_t rs = o.seq % kRecvSlots;
+    if (o.owner != o.rank) {
+        if (o.seq >= kRecvSlots && !wait_count(&sh->credit[rs], o.seq + 1u - kRecvSlots, wc)) return false;
+        const uint32_t to = peer_addr(&sh->recv[rs][0][0], (uint32_t)o.owner);
 #pragma unroll
         for (int q = 0; q < NR / 8; ++q) {
             const int n = (lane >> 2) + 8 * q;
-            if (n < o.N) store_tile(st, first + tl * G, n, t2, r[q], o, sh->tag_base);
+            if (n < o.N) st_cluster_f2(to + (uint32_t)(n * 4 + (lane & 3)) * 8u, make_float2(r[q][0], r[q][1]));
+        }
+        __syncwarp();
+        if (lane == 0) st_release_cluster(peer_addr(&sh->recv_seq[rs], (uint32_t)o.owner), o.seq + 1u);
+        return true;
+    }
+    if (!o.alone) {
+        if (!wait_count(&sh->recv_seq[rs], o.seq + 1u, wc)) return false;
+#pragma unroll
+        for (int q = 0; q < NR / 8; ++q) {
+            const int n = (lane >> 2) + 8 * q;
+            const float2 v = sh->recv[rs][n < o.N ? n : 0][lane & 3];
+            r[q][0] += v.x;
+            r[q][1] += v.y;
+        }
+        __syncwarp();
+        if (lane == 0) st_release_cluster(peer_addr(&sh->credit[rs], (uint32_t)(o.rank ^ 1)), o.seq + 1u);
+    }
+    if (!st.pair) {
+        const CMat& md = st.mat[o.mat];
+        void* yp = (o.y_out && o.mat == 0) ? o.y_out : md.y;
+#pragma unroll
+        for (int q = 0; q < NR / 8; ++q) {
+            const int n = (lane >> 2) + 8 * q;
+            if (n < o.N) store_tile(md, yp, o.t0 + o.j, o.n0 + n, t2, r[q]);
         }
         return true;
     }
-    const unsigned int pair = (ord - (unsigned int)(tl & 1)) >> 1;   // gate tiles are the even ones of the stage, each followed by its up tile
-    const unsigned int gs = pair % kPairSlots;
-    if (!(tl & 1)) {
-        // the gate slot's previous pair must have been finished (one of an earlier stage has been)
-        if (tl >= 2 * kPairSlots && !wait_count(&sh->finished[(ord + 1u) % kPartSlots], ord + 2u - 2u * kPairSlots, wc)) return false;
+    // gate tiles of a run wait in gate[] for the up tiles of the run that follows.  (A slot's next gate tile comes a
+    // multiple of kPartSlots tiles after the slot's up tile, so it cannot be complete before that one was finished.)
+    const unsigned int gs = (unsigned int)o.j % kPairSlots;
+    if (o.mat == 0) {
 #pragma unroll
         for (int q = 0; q < NR / 8; ++q) {
             const int n = (lane >> 2) + 8 * q;
@@ -511,14 +532,14 @@ __device__ __noinline__ bool finish_tile(CellShared* sh, const CStage& st, const
         }
         __threadfence_block();
         __syncwarp();
-        if (lane == 0) *(volatile unsigned int*)&sh->gate_done[gs] = pair + 1u;
+        if (lane == 0) *(volatile unsigned int*)&sh->gate_done[gs] = o.pair + 1u;
         return true;
     }
-    if (!wait_count(&sh->gate_done[gs], pair + 1u, wc)) return false;
+    if (!wait_count(&sh->gate_done[gs], o.pair + 1u, wc)) return false;
 #pragma unroll
     for (int q = 0; q < NR / 8; ++q) {
         const int n = (lane >> 2) + 8 * q;
-        if (n < o.N) store_pair(st, first + (tl >> 1) * G, n, t2, &sh->gate[gs][n][t2], r[q], o, sh->tag_base);
+        if (n < o.N) store_pair(st, o.t0 + o.j, o.n0 + n, t2, &sh->gate[gs][n][t2], r[q]);
     }
     return true;
 }
@@ -531,31 +552,33 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr uint32_t kPartOff = (uint32_t)((sizeof(CellShared) + 127) & ~127);
     CellShared* sh = (CellShared*)smem;
-    const uint32_t xoff0 = kPartOff + (uint32_t)(kPartSlots * a.part_bytes);
-    const uint32_t ring_off = xoff0 + (uint32_t)a.xbuf_bytes[0] + (uint32_t)a.xbuf_bytes[1];
+    const uint32_t xoff = kPartOff + (uint32_t)((a.part_mask + 1) * a.part_bytes);
+    const uint32_t ring_off = xoff + (uint32_t)a.xbuf_bytes;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int cta = blockIdx.x, G = gridDim.x;
+    const int rank = blockIdx.x & 1, cluster = blockIdx.x >> 1, clusters = gridDim.x >> 1;
+    const int G = gridDim.x;
     const int N = a.N;
     const uint32_t NS = (uint32_t)a.n_slots;
 
-    if (tid < kCellWarps * kCellSlots) {
+    if (tid < kCellGroups * kGroupSlots) {
         mbar_init(smem_u32(&sh->full[0][0]) + 8 * tid, 1);
-        mbar_init(smem_u32(&sh->empty[0][0]) + 8 * tid, 1);
+        mbar_init(smem_u32(&sh->empty[0][0]) + 8 * tid, kChunkCells);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    } else if (tid < kCellWarps * kCellSlots + kPairSlots) {
-        const int i = tid - kCellWarps * kCellSlots;
+    } else if (tid == 32) {
+        mbar_init(smem_u32(&sh->xfull), 1);
+        mbar_init(smem_u32(&sh->left), kCellWarps);
+        mbar_init(smem_u32(&sh->csync), kCellWarps);
+        sh->abort_flag = 0;
+        sh->stage_tiles = 0u;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    } else if (tid >= 64 && tid < 64 + kPairSlots) {
+        const int i = tid - 64;
         sh->gate_done[i] = 0u;
         if (i < kPartSlots) sh->arrived[i] = sh->finished[i] = 0u;
-        if (i == 0) {
-            sh->abort_flag = 0;
-            sh->stage_dead[0] = sh->stage_dead[1] = 0;
-            sh->stage_tiles = 0u;
-        }
-    } else if (tid >= 160 && tid < 160 + kPanelRows) {
-        const int n = tid - 160;
-        sh->tag_base[n] = (a.tagged && n < N) ? ((*(volatile unsigned int*)(a.rowseq + a.n0 + n)) & 0xFFu) << 8 : 0u;
+        if (i < kRecvSlots) sh->recv_seq[i] = sh->credit[i] = 0u;
     }
     __syncthreads();
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");    // waited for before the first access to the other CTA
 
     WaitCtx wc;
     wc.abort_flag = &sh->abort_flag;
@@ -563,96 +586,79 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
 
     if (warp == kCellWarps) {
         // ---------------------------------------------------------------------- producer
-        // Rounds of up to 15 cells, one per lane, through all stages.  A round's directory entries are loaded four rounds
-        // ahead and a stage's fields one stage ahead, so the latencies stay off the ring's critical path.
-        struct PStage {
-            int count, D, nsub, first, n_cells;
-            int T[kMaxFused - 1];
-            const uint32_t* off[kMaxFused];
-            const unsigned char* cells[kMaxFused];
+        // Rounds of one chunk per group; lane 5 g + j stands for cell j of group g's chunk.  A round's directory entries are
+        // loaded four rounds ahead, so their latency (and a stage's fields') stays off the ring's critical path.
+        struct PRound {
+            uint32_t o0, o1;                 // directory entries of the lane's cell; equal: none
+            const unsigned char* cells;
         };
-        struct PCell {
-            uint32_t bytes;
-            const unsigned char* src;
-        };
-        auto stage_of = [&](const CStage& st) {
-            PStage p;
-            p.count = st.count;
-            p.D = st.D;
-            p.nsub = st.pair ? 2 : 1;
-            p.first = cta - st.rot + (cta < st.rot ? G : 0);
-            p.n_cells = (st.tiles_div + (p.first < st.tiles_rem ? 1 : 0)) * p.nsub * p.D;
-#pragma unroll
-            for (int m = 0; m < kMaxFused; ++m) {
-                if (m + 1 < kMaxFused) p.T[m] = st.mat[m].T;
-                p.off[m] = st.mat[m].off;
-                p.cells[m] = st.mat[m].cells;
-            }
-            return p;
-        };
-        auto load_stage = [&](int s) { return a.ext ? stage_of(a.ext[s]) : stage_of(a.inl[MAXS == 1 ? 0 : s]); };
-        // position of the look-ahead: stage sa (fields in `cur`), first cell of the next round ia, warp that gets cell 0 fb
-        int sa = 0, ia = 0, fb = 0;
-        PStage cur = load_stage(0);
-        PStage nxt = a.n_stages > 1 ? load_stage(1) : cur;
+        const int grp = lane / kChunkCells, cj = lane - grp * kChunkCells;
+        int sa = 0, qa = 0, n = 0, n_chunks = 0, gb = 0;
+        const uint32_t* off = nullptr;
+        const unsigned char* cells = nullptr;
+        const CStage* cur = a.ext ? a.ext : &a.inl[0];
+        TileRuns runs(cluster, clusters, cur->rot, cur->tiles_div, cur->tiles_rem);
         auto load_round = [&]() {
-            PCell c;
-            c.bytes = 0u;
-            c.src = nullptr;
-            while (sa < a.n_stages && ia >= cur.n_cells) {       // on to the next stage that has cells for this CTA
-                fb = (fb + cur.n_cells) % kCellWarps;
-                ++sa;
-                ia = 0;
-                cur = nxt;
-                if (sa + 1 < a.n_stages) nxt = load_stage(sa + 1);
-            }
-            if (sa >= a.n_stages) return c;
-            const int r = lane - fb;
-            const int i = ia + (r < 0 ? r + kCellWarps : r);
-            if (lane < kCellWarps && i < cur.n_cells) {
-                const int tl = i / cur.D, d = i - tl * cur.D;
-                int mi = 0, v;
-                if (cur.nsub == 2) {
-                    mi = tl & 1;
-                    v = cur.first + (tl >> 1) * G;
-                } else {
-                    v = cur.first + tl * G;
-#pragma unroll
-                    for (int m = 0; m + 1 < kMaxFused; ++m)
-                        if (mi == m && m + 1 < cur.count && v >= cur.T[m]) { v -= cur.T[m]; mi = m + 1; }
+            PRound c;
+            c.o0 = c.o1 = 0u;
+            c.cells = nullptr;
+            while (qa >= n_chunks) {         // on to the next run of tiles, the next stage
+                gb = (gb + n_chunks) % kCellGroups;
+                qa = n = n_chunks = 0;
+                int mat, t0, nt;
+                if (runs.next(cur->pair, cur->count, cur->mat[0].T, cur->mat[1].T, cur->mat[2].T, mat, t0, nt)) {
+                    const CMat& md = cur->mat[mat];
+                    const int Dr = share_cells(cur->D, rank);
+                    n = nt * Dr;
+                    n_chunks = (n + kChunkCells - 1) / kChunkCells;
+                    cells = md.cells;
+                    off = md.off + (rank ? (size_t)md.T * share_cells(cur->D, 0) : 0) + (size_t)t0 * Dr;
+                    continue;
                 }
-                const uint32_t* off = cur.off[0];
-                const unsigned char* ce = cur.cells[0];
-#pragma unroll
-                for (int m = 1; m < kMaxFused; ++m)
-                    if (mi == m) { off = cur.off[m]; ce = cur.cells[m]; }
-                const uint32_t o0 = __ldg(off + (size_t)v * cur.D + d), o1 = __ldg(off + (size_t)v * cur.D + d + 1);
-                c.bytes = (o1 - o0) * 32u;
-                c.src = ce + (size_t)o0 * 32;
+                if (++sa >= a.n_stages) return c;
+                ++cur;
+                runs = TileRuns(cluster, clusters, cur->rot, cur->tiles_div, cur->tiles_rem);
             }
-            ia += kCellWarps;
+            int g = grp - gb;
+            if (g < 0) g += kCellGroups;
+            const int i = (qa + g) * kChunkCells + cj;
+            if (lane < kCellWarps && i < n) {
+                c.o0 = __ldg(off + i);
+                c.o1 = __ldg(off + i + 1);
+            }
+            c.cells = cells;
+            qa += kCellGroups;
             return c;
         };
         // weights are read once: with several stages their lines leave L2 first, so that the stream does not push out
-        // the small, shared, re-read hand-off words
+        // the small, shared, re-read activations
         const uint64_t policy = l2_evict_first();
         const bool hinted = a.n_stages > 1;
-        const uint32_t bar = 8u * (uint32_t)kCellSlots * (uint32_t)lane;
-        const uint32_t full0 = smem_u32(&sh->full[0][0]) + bar, empty0 = smem_u32(&sh->empty[0][0]) + bar;
-        const uint32_t ring = smem_u32(smem) + ring_off + (uint32_t)lane * NS * (uint32_t)a.slot_bytes;
-        uint32_t slot = 0, phase = 1, issued = 0;                // of this lane's warp
+        const int bg = grp < kCellGroups ? grp : 0;
+        const uint32_t full0 = smem_u32(&sh->full[bg][0]), empty0 = smem_u32(&sh->empty[bg][0]);
+        const uint32_t ring = smem_u32(smem) + ring_off + (uint32_t)bg * NS * (uint32_t)a.chunk_bytes;
+        uint32_t slot = 0, phase = 1, issued = 0;                // of the lane's group
         bool ok = true;
-        PCell c0 = load_round(), c1 = load_round(), c2 = load_round(), c3 = load_round();
-        while (__any_sync(0xFFFFFFFFu, (c0.bytes | c1.bytes | c2.bytes | c3.bytes) != 0u)) {
+        PRound c0 = load_round(), c1 = load_round(), c2 = load_round(), c3 = load_round();
+        while (c0.cells) {
+            const bool mine = c0.o1 != c0.o0;
+            const uint32_t start = __shfl_sync(0xFFFFFFFFu, c0.o0, bg * kChunkCells);
+            uint32_t end = start;
+#pragma unroll
+            for (int k = 0; k < kChunkCells; ++k) end = max(end, __shfl_sync(0xFFFFFFFFu, c0.o1, bg * kChunkCells + k));
+            const bool busy = lane < kCellWarps && end != start;   // the group has a chunk in this round
             bool good = true;
-            if (c0.bytes) good = wait_phase(empty0 + 8 * slot, phase, wc);
+            if (busy) good = wait_phase(empty0 + 8 * slot, phase, wc);
             if (!__all_sync(0xFFFFFFFFu, good)) { ok = false; break; }
-            if (c0.bytes) {
-                sh->rows[lane][slot] = (int)(c0.bytes - kCellHeaderBytes) >> 7;
-                mbar_expect_tx(full0 + 8 * slot, c0.bytes);
-                const uint32_t dst = ring + slot * (uint32_t)a.slot_bytes;
-                if (hinted) bulk_g2s(dst, c0.src, c0.bytes, full0 + 8 * slot, policy);
-                else bulk_g2s(dst, c0.src, c0.bytes, full0 + 8 * slot);
+            if (mine) sh->cell[bg][slot][cj] = ((c0.o0 - start) << 13) | (((c0.o1 - c0.o0) * 32u - kCellHeaderBytes) >> 7);
+            __syncwarp();
+            if (busy) {
+                if (cj == 0) {
+                    const uint32_t bytes = (end - start) * 32u, dst = ring + slot * (uint32_t)a.chunk_bytes;
+                    mbar_expect_tx(full0 + 8 * slot, bytes);
+                    if (hinted) bulk_g2s(dst, c0.cells + (size_t)start * 32, bytes, full0 + 8 * slot, policy);
+                    else bulk_g2s(dst, c0.cells + (size_t)start * 32, bytes, full0 + 8 * slot);
+                }
                 ++issued;
                 if (++slot == NS) { slot = 0; phase ^= 1u; }
             }
@@ -662,7 +668,7 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
             c2 = c3;
             c3 = load_round();
         }
-        if (!ok && lane < kCellWarps) {
+        if (!ok && lane < kCellWarps && cj == 0) {
             // give the copies already issued time to land before this CTA's memory is released
             for (uint32_t t = issued > NS ? issued - NS : 0u; t != issued; ++t) {
                 const long long t0 = clock64();
@@ -670,162 +676,217 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                     if (clock64() - t0 > wc.budget) break;
             }
         }
-    } else {
-        // ---------------------------------------------------------------------- consumers
-        const int ctid = tid;
-        struct CUse {
-            const uint16_t* x;
-            int K, D, nsub, first, n_tiles, tagged_in;
-        };
-        auto use_of = [&](const CStage& st) {
-            CUse c;
-            c.x = st.x;
-            c.K = st.K;
-            c.D = st.D;
-            c.nsub = st.pair ? 2 : 1;
-            c.first = cta - st.rot + (cta < st.rot ? G : 0);
-            c.n_tiles = (st.tiles_div + (c.first < st.tiles_rem ? 1 : 0)) * c.nsub;
-            c.tagged_in = st.tagged_in;
-            return c;
-        };
-        auto load_use = [&](int s) { return a.ext ? use_of(a.ext[s]) : use_of(a.inl[MAXS == 1 ? 0 : s]); };
-        auto fetch_stage = [&](int s) {                          // one warp: the descriptor for those who finish tiles
+        __syncwarp();
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    } else if (warp > kCellWarps) {
+        // ---------------------------------------------------------------------- service warp
+        const uint32_t xfull = smem_u32(&sh->xfull);
+        auto fetch_stage = [&](int s) {
             uint32_t* dst = (uint32_t*)&sh->stage[s & 1];
             for (int i = lane; i < (int)(sizeof(CStage) / 4); i += 32)
                 dst[i] = a.ext ? ((const uint32_t*)(a.ext + s))[i] : ((const uint32_t*)&a.inl[s])[i];
+            __syncwarp();
         };
-        const uint32_t full0 = smem_u32(&sh->full[warp][0]), empty0 = smem_u32(&sh->empty[warp][0]);
-        const uint32_t ring = ring_off + (uint32_t)warp * NS * (uint32_t)a.slot_bytes;
+        if (MAXS > 1) fetch_stage(0);
+        bool landed = true;
+        for (int s = 0; s < a.n_stages; ++s) {
+            const CStage& st = MAXS == 1 ? a.inl[0] : sh->stage[s & 1];
+            const int Dr = share_cells(st.D, rank), xb = rank ? share_cells(st.D, 0) * kCellCols : 0;
+            const int Kr = min(st.K - xb, Dr * kCellCols);
+            const uint16_t* x = (s == 0 && a.x_in) ? a.x_in : st.x;
+            const bool bulk = x && (st.K & 7) == 0 && (((uintptr_t)x) & 15) == 0 && Kr > 0;
+            if (s > 0) {
+                // every CTA has written the previous stage's outputs (and has read its activations)
+                bool ok = true;
+                if (lane == 0) ok = grid_wait(a.gbar, (unsigned int)s * (unsigned int)G, wc);
+                if (!__all_sync(0xFFFFFFFFu, ok)) break;
+                // ... and this CTA's consumers have left the stage, those without a tile in it among them
+                if (!wait_phase_warp(smem_u32(&sh->left), (uint32_t)(s - 1) & 1u, wc)) break;
+                __threadfence();
+                asm volatile("fence.proxy.async;" ::: "memory");     // ... written through the generic proxy, read by bulk copies
+            }
+            if (lane == 0) {
+                if (bulk) mbar_expect_tx(xfull, (uint32_t)(N * Kr * 2));
+                else mbar_arrive(xfull);
+            }
+            __syncwarp();
+            if (bulk && lane < N) {
+                int n = lane + cluster;                          // (not all CTAs ask for the same row first)
+                n -= n / N * N;
+                bulk_g2s(smem_u32(smem) + xoff + (uint32_t)(n * (2 * Dr * kCellCols + 64)), x + (size_t)(a.n0 + n) * st.K + xb, (uint32_t)(Kr * 2), xfull);
+            }
+            landed = !bulk;
+            if (s + 1 < a.n_stages) {
+                // a CTA that finishes no tile of the stage arrives for it at once
+                int owned = 0, mat, t0, nt;
+                TileRuns runs(cluster, clusters, st.rot, st.tiles_div, st.tiles_rem);
+                while (runs.next(st.pair, st.count, st.mat[0].T, st.mat[1].T, st.mat[2].T, mat, t0, nt))
+                    owned += st.D == 1 ? (rank ? 0 : nt) : (nt + 1 - rank) >> 1;
+                if (owned == 0 && lane == 0) atomicAdd(a.gbar, 1u);
+                fetch_stage(s + 1);
+            } else if (bulk) {
+                landed = wait_phase_warp(xfull, (uint32_t)s & 1u, wc);
+            }
+        }
+        if (!landed) {                                           // a wait ran out: give the rows in flight time to land
+            const long long t0 = clock64();
+            while (clock64() - t0 < 200000) {}
+        }
+        __syncwarp();
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    } else {
+        // ---------------------------------------------------------------------- consumers
+        const int ctid = tid;
+        const int grp = warp / kChunkCells, cj = warp - grp * kChunkCells;
+        const uint32_t full0 = smem_u32(&sh->full[grp][0]), empty0 = smem_u32(&sh->empty[grp][0]);
+        const uint32_t xfull = smem_u32(&sh->xfull);
+        const uint32_t ring = ring_off + (uint32_t)grp * NS * (uint32_t)a.chunk_bytes;
         const int g = lane >> 2;
         const int xrow = g < N ? g : 0, xrow8 = g + 8 < N ? g + 8 : 0;   // rows beyond N repeat row 0; their sums are never read
+        ConsumerSync sync;
+        sync.bar = smem_u32(&sh->csync);
+        sync.phase = 0;
         uint32_t slot = 0, phase = 0;
-        unsigned int ord0 = 0;                                   // tiles of the CTA before this stage
-        int fb = 0;                                              // the warp that gets the stage's first cell
+        unsigned int ord0 = 0, seq0 = 0, seq1 = 0, pair0 = 0;    // tiles, tiles sent to CTA 0 / 1, pairs before this run
+        int gb = 0;                                              // the group that gets the run's first chunk
+        bool joined = false;                                     // the other CTA of the cluster has started
         bool failed = false;
-        CUse use = load_use(0);
-        if (MAXS > 1 && warp == kCellWarps - 1) fetch_stage(0);  // visible behind the first staging barrier
-        for (int s = 0; s < a.n_stages; ++s) {
-            const int K = use.K, D = use.D;
-            const uint32_t xoff = xoff0 + ((s & 1) && a.xbuf_bytes[1] ? (uint32_t)a.xbuf_bytes[0] : 0u);
-            const int Kp = D * kCellCols;
-            XRows xr;
-            xr.buf = smem + xoff;
-            xr.K = K;
-            xr.pitch = 2 * Kp + 64;                              // a multiple of 64 that is not one of 128: rows of one
-            xr.N = N;                                            // 128-bit read fall into different banks
-            const bool first_x = s == 0 && a.x_in;
-            const uint16_t* x = first_x ? a.x_in : use.x;
-            if (s > 0 && (!a.xbuf_bytes[1] || !a.tagged)) {
-                // one buffer: everybody has left the previous stage's rows.  Grid barrier: every CTA has written the
-                // previous stage's outputs; one that has no tiles now arrives for this stage at once.
-                if (!a.tagged && ctid == 0) {
-                    grid_wait(a.gbar, (unsigned int)s * (unsigned int)G, wc);
-                    if (use.n_tiles == 0 && s + 1 < a.n_stages) atomicAdd(a.gbar, 1u);
-                }
-                consumer_sync();
-            } else if (s == 0 && !a.tagged && a.n_stages > 1 && use.n_tiles == 0 && ctid == 0) {
-                atomicAdd(a.gbar, 1u);
-            }
-            const size_t go = (size_t)a.n0 * K;
-            if (a.tagged && use.tagged_in && !first_x) {
-                stage_tagged(xr, (const uint32_t*)x + go, (uint32_t)s, sh->tag_base, wc, ctid);
-            } else if (x) {
-                stage_plain(xr, x + go, nullptr, nullptr, nullptr, ctid);
-            } else {
-                const CStage& st = a.inl[MAXS == 1 ? 0 : s];     // (glue mode: inline programs only)
-                stage_plain(xr, nullptr, st.g + go, st.u + go, st.t_out ? st.t_out + go : nullptr, ctid);
-            }
-            for (int n = 0; n < N; ++n)
-                for (int i = K + ctid; i < Kp; i += kCellConsumers) *(uint16_t*)(xr.buf + (size_t)n * xr.pitch + 2 * i) = 0;
-            if constexpr (FOLD) {
-                if (a.fold[MAXS == 1 ? 0 : s].norm_w) fold_norm(xr, a.fold[MAXS == 1 ? 0 : s], a.n0, sh->red, ctid);
-            }
-            if (ctid == 0) sh->stage_dead[s & 1] = sh->abort_flag;
-            consumer_sync();
-            if (sh->stage_dead[s & 1]) break;
-            const int n_tiles = use.n_tiles, first = use.first, n_cells = n_tiles * D;
-            if (s + 1 < a.n_stages) {
-                use = load_use(s + 1);
-                if (warp == kCellWarps - 1) fetch_stage(s + 1);
+        for (int s = 0; s < a.n_stages && !failed; ++s) {
+            if (!wait_phase_warp(xfull, (uint32_t)s & 1u, wc)) break;
+            if (!joined) {
+                asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+                joined = true;
             }
             const CStage& st = MAXS == 1 ? a.inl[0] : sh->stage[s & 1];
-            TileOut to;
-            to.n0 = a.n0;
-            to.N = N;
-            to.tagged = a.tagged;
-            to.tag = (uint32_t)(s + 1);
-            to.y_out = s == a.n_stages - 1 ? a.y_out : nullptr;
-
-            const int C = D < kCellWarps ? D : kCellWarps;
-            const uint32_t xl = xoff + (uint32_t)(xrow * xr.pitch) + 16u * (lane & 3), xl8 = xoff + (uint32_t)(xrow8 * xr.pitch) + 16u * (lane & 3);
-            int i = warp - fb;
-            if (i < 0) i += kCellWarps;
-            int tl = i / D, d = i - tl * D, c0 = d;
-            float af[4] = {0.f, 0.f, 0.f, 0.f}, ab[4] = {0.f, 0.f, 0.f, 0.f};
-            while (i < n_cells && !failed) {   // (after a failure the barriers ahead are attended; thread 0 reads abort_flag there)
-                if (!wait_phase_warp(full0 + 8 * slot, phase, wc)) { failed = true; break; }
-                const uint32_t cell = ring + slot * (uint32_t)a.slot_bytes;
-                {
-                    const uint32_t H = (uint32_t)sh->rows[warp][slot];
-                    const uint32_t ma = *(const uint32_t*)(smem + cell + 4 * lane), mb = *(const uint32_t*)(smem + cell + 128 + 4 * lane);
-                    const uint32_t pi = *(smem + cell + 256 + lane);
-                    const uint32_t xd = (uint32_t)d * (2 * kCellCols), v0 = cell + kCellHeaderBytes;
-                    half_cell<NR, 1>(smem, ma, v0 + 4u * lane, xl + xd, xl8 + xd, af, ab);
-                    if (d * kCellCols + kHalfCols < K)
-                        half_cell<NR, -1>(smem, mb, v0 + (H - 1u) * 128u + pi, xl + xd + 2 * kHalfCols, xl8 + xd + 2 * kHalfCols, af, ab);
+            const int D = st.D, K = st.K, Dr = share_cells(D, rank), xb = rank ? share_cells(D, 0) * kCellCols : 0;
+            const int Kp = Dr * kCellCols, Kr = min(K - xb, Kp);
+            const int pitch = 2 * Kp + 64;                       // a multiple of 64 that is not one of 128: rows of one
+                                                                 // 128-bit read fall into different banks
+            const uint16_t* x = (s == 0 && a.x_in) ? a.x_in : st.x;
+            const bool bulk = x && (K & 7) == 0 && (((uintptr_t)x) & 15) == 0;
+            const bool norm = FOLD && a.fold[MAXS == 1 ? 0 : s].norm_w;
+            if ((!bulk || Kr < Kp || norm) && Kr > 0) {
+                XRows xr;
+                xr.buf = smem + xoff;
+                xr.pitch = pitch;
+                xr.K = Kr;
+                xr.N = N;
+                xr.ld = K;
+                const size_t go = (size_t)a.n0 * K + xb;
+                const bool pub = cluster == 0;
+                if (!bulk) stage_rows(xr, x ? x + go : nullptr, x ? nullptr : st.g + go, x ? nullptr : st.u + go,
+                                      !x && pub && st.t_out ? st.t_out + go : nullptr, ctid);
+                for (int n = 0; n < N; ++n)
+                    for (int i = Kr + ctid; i < Kp; i += kCellConsumers) *(uint16_t*)(xr.buf + (size_t)n * pitch + 2 * i) = 0;
+                if constexpr (FOLD) {
+                    if (norm && !fold_norm(xr, a.fold[MAXS == 1 ? 0 : s], x + (size_t)a.n0 * K, a.n0, xb, pub, sh->red, sync, wc, ctid)) break;
                 }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(empty0 + 8 * slot);
-                if (++slot == NS) { slot = 0; phase ^= 1u; }
-                i += kCellWarps;
-                d += kCellWarps;
-                if (d < D) continue;                             // the next cell belongs to the same tile
-                // the tile's sums go to shared memory; who completes them finishes the tile
-                const unsigned int ord = ord0 + (unsigned int)tl;
-                const uint32_t ps = ord % kPartSlots;
-                if (ord >= kPartSlots && !wait_count(&sh->finished[ps], ord + 1u - kPartSlots, wc)) { failed = true; break; }
-                unsigned char* part = smem + kPartOff + ps * (uint32_t)a.part_bytes;
-                {
-                    unsigned char* p = part + (uint32_t)(c0 * N + g) * 32u + (lane & 3) * 8;
-                    if (g < N) *(float2*)p = make_float2(af[0] + ab[0], af[1] + ab[1]);
-                    if (NR > 8 && g + 8 < N) *(float2*)(p + 256) = make_float2(af[2] + ab[2], af[3] + ab[3]);
-                }
-#pragma unroll
-                for (int k = 0; k < 4; ++k) af[k] = ab[k] = 0.f;
-                __threadfence_block();
-                __syncwarp();
-                unsigned int before = 0;
-                if (lane == 0) before = atomicAdd(&sh->arrived[ps], 1u);
-                before = __shfl_sync(0xFFFFFFFFu, before, 0);
-                if (before == (unsigned int)C - 1u) {
-                    __threadfence_block();
-                    if (!finish_tile<NR>(sh, st, part, C, tl, ord, first, G, to, wc, lane)) { failed = true; break; }
-                    const bool barrier = !a.tagged && s + 1 < a.n_stages;
-                    if (barrier) __threadfence();                // the tile's outputs are visible before the grid barrier counts them
-                    __syncwarp();
-                    if (lane == 0) {
-                        sh->arrived[ps] = 0u;
-                        __threadfence_block();
-                        *(volatile unsigned int*)&sh->finished[ps] = ord + 1u;
-                        if (barrier && atomicAdd(&sh->stage_tiles, 1u) + 1u == (unsigned int)n_tiles) {
-                            sh->stage_tiles = 0u;                // nobody of this CTA is past the barrier yet
-                            __threadfence();
-                            atomicAdd(a.gbar, 1u);
-                        }
+                if (!sync(wc, lane)) break;
+            }
+            TileJob job;
+            job.n0 = a.n0;
+            job.N = N;
+            job.y_out = s == a.n_stages - 1 ? a.y_out : nullptr;
+            job.C = Dr < kCellWarps ? Dr : kCellWarps;
+            job.rank = rank;
+            job.alone = D == 1;
+            const bool barrier = s + 1 < a.n_stages;
+            int owned = 0;                                       // tiles this CTA finishes in the stage
+            if (barrier) {
+                int mat, t0, nt;
+                TileRuns runs(cluster, clusters, st.rot, st.tiles_div, st.tiles_rem);
+                while (runs.next(st.pair, st.count, st.mat[0].T, st.mat[1].T, st.mat[2].T, mat, t0, nt))
+                    owned += D == 1 ? (rank ? 0 : nt) : (nt + 1 - rank) >> 1;
+            }
+            const uint32_t xl = xoff + (uint32_t)(xrow * pitch) + 16u * (lane & 3), xl8 = xoff + (uint32_t)(xrow8 * pitch) + 16u * (lane & 3);
+            TileRuns runs(cluster, clusters, st.rot, st.tiles_div, st.tiles_rem);
+            int nt;
+            while (!failed && runs.next(st.pair, st.count, st.mat[0].T, st.mat[1].T, st.mat[2].T, job.mat, job.t0, nt)) {
+                const int n = nt * Dr, n_chunks = (n + kChunkCells - 1) / kChunkCells;
+                int q = grp - gb;
+                if (q < 0) q += kCellGroups;
+                int i = q * kChunkCells + cj;
+                int tl = Dr > 0 ? i / Dr : 0, d = i - tl * Dr, c0 = d;
+                float af[4] = {0.f, 0.f, 0.f, 0.f}, ab[4] = {0.f, 0.f, 0.f, 0.f};
+                for (; q < n_chunks; q += kCellGroups, i += kCellWarps) {
+                    if (!wait_phase_warp(full0 + 8 * slot, phase, wc)) { failed = true; break; }
+                    if (i < n) {
+                        const uint32_t where = sh->cell[grp][slot][cj];
+                        const uint32_t cell = ring + slot * (uint32_t)a.chunk_bytes + (where >> 8), H = where & 0xFFu;
+                        const uint32_t ma = *(const uint32_t*)(smem + cell + 4 * lane), mb = *(const uint32_t*)(smem + cell + 128 + 4 * lane);
+                        const uint32_t pi = *(smem + cell + 256 + lane);
+                        const uint32_t xd = (uint32_t)d * (2 * kCellCols), v0 = cell + kCellHeaderBytes;
+                        half_cell<NR, 1>(smem, ma, v0 + 4u * lane, xl + xd, xl8 + xd, af, ab);
+                        if (d * kCellCols + kHalfCols < Kr)
+                            half_cell<NR, -1>(smem, mb, v0 + (H - 1u) * 128u + pi, xl + xd + 2 * kHalfCols, xl8 + xd + 2 * kHalfCols, af, ab);
                     }
                     __syncwarp();
+                    if (lane == 0) mbar_arrive(empty0 + 8 * slot);
+                    if (++slot == NS) { slot = 0; phase ^= 1u; }
+                    if (i >= n) continue;
+                    d += kCellWarps;
+                    if (d < Dr) continue;                        // the next cell belongs to the same tile
+                    // the tile's sums go to shared memory; who completes them finishes the tile
+                    job.ord = ord0 + (unsigned int)tl;
+                    const uint32_t ps = job.ord & (unsigned int)a.part_mask;
+                    if (job.ord > (unsigned int)a.part_mask && !wait_count(&sh->finished[ps], job.ord - (unsigned int)a.part_mask, wc)) { failed = true; break; }
+                    unsigned char* part = smem + kPartOff + ps * (uint32_t)a.part_bytes;
+                    {
+                        unsigned char* p = part + (uint32_t)(c0 * N + g) * 32u + (lane & 3) * 8;
+                        if (g < N) *(float2*)p = make_float2(af[0] + ab[0], af[1] + ab[1]);
+                        if (NR > 8 && g + 8 < N) *(float2*)(p + 256) = make_float2(af[2] + ab[2], af[3] + ab[3]);
+                    }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) af[k] = ab[k] = 0.f;
+                    __threadfence_block();
+                    __syncwarp();
+                    unsigned int before = 0;
+                    if (lane == 0) before = atomicAdd(&sh->arrived[ps], 1u);
+                    before = __shfl_sync(0xFFFFFFFFu, before, 0);
+                    if (before == (unsigned int)job.C - 1u) {
+                        __threadfence_block();
+                        job.j = tl;
+                        job.owner = job.alone ? 0 : tl & 1;
+                        job.seq = (job.owner ? seq1 : seq0) + (unsigned int)(tl >> 1);
+                        job.pair = pair0 + (unsigned int)tl;
+                        if (!finish_tile<NR>(sh, st, part, job, wc, lane)) { failed = true; break; }
+                        const bool count = barrier && job.owner == rank;
+                        if (count) __threadfence();              // the tile's outputs are visible before the grid barrier counts them
+                        __syncwarp();
+                        if (lane == 0) {
+                            sh->arrived[ps] = 0u;
+                            __threadfence_block();
+                            *(volatile unsigned int*)&sh->finished[ps] = job.ord + 1u;
+                            if (count && atomicAdd(&sh->stage_tiles, 1u) + 1u == (unsigned int)owned) {
+                                sh->stage_tiles = 0u;            // nobody is past the barrier yet
+                                __threadfence();
+                                atomicAdd(a.gbar, 1u);
+                            }
+                        }
+                        __syncwarp();
+                    }
+                    do { d -= Dr; ++tl; } while (d >= Dr);
+                    c0 = d;
                 }
-                do { d -= D; ++tl; } while (d >= D);
-                c0 = d;
+                gb = (gb + n_chunks) % kCellGroups;
+                if (Dr > 0) ord0 += (unsigned int)nt;            // (tiles this CTA has no cells of take no slot)
+                if (!job.alone) {                                // (only what is sent is numbered)
+                    seq0 += (unsigned int)(nt + 1) >> 1;
+                    seq1 += (unsigned int)nt >> 1;
+                }
+                if (st.pair && job.mat == 1) pair0 += (unsigned int)nt;
             }
-            ord0 += (unsigned int)n_tiles;
-            fb = (fb + n_cells) % kCellWarps;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&sh->left));
         }
+        __syncwarp();
+        if (!joined) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
     }
 
-    // ---- exit: every role comes here
+    // ---- exit: every role comes here; nobody leaves while the other CTA may still write to this one's memory
     __syncwarp();
-    __syncthreads();
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
     if (tid != 0) return;
     if (sh->abort_flag) {   // a bounded wait ran out somewhere in this CTA
         if (a.err) atomicExch(a.err, 1);
@@ -837,8 +898,6 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         if (prev == (unsigned int)G - 1u) {
             atomicExch(a.gbar, 0u);
             atomicExch(a.gbar + 32, 0u);
-            if (a.tagged)   // the launch's activation rows have been produced once more: their next tags differ
-                for (int n = 0; n < N; ++n) atomicAdd(a.rowseq + a.n0 + n, 1u);
         }
     }
 }

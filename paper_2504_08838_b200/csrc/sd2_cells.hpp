@@ -19,8 +19,11 @@
 //     in half 0 to lanes with few in half 1, which keeps H close to the mean (18.7 rows where 18.0 words are used,
 //     at 50 % density).  Whatever rows 32 lanes read, they read 32 different banks.
 //
+// Two CTAs share a tile: one takes the first ceil(D / 2) cells of its columns, the other the rest.  The cells of each
+// share stand together, tile by tile, so that a CTA's run of tiles is one run of bytes.
+//
 //   cell    u32 mask[2][32], u8 pi[32] (4 x column), u32 words[H][32]
-//   sec0    u32 cell_off[T * D + 1] (32-byte units into sec1), cells in order of tile, then column
+//   sec0    u32 cell_off[T * D + 1] (32-byte units into sec1), in order of share, then tile, then column
 //   sec1    cells
 
 #pragma once
@@ -34,10 +37,15 @@ constexpr int kCellCols = 256;
 constexpr int kHalfCols = 128;
 constexpr int kCellHeaderBytes = 2 * 128 + 32;
 
+constexpr int kChunkCells = 5;        // consecutive cells of a share that travel in one copy, at most
+
 struct CellGeom {
     int64_t T;        // row tiles
     int D;            // cells per tile
 };
+
+// cells of share r (0, 1) of a tile
+SD2_HD int share_cells(int D, int r) { return r == 0 ? (D + 1) / 2 : D / 2; }
 
 inline CellGeom cell_geometry(int64_t M, int64_t K)
 {
@@ -50,7 +58,7 @@ inline CellGeom cell_geometry(int64_t M, int64_t K)
 struct CellImage {
     uint8_t* data = nullptr;       // sec0 padded to 256 bytes, then sec1 (malloc)
     size_t sec1_off = 0, bytes = 0;
-    int max_cell = 0;              // bytes of the largest cell
+    int max_chunk = 0;             // bytes of the largest run of kChunkCells cells
     int status = 0;
 };
 
@@ -122,26 +130,29 @@ inline CellImage pack_cells(const uint16_t* W, const uint8_t* mask, int64_t M, i
     const int64_t n_cells = g.T * g.D;
     if (n_cells > 0x3FFFFFFF) { im.status = -2; return im; }
     const size_t sec1_off = align256((size_t)(n_cells + 1) * 4);
-    std::vector<std::vector<uint8_t>> tiles((size_t)g.T);
+    std::vector<std::vector<uint8_t>> tiles((size_t)g.T * 2);
     std::vector<uint32_t> off((size_t)n_cells + 1);       // first the cells' sizes, then their places
-    int max_cell = 0;
-#pragma omp parallel for schedule(dynamic, 4) reduction(max : max_cell)
-    for (int64_t i = 0; i < g.T; ++i) {
-        std::vector<uint8_t>& out = tiles[(size_t)i];
-        out.reserve((size_t)g.D * 3072);
-        for (int d = 0; d < g.D; ++d) {
-            const size_t start = out.size();
-            pack_cell(W, mask, M, K, i * kTileRows, (int64_t)d * kCellCols, out);
-            const int bytes = (int)(out.size() - start);
-            off[(size_t)(i * g.D + d)] = (uint32_t)(bytes / 32);
-            if (bytes > max_cell) max_cell = bytes;
+    const int64_t first_cell[2] = {0, g.T * share_cells(g.D, 0)};
+#pragma omp parallel for schedule(dynamic, 4)
+    for (int64_t i = 0; i < g.T; ++i)
+        for (int r = 0, d = 0; r < 2; ++r) {
+            const int n = share_cells(g.D, r);
+            std::vector<uint8_t>& out = tiles[(size_t)(r * g.T + i)];
+            out.reserve((size_t)n * 3072);
+            for (int j = 0; j < n; ++j, ++d) {
+                const size_t start = out.size();
+                pack_cell(W, mask, M, K, i * kTileRows, (int64_t)d * kCellCols, out);
+                off[(size_t)(first_cell[r] + i * n + j)] = (uint32_t)((out.size() - start) / 32);
+            }
         }
-    }
     uint64_t units = 0;
+    uint32_t max_run = 0;
     for (int64_t c = 0; c < n_cells; ++c) {
         const uint32_t n = off[(size_t)c];
         off[(size_t)c] = (uint32_t)units;
         units += n;
+        const uint32_t from = c >= kChunkCells - 1 ? off[(size_t)(c - (kChunkCells - 1))] : 0u;
+        if ((uint32_t)units - from > max_run) max_run = (uint32_t)units - from;
     }
     if (units > 0xFFFFFFF0ull) { im.status = -2; return im; }
     off[(size_t)n_cells] = (uint32_t)units;
@@ -151,10 +162,13 @@ inline CellImage pack_cells(const uint16_t* W, const uint8_t* mask, int64_t M, i
     std::memcpy(im.data, off.data(), off.size() * 4);
 #pragma omp parallel for schedule(static)
     for (int64_t i = 0; i < g.T; ++i)
-        std::memcpy(im.data + sec1_off + (size_t)off[(size_t)(i * g.D)] * 32, tiles[(size_t)i].data(), tiles[(size_t)i].size());
+        for (int r = 0; r < 2; ++r) {
+            const std::vector<uint8_t>& src = tiles[(size_t)(r * g.T + i)];
+            if (!src.empty()) std::memcpy(im.data + sec1_off + (size_t)off[(size_t)(first_cell[r] + i * share_cells(g.D, r))] * 32, src.data(), src.size());
+        }
     im.sec1_off = sec1_off;
     im.bytes = sec1_off + (size_t)units * 32;
-    im.max_cell = max_cell;
+    im.max_chunk = (int)(max_run * 32u);
     return im;
 }
 
