@@ -597,8 +597,8 @@ bool plan_cells(int n, const CellNeeds& needs, CellPlan* p)
     p->part_bytes = (needs.parts * n * 32 + 127) & ~127;
     p->chunk_bytes = (needs.max_chunk + 127) & ~127;
     p->xbuf_bytes = (n * needs.pitch + 127) & ~127;
-    for (p->n_parts = kPartSlots; p->n_parts >= 2; p->n_parts >>= 1) {
-        const int ring = kSmemMax - kCellFixedBytes - p->n_parts * p->part_bytes - p->xbuf_bytes;
+    for (p->n_parts = kPartSlots; p->n_parts >= 1; p->n_parts >>= 1) {     // (per finisher)
+        const int ring = kSmemMax - kCellFixedBytes - 2 * p->n_parts * p->part_bytes - p->xbuf_bytes;
         p->n_slots = ring > 0 ? ring / (kCellGroups * p->chunk_bytes) : 0;
         if (p->n_slots > kGroupSlots) p->n_slots = kGroupSlots;
         if (p->n_slots >= 2) return true;
@@ -706,7 +706,7 @@ sd2_status run_cell_panels(CArgs<kMaxStagesInline>& a, int64_t N, const CellNeed
         a.xbuf_bytes = p.xbuf_bytes;
         a.chunk_bytes = p.chunk_bytes;
         a.n_slots = p.n_slots;
-        const int smem = kCellFixedBytes + p.n_parts * p.part_bytes + p.xbuf_bytes + kCellGroups * p.n_slots * p.chunk_bytes;
+        const int smem = kCellFixedBytes + 2 * p.n_parts * p.part_bytes + p.xbuf_bytes + kCellGroups * p.n_slots * p.chunk_bytes;
         sd2_status st;
         if (a.n_stages == 1) {
             static_cast<CArgsBase&>(one) = a;

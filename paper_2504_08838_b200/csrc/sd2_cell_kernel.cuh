@@ -13,9 +13,12 @@
 //   15 consumers, in three groups of five.  A chunk of five cells goes to a group, a cell to each of its warps.  A warp
 //              expands its cell in registers and multiplies it with mma.m16n8k16: the activation rows are the A operand
 //              (16 rows), eight weight rows the B operand, so the expanded weights never pass through shared memory.  At
-//              the end of a tile a warp leaves its 8 x N partial sums in shared memory; the warp that brings the last
-//              of a tile's contributions adds them up in one fixed order (so a row's result depends neither on the
-//              launch nor on N), and sends or stores them.
+//              the end of a tile a warp leaves its 8 x N partial sums in shared memory and goes on.
+//   2 finishers: one takes the tiles this CTA finishes, one those it sends, each in order.  They add a tile's partial sums
+//              up in one fixed order (so a row's result depends neither on the launch nor on N).  The sums for the other
+//              CTA travel as asynchronous stores that count bytes on its mbarrier.  (When the consumer that brought a
+//              tile's last contribution finished it, with flags and fences, it was away for 2400 to 7000 cycles per
+//              tile: 80 us for 48 rows of an 8192 x 2048 matrix.)
 //   1 producer: one bulk asynchronous copy per chunk (13 KB at 50 % density) into the group's own ring slots.  Copies of
 //              single cells (2.7 KB) took 147 cycles each to start, 18 bytes per clock; HBM brings 23.  Nothing waits for a
 //              stage boundary: while the previous stage finishes, the next stages' weights land.
@@ -39,9 +42,10 @@ constexpr int kCellWarps = 15;
 constexpr int kCellGroups = 3;
 static_assert(kCellWarps == kCellGroups * kChunkCells, "a group has a warp for every cell of a chunk");
 constexpr int kCellConsumers = kCellWarps * 32;
-constexpr int kCellThreads = kCellConsumers + 64;
+constexpr int kProducerWarp = kCellWarps, kServiceWarp = kCellWarps + 1, kOwnWarp = kCellWarps + 2, kSendWarp = kCellWarps + 3;
+constexpr int kCellThreads = 32 * (kCellWarps + 4);
 constexpr int kGroupSlots = 4;              // chunks in flight per group, at most
-constexpr int kPartSlots = 4;               // tiles whose partial sums may be incomplete, at most
+constexpr int kPartSlots = 4;               // tiles of a finisher whose partial sums may wait, at most
 constexpr int kRecvSlots = 4;               // sums from the other CTA that wait to be used
 constexpr int kPairSlots = 8;               // gate tiles whose results wait for the up tile's
 constexpr int kPanelRows = 16;              // activation rows of a launch, at most
@@ -84,7 +88,7 @@ struct CArgsBase {
     int n_stages;
     int N;                          // activation rows of this launch
     int n0;                         // first activation row: every X / Y pointer is advanced by n0 rows
-    int part_bytes, part_mask;      // shared memory: one tile's partial sums, number of such slots - 1 (a power of two)
+    int part_bytes, part_mask;      // shared memory: one tile's partial sums, number of such slots per finisher - 1 (a power of two)
     int xbuf_bytes;                 // staged activations
     int chunk_bytes, n_slots;       // a ring slot, slots per group
     int fold_any;                   // host side: launch the FOLD instance
@@ -101,17 +105,15 @@ struct CellShared {
     unsigned long long full[kCellGroups][kGroupSlots];    // a chunk landed
     unsigned long long empty[kCellGroups][kGroupSlots];   // ... and has been consumed
     unsigned long long xfull;                           // the stage's activations have landed, its descriptor is there
-    unsigned long long left;                            // all consumers have left the stage: its descriptor and rows are free
+    unsigned long long left;                            // consumers and finishers have left the stage: its descriptor and rows are free
     unsigned long long csync;                           // all consumers have come this far
     uint32_t cell[kCellGroups][kGroupSlots][kChunkCells]; // of each cell of the chunk: byte offset << 8 | H
-    unsigned int arrived[kPartSlots];                   // contributions to the tile in the slot so far
-    unsigned int finished[kPartSlots];                  // 1 + number of the last tile that was finished in the slot
-    unsigned int recv_seq[kRecvSlots];                  // 1 + number of the last sums the other CTA has put into recv[]
-    unsigned int credit[kRecvSlots];                    // 1 + number of the last sums the other CTA has taken out of its recv[]
-    unsigned int gate_done[kPairSlots];                 // 1 + number of the last gate tile whose results are in gate[]
+    unsigned long long pfull[2][kPartSlots];            // a tile's partial sums are complete: [0] to be sent, [1] to be finished here
+    unsigned long long rfull[kRecvSlots];               // sums from the other CTA have landed in recv[]
+    unsigned long long credit[kRecvSlots];              // ... the other CTA has taken ours out of its recv[]
+    unsigned int freed[2][kPartSlots];                  // how often the slot's sums have been read
     uint16_t gate[kPairSlots][kPanelRows][kTileRows];   // bf16 results of gate tiles
     float2 recv[kRecvSlots][kPanelRows][kTileRows / 2];
-    unsigned int stage_tiles;                           // tiles of the stage finished so far by this CTA
     int abort_flag;                                     // any warp: a bounded wait ran out
     float red[2][kCellWarps];                           // FOLD: per-warp partial sums of squares of two rows
     CStage stage[2];                                    // descriptors of the current and the next stage
@@ -125,28 +127,23 @@ __device__ __forceinline__ bool wait_phase_warp(uint32_t bar, uint32_t parity, c
     return __all_sync(0xFFFFFFFFu, ok);
 }
 
-__device__ __forceinline__ unsigned int ld_acquire_shared(const unsigned int* p)
-{
-    unsigned int v;
-    asm volatile("ld.acquire.cluster.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(smem_u32(p)) : "memory");
-    return v;
-}
-
 // Until the shared counter at p has reached `want` (one warp, together).
 __device__ __forceinline__ bool wait_count(const unsigned int* p, unsigned int want, const WaitCtx& w)
 {
     bool ok = true;
-    if ((int)(ld_acquire_shared(p) - want) < 0) {
+    if ((int)(*(const volatile unsigned int*)p - want) < 0) {
         const long long t0 = clock64();
         uint32_t it = 0;
-        while ((int)(ld_acquire_shared(p) - want) < 0) {
+        while ((int)(*(const volatile unsigned int*)p - want) < 0) {
             if ((++it & 15u) == 0u) {
                 if (*w.abort_flag) { ok = false; break; }
                 if (clock64() - t0 > w.budget) { *w.abort_flag = 1; ok = false; break; }
             }
         }
     }
-    return __all_sync(0xFFFFFFFFu, ok);
+    ok = __all_sync(0xFFFFFFFFu, ok);
+    __threadfence_block();
+    return ok;
 }
 
 // Until `target` arrivals have been counted.  false: the wait budget is out.
@@ -170,13 +167,18 @@ __device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t rank)
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
     return a;
 }
-__device__ __forceinline__ void st_cluster_f2(uint32_t a, float2 v)
+// eight bytes into the other CTA's shared memory, counted on its mbarrier when they are there
+__device__ __forceinline__ void st_async_f2(uint32_t a, float2 v, uint32_t bar)
 {
-    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(a), "f"(v.x), "f"(v.y) : "memory");
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(a), "f"(v.x), "f"(v.y), "r"(bar) : "memory");
 }
-__device__ __forceinline__ void st_release_cluster(uint32_t a, unsigned int v)
+__device__ __forceinline__ void mbar_arrive_remote(uint32_t bar)
 {
-    asm volatile("st.release.cluster.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t n)
+{
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(n) : "memory");
 }
 
 // The runs of consecutive tiles of one weight that a cluster works through in a stage, in order.
@@ -416,19 +418,6 @@ __device__ __noinline__ bool fold_norm(const XRows& r, const SFold& f, const uin
 
 // ---- finishing a tile ---------------------------------------------------------------------
 
-struct TileJob {
-    int n0, N;
-    void* y_out;             // replaces mat[0].y (last stage), or NULL
-    int mat, t0;             // weight and first tile of the run
-    int j;                   // tile of the run
-    unsigned int ord;        // number of the tile among those this CTA contributes to
-    unsigned int seq;        // ... among those that are sent to the CTA that finishes it
-    unsigned int pair;       // gate|up: number of the pair in the program
-    int C;                   // contributions of this CTA
-    int owner, rank;         // who finishes the tile (j & 1, or 0 where only that CTA has cells), this CTA
-    int alone;               // the other CTA has no cells
-};
-
 // Rows 2 t and 2 t + 1 (values r) of tile v of weight md for panel row n.
 __device__ __forceinline__ void store_tile(const CMat& md, void* yp, int v, int n, int t2, const float (&r)[2])
 {
@@ -460,25 +449,22 @@ __device__ __forceinline__ void store_pair(const CStage& st, int v, int n, int t
     }
 }
 
-// The warp that brought this CTA's last contribution to a tile: adds the contributions up (four running sums, then one
-// tree: an order that depends neither on N nor on the CTA), then sends the sums to the CTA that finishes the tile, or
-// adds what the other CTA has sent and stores.
+// The sum of a tile's C contributions of this CTA, N x 8 fp32 each: four running sums, then one tree, an order that
+// depends neither on N nor on the CTA.  Lane 4 n + t gets weight rows 2 t and 2 t + 1 of panel rows n and n + 8.
 template <int NR>
-__device__ __noinline__ bool finish_tile(CellShared* sh, const CStage& st, const unsigned char* part, const TileJob& o, const WaitCtx& wc, int lane)
+__device__ __forceinline__ void sum_parts(const unsigned char* part, int C, int N, int lane, float (&r)[NR / 8][2])
 {
-    const int t2 = (lane & 3) * 2;
-    const uint32_t part_row = (uint32_t)o.N * 32u;               // bytes of one contribution: N x 8 fp32
-    float r[NR / 8][2];
+    const uint32_t part_row = (uint32_t)N * 32u;
 #pragma unroll
     for (int q = 0; q < NR / 8; ++q) {
         const int n = (lane >> 2) + 8 * q;
-        const unsigned char* p = part + (n < o.N ? n : 0) * 32 + t2 * 4;
+        const unsigned char* p = part + (n < N ? n : 0) * 32 + (lane & 3) * 8;
         float2 acc[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) acc[k] = make_float2(0.f, 0.f);
 #pragma unroll
         for (int c = 0; c < kCellWarps; ++c)
-            if (c < o.C) {
+            if (c < C) {
                 const float2 v = *(const float2*)(p + (uint32_t)c * part_row);
                 acc[c & 3].x += v.x;
                 acc[c & 3].y += v.y;
@@ -486,62 +472,6 @@ __device__ __noinline__ bool finish_tile(CellShared* sh, const CStage& st, const
         r[q][0] = (acc[0].x + acc[1].x) + (acc[2].x + acc[3].x);
         r[q][1] = (acc[0].y + acc[1].y) + (acc[2].y + acc[3].y);
     }
-    const uint32_t rs = o.seq % kRecvSlots;
-    if (o.owner != o.rank) {
-        if (o.seq >= kRecvSlots && !wait_count(&sh->credit[rs], o.seq + 1u - kRecvSlots, wc)) return false;
-        const uint32_t to = peer_addr(&sh->recv[rs][0][0], (uint32_t)o.owner);
-#pragma unroll
-        for (int q = 0; q < NR / 8; ++q) {
-            const int n = (lane >> 2) + 8 * q;
-            if (n < o.N) st_cluster_f2(to + (uint32_t)(n * 4 + (lane & 3)) * 8u, make_float2(r[q][0], r[q][1]));
-        }
-        __syncwarp();
-        if (lane == 0) st_release_cluster(peer_addr(&sh->recv_seq[rs], (uint32_t)o.owner), o.seq + 1u);
-        return true;
-    }
-    if (!o.alone) {
-        if (!wait_count(&sh->recv_seq[rs], o.seq + 1u, wc)) return false;
-#pragma unroll
-        for (int q = 0; q < NR / 8; ++q) {
-            const int n = (lane >> 2) + 8 * q;
-            const float2 v = sh->recv[rs][n < o.N ? n : 0][lane & 3];
-            r[q][0] += v.x;
-            r[q][1] += v.y;
-        }
-        __syncwarp();
-        if (lane == 0) st_release_cluster(peer_addr(&sh->credit[rs], (uint32_t)(o.rank ^ 1)), o.seq + 1u);
-    }
-    if (!st.pair) {
-        const CMat& md = st.mat[o.mat];
-        void* yp = (o.y_out && o.mat == 0) ? o.y_out : md.y;
-#pragma unroll
-        for (int q = 0; q < NR / 8; ++q) {
-            const int n = (lane >> 2) + 8 * q;
-            if (n < o.N) store_tile(md, yp, o.t0 + o.j, o.n0 + n, t2, r[q]);
-        }
-        return true;
-    }
-    // gate tiles of a run wait in gate[] for the up tiles of the run that follows.  (A slot's next gate tile comes a
-    // multiple of kPartSlots tiles after the slot's up tile, so it cannot be complete before that one was finished.)
-    const unsigned int gs = (unsigned int)o.j % kPairSlots;
-    if (o.mat == 0) {
-#pragma unroll
-        for (int q = 0; q < NR / 8; ++q) {
-            const int n = (lane >> 2) + 8 * q;
-            if (n < o.N) *(uint32_t*)&sh->gate[gs][n][t2] = (uint32_t)f32_to_bf16_rne(r[q][0]) | ((uint32_t)f32_to_bf16_rne(r[q][1]) << 16);
-        }
-        __threadfence_block();
-        __syncwarp();
-        if (lane == 0) *(volatile unsigned int*)&sh->gate_done[gs] = o.pair + 1u;
-        return true;
-    }
-    if (!wait_count(&sh->gate_done[gs], o.pair + 1u, wc)) return false;
-#pragma unroll
-    for (int q = 0; q < NR / 8; ++q) {
-        const int n = (lane >> 2) + 8 * q;
-        if (n < o.N) store_pair(st, o.t0 + o.j, o.n0 + n, t2, &sh->gate[gs][n][t2], r[q]);
-    }
-    return true;
 }
 
 // ---- the kernel ---------------------------------------------------------------------------
@@ -552,7 +482,7 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr uint32_t kPartOff = (uint32_t)((sizeof(CellShared) + 127) & ~127);
     CellShared* sh = (CellShared*)smem;
-    const uint32_t xoff = kPartOff + (uint32_t)((a.part_mask + 1) * a.part_bytes);
+    const uint32_t xoff = kPartOff + (uint32_t)(2 * (a.part_mask + 1) * a.part_bytes);
     const uint32_t ring_off = xoff + (uint32_t)a.xbuf_bytes;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = blockIdx.x & 1, cluster = blockIdx.x >> 1, clusters = gridDim.x >> 1;
@@ -566,25 +496,28 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     } else if (tid == 32) {
         mbar_init(smem_u32(&sh->xfull), 1);
-        mbar_init(smem_u32(&sh->left), kCellWarps);
+        mbar_init(smem_u32(&sh->left), kCellWarps + 2);
         mbar_init(smem_u32(&sh->csync), kCellWarps);
         sh->abort_flag = 0;
-        sh->stage_tiles = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    } else if (tid >= 64 && tid < 64 + kPairSlots) {
-        const int i = tid - 64;
-        sh->gate_done[i] = 0u;
-        if (i < kPartSlots) sh->arrived[i] = sh->finished[i] = 0u;
-        if (i < kRecvSlots) sh->recv_seq[i] = sh->credit[i] = 0u;
+    } else if (tid >= 64 && tid < 64 + 2 * kPartSlots) {
+        mbar_init(smem_u32(&sh->pfull[0][0]) + 8 * (tid - 64), kCellWarps);
+        (&sh->freed[0][0])[tid - 64] = 0u;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    } else if (tid >= 96 && tid < 96 + kRecvSlots) {
+        mbar_init(smem_u32(&sh->rfull[tid - 96]), 1);
+        mbar_init(smem_u32(&sh->credit[tid - 96]), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
-    asm volatile("barrier.cluster.arrive.release;" ::: "memory");    // waited for before the first access to the other CTA
+    // waited for before the first access to the other CTA (only its mbarriers have to be there: fence.mbarrier_init above)
+    asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
 
     WaitCtx wc;
     wc.abort_flag = &sh->abort_flag;
     wc.budget = a.wait_cycles;
 
-    if (warp == kCellWarps) {
+    if (warp == kProducerWarp) {
         // ---------------------------------------------------------------------- producer
         // Rounds of one chunk per group; lane 5 g + j stands for cell j of group g's chunk.  A round's directory entries are
         // loaded four rounds ahead, so their latency (and a stage's fields') stays off the ring's critical path.
@@ -596,8 +529,9 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         int sa = 0, qa = 0, n = 0, n_chunks = 0, gb = 0;
         const uint32_t* off = nullptr;
         const unsigned char* cells = nullptr;
-        const CStage* cur = a.ext ? a.ext : &a.inl[0];
-        TileRuns runs(cluster, clusters, cur->rot, cur->tiles_div, cur->tiles_rem);
+        // (fields one by one, so that inline descriptors are read as kernel arguments and not through a generic pointer)
+#define SD2_FIELD(f) (a.ext ? a.ext[sa].f : a.inl[MAXS == 1 ? 0 : sa].f)
+        TileRuns runs(cluster, clusters, SD2_FIELD(rot), SD2_FIELD(tiles_div), SD2_FIELD(tiles_rem));
         auto load_round = [&]() {
             PRound c;
             c.o0 = c.o1 = 0u;
@@ -606,18 +540,16 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                 gb = (gb + n_chunks) % kCellGroups;
                 qa = n = n_chunks = 0;
                 int mat, t0, nt;
-                if (runs.next(cur->pair, cur->count, cur->mat[0].T, cur->mat[1].T, cur->mat[2].T, mat, t0, nt)) {
-                    const CMat& md = cur->mat[mat];
-                    const int Dr = share_cells(cur->D, rank);
+                if (runs.next(SD2_FIELD(pair), SD2_FIELD(count), SD2_FIELD(mat[0].T), SD2_FIELD(mat[1].T), SD2_FIELD(mat[2].T), mat, t0, nt)) {
+                    const int D = SD2_FIELD(D), Dr = share_cells(D, rank);
                     n = nt * Dr;
                     n_chunks = (n + kChunkCells - 1) / kChunkCells;
-                    cells = md.cells;
-                    off = md.off + (rank ? (size_t)md.T * share_cells(cur->D, 0) : 0) + (size_t)t0 * Dr;
+                    cells = SD2_FIELD(mat[mat].cells);
+                    off = SD2_FIELD(mat[mat].off) + (rank ? (size_t)SD2_FIELD(mat[mat].T) * share_cells(D, 0) : 0) + (size_t)t0 * Dr;
                     continue;
                 }
                 if (++sa >= a.n_stages) return c;
-                ++cur;
-                runs = TileRuns(cluster, clusters, cur->rot, cur->tiles_div, cur->tiles_rem);
+                runs = TileRuns(cluster, clusters, SD2_FIELD(rot), SD2_FIELD(tiles_div), SD2_FIELD(tiles_rem));
             }
             int g = grp - gb;
             if (g < 0) g += kCellGroups;
@@ -678,7 +610,7 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         }
         __syncwarp();
         asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-    } else if (warp > kCellWarps) {
+    } else if (warp == kServiceWarp) {
         // ---------------------------------------------------------------------- service warp
         const uint32_t xfull = smem_u32(&sh->xfull);
         auto fetch_stage = [&](int s) {
@@ -687,10 +619,10 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                 dst[i] = a.ext ? ((const uint32_t*)(a.ext + s))[i] : ((const uint32_t*)&a.inl[s])[i];
             __syncwarp();
         };
-        if (MAXS > 1) fetch_stage(0);
+        fetch_stage(0);
         bool landed = true;
         for (int s = 0; s < a.n_stages; ++s) {
-            const CStage& st = MAXS == 1 ? a.inl[0] : sh->stage[s & 1];
+            const CStage& st = sh->stage[s & 1];
             const int Dr = share_cells(st.D, rank), xb = rank ? share_cells(st.D, 0) * kCellCols : 0;
             const int Kr = min(st.K - xb, Dr * kCellCols);
             const uint16_t* x = (s == 0 && a.x_in) ? a.x_in : st.x;
@@ -700,7 +632,7 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                 bool ok = true;
                 if (lane == 0) ok = grid_wait(a.gbar, (unsigned int)s * (unsigned int)G, wc);
                 if (!__all_sync(0xFFFFFFFFu, ok)) break;
-                // ... and this CTA's consumers have left the stage, those without a tile in it among them
+                // ... and this CTA's warps have left the stage, those without a tile in it among them
                 if (!wait_phase_warp(smem_u32(&sh->left), (uint32_t)(s - 1) & 1u, wc)) break;
                 __threadfence();
                 asm volatile("fence.proxy.async;" ::: "memory");     // ... written through the generic proxy, read by bulk copies
@@ -717,12 +649,6 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
             }
             landed = !bulk;
             if (s + 1 < a.n_stages) {
-                // a CTA that finishes no tile of the stage arrives for it at once
-                int owned = 0, mat, t0, nt;
-                TileRuns runs(cluster, clusters, st.rot, st.tiles_div, st.tiles_rem);
-                while (runs.next(st.pair, st.count, st.mat[0].T, st.mat[1].T, st.mat[2].T, mat, t0, nt))
-                    owned += st.D == 1 ? (rank ? 0 : nt) : (nt + 1 - rank) >> 1;
-                if (owned == 0 && lane == 0) atomicAdd(a.gbar, 1u);
                 fetch_stage(s + 1);
             } else if (bulk) {
                 landed = wait_phase_warp(xfull, (uint32_t)s & 1u, wc);
@@ -734,6 +660,86 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         }
         __syncwarp();
         asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    } else if (warp > kServiceWarp) {
+        // ---------------------------------------------------------------------- finishers
+        const int own = warp == kOwnWarp ? 1 : 0;
+        const uint32_t PM = (uint32_t)a.part_mask;
+        const uint32_t pfull0 = smem_u32(&sh->pfull[own][0]);
+        const unsigned char* parts = smem + kPartOff + (uint32_t)own * (PM + 1u) * (uint32_t)a.part_bytes;
+        const int t2 = (lane & 3) * 2;
+        uint32_t done = 0, seq = 0;                              // tiles of this warp so far; those that were exchanged
+        bool ok = true;
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+        for (int s = 0; s < a.n_stages && ok; ++s) {
+            if (!wait_phase_warp(smem_u32(&sh->xfull), (uint32_t)s & 1u, wc)) break;
+            const CStage& st = sh->stage[s & 1];
+            const int D = st.D, Dr = share_cells(D, rank), C = Dr < kCellWarps ? Dr : kCellWarps;
+            const bool alone = D == 1;
+            TileRuns runs(cluster, clusters, st.rot, st.tiles_div, st.tiles_rem);
+            int mat, t0, nt;
+            while (ok && runs.next(st.pair, st.count, st.mat[0].T, st.mat[1].T, st.mat[2].T, mat, t0, nt)) {
+                if (alone && (rank || !own)) continue;           // CTA 0 has all the cells and finishes all the tiles
+                for (int j = alone ? 0 : own ? rank : rank ^ 1; j < nt; j += alone ? 1 : 2, ++done) {
+                    const uint32_t ps = done & PM, use = done / (PM + 1u);
+                    if (!(ok = wait_phase_warp(pfull0 + 8 * ps, use & 1u, wc))) break;
+                    float r[NR / 8][2];
+                    sum_parts<NR>(parts + ps * (uint32_t)a.part_bytes, C, N, lane, r);
+                    __syncwarp();
+                    if (lane == 0) *(volatile unsigned int*)&sh->freed[own][ps] = use + 1u;
+                    const uint32_t rs = seq % kRecvSlots, ru = seq / kRecvSlots;
+                    if (!own) {
+                        if (ru > 0 && !(ok = wait_phase_warp(smem_u32(&sh->credit[rs]), (ru - 1u) & 1u, wc))) break;
+                        const uint32_t to = peer_addr(&sh->recv[rs][0][0], (uint32_t)(rank ^ 1)), bar = peer_addr(&sh->rfull[rs], (uint32_t)(rank ^ 1));
+#pragma unroll
+                        for (int q = 0; q < NR / 8; ++q) {
+                            const int n = (lane >> 2) + 8 * q;
+                            if (n < N) st_async_f2(to + (uint32_t)(n * 4 + (lane & 3)) * 8u, make_float2(r[q][0], r[q][1]), bar);
+                        }
+                        ++seq;
+                        continue;
+                    }
+                    if (!alone) {
+                        if (lane == 0) mbar_expect_tx(smem_u32(&sh->rfull[rs]), (uint32_t)N * 32u);
+                        __syncwarp();
+                        if (!(ok = wait_phase_warp(smem_u32(&sh->rfull[rs]), ru & 1u, wc))) break;
+#pragma unroll
+                        for (int q = 0; q < NR / 8; ++q) {
+                            const int n = (lane >> 2) + 8 * q;
+                            const float2 v = sh->recv[rs][n < N ? n : 0][lane & 3];
+                            r[q][0] += v.x;
+                            r[q][1] += v.y;
+                        }
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive_remote(peer_addr(&sh->credit[rs], (uint32_t)(rank ^ 1)));
+                        ++seq;
+                    }
+#pragma unroll
+                    for (int q = 0; q < NR / 8; ++q) {
+                        const int n = (lane >> 2) + 8 * q;
+                        if (n >= N) continue;
+                        if (!st.pair) {
+                            const CMat& md = st.mat[mat];
+                            store_tile(md, s == a.n_stages - 1 && a.y_out && mat == 0 ? a.y_out : md.y, t0 + j, a.n0 + n, t2, r[q]);
+                        } else {
+                            // gate tiles of a run wait for the up tiles of the run that follows, written and read by the same lane
+                            uint16_t* gt = &sh->gate[j % kPairSlots][n][t2];
+                            if (mat == 0) *(uint32_t*)gt = (uint32_t)f32_to_bf16_rne(r[q][0]) | ((uint32_t)f32_to_bf16_rne(r[q][1]) << 16);
+                            else store_pair(st, t0 + j, a.n0 + n, t2, gt, r[q]);
+                        }
+                    }
+                }
+            }
+            if (own && ok && s + 1 < a.n_stages) {
+                __threadfence();                                 // this CTA's outputs are visible before the grid barrier counts it
+                __syncwarp();
+                if (lane == 0) {
+                    __threadfence();
+                    atomicAdd(a.gbar, 1u);
+                }
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&sh->left));
+        }
     } else {
         // ---------------------------------------------------------------------- consumers
         const int ctid = tid;
@@ -747,17 +753,12 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         sync.bar = smem_u32(&sh->csync);
         sync.phase = 0;
         uint32_t slot = 0, phase = 0;
-        unsigned int ord0 = 0, seq0 = 0, seq1 = 0, pair0 = 0;    // tiles, tiles sent to CTA 0 / 1, pairs before this run
+        uint32_t cnt[2] = {0, 0};                                // tiles of each finisher before this run
         int gb = 0;                                              // the group that gets the run's first chunk
-        bool joined = false;                                     // the other CTA of the cluster has started
         bool failed = false;
         for (int s = 0; s < a.n_stages && !failed; ++s) {
             if (!wait_phase_warp(xfull, (uint32_t)s & 1u, wc)) break;
-            if (!joined) {
-                asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-                joined = true;
-            }
-            const CStage& st = MAXS == 1 ? a.inl[0] : sh->stage[s & 1];
+            const CStage& st = sh->stage[s & 1];
             const int D = st.D, K = st.K, Dr = share_cells(D, rank), xb = rank ? share_cells(D, 0) * kCellCols : 0;
             const int Kp = Dr * kCellCols, Kr = min(K - xb, Kp);
             const int pitch = 2 * Kp + 64;                       // a multiple of 64 that is not one of 128: rows of one
@@ -783,25 +784,12 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                 }
                 if (!sync(wc, lane)) break;
             }
-            TileJob job;
-            job.n0 = a.n0;
-            job.N = N;
-            job.y_out = s == a.n_stages - 1 ? a.y_out : nullptr;
-            job.C = Dr < kCellWarps ? Dr : kCellWarps;
-            job.rank = rank;
-            job.alone = D == 1;
-            const bool barrier = s + 1 < a.n_stages;
-            int owned = 0;                                       // tiles this CTA finishes in the stage
-            if (barrier) {
-                int mat, t0, nt;
-                TileRuns runs(cluster, clusters, st.rot, st.tiles_div, st.tiles_rem);
-                while (runs.next(st.pair, st.count, st.mat[0].T, st.mat[1].T, st.mat[2].T, mat, t0, nt))
-                    owned += D == 1 ? (rank ? 0 : nt) : (nt + 1 - rank) >> 1;
-            }
+            const uint32_t C = (uint32_t)(Dr < kCellWarps ? Dr : kCellWarps);
+            const bool alone = D == 1;
             const uint32_t xl = xoff + (uint32_t)(xrow * pitch) + 16u * (lane & 3), xl8 = xoff + (uint32_t)(xrow8 * pitch) + 16u * (lane & 3);
             TileRuns runs(cluster, clusters, st.rot, st.tiles_div, st.tiles_rem);
-            int nt;
-            while (!failed && runs.next(st.pair, st.count, st.mat[0].T, st.mat[1].T, st.mat[2].T, job.mat, job.t0, nt)) {
+            int mat, t0, nt;
+            while (!failed && runs.next(st.pair, st.count, st.mat[0].T, st.mat[1].T, st.mat[2].T, mat, t0, nt)) {
                 const int n = nt * Dr, n_chunks = (n + kChunkCells - 1) / kChunkCells;
                 int q = grp - gb;
                 if (q < 0) q += kCellGroups;
@@ -826,61 +814,38 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                     if (i >= n) continue;
                     d += kCellWarps;
                     if (d < Dr) continue;                        // the next cell belongs to the same tile
-                    // the tile's sums go to shared memory; who completes them finishes the tile
-                    job.ord = ord0 + (unsigned int)tl;
-                    const uint32_t ps = job.ord & (unsigned int)a.part_mask;
-                    if (job.ord > (unsigned int)a.part_mask && !wait_count(&sh->finished[ps], job.ord - (unsigned int)a.part_mask, wc)) { failed = true; break; }
-                    unsigned char* part = smem + kPartOff + ps * (uint32_t)a.part_bytes;
+                    // the tile's sums go to the finisher in charge
                     {
-                        unsigned char* p = part + (uint32_t)(c0 * N + g) * 32u + (lane & 3) * 8;
+                        const int own = alone || (tl & 1) == rank ? 1 : 0;
+                        const uint32_t k = (own ? cnt[1] : cnt[0]) + (uint32_t)(alone ? tl : tl >> 1);
+                        const uint32_t ps = k & (uint32_t)a.part_mask, use = k / ((uint32_t)a.part_mask + 1u);
+                        if (use > 0 && !wait_count(&sh->freed[own][ps], use, wc)) { failed = true; break; }
+                        unsigned char* p = smem + kPartOff + ((uint32_t)own * ((uint32_t)a.part_mask + 1u) + ps) * (uint32_t)a.part_bytes +
+                                           (uint32_t)(c0 * N + g) * 32u + (lane & 3) * 8;
                         if (g < N) *(float2*)p = make_float2(af[0] + ab[0], af[1] + ab[1]);
                         if (NR > 8 && g + 8 < N) *(float2*)(p + 256) = make_float2(af[2] + ab[2], af[3] + ab[3]);
-                    }
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) af[k] = ab[k] = 0.f;
-                    __threadfence_block();
-                    __syncwarp();
-                    unsigned int before = 0;
-                    if (lane == 0) before = atomicAdd(&sh->arrived[ps], 1u);
-                    before = __shfl_sync(0xFFFFFFFFu, before, 0);
-                    if (before == (unsigned int)job.C - 1u) {
-                        __threadfence_block();
-                        job.j = tl;
-                        job.owner = job.alone ? 0 : tl & 1;
-                        job.seq = (job.owner ? seq1 : seq0) + (unsigned int)(tl >> 1);
-                        job.pair = pair0 + (unsigned int)tl;
-                        if (!finish_tile<NR>(sh, st, part, job, wc, lane)) { failed = true; break; }
-                        const bool count = barrier && job.owner == rank;
-                        if (count) __threadfence();              // the tile's outputs are visible before the grid barrier counts them
+                        for (int m = 0; m < 4; ++m) af[m] = ab[m] = 0.f;
                         __syncwarp();
-                        if (lane == 0) {
-                            sh->arrived[ps] = 0u;
-                            __threadfence_block();
-                            *(volatile unsigned int*)&sh->finished[ps] = job.ord + 1u;
-                            if (count && atomicAdd(&sh->stage_tiles, 1u) + 1u == (unsigned int)owned) {
-                                sh->stage_tiles = 0u;            // nobody is past the barrier yet
-                                __threadfence();
-                                atomicAdd(a.gbar, 1u);
-                            }
-                        }
-                        __syncwarp();
+                        // the C contributions make 15 arrivals between them
+                        if (lane == 0) mbar_arrive_n(smem_u32(&sh->pfull[own][ps]), c0 == 0 ? kCellWarps + 1u - C : 1u);
                     }
                     do { d -= Dr; ++tl; } while (d >= Dr);
                     c0 = d;
                 }
                 gb = (gb + n_chunks) % kCellGroups;
-                if (Dr > 0) ord0 += (unsigned int)nt;            // (tiles this CTA has no cells of take no slot)
-                if (!job.alone) {                                // (only what is sent is numbered)
-                    seq0 += (unsigned int)(nt + 1) >> 1;
-                    seq1 += (unsigned int)nt >> 1;
+                if (alone) {
+                    cnt[1] += rank ? 0u : (uint32_t)nt;
+                } else {                                         // tile j is finished by CTA j & 1
+                    cnt[1] += (uint32_t)(nt + 1 - rank) >> 1;
+                    cnt[0] += (uint32_t)(nt + rank) >> 1;
                 }
-                if (st.pair && job.mat == 1) pair0 += (unsigned int)nt;
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&sh->left));
         }
         __syncwarp();
-        if (!joined) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
     }
 
     // ---- exit: every role comes here; nobody leaves while the other CTA may still write to this one's memory
