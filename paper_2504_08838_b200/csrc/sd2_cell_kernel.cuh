@@ -517,6 +517,8 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
     wc.abort_flag = &sh->abort_flag;
     wc.budget = a.wait_cycles;
 
+    // field f of stage sa (one by one, so that inline descriptors are read as kernel arguments, not through a generic pointer)
+#define SD2_FIELD(f) (a.ext ? a.ext[sa].f : a.inl[MAXS == 1 ? 0 : sa].f)
     if (warp == kProducerWarp) {
         // ---------------------------------------------------------------------- producer
         // Rounds of one chunk per group; lane 5 g + j stands for cell j of group g's chunk.  A round's directory entries are
@@ -529,8 +531,6 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         int sa = 0, qa = 0, n = 0, n_chunks = 0, gb = 0;
         const uint32_t* off = nullptr;
         const unsigned char* cells = nullptr;
-        // (fields one by one, so that inline descriptors are read as kernel arguments and not through a generic pointer)
-#define SD2_FIELD(f) (a.ext ? a.ext[sa].f : a.inl[MAXS == 1 ? 0 : sa].f)
         TileRuns runs(cluster, clusters, SD2_FIELD(rot), SD2_FIELD(tiles_div), SD2_FIELD(tiles_rem));
         auto load_round = [&]() {
             PRound c;
@@ -619,14 +619,16 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                 dst[i] = a.ext ? ((const uint32_t*)(a.ext + s))[i] : ((const uint32_t*)&a.inl[s])[i];
             __syncwarp();
         };
-        fetch_stage(0);
         bool landed = true;
         for (int s = 0; s < a.n_stages; ++s) {
+            // (the first stage's rows are on their way before its descriptor has been copied to shared memory)
+            const int sa = s;
             const CStage& st = sh->stage[s & 1];
-            const int Dr = share_cells(st.D, rank), xb = rank ? share_cells(st.D, 0) * kCellCols : 0;
-            const int Kr = min(st.K - xb, Dr * kCellCols);
-            const uint16_t* x = (s == 0 && a.x_in) ? a.x_in : st.x;
-            const bool bulk = x && (st.K & 7) == 0 && (((uintptr_t)x) & 15) == 0 && Kr > 0;
+            const int D = s == 0 ? SD2_FIELD(D) : st.D, K = s == 0 ? SD2_FIELD(K) : st.K;
+            const int Dr = share_cells(D, rank), xb = rank ? share_cells(D, 0) * kCellCols : 0;
+            const int Kr = min(K - xb, Dr * kCellCols);
+            const uint16_t* x = s == 0 ? (a.x_in ? a.x_in : SD2_FIELD(x)) : st.x;
+            const bool bulk = x && (K & 7) == 0 && (((uintptr_t)x) & 15) == 0 && Kr > 0;
             if (s > 0) {
                 // every CTA has written the previous stage's outputs (and has read its activations)
                 bool ok = true;
@@ -637,15 +639,16 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                 __threadfence();
                 asm volatile("fence.proxy.async;" ::: "memory");     // ... written through the generic proxy, read by bulk copies
             }
-            if (lane == 0) {
-                if (bulk) mbar_expect_tx(xfull, (uint32_t)(N * Kr * 2));
-                else mbar_arrive(xfull);
-            }
-            __syncwarp();
             if (bulk && lane < N) {
                 int n = lane + cluster;                          // (not all CTAs ask for the same row first)
                 n -= n / N * N;
-                bulk_g2s(smem_u32(smem) + xoff + (uint32_t)(n * (2 * Dr * kCellCols + 64)), x + (size_t)(a.n0 + n) * st.K + xb, (uint32_t)(Kr * 2), xfull);
+                bulk_g2s(smem_u32(smem) + xoff + (uint32_t)(n * (2 * Dr * kCellCols + 64)), x + (size_t)(a.n0 + n) * K + xb, (uint32_t)(Kr * 2), xfull);
+            }
+            __syncwarp();
+            if (s == 0) fetch_stage(0);
+            if (lane == 0) {
+                if (bulk) mbar_expect_tx(xfull, (uint32_t)(N * Kr * 2));
+                else mbar_arrive(xfull);
             }
             landed = !bulk;
             if (s + 1 < a.n_stages) {
