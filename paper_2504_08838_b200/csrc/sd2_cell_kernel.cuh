@@ -113,7 +113,7 @@ struct CellShared {
     unsigned long long credit[kRecvSlots];              // ... the other CTA has taken ours out of its recv[]
     unsigned int freed[2][kPartSlots];                  // how often the slot's sums have been read
     uint16_t gate[kPairSlots][kPanelRows][kTileRows];   // bf16 results of gate tiles
-    float2 recv[kRecvSlots][kPanelRows][kTileRows / 2];
+    float4 recv[kRecvSlots][kPanelRows * kTileRows / 4];
     int abort_flag;                                     // any warp: a bounded wait ran out
     float red[2][kCellWarps];                           // FOLD: per-warp partial sums of squares of two rows
     CStage stage[2];                                    // descriptors of the current and the next stage
@@ -167,10 +167,14 @@ __device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t rank)
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
     return a;
 }
-// eight bytes into the other CTA's shared memory, counted on its mbarrier when they are there
-__device__ __forceinline__ void st_async_f2(uint32_t a, float2 v, uint32_t bar)
+// NV floats into the other CTA's shared memory, counted in bytes on its mbarrier when they are there
+template <int NV>
+__device__ __forceinline__ void st_async(uint32_t a, const float (&v)[NV], uint32_t bar)
 {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(a), "f"(v.x), "f"(v.y), "r"(bar) : "memory");
+    if (NV == 4)
+        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(a), "f"(v[0]), "f"(v[1]), "f"(v[NV - 2]), "f"(v[NV - 1]), "r"(bar) : "memory");
+    else
+        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(a), "f"(v[0]), "f"(v[1]), "r"(bar) : "memory");
 }
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t bar)
 {
@@ -418,60 +422,54 @@ __device__ __noinline__ bool fold_norm(const XRows& r, const SFold& f, const uin
 
 // ---- finishing a tile ---------------------------------------------------------------------
 
-// Rows 2 t and 2 t + 1 (values r) of tile v of weight md for panel row n.
-__device__ __forceinline__ void store_tile(const CMat& md, void* yp, int v, int n, int t2, const float (&r)[2])
+// A finisher shares its scheduler with four or five busy warps and gets an instruction in every few cycles, so what counts
+// here is the number of instructions per tile.  Lane l holds the NR / 4 results that stand together at l * NR bytes of a
+// contribution (N x 8 fp32): panel row l * NR / 32, NR / 4 consecutive weight rows.
+
+// The sum of a tile's C contributions: four running sums, then one tree, an order that depends neither on N nor on the CTA.
+template <int NV>
+__device__ __forceinline__ void sum_parts(const unsigned char* p, int C, uint32_t part_row, float (&r)[NV])
 {
-    const size_t M = (size_t)md.M;
+    float acc[4][NV];
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        const size_t row = (size_t)v * kTileRows + t2 + j;
-        if (row >= M) break;
-        const size_t at = (size_t)n * M + row;
-        if (md.y_f32) ((float*)yp)[at] = r[j];
-        else ((uint16_t*)yp)[at] = f32_to_bf16_rne(r[j]);
+    for (int k = 0; k < 4; ++k)
+#pragma unroll
+        for (int j = 0; j < NV; ++j) acc[k][j] = 0.f;
+    for (int c = 0; c < C; c += 4) {
+        float v[4][NV];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (NV == 4) *(float4*)v[k] = *(const float4*)(p + (uint32_t)min(c + k, C - 1) * part_row);
+            else *(float2*)v[k] = *(const float2*)(p + (uint32_t)min(c + k, C - 1) * part_row);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+#pragma unroll
+            for (int j = 0; j < NV; ++j) acc[k][j] += c + k < C ? v[k][j] : 0.f;
     }
+#pragma unroll
+    for (int j = 0; j < NV; ++j) r[j] = (acc[0][j] + acc[1][j]) + (acc[2][j] + acc[3][j]);
 }
 
-// The same for an up tile: g, u as plain bf16 (where asked for) and t = silu(g) * u.
-__device__ __forceinline__ void store_pair(const CStage& st, int v, int n, int t2, const uint16_t* g, const float (&r)[2])
+__device__ __forceinline__ uint32_t bf16_pair(float lo, float hi)
 {
-    const size_t M = (size_t)st.mat[0].M;
-    uint16_t *gp = (uint16_t*)st.mat[0].y, *up = (uint16_t*)st.mat[1].y, *tp = st.t_out;
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-        const size_t row = (size_t)v * kTileRows + t2 + j;
-        if (row >= M) break;
-        const size_t at = (size_t)n * M + row;
-        const uint16_t gb = g[j], ub = f32_to_bf16_rne(r[j]);
-        if (tp) tp[at] = silu_mul_bits(gb, ub);
-        if (gp) gp[at] = gb;
-        if (up) up[at] = ub;
-    }
+    uint32_t d;
+    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
+    return d;
 }
 
-// The sum of a tile's C contributions of this CTA, N x 8 fp32 each: four running sums, then one tree, an order that
-// depends neither on N nor on the CTA.  Lane 4 n + t gets weight rows 2 t and 2 t + 1 of panel rows n and n + 8.
-template <int NR>
-__device__ __forceinline__ void sum_parts(const unsigned char* part, int C, int N, int lane, float (&r)[NR / 8][2])
+// NV consecutive bf16 values to p, of which `n` exist; vec: p is aligned to 2 NV bytes
+template <int NV>
+__device__ __forceinline__ void store_bf16(uint16_t* p, const uint32_t (&v)[NV / 2], int n, bool vec)
 {
-    const uint32_t part_row = (uint32_t)N * 32u;
-#pragma unroll
-    for (int q = 0; q < NR / 8; ++q) {
-        const int n = (lane >> 2) + 8 * q;
-        const unsigned char* p = part + (n < N ? n : 0) * 32 + (lane & 3) * 8;
-        float2 acc[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) acc[k] = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int c = 0; c < kCellWarps; ++c)
-            if (c < C) {
-                const float2 v = *(const float2*)(p + (uint32_t)c * part_row);
-                acc[c & 3].x += v.x;
-                acc[c & 3].y += v.y;
-            }
-        r[q][0] = (acc[0].x + acc[1].x) + (acc[2].x + acc[3].x);
-        r[q][1] = (acc[0].y + acc[1].y) + (acc[2].y + acc[3].y);
+    if (vec && n >= NV) {
+        if (NV == 4) *(uint2*)p = make_uint2(v[0], v[NV / 2 - 1]);
+        else *(uint32_t*)p = v[0];
+        return;
     }
+#pragma unroll
+    for (int j = 0; j < NV; ++j)
+        if (j < n) p[j] = (uint16_t)(v[j / 2] >> (16 * (j & 1)));
 }
 
 // ---- the kernel ---------------------------------------------------------------------------
@@ -565,7 +563,11 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         // weights are read once: with several stages their lines leave L2 first, so that the stream does not push out
         // the small, shared, re-read activations
         const uint64_t policy = l2_evict_first();
+#ifdef SD2_NOHINT
+        const bool hinted = false;
+#else
         const bool hinted = a.n_stages > 1;
+#endif
         const int bg = grp < kCellGroups ? grp : 0;
         const uint32_t full0 = smem_u32(&sh->full[bg][0]), empty0 = smem_u32(&sh->empty[bg][0]);
         const uint32_t ring = smem_u32(smem) + ring_off + (uint32_t)bg * NS * (uint32_t)a.chunk_bytes;
@@ -669,69 +671,90 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         const uint32_t PM = (uint32_t)a.part_mask;
         const uint32_t pfull0 = smem_u32(&sh->pfull[own][0]);
         const unsigned char* parts = smem + kPartOff + (uint32_t)own * (PM + 1u) * (uint32_t)a.part_bytes;
-        const int t2 = (lane & 3) * 2;
-        uint32_t done = 0, seq = 0;                              // tiles of this warp so far; those that were exchanged
+        constexpr int NV = NR / 4;
+        const int n = lane * NR / 32, r0 = lane * NV % kTileRows;   // panel row, first weight row of the tile
+        const bool mine = n < N;
+        const uint32_t part_row = (uint32_t)N * 32u, lane_off = mine ? (uint32_t)(lane * NR) : 0u;
+        const uint32_t peer_recv = peer_addr(&sh->recv[0][0], (uint32_t)(rank ^ 1)) + (uint32_t)(lane * NR);
+        const uint32_t peer_rfull = peer_addr(&sh->rfull[0], (uint32_t)(rank ^ 1)), peer_credit = peer_addr(&sh->credit[0], (uint32_t)(rank ^ 1));
+        const uint32_t rfull0 = smem_u32(&sh->rfull[0]), credit0 = smem_u32(&sh->credit[0]);
+        constexpr uint32_t kRecvBytes = (uint32_t)sizeof(sh->recv[0]);
+        uint32_t ps = 0, use = 0, rs = 0, ru = 0;                // slot of partial sums and its use, the same for exchanged sums
         bool ok = true;
         asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
         for (int s = 0; s < a.n_stages && ok; ++s) {
             if (!wait_phase_warp(smem_u32(&sh->xfull), (uint32_t)s & 1u, wc)) break;
             const CStage& st = sh->stage[s & 1];
             const int D = st.D, Dr = share_cells(D, rank), C = Dr < kCellWarps ? Dr : kCellWarps;
-            const bool alone = D == 1;
+            const bool alone = D == 1, pair = st.pair != 0;
             TileRuns runs(cluster, clusters, st.rot, st.tiles_div, st.tiles_rem);
             int mat, t0, nt;
-            while (ok && runs.next(st.pair, st.count, st.mat[0].T, st.mat[1].T, st.mat[2].T, mat, t0, nt)) {
+            while (ok && runs.next(pair, st.count, st.mat[0].T, st.mat[1].T, st.mat[2].T, mat, t0, nt)) {
                 if (alone && (rank || !own)) continue;           // CTA 0 has all the cells and finishes all the tiles
-                for (int j = alone ? 0 : own ? rank : rank ^ 1; j < nt; j += alone ? 1 : 2, ++done) {
-                    const uint32_t ps = done & PM, use = done / (PM + 1u);
+                const CMat& md = st.mat[mat];
+                const int M = md.M;
+                const bool f32 = md.y_f32 != 0, vec = (M & 3) == 0;
+                unsigned char* y = (unsigned char*)(s == a.n_stages - 1 && a.y_out && mat == 0 ? a.y_out : md.y);
+                const size_t at0 = (size_t)(a.n0 + n) * M + (size_t)t0 * kTileRows + r0;
+                const bool yvec = vec && (((uintptr_t)y) & 15) == 0;
+                for (int j = alone ? 0 : own ? rank : rank ^ 1; j < nt; j += alone ? 1 : 2) {
                     if (!(ok = wait_phase_warp(pfull0 + 8 * ps, use & 1u, wc))) break;
-                    float r[NR / 8][2];
-                    sum_parts<NR>(parts + ps * (uint32_t)a.part_bytes, C, N, lane, r);
+                    float r[NV];
+                    sum_parts<NV>(parts + ps * (uint32_t)a.part_bytes + lane_off, C, part_row, r);
                     __syncwarp();
                     if (lane == 0) *(volatile unsigned int*)&sh->freed[own][ps] = use + 1u;
-                    const uint32_t rs = seq % kRecvSlots, ru = seq / kRecvSlots;
+                    if (++ps > PM) { ps = 0; ++use; }
                     if (!own) {
-                        if (ru > 0 && !(ok = wait_phase_warp(smem_u32(&sh->credit[rs]), (ru - 1u) & 1u, wc))) break;
-                        const uint32_t to = peer_addr(&sh->recv[rs][0][0], (uint32_t)(rank ^ 1)), bar = peer_addr(&sh->rfull[rs], (uint32_t)(rank ^ 1));
-#pragma unroll
-                        for (int q = 0; q < NR / 8; ++q) {
-                            const int n = (lane >> 2) + 8 * q;
-                            if (n < N) st_async_f2(to + (uint32_t)(n * 4 + (lane & 3)) * 8u, make_float2(r[q][0], r[q][1]), bar);
-                        }
-                        ++seq;
+                        if (ru > 0 && !(ok = wait_phase_warp(credit0 + 8 * rs, (ru - 1u) & 1u, wc))) break;
+                        if (mine) st_async<NV>(peer_recv + rs * kRecvBytes, r, peer_rfull + 8 * rs);
+                        if (++rs == kRecvSlots) { rs = 0; ++ru; }
                         continue;
                     }
                     if (!alone) {
-                        if (lane == 0) mbar_expect_tx(smem_u32(&sh->rfull[rs]), (uint32_t)N * 32u);
-                        __syncwarp();
-                        if (!(ok = wait_phase_warp(smem_u32(&sh->rfull[rs]), ru & 1u, wc))) break;
+                        if (lane == 0) mbar_expect_tx(rfull0 + 8 * rs, part_row);
+                        if (!(ok = wait_phase_warp(rfull0 + 8 * rs, ru & 1u, wc))) break;
+                        float v[NV];
+                        if (NV == 4) *(float4*)v = *(const float4*)((const unsigned char*)&sh->recv[rs][0] + lane_off);
+                        else *(float2*)v = *(const float2*)((const unsigned char*)&sh->recv[rs][0] + lane_off);
 #pragma unroll
-                        for (int q = 0; q < NR / 8; ++q) {
-                            const int n = (lane >> 2) + 8 * q;
-                            const float2 v = sh->recv[rs][n < N ? n : 0][lane & 3];
-                            r[q][0] += v.x;
-                            r[q][1] += v.y;
-                        }
+                        for (int k = 0; k < NV; ++k) r[k] += v[k];
                         __syncwarp();
-                        if (lane == 0) mbar_arrive_remote(peer_addr(&sh->credit[rs], (uint32_t)(rank ^ 1)));
-                        ++seq;
+                        if (lane == 0) mbar_arrive_remote(peer_credit + 8 * rs);
+                        if (++rs == kRecvSlots) { rs = 0; ++ru; }
                     }
-#pragma unroll
-                    for (int q = 0; q < NR / 8; ++q) {
-                        const int n = (lane >> 2) + 8 * q;
-                        if (n >= N) continue;
-                        if (!st.pair) {
-                            const CMat& md = st.mat[mat];
-                            store_tile(md, s == a.n_stages - 1 && a.y_out && mat == 0 ? a.y_out : md.y, t0 + j, a.n0 + n, t2, r[q]);
+                    const int left = M - (t0 + j) * kTileRows - r0;          // rows of the lane that exist
+                    if (!mine || left <= 0) continue;
+                    const size_t at = at0 + (size_t)j * kTileRows;
+                    if (f32) {
+                        if (yvec && left >= NV) {
+                            if (NV == 4) *(float4*)((float*)y + at) = *(const float4*)r;
+                            else *(float2*)((float*)y + at) = *(const float2*)r;
                         } else {
-                            // gate tiles of a run wait for the up tiles of the run that follows, written and read by the same lane
-                            uint16_t* gt = &sh->gate[j % kPairSlots][n][t2];
-                            if (mat == 0) *(uint32_t*)gt = (uint32_t)f32_to_bf16_rne(r[q][0]) | ((uint32_t)f32_to_bf16_rne(r[q][1]) << 16);
-                            else store_pair(st, t0 + j, a.n0 + n, t2, gt, r[q]);
+#pragma unroll
+                            for (int k = 0; k < NV; ++k)
+                                if (k < left) ((float*)y)[at + k] = r[k];
+                        }
+                        continue;
+                    }
+                    uint32_t b[NV / 2];
+#pragma unroll
+                    for (int k = 0; k < NV / 2; ++k) b[k] = bf16_pair(r[2 * k], r[2 * k + 1]);
+                    if (y) store_bf16<NV>((uint16_t*)y + at, b, left, yvec);
+                    if (pair) {
+                        // gate tiles of a run wait for the up tiles of the run that follows, written and read by the same lane
+                        uint32_t* gt = (uint32_t*)&sh->gate[j % kPairSlots][0][0] + lane * (NV / 2);
+                        if (mat == 0) {
+#pragma unroll
+                            for (int k = 0; k < NV / 2; ++k) gt[k] = b[k];
+                        } else if (st.t_out) {
+#pragma unroll
+                            for (int k = 0; k < NV / 2; ++k) b[k] = silu_mul_pair(gt[k], b[k]);
+                            store_bf16<NV>(st.t_out + at, b, left, vec && (((uintptr_t)st.t_out) & 15) == 0);
                         }
                     }
                 }
             }
+            __syncwarp();
             if (own && ok && s + 1 < a.n_stages) {
                 __threadfence();                                 // this CTA's outputs are visible before the grid barrier counts it
                 __syncwarp();
