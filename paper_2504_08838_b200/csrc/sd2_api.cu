@@ -589,12 +589,12 @@ struct CellPlan {
     int part_bytes, n_parts, xbuf_bytes, chunk_bytes, n_slots;
 };
 
-constexpr int kCellFixedBytes = (int)((sizeof(CellShared) + 127) & ~127) + kRingGuardBytes;
+constexpr int kCellFixedBytes = (int)((sizeof(CellShared) + 127) & ~127);
 
 // Shared memory of a launch of n rows.  false: not even two chunks per group fit beside the staged rows.
 bool plan_cells(int n, const CellNeeds& needs, CellPlan* p)
 {
-    p->part_bytes = (needs.parts * n * 32 + 127) & ~127;
+    p->part_bytes = (needs.parts * n * kPartPitch + 127) & ~127;
     p->chunk_bytes = (needs.max_chunk + 127) & ~127;
     p->xbuf_bytes = (n * needs.pitch + 127) & ~127;
     for (p->n_parts = kPartSlots; p->n_parts >= 1; p->n_parts >>= 1) {     // (per finisher)

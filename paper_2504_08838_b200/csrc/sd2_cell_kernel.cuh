@@ -5,28 +5,29 @@
 // Consecutive stages depend on each other; a grid-wide barrier separates them.  (Tagged words, the hand-off of
 // sd2_kernels.cuh, double the bytes every CTA has to fetch, which is what a panel of rows cannot afford.)
 //
-// CTAs work in clusters of two.  A cluster owns a run of 8-row tiles; each of its CTAs multiplies one half of the
+// CTAs work in clusters of two.  A cluster owns a run of 16-row tiles; each of its CTAs multiplies one half of the
 // columns, so it stages half of the activations only (they are the largest thing in shared memory, and every CTA
 // fetches them through L2), and sends its sums of every other tile to the CTA that finishes that tile.
 //
-// Warps of a CTA:
-//   15 consumers, in three groups of five.  A chunk of five cells goes to a group, a cell to each of its warps.  A warp
-//              expands its cell in registers and multiplies it with mma.m16n8k16: the activation rows are the A operand
-//              (16 rows), eight weight rows the B operand, so the expanded weights never pass through shared memory.  At
-//              the end of a tile a warp leaves its 8 x N partial sums in shared memory and goes on.
+// Warps of a CTA (sixteen, four per scheduler):
+//   12 consumers, in three groups of four.  A chunk of four cells goes to a group, a cell to each of its warps.  A warp
+//              expands its cell in registers and multiplies it with mma.m16n8k16: sixteen weight rows are the A operand,
+//              eight (twice eight) activation rows the B operand, so the expanded weights never pass through shared
+//              memory.  At the end of a tile a warp leaves its 16 x N partial sums in shared memory and goes on.
 //   2 finishers: one takes the tiles this CTA finishes, one those it sends, each in order.  They add a tile's partial sums
 //              up in one fixed order (so a row's result depends neither on the launch nor on N).  The sums for the other
 //              CTA travel as asynchronous stores that count bytes on its mbarrier.  (When the consumer that brought a
 //              tile's last contribution finished it, with flags and fences, it was away for 2400 to 7000 cycles per
 //              tile: 80 us for 48 rows of an 8192 x 2048 matrix.)
 //   1 producer: one bulk asynchronous copy per chunk (13 KB at 50 % density) into the group's own ring slots.  Copies of
-//              single cells (2.7 KB) took 147 cycles each to start, 18 bytes per clock; HBM brings 23.  Nothing waits for a
-//              stage boundary: while the previous stage finishes, the next stages' weights land.
+//              13 KB reach 7 TB/s with 118 KB in flight per SM, 6.5 TB/s with 52 KB; copies of single cells of 2.7 KB
+//              1.6 TB/s from one thread (measured).  Nothing waits for a stage boundary: while the previous stage
+//              finishes, the next stages' weights land.
 //   1 service warp: waits for the grid barrier, starts the bulk copies of the stage's activation rows, and fetches the
 //              next stage's descriptor.
 //
-// What bounds it: the expansion, about 75 permute / logic instructions per warp and 1024 slots, which an SM retires at
-// two per clock (measured): 27 slots per clock and SM at most, against 17 that arrive from HBM at 50 % density.
+// What bounds it: HBM for large matrices (15 slots per clock and SM at 50 % density against 33 that twelve warps
+// expand), start-up and the stages' hand-off for small ones.
 //
 // Every wait (ring barriers, counters, grid barrier) is bounded by a cycle budget: when it runs out the CTA raises the
 // error word and winds down instead of hanging.
@@ -38,7 +39,7 @@
 
 namespace sd2 {
 
-constexpr int kCellWarps = 15;
+constexpr int kCellWarps = 12;
 constexpr int kCellGroups = 3;
 static_assert(kCellWarps == kCellGroups * kChunkCells, "a group has a warp for every cell of a chunk");
 constexpr int kCellConsumers = kCellWarps * 32;
@@ -49,7 +50,8 @@ constexpr int kPartSlots = 4;               // tiles of a finisher whose partial
 constexpr int kRecvSlots = 4;               // sums from the other CTA that wait to be used
 constexpr int kPairSlots = 8;               // gate tiles whose results wait for the up tile's
 constexpr int kPanelRows = 16;              // activation rows of a launch, at most
-constexpr int kRingGuardBytes = 256;        // the two words read past a cell's last row may lie behind the ring
+// A contribution to a tile is N rows of 16 fp32, 80 bytes apart: the lanes of a fragment store then hit 32 banks.
+constexpr int kPartPitch = 80;
 
 struct CMat {
     const uint32_t* off;           // [T * D + 1], 32-byte units into `cells`
@@ -113,7 +115,7 @@ struct CellShared {
     unsigned long long credit[kRecvSlots];              // ... the other CTA has taken ours out of its recv[]
     unsigned int freed[2][kPartSlots];                  // how often the slot's sums have been read
     uint16_t gate[kPairSlots][kPanelRows][kTileRows];   // bf16 results of gate tiles
-    float4 recv[kRecvSlots][kPanelRows * kTileRows / 4];
+    float4 recv[kRecvSlots][kPanelRows][kTileRows / 4];
     int abort_flag;                                     // any warp: a bounded wait ran out
     float red[2][kCellWarps];                           // FOLD: per-warp partial sums of squares of two rows
     CStage stage[2];                                    // descriptors of the current and the next stage
@@ -167,14 +169,10 @@ __device__ __forceinline__ uint32_t peer_addr(const void* p, uint32_t rank)
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
     return a;
 }
-// NV floats into the other CTA's shared memory, counted in bytes on its mbarrier when they are there
-template <int NV>
-__device__ __forceinline__ void st_async(uint32_t a, const float (&v)[NV], uint32_t bar)
+// four floats into the other CTA's shared memory, counted in bytes on its mbarrier when they are there
+__device__ __forceinline__ void st_async(uint32_t a, const float (&v)[4], uint32_t bar)
 {
-    if (NV == 4)
-        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(a), "f"(v[0]), "f"(v[1]), "f"(v[NV - 2]), "f"(v[NV - 1]), "r"(bar) : "memory");
-    else
-        asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(a), "f"(v[0]), "f"(v[1]), "r"(bar) : "memory");
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(a), "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "r"(bar) : "memory");
 }
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t bar)
 {
@@ -223,13 +221,6 @@ struct TileRuns {
 
 // ---- expanding a cell -----------------------------------------------------------------
 
-__device__ __forceinline__ uint32_t prmt(uint32_t a, uint32_t b, uint32_t s)
-{
-    uint32_t d;
-    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(d) : "r"(a), "r"(b), "r"(s));
-    return d;
-}
-
 // c + 128 * byte K8 of p (SGN = 1) or c - 128 * byte K8 of p (SGN = -1): one integer dot-product instruction
 template <int SGN, int K8>
 __device__ __forceinline__ uint32_t byte_times_128(uint32_t p, uint32_t c)
@@ -248,52 +239,43 @@ __device__ __forceinline__ void mma_rows(float (&d)[4], uint32_t a0, uint32_t a1
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// Selector tables for prmt, indexed by the two mask bits of a pair of slots (bit 0: low slot kept).  Bytes 0-3 serve
-// front pairs (the next halfword of the stream is the low half of the window), bytes 4-7 back pairs (it is the high
-// half).  S: places the window's halfwords in the pair's register, zeros (bytes 4..7 of prmt's second operand) for
-// dropped slots.  H: moves the window on by the pair's kept halfwords.
-constexpr uint32_t kSFrontLo = 0x10441044u, kSFrontHi = 0x32104444u, kSBackLo = 0x10443244u, kSBackHi = 0x32324444u;
-constexpr uint32_t kHFrontLo = 0x54323210u, kHFrontHi = 0x76545432u, kHBackLo = 0x10323254u, kHBackHi = 0x32545476u;
-
-// Half a cell: eight mma steps.  m: the lane's mask; base: byte offset in shared memory of the lane's first word (words
-// 128 bytes apart, upward for SGN = 1); xo, xo8: byte offsets of the lane's first eight activations in rows g and g + 8.
-template <int NR, int SGN>
-__device__ __forceinline__ void half_cell(const unsigned char* smem, uint32_t m, uint32_t base, uint32_t xo, uint32_t xo8,
-                                          float (&af)[4], float (&ab)[4])
+// One unit of a row: its four pairs' words, zero where a pair has none.  nib: the unit's mask bits; at: shared address of
+// the row's next word (words 128 bytes apart, upward for SGN = 1), moved on.
+template <int SGN>
+__device__ __forceinline__ void load_pairs(uint32_t nib, uint32_t& at, uint32_t (&w)[4])
 {
-    // words of each unit: (kept + 1) / 2, then their running sum, one byte per unit
-    const uint32_t p2 = m - ((m >> 1) & 0x55555555u);
-    const uint32_t p4 = (p2 & 0x33333333u) + ((p2 >> 2) & 0x33333333u);
-    const uint32_t p8 = (p4 + (p4 >> 4)) & 0x0F0F0F0Fu;
-    const uint32_t ends = (((p8 + 0x01010101u) >> 1) & 0x07070707u) * 0x01010101u;
-    // selectors of the first (E) and second (O) pair of every group of four slots, byte-wise by table
-    const uint32_t E = (m & 0x33333333u) | 0x40404040u, O = ((m >> 2) & 0x33333333u) | 0x40404040u;
-    constexpr uint32_t kStep = (uint32_t)(128 * SGN);
-    uint32_t start = base;
+    // byte i: words of pairs 0..i
+    const uint32_t upto = ((nib * 0x00204081u) & 0x01010101u) * 0x01010101u;
+    const uint32_t a1 = byte_times_128<SGN, 0>(upto, at), a2 = byte_times_128<SGN, 1>(upto, at), a3 = byte_times_128<SGN, 2>(upto, at);
+    asm volatile("{\n\t.reg .pred p0, p1, p2, p3;\n\t.reg .b32 t0, t1, t2, t3;\n\t"
+                 "and.b32 t0, %8, 1;\n\tand.b32 t1, %8, 2;\n\tand.b32 t2, %8, 4;\n\tand.b32 t3, %8, 8;\n\t"
+                 "setp.ne.u32 p0, t0, 0;\n\tsetp.ne.u32 p1, t1, 0;\n\tsetp.ne.u32 p2, t2, 0;\n\tsetp.ne.u32 p3, t3, 0;\n\t"
+                 "mov.b32 %0, 0;\n\tmov.b32 %1, 0;\n\tmov.b32 %2, 0;\n\tmov.b32 %3, 0;\n\t"
+                 "@p0 ld.shared.u32 %0, [%4];\n\t@p1 ld.shared.u32 %1, [%5];\n\t@p2 ld.shared.u32 %2, [%6];\n\t@p3 ld.shared.u32 %3, [%7];\n\t}"
+                 : "=&r"(w[0]), "=&r"(w[1]), "=&r"(w[2]), "=&r"(w[3])
+                 : "r"(at), "r"(a1), "r"(a2), "r"(a3), "r"(nib)
+                 : "memory");
+    at = byte_times_128<SGN, 3>(upto, at);
+}
+
+// One cell: eight mma steps for each eight activation rows.  m: the lane's mask; lo, hi: shared addresses of the first
+// words of its rows g and g + 8; xo, xo8: of the first eight activations of panel rows g and g + 8.
+// Two sets of sums per eight rows keep two chains of mma in flight.
+template <int NR>
+__device__ __forceinline__ void multiply_cell(uint32_t m, uint32_t lo, uint32_t hi, uint32_t xo, uint32_t xo8, float (&c)[NR / 4][4])
+{
 #pragma unroll
-    for (int t = 0; t < 2; ++t) {
-        const uint32_t e = E >> (16 * t), o = O >> (16 * t);
-        const uint32_t sl = prmt(kSFrontLo, kSBackLo, e), sh = prmt(kSFrontHi, kSBackHi, e);
-        const uint32_t hl = prmt(kHFrontLo, kHBackLo, e), hh = prmt(kHFrontHi, kHBackHi, e);
-        const uint32_t ol = prmt(kSFrontLo, kSBackLo, o), oh = prmt(kSFrontHi, kSBackHi, o);
-#pragma unroll
-        for (int v = 0; v < 2; ++v) {
-            const int u = 2 * t + v;
-            const uint32_t end = u == 0 ? byte_times_128<SGN, 0>(ends, base) : u == 1 ? byte_times_128<SGN, 1>(ends, base)
-                               : u == 2 ? byte_times_128<SGN, 2>(ends, base) : byte_times_128<SGN, 3>(ends, base);
-            const uint32_t wa = *(const uint32_t*)(smem + start), wb = *(const uint32_t*)(smem + (start + kStep));
-            const uint32_t wz = *(const uint32_t*)(smem + (end - kStep)), wy = *(const uint32_t*)(smem + (end - 2 * kStep));
-            const uint4 xv = *(const uint4*)(smem + (xo + 64u * u));
-            uint4 xw = make_uint4(0u, 0u, 0u, 0u);
-            if (NR > 8) xw = *(const uint4*)(smem + (xo8 + 64u * u));
-            const uint32_t pf = v == 0 ? 0x0040u : 0x0062u, pb = v == 0 ? 0x0051u : 0x0073u;   // byte k of the low and of the high result
-            const uint32_t f0 = prmt(wa, 0u, prmt(sl, sh, pf));
-            const uint32_t f1 = prmt(prmt(wa, wb, prmt(hl, hh, pf)), 0u, prmt(ol, oh, pf));
-            mma_rows(af, xv.x, xw.x, xv.y, xw.y, f0, f1);
-            const uint32_t b0 = prmt(wz, 0u, prmt(sl, sh, pb));
-            const uint32_t b1 = prmt(prmt(wy, wz, prmt(hl, hh, pb)), 0u, prmt(ol, oh, pb));
-            mma_rows(ab, xv.z, xw.z, xv.w, xw.w, b0, b1);
-            start = end;
+    for (int u = 0; u < 4; ++u) {
+        uint32_t a[4], b[4];
+        load_pairs<1>((m >> (4 * u)) & 0xFu, lo, a);
+        load_pairs<-1>((m >> (16 + 4 * u)) & 0xFu, hi, b);
+        const uint4 x = lds_v4(xo + 64u * u);
+        mma_rows(c[0], a[0], b[0], a[1], b[1], x.x, x.y);
+        mma_rows(c[1], a[2], b[2], a[3], b[3], x.z, x.w);
+        if (NR > 8) {
+            const uint4 y = lds_v4(xo8 + 64u * u);
+            mma_rows(c[NR / 4 - 2], a[0], b[0], a[1], b[1], y.x, y.y);
+            mma_rows(c[NR / 4 - 1], a[2], b[2], a[3], b[3], y.z, y.w);
         }
     }
 }
@@ -422,33 +404,32 @@ __device__ __noinline__ bool fold_norm(const XRows& r, const SFold& f, const uin
 
 // ---- finishing a tile ---------------------------------------------------------------------
 
-// A finisher shares its scheduler with four or five busy warps and gets an instruction in every few cycles, so what counts
-// here is the number of instructions per tile.  Lane l holds the NR / 4 results that stand together at l * NR bytes of a
-// contribution (N x 8 fp32): panel row l * NR / 32, NR / 4 consecutive weight rows.
+// A finisher shares its scheduler with busy warps and gets an instruction in every few cycles, so what counts here is the
+// number of instructions per tile.  Lane 4 n + t holds weight rows 4 t .. 4 t + 3 of panel rows n and n + 8.
 
 // The sum of a tile's C contributions: four running sums, then one tree, an order that depends neither on N nor on the CTA.
-template <int NV>
-__device__ __forceinline__ void sum_parts(const unsigned char* p, int C, uint32_t part_row, float (&r)[NV])
+__device__ __forceinline__ void sum_parts(const unsigned char* p, int C, uint32_t part_row, float (&r)[4])
 {
-    float acc[4][NV];
+    float acc[4][4];
 #pragma unroll
     for (int k = 0; k < 4; ++k)
 #pragma unroll
-        for (int j = 0; j < NV; ++j) acc[k][j] = 0.f;
+        for (int j = 0; j < 4; ++j) acc[k][j] = 0.f;
     for (int c = 0; c < C; c += 4) {
-        float v[4][NV];
+        float4 v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = *(const float4*)(p + (uint32_t)min(c + k, C - 1) * part_row);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            if (NV == 4) *(float4*)v[k] = *(const float4*)(p + (uint32_t)min(c + k, C - 1) * part_row);
-            else *(float2*)v[k] = *(const float2*)(p + (uint32_t)min(c + k, C - 1) * part_row);
+            const bool there = c + k < C;
+            acc[k][0] += there ? v[k].x : 0.f;
+            acc[k][1] += there ? v[k].y : 0.f;
+            acc[k][2] += there ? v[k].z : 0.f;
+            acc[k][3] += there ? v[k].w : 0.f;
         }
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-#pragma unroll
-            for (int j = 0; j < NV; ++j) acc[k][j] += c + k < C ? v[k][j] : 0.f;
     }
 #pragma unroll
-    for (int j = 0; j < NV; ++j) r[j] = (acc[0][j] + acc[1][j]) + (acc[2][j] + acc[3][j]);
+    for (int j = 0; j < 4; ++j) r[j] = (acc[0][j] + acc[1][j]) + (acc[2][j] + acc[3][j]);
 }
 
 __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi)
@@ -458,18 +439,17 @@ __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi)
     return d;
 }
 
-// NV consecutive bf16 values to p, of which `n` exist; vec: p is aligned to 2 NV bytes
-template <int NV>
-__device__ __forceinline__ void store_bf16(uint16_t* p, const uint32_t (&v)[NV / 2], int n, bool vec)
+// four consecutive bf16 values to p, of which `n` exist; vec: p is aligned to eight bytes
+__device__ __forceinline__ void store_bf16(uint16_t* p, uint2 v, int n, bool vec)
 {
-    if (vec && n >= NV) {
-        if (NV == 4) *(uint2*)p = make_uint2(v[0], v[NV / 2 - 1]);
-        else *(uint32_t*)p = v[0];
+    if (vec && n >= 4) {
+        *(uint2*)p = v;
         return;
     }
-#pragma unroll
-    for (int j = 0; j < NV; ++j)
-        if (j < n) p[j] = (uint16_t)(v[j / 2] >> (16 * (j & 1)));
+    if (n > 0) p[0] = (uint16_t)v.x;
+    if (n > 1) p[1] = (uint16_t)(v.x >> 16);
+    if (n > 2) p[2] = (uint16_t)v.y;
+    if (n > 3) p[3] = (uint16_t)(v.y >> 16);
 }
 
 // ---- the kernel ---------------------------------------------------------------------------
@@ -519,14 +499,15 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
 #define SD2_FIELD(f) (a.ext ? a.ext[sa].f : a.inl[MAXS == 1 ? 0 : sa].f)
     if (warp == kProducerWarp) {
         // ---------------------------------------------------------------------- producer
-        // Rounds of one chunk per group; lane 5 g + j stands for cell j of group g's chunk.  A round's directory entries are
-        // loaded four rounds ahead, so their latency (and a stage's fields') stays off the ring's critical path.
+        // The chunks of all stages, numbered through, go to the groups in turn; a round is one chunk per group.  Lane
+        // 4 g + j stands for cell j of group g's chunk.  A round's directory entries are loaded four rounds ahead, so
+        // their latency (and a stage's fields') stays off the ring's critical path.
         struct PRound {
             uint32_t o0, o1;                 // directory entries of the lane's cell; equal: none
-            const unsigned char* cells;
+            const unsigned char* cells;      // NULL: the lane's group has come to the end
         };
         const int grp = lane / kChunkCells, cj = lane - grp * kChunkCells;
-        int sa = 0, qa = 0, n = 0, n_chunks = 0, gb = 0;
+        int sa = 0, q = grp, n = 0, n_chunks = 0;                // stage, chunk of the current run of tiles, the run's cells and chunks
         const uint32_t* off = nullptr;
         const unsigned char* cells = nullptr;
         TileRuns runs(cluster, clusters, SD2_FIELD(rot), SD2_FIELD(tiles_div), SD2_FIELD(tiles_rem));
@@ -534,9 +515,10 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
             PRound c;
             c.o0 = c.o1 = 0u;
             c.cells = nullptr;
-            while (qa >= n_chunks) {         // on to the next run of tiles, the next stage
-                gb = (gb + n_chunks) % kCellGroups;
-                qa = n = n_chunks = 0;
+            if (grp >= kCellGroups || sa >= a.n_stages) return c;
+            while (q >= n_chunks) {          // on to the next run of tiles, the next stage
+                q -= n_chunks;
+                n = n_chunks = 0;
                 int mat, t0, nt;
                 if (runs.next(SD2_FIELD(pair), SD2_FIELD(count), SD2_FIELD(mat[0].T), SD2_FIELD(mat[1].T), SD2_FIELD(mat[2].T), mat, t0, nt)) {
                     const int D = SD2_FIELD(D), Dr = share_cells(D, rank);
@@ -549,32 +531,26 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                 if (++sa >= a.n_stages) return c;
                 runs = TileRuns(cluster, clusters, SD2_FIELD(rot), SD2_FIELD(tiles_div), SD2_FIELD(tiles_rem));
             }
-            int g = grp - gb;
-            if (g < 0) g += kCellGroups;
-            const int i = (qa + g) * kChunkCells + cj;
-            if (lane < kCellWarps && i < n) {
+            const int i = q * kChunkCells + cj;
+            if (i < n) {
                 c.o0 = __ldg(off + i);
                 c.o1 = __ldg(off + i + 1);
             }
             c.cells = cells;
-            qa += kCellGroups;
+            q += kCellGroups;
             return c;
         };
         // weights are read once: with several stages their lines leave L2 first, so that the stream does not push out
         // the small, shared, re-read activations
         const uint64_t policy = l2_evict_first();
-#ifdef SD2_NOHINT
-        const bool hinted = false;
-#else
         const bool hinted = a.n_stages > 1;
-#endif
         const int bg = grp < kCellGroups ? grp : 0;
         const uint32_t full0 = smem_u32(&sh->full[bg][0]), empty0 = smem_u32(&sh->empty[bg][0]);
         const uint32_t ring = smem_u32(smem) + ring_off + (uint32_t)bg * NS * (uint32_t)a.chunk_bytes;
         uint32_t slot = 0, phase = 1, issued = 0;                // of the lane's group
         bool ok = true;
         PRound c0 = load_round(), c1 = load_round(), c2 = load_round(), c3 = load_round();
-        while (c0.cells) {
+        while (__any_sync(0xFFFFFFFFu, c0.cells != nullptr)) {
             const bool mine = c0.o1 != c0.o0;
             const uint32_t start = __shfl_sync(0xFFFFFFFFu, c0.o0, bg * kChunkCells);
             uint32_t end = start;
@@ -671,11 +647,9 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         const uint32_t PM = (uint32_t)a.part_mask;
         const uint32_t pfull0 = smem_u32(&sh->pfull[own][0]);
         const unsigned char* parts = smem + kPartOff + (uint32_t)own * (PM + 1u) * (uint32_t)a.part_bytes;
-        constexpr int NV = NR / 4;
-        const int n = lane * NR / 32, r0 = lane * NV % kTileRows;   // panel row, first weight row of the tile
-        const bool mine = n < N;
-        const uint32_t part_row = (uint32_t)N * 32u, lane_off = mine ? (uint32_t)(lane * NR) : 0u;
-        const uint32_t peer_recv = peer_addr(&sh->recv[0][0], (uint32_t)(rank ^ 1)) + (uint32_t)(lane * NR);
+        const int n0 = lane >> 2, r0 = (lane & 3) * 4;
+        const uint32_t part_row = (uint32_t)(N * kPartPitch), recv_off = (uint32_t)lane * 16u;
+        const uint32_t peer_recv = peer_addr(&sh->recv[0][0][0], (uint32_t)(rank ^ 1)) + recv_off;
         const uint32_t peer_rfull = peer_addr(&sh->rfull[0], (uint32_t)(rank ^ 1)), peer_credit = peer_addr(&sh->credit[0], (uint32_t)(rank ^ 1));
         const uint32_t rfull0 = smem_u32(&sh->rfull[0]), credit0 = smem_u32(&sh->credit[0]);
         constexpr uint32_t kRecvBytes = (uint32_t)sizeof(sh->recv[0]);
@@ -695,61 +669,62 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                 const int M = md.M;
                 const bool f32 = md.y_f32 != 0, vec = (M & 3) == 0;
                 unsigned char* y = (unsigned char*)(s == a.n_stages - 1 && a.y_out && mat == 0 ? a.y_out : md.y);
-                const size_t at0 = (size_t)(a.n0 + n) * M + (size_t)t0 * kTileRows + r0;
                 const bool yvec = vec && (((uintptr_t)y) & 15) == 0;
                 for (int j = alone ? 0 : own ? rank : rank ^ 1; j < nt; j += alone ? 1 : 2) {
                     if (!(ok = wait_phase_warp(pfull0 + 8 * ps, use & 1u, wc))) break;
-                    float r[NV];
-                    sum_parts<NV>(parts + ps * (uint32_t)a.part_bytes + lane_off, C, part_row, r);
+                    float r[NR / 8][4];
+#pragma unroll
+                    for (int h = 0; h < NR / 8; ++h)
+                        sum_parts(parts + ps * (uint32_t)a.part_bytes + (uint32_t)(min(n0 + 8 * h, N - 1) * kPartPitch + r0 * 4), C, part_row, r[h]);
                     __syncwarp();
                     if (lane == 0) *(volatile unsigned int*)&sh->freed[own][ps] = use + 1u;
                     if (++ps > PM) { ps = 0; ++use; }
                     if (!own) {
                         if (ru > 0 && !(ok = wait_phase_warp(credit0 + 8 * rs, (ru - 1u) & 1u, wc))) break;
-                        if (mine) st_async<NV>(peer_recv + rs * kRecvBytes, r, peer_rfull + 8 * rs);
+#pragma unroll
+                        for (int h = 0; h < NR / 8; ++h)
+                            if (n0 + 8 * h < N) st_async(peer_recv + rs * kRecvBytes + 512u * h, r[h], peer_rfull + 8 * rs);
                         if (++rs == kRecvSlots) { rs = 0; ++ru; }
                         continue;
                     }
                     if (!alone) {
-                        if (lane == 0) mbar_expect_tx(rfull0 + 8 * rs, part_row);
+                        if (lane == 0) mbar_expect_tx(rfull0 + 8 * rs, (uint32_t)N * 64u);
                         if (!(ok = wait_phase_warp(rfull0 + 8 * rs, ru & 1u, wc))) break;
-                        float v[NV];
-                        if (NV == 4) *(float4*)v = *(const float4*)((const unsigned char*)&sh->recv[rs][0] + lane_off);
-                        else *(float2*)v = *(const float2*)((const unsigned char*)&sh->recv[rs][0] + lane_off);
 #pragma unroll
-                        for (int k = 0; k < NV; ++k) r[k] += v[k];
+                        for (int h = 0; h < NR / 8; ++h) {
+                            const float4 v = *(const float4*)((const unsigned char*)&sh->recv[rs][0][0] + recv_off + 512u * h);
+                            r[h][0] += v.x;
+                            r[h][1] += v.y;
+                            r[h][2] += v.z;
+                            r[h][3] += v.w;
+                        }
                         __syncwarp();
                         if (lane == 0) mbar_arrive_remote(peer_credit + 8 * rs);
                         if (++rs == kRecvSlots) { rs = 0; ++ru; }
                     }
                     const int left = M - (t0 + j) * kTileRows - r0;          // rows of the lane that exist
-                    if (!mine || left <= 0) continue;
-                    const size_t at = at0 + (size_t)j * kTileRows;
-                    if (f32) {
-                        if (yvec && left >= NV) {
-                            if (NV == 4) *(float4*)((float*)y + at) = *(const float4*)r;
-                            else *(float2*)((float*)y + at) = *(const float2*)r;
-                        } else {
 #pragma unroll
-                            for (int k = 0; k < NV; ++k)
-                                if (k < left) ((float*)y)[at + k] = r[k];
+                    for (int h = 0; h < NR / 8; ++h) {
+                        const int n = n0 + 8 * h;
+                        if (n >= N || left <= 0) continue;
+                        const size_t at = (size_t)(a.n0 + n) * M + (size_t)(t0 + j) * kTileRows + r0;
+                        if (f32) {
+                            if (yvec && left >= 4) {
+                                *(float4*)((float*)y + at) = make_float4(r[h][0], r[h][1], r[h][2], r[h][3]);
+                            } else {
+#pragma unroll
+                                for (int k = 0; k < 4; ++k)
+                                    if (k < left) ((float*)y)[at + k] = r[h][k];
+                            }
+                            continue;
                         }
-                        continue;
-                    }
-                    uint32_t b[NV / 2];
-#pragma unroll
-                    for (int k = 0; k < NV / 2; ++k) b[k] = bf16_pair(r[2 * k], r[2 * k + 1]);
-                    if (y) store_bf16<NV>((uint16_t*)y + at, b, left, yvec);
-                    if (pair) {
-                        // gate tiles of a run wait for the up tiles of the run that follows, written and read by the same lane
-                        uint32_t* gt = (uint32_t*)&sh->gate[j % kPairSlots][0][0] + lane * (NV / 2);
-                        if (mat == 0) {
-#pragma unroll
-                            for (int k = 0; k < NV / 2; ++k) gt[k] = b[k];
-                        } else if (st.t_out) {
-#pragma unroll
-                            for (int k = 0; k < NV / 2; ++k) b[k] = silu_mul_pair(gt[k], b[k]);
-                            store_bf16<NV>(st.t_out + at, b, left, vec && (((uintptr_t)st.t_out) & 15) == 0);
+                        const uint2 b = make_uint2(bf16_pair(r[h][0], r[h][1]), bf16_pair(r[h][2], r[h][3]));
+                        if (y) store_bf16((uint16_t*)y + at, b, left, yvec);
+                        if (pair) {
+                            // gate tiles of a run wait for the up tiles of the run that follows, written and read by the same lane
+                            uint2* gt = (uint2*)&sh->gate[j % kPairSlots][n][r0];
+                            if (mat == 0) *gt = b;
+                            else if (st.t_out) store_bf16(st.t_out + at, make_uint2(silu_mul_pair(gt->x, b.x), silu_mul_pair(gt->y, b.y)), left, vec && (((uintptr_t)st.t_out) & 15) == 0);
                         }
                     }
                 }
@@ -772,7 +747,8 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         const int grp = warp / kChunkCells, cj = warp - grp * kChunkCells;
         const uint32_t full0 = smem_u32(&sh->full[grp][0]), empty0 = smem_u32(&sh->empty[grp][0]);
         const uint32_t xfull = smem_u32(&sh->xfull);
-        const uint32_t ring = ring_off + (uint32_t)grp * NS * (uint32_t)a.chunk_bytes;
+        const uint32_t sbase = smem_u32(smem);
+        const uint32_t ring = sbase + ring_off + (uint32_t)grp * NS * (uint32_t)a.chunk_bytes;
         const int g = lane >> 2;
         const int xrow = g < N ? g : 0, xrow8 = g + 8 < N ? g + 8 : 0;   // rows beyond N repeat row 0; their sums are never read
         ConsumerSync sync;
@@ -812,7 +788,7 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
             }
             const uint32_t C = (uint32_t)(Dr < kCellWarps ? Dr : kCellWarps);
             const bool alone = D == 1;
-            const uint32_t xl = xoff + (uint32_t)(xrow * pitch) + 16u * (lane & 3), xl8 = xoff + (uint32_t)(xrow8 * pitch) + 16u * (lane & 3);
+            const uint32_t xl = sbase + xoff + (uint32_t)(xrow * pitch) + 16u * (lane & 3), xl8 = sbase + xoff + (uint32_t)(xrow8 * pitch) + 16u * (lane & 3);
             TileRuns runs(cluster, clusters, st.rot, st.tiles_div, st.tiles_rem);
             int mat, t0, nt;
             while (!failed && runs.next(st.pair, st.count, st.mat[0].T, st.mat[1].T, st.mat[2].T, mat, t0, nt)) {
@@ -821,18 +797,20 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                 if (q < 0) q += kCellGroups;
                 int i = q * kChunkCells + cj;
                 int tl = Dr > 0 ? i / Dr : 0, d = i - tl * Dr, c0 = d;
-                float af[4] = {0.f, 0.f, 0.f, 0.f}, ab[4] = {0.f, 0.f, 0.f, 0.f};
+                float acc[NR / 4][4];
+#pragma unroll
+                for (int m = 0; m < NR / 4; ++m)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) acc[m][k] = 0.f;
                 for (; q < n_chunks; q += kCellGroups, i += kCellWarps) {
                     if (!wait_phase_warp(full0 + 8 * slot, phase, wc)) { failed = true; break; }
                     if (i < n) {
                         const uint32_t where = sh->cell[grp][slot][cj];
                         const uint32_t cell = ring + slot * (uint32_t)a.chunk_bytes + (where >> 8), H = where & 0xFFu;
-                        const uint32_t ma = *(const uint32_t*)(smem + cell + 4 * lane), mb = *(const uint32_t*)(smem + cell + 128 + 4 * lane);
-                        const uint32_t pi = *(smem + cell + 256 + lane);
-                        const uint32_t xd = (uint32_t)d * (2 * kCellCols), v0 = cell + kCellHeaderBytes;
-                        half_cell<NR, 1>(smem, ma, v0 + 4u * lane, xl + xd, xl8 + xd, af, ab);
-                        if (d * kCellCols + kHalfCols < Kr)
-                            half_cell<NR, -1>(smem, mb, v0 + (H - 1u) * 128u + pi, xl + xd + 2 * kHalfCols, xl8 + xd + 2 * kHalfCols, af, ab);
+                        const uint32_t m = lds_u32(cell + 4 * lane), v0 = cell + kCellHeaderBytes;
+                        const uint32_t pi = *(smem + (cell - sbase) + 128 + lane);
+                        const uint32_t xd = (uint32_t)d * (2 * kCellCols);
+                        multiply_cell<NR>(m, v0 + 4u * lane, v0 + (H - 1u) * 128u + pi, xl + xd, xl8 + xd, acc);
                     }
                     __syncwarp();
                     if (lane == 0) mbar_arrive(empty0 + 8 * slot);
@@ -846,14 +824,24 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                         const uint32_t k = (own ? cnt[1] : cnt[0]) + (uint32_t)(alone ? tl : tl >> 1);
                         const uint32_t ps = k & (uint32_t)a.part_mask, use = k / ((uint32_t)a.part_mask + 1u);
                         if (use > 0 && !wait_count(&sh->freed[own][ps], use, wc)) { failed = true; break; }
-                        unsigned char* p = smem + kPartOff + ((uint32_t)own * ((uint32_t)a.part_mask + 1u) + ps) * (uint32_t)a.part_bytes +
-                                           (uint32_t)(c0 * N + g) * 32u + (lane & 3) * 8;
-                        if (g < N) *(float2*)p = make_float2(af[0] + ab[0], af[1] + ab[1]);
-                        if (NR > 8 && g + 8 < N) *(float2*)(p + 256) = make_float2(af[2] + ab[2], af[3] + ab[3]);
+                        float* p = (float*)(smem + kPartOff + ((uint32_t)own * ((uint32_t)a.part_mask + 1u) + ps) * (uint32_t)a.part_bytes +
+                                            (uint32_t)(c0 * N * kPartPitch)) + g;
 #pragma unroll
-                        for (int m = 0; m < 4; ++m) af[m] = ab[m] = 0.f;
+                        for (int h = 0; h < NR / 8; ++h)
+#pragma unroll
+                            for (int k = 0; k < 2; ++k) {
+                                const int n = (lane & 3) * 2 + k + 8 * h;
+                                if (n < N) {
+                                    p[n * (kPartPitch / 4)] = acc[2 * h][k] + acc[2 * h + 1][k];
+                                    p[n * (kPartPitch / 4) + 8] = acc[2 * h][k + 2] + acc[2 * h + 1][k + 2];
+                                }
+                            }
+#pragma unroll
+                        for (int m = 0; m < NR / 4; ++m)
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) acc[m][k] = 0.f;
                         __syncwarp();
-                        // the C contributions make 15 arrivals between them
+                        // the C contributions make 12 arrivals between them
                         if (lane == 0) mbar_arrive_n(smem_u32(&sh->pfull[own][ps]), c0 == 0 ? kCellWarps + 1u - C : 1u);
                     }
                     do { d -= Dr; ++tl; } while (d >= Dr);

@@ -1,28 +1,26 @@
 // Cells: the device layout of a GAP4 handle for panels of activation rows, in the order of a tensor-core operand.
 //
 // The strip layout (sd2_format.hpp) is built to be gathered from, entry by entry; its work grows with every activation
-// row.  For several rows a handle also keeps this one: a bitmask (one bit per dense slot) plus the packed kept values,
-// arranged so that a warp turns a compressed cell into the B fragments of mma.m16n8k16 (8 weight rows x 16 columns)
-// with table look-ups by byte permutation, whatever the pattern:
+// row.  For several rows a handle also keeps this one, which a warp turns into the A fragments of mma.m16n8k16 (16 weight
+// rows x 16 columns) whatever the pattern:
 //
-//   - Rows are cut into tiles of 8, columns into cells of 256 = two halves of 128.  A warp takes one cell of one
-//     tile.  Lane l = 4 g + t holds weight row g; of half h it owns, for u = 0..3, the eight columns
-//     128 h + 32 u + 8 t + i, i = 0..7: a *unit*.  Slots 0..3 of a unit feed one mma step, slots 4..7 the next.
-//   - mask[h][l] has bit 8 u + i set iff the slot is kept.
-//   - A unit's kept values fill whole 32-bit words from both ends: slots 0..3 from the front (a pair of slots that are
-//     both kept takes two halfwords, low slot first; a single one takes one), slots 4..7 from the back (a pair's
-//     high slot takes the later halfword).  An odd count leaves one halfword of zero in the middle.  So the four
-//     values a step needs sit in the first two or the last two words of the unit, at a place that follows from the
-//     mask alone, and two byte permutations per register put them (and zeros) where the tensor core wants them.
-//   - The words of a lane's four units of half 0 stand one above the other in column l of a matrix of H rows x 32
-//     words, from row 0 up; those of half 1 in column pi(l), from row H - 1 down.  pi matches lanes with many words
-//     in half 0 to lanes with few in half 1, which keeps H close to the mean (18.7 rows where 18.0 words are used,
-//     at 50 % density).  Whatever rows 32 lanes read, they read 32 different banks.
+//   - Rows are cut into tiles of 16, columns into cells of 128.  A warp takes one cell of one tile.  Lane l = 4 g + t holds
+//     weight rows g and g + 8; of each it owns, for u = 0..3, the eight columns 32 u + 8 t + i, i = 0..7: four *pairs*
+//     of neighbours.  Pairs 0 and 1 of a unit feed one mma step, pairs 2 and 3 the next.
+//   - A pair of which anything is kept is one 32-bit word (the low column in the low half, zero for a dropped one); the
+//     others take no room.  mask[l] has bit 16 r + 4 u + i set iff pair i of unit u of row g + 8 r has a word.
+//   - The words of a lane's row g stand one above the other in column l of a matrix of H rows x 32 words, from row 0 up;
+//     those of row g + 8 in column pi(l), from row H - 1 down.  pi matches lanes with many words in one row to lanes
+//     with few in the other, which keeps H close to the mean.  Whatever rows 32 lanes read, they read 32 different banks.
+//
+// Bytes per dense slot at 50 % density: 1.61 (three of four pairs have a word; the strips take 1.28).  Packing the values
+// without the pairs' zeros takes 1.39, but its expansion by byte permutations ran at 18 slots per clock and SM; this
+// one, a predicated load per pair, runs at 33 (29 for sixteen activation rows), and HBM brings 15.
 //
 // Two CTAs share a tile: one takes the first ceil(D / 2) cells of its columns, the other the rest.  The cells of each
 // share stand together, tile by tile, so that a CTA's run of tiles is one run of bytes.
 //
-//   cell    u32 mask[2][32], u8 pi[32] (4 x column), u32 words[H][32]
+//   cell    u32 mask[32], u8 pi[32] (4 x column), u32 words[H][32]
 //   sec0    u32 cell_off[T * D + 1] (32-byte units into sec1), in order of share, then tile, then column
 //   sec1    cells
 
@@ -32,12 +30,11 @@
 
 namespace sd2 {
 
-constexpr int kTileRows = 8;
-constexpr int kCellCols = 256;
-constexpr int kHalfCols = 128;
-constexpr int kCellHeaderBytes = 2 * 128 + 32;
+constexpr int kTileRows = 16;
+constexpr int kCellCols = 128;
+constexpr int kCellHeaderBytes = 128 + 32;
 
-constexpr int kChunkCells = 5;        // consecutive cells of a share that travel in one copy, at most
+constexpr int kChunkCells = 4;        // consecutive cells of a share that travel in one copy, at most
 
 struct CellGeom {
     int64_t T;        // row tiles
@@ -65,57 +62,47 @@ struct CellImage {
 // One cell of the tile that starts at row m0, columns from k0; appended to `out`.
 inline void pack_cell(const uint16_t* W, const uint8_t* mask, int64_t M, int64_t K, int64_t m0, int64_t k0, std::vector<uint8_t>& out)
 {
-    uint32_t bits[2][32];
+    uint32_t bits[32];
     uint32_t words[2][32][16];
     uint8_t n_words[2][32];
     std::memset(bits, 0, sizeof bits);
     std::memset(n_words, 0, sizeof n_words);
-    for (int g = 0; g < kTileRows && m0 + g < M; ++g) {
-        const uint16_t* wr = W + (m0 + g) * K;
-        const uint8_t* mr = mask ? mask + (m0 + g) * K : nullptr;
-        for (int h = 0; h < 2; ++h)
-            for (int u = 0; u < 4; ++u)
-                for (int t = 0; t < 4; ++t) {
-                    const int l = 4 * g + t;
-                    const int64_t c0 = k0 + kHalfCols * h + 32 * u + 8 * t;
-                    const int nc = c0 >= K ? 0 : (int)(K - c0 < 8 ? K - c0 : 8);
-                    uint32_t b = 0;
-                    if (mr) { for (int i = 0; i < nc; ++i) b |= (mr[c0 + i] ? 1u : 0u) << i; }
-                    else { for (int i = 0; i < nc; ++i) b |= ((wr[c0 + i] & 0x7FFF) ? 1u : 0u) << i; }
-                    if (!b) continue;
-                    bits[h][l] |= b << (8 * u);
-                    const int nw = (__builtin_popcount(b) + 1) / 2;
-                    uint16_t hw[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-                    int f = 0, e = 2 * nw - 1;
-                    for (int i = 0; i < 4; ++i)
-                        if (b >> i & 1) hw[f++] = wr[c0 + i];
-                    for (int i = 4; i < 8; i += 2) {
-                        if (b >> (i + 1) & 1) hw[e--] = wr[c0 + i + 1];
-                        if (b >> i & 1) hw[e--] = wr[c0 + i];
-                    }
-                    std::memcpy(words[h][l] + n_words[h][l], hw, (size_t)nw * 4);
-                    n_words[h][l] = (uint8_t)(n_words[h][l] + nw);
-                }
+    for (int row = 0; row < kTileRows && m0 + row < M; ++row) {
+        const uint16_t* wr = W + (m0 + row) * K;
+        const uint8_t* mr = mask ? mask + (m0 + row) * K : nullptr;
+        const int r = row >> 3;
+        const int64_t left = K - k0;
+        const int cols = left < kCellCols ? (int)left : kCellCols;
+        for (int c = 0; c < cols; c += 2) {
+            const int l = 4 * (row & 7) + ((c >> 3) & 3);
+            const bool two = c + 1 < cols;
+            const uint32_t lo = wr[k0 + c], hi = two ? wr[k0 + c + 1] : 0u;
+            const bool klo = mr ? mr[k0 + c] != 0 : (lo & 0x7FFF) != 0;
+            const bool khi = two && (mr ? mr[k0 + c + 1] != 0 : (hi & 0x7FFF) != 0);
+            if (!klo && !khi) continue;
+            bits[l] |= 1u << (16 * r + 4 * (c >> 5) + ((c >> 1) & 3));
+            words[r][l][n_words[r][l]++] = (klo ? lo : 0u) | (khi ? hi << 16 : 0u);
+        }
     }
-    // lanes of half 0 by words, most first; lanes of half 1 by words, fewest first; equal ranks share a column
-    int col_of_rank[32], r = 0, H = 0;
+    // lanes by the words of their first row, most first, and by those of their second, fewest first; equal ranks share a column
+    int col_of_rank[32], k = 0, H = 0;
     for (int n = 16; n >= 0; --n)
         for (int l = 0; l < 32; ++l)
-            if (n_words[0][l] == n) col_of_rank[r++] = l;
+            if (n_words[0][l] == n) col_of_rank[k++] = l;
     uint8_t pi[32];
-    r = 0;
+    k = 0;
     for (int n = 0; n <= 16; ++n)
         for (int l = 0; l < 32; ++l)
             if (n_words[1][l] == n) {
-                const int c = col_of_rank[r++];
+                const int c = col_of_rank[k++];
                 pi[l] = (uint8_t)(4 * c);
                 if (n_words[0][c] + n > H) H = n_words[0][c] + n;
             }
     const size_t at = out.size();
     out.resize(at + kCellHeaderBytes + (size_t)H * 128, 0);
     uint8_t* p = out.data() + at;
-    std::memcpy(p, bits, 256);
-    std::memcpy(p + 256, pi, 32);
+    std::memcpy(p, bits, 128);
+    std::memcpy(p + 128, pi, 32);
     uint32_t* v = (uint32_t*)(p + kCellHeaderBytes);
     for (int l = 0; l < 32; ++l) {
         for (int w = 0; w < n_words[0][l]; ++w) v[(size_t)w * 32 + l] = words[0][l][w];
