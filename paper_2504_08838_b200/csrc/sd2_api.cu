@@ -597,11 +597,14 @@ bool plan_cells(int n, const CellNeeds& needs, CellPlan* p)
     p->part_bytes = (needs.parts * n * kPartPitch + 127) & ~127;
     p->chunk_bytes = (needs.max_chunk + 127) & ~127;
     p->xbuf_bytes = (n * needs.pitch + 127) & ~127;
-    for (p->n_parts = kPartSlots; p->n_parts >= 1; p->n_parts >>= 1) {     // (per finisher)
-        const int ring = kSmemMax - kCellFixedBytes - 2 * p->n_parts * p->part_bytes - p->xbuf_bytes;
+    // (n_parts: per finisher) the ring comes first: nine chunks in flight cover HBM's latency, then sums may wait, then more
+    static const int tries[][2] = {{4, 4}, {3, 2}, {3, 1}, {2, 1}};
+    for (const int* t : tries) {
+        const int ring = kSmemMax - kCellFixedBytes - 2 * t[1] * p->part_bytes - p->xbuf_bytes;
+        p->n_parts = t[1];
         p->n_slots = ring > 0 ? ring / (kCellGroups * p->chunk_bytes) : 0;
         if (p->n_slots > kGroupSlots) p->n_slots = kGroupSlots;
-        if (p->n_slots >= 2) return true;
+        if (p->n_slots >= t[0]) return true;
     }
     return false;
 }

@@ -148,12 +148,19 @@ __device__ __forceinline__ bool wait_count(const unsigned int* p, unsigned int w
     return ok;
 }
 
+__device__ __forceinline__ unsigned int ld_relaxed_gpu(const unsigned int* p)
+{
+    unsigned int v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
 // Until `target` arrivals have been counted.  false: the wait budget is out.
 __device__ __forceinline__ bool grid_wait(const unsigned int* gbar, unsigned int target, const WaitCtx& w)
 {
     const long long t0 = clock64();
     uint32_t it = 0;
-    while ((int)(ld_acquire_gpu(gbar) - target) < 0) {
+    while ((int)(ld_relaxed_gpu(gbar) - target) < 0) {           // (the caller fences once it is through)
         if ((++it & 15u) == 0u) {
             if (*w.abort_flag) return false;
             if (clock64() - t0 > w.budget) { *w.abort_flag = 1; return false; }
@@ -499,25 +506,35 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
 #define SD2_FIELD(f) (a.ext ? a.ext[sa].f : a.inl[MAXS == 1 ? 0 : sa].f)
     if (warp == kProducerWarp) {
         // ---------------------------------------------------------------------- producer
-        // The chunks of all stages, numbered through, go to the groups in turn; a round is one chunk per group.  Lane
-        // 4 g + j stands for cell j of group g's chunk.  A round's directory entries are loaded four rounds ahead, so
-        // their latency (and a stage's fields') stays off the ring's critical path.
-        struct PRound {
+        // The chunks of all stages, numbered through, go to the groups in turn.  Directory entries come in batches of eight
+        // chunks (lane 4 k + j: cell j of the batch's chunk k), loaded a batch ahead, so their latency and a stage's fields'
+        // stay off the ring's critical path.  (Like the finishers this warp gets an instruction in every few cycles only.)
+        constexpr int kBatch = 32 / kChunkCells;
+        struct PBatch {
             uint32_t o0, o1;                 // directory entries of the lane's cell; equal: none
-            const unsigned char* cells;      // NULL: the lane's group has come to the end
+            const unsigned char* cells;      // NULL: the end has come
         };
-        const int grp = lane / kChunkCells, cj = lane - grp * kChunkCells;
-        int sa = 0, q = grp, n = 0, n_chunks = 0;                // stage, chunk of the current run of tiles, the run's cells and chunks
+        const int bk = lane / kChunkCells, bj = lane - bk * kChunkCells;
+        int sa = 0, run0 = 0, n = 0, n_chunks = 0;               // stage; first chunk of the run of tiles, its cells and chunks
         const uint32_t* off = nullptr;
         const unsigned char* cells = nullptr;
         TileRuns runs(cluster, clusters, SD2_FIELD(rot), SD2_FIELD(tiles_div), SD2_FIELD(tiles_rem));
-        auto load_round = [&]() {
-            PRound c;
+        auto load_batch = [&](int first) {
+            PBatch c;
             c.o0 = c.o1 = 0u;
             c.cells = nullptr;
-            if (grp >= kCellGroups || sa >= a.n_stages) return c;
-            while (q >= n_chunks) {          // on to the next run of tiles, the next stage
-                q -= n_chunks;
+            while (true) {
+                const int q = first + bk - run0;
+                if (q >= 0 && q < n_chunks) {
+                    const int i = q * kChunkCells + bj;
+                    if (i < n) {
+                        c.o0 = __ldg(off + i);
+                        c.o1 = __ldg(off + i + 1);
+                    }
+                    c.cells = cells;
+                }
+                if (run0 + n_chunks >= first + kBatch || sa >= a.n_stages) return c;
+                run0 += n_chunks;            // on to the next run of tiles, the next stage
                 n = n_chunks = 0;
                 int mat, t0, nt;
                 if (runs.next(SD2_FIELD(pair), SD2_FIELD(count), SD2_FIELD(mat[0].T), SD2_FIELD(mat[1].T), SD2_FIELD(mat[2].T), mat, t0, nt)) {
@@ -526,63 +543,57 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                     n_chunks = (n + kChunkCells - 1) / kChunkCells;
                     cells = SD2_FIELD(mat[mat].cells);
                     off = SD2_FIELD(mat[mat].off) + (rank ? (size_t)SD2_FIELD(mat[mat].T) * share_cells(D, 0) : 0) + (size_t)t0 * Dr;
-                    continue;
+                } else if (++sa < a.n_stages) {
+                    runs = TileRuns(cluster, clusters, SD2_FIELD(rot), SD2_FIELD(tiles_div), SD2_FIELD(tiles_rem));
                 }
-                if (++sa >= a.n_stages) return c;
-                runs = TileRuns(cluster, clusters, SD2_FIELD(rot), SD2_FIELD(tiles_div), SD2_FIELD(tiles_rem));
             }
-            const int i = q * kChunkCells + cj;
-            if (i < n) {
-                c.o0 = __ldg(off + i);
-                c.o1 = __ldg(off + i + 1);
-            }
-            c.cells = cells;
-            q += kCellGroups;
-            return c;
         };
         // weights are read once: with several stages their lines leave L2 first, so that the stream does not push out
         // the small, shared, re-read activations
         const uint64_t policy = l2_evict_first();
         const bool hinted = a.n_stages > 1;
-        const int bg = grp < kCellGroups ? grp : 0;
-        const uint32_t full0 = smem_u32(&sh->full[bg][0]), empty0 = smem_u32(&sh->empty[bg][0]);
-        const uint32_t ring = smem_u32(smem) + ring_off + (uint32_t)bg * NS * (uint32_t)a.chunk_bytes;
-        uint32_t slot = 0, phase = 1, issued = 0;                // of the lane's group
+        const uint32_t full0 = smem_u32(&sh->full[0][0]), empty0 = smem_u32(&sh->empty[0][0]), ring = smem_u32(smem) + ring_off;
+        uint32_t slot = 0, phase = 1, issued = 0;
+        int grp = 0;
         bool ok = true;
-        PRound c0 = load_round(), c1 = load_round(), c2 = load_round(), c3 = load_round();
-        while (__any_sync(0xFFFFFFFFu, c0.cells != nullptr)) {
-            const bool mine = c0.o1 != c0.o0;
-            const uint32_t start = __shfl_sync(0xFFFFFFFFu, c0.o0, bg * kChunkCells);
-            uint32_t end = start;
+        PBatch cur = load_batch(0);
+        for (int first = 0; ok; first += kBatch) {
+            const PBatch next = load_batch(first + kBatch);
+            // first and last directory entry of the lane's chunk
+            const uint32_t start = __shfl_sync(0xFFFFFFFFu, cur.o0, lane & ~(kChunkCells - 1));
+            uint32_t end = cur.o1;
 #pragma unroll
-            for (int k = 0; k < kChunkCells; ++k) end = max(end, __shfl_sync(0xFFFFFFFFu, c0.o1, bg * kChunkCells + k));
-            const bool busy = lane < kCellWarps && end != start;   // the group has a chunk in this round
-            bool good = true;
-            if (busy) good = wait_phase(empty0 + 8 * slot, phase, wc);
-            if (!__all_sync(0xFFFFFFFFu, good)) { ok = false; break; }
-            if (mine) sh->cell[bg][slot][cj] = ((c0.o0 - start) << 13) | (((c0.o1 - c0.o0) * 32u - kCellHeaderBytes) >> 7);
-            __syncwarp();
-            if (busy) {
-                if (cj == 0) {
-                    const uint32_t bytes = (end - start) * 32u, dst = ring + slot * (uint32_t)a.chunk_bytes;
-                    mbar_expect_tx(full0 + 8 * slot, bytes);
-                    if (hinted) bulk_g2s(dst, c0.cells + (size_t)start * 32, bytes, full0 + 8 * slot, policy);
-                    else bulk_g2s(dst, c0.cells + (size_t)start * 32, bytes, full0 + 8 * slot);
+            for (int k = 1; k < kChunkCells; k <<= 1) end = max(end, __shfl_xor_sync(0xFFFFFFFFu, end, k));
+            const uint32_t mine = ((cur.o0 - start) << 13) | (((cur.o1 - cur.o0) * 32u - kCellHeaderBytes) >> 7);
+            const unsigned there = __ballot_sync(0xFFFFFFFFu, cur.cells != nullptr);
+            for (int k = 0; k < kBatch; ++k) {
+                if (!(there >> (k * kChunkCells) & 1u)) break;
+                const uint32_t s = (uint32_t)(grp * kGroupSlots) + slot;
+                if (!wait_phase_warp(empty0 + 8 * s, phase, wc)) { ok = false; break; }
+                if (bk == k && cur.o1 != cur.o0) (&sh->cell[0][0][0])[s * kChunkCells + bj] = mine;
+                __syncwarp();
+                if (lane == k * kChunkCells) {
+                    const uint32_t bytes = (end - start) * 32u, dst = ring + ((uint32_t)grp * NS + slot) * (uint32_t)a.chunk_bytes;
+                    mbar_expect_tx(full0 + 8 * s, bytes);
+                    if (hinted) bulk_g2s(dst, cur.cells + (size_t)start * 32, bytes, full0 + 8 * s, policy);
+                    else bulk_g2s(dst, cur.cells + (size_t)start * 32, bytes, full0 + 8 * s);
                 }
+                __syncwarp();
                 ++issued;
-                if (++slot == NS) { slot = 0; phase ^= 1u; }
+                if (++grp == kCellGroups) {
+                    grp = 0;
+                    if (++slot == NS) { slot = 0; phase ^= 1u; }
+                }
             }
-            __syncwarp();
-            c0 = c1;
-            c1 = c2;
-            c2 = c3;
-            c3 = load_round();
+            if (there != 0xFFFFFFFFu) break;
+            cur = next;
         }
-        if (!ok && lane < kCellWarps && cj == 0) {
+        if (!ok && lane == 0) {
             // give the copies already issued time to land before this CTA's memory is released
-            for (uint32_t t = issued > NS ? issued - NS : 0u; t != issued; ++t) {
+            for (uint32_t c = issued > kCellGroups * NS ? issued - kCellGroups * NS : 0u; c != issued; ++c) {
+                const uint32_t u = c / kCellGroups, s = (c % kCellGroups) * kGroupSlots + u % NS;
                 const long long t0 = clock64();
-                while (!mbar_try_wait(full0 + 8 * (t % NS), (t / NS) & 1u))
+                while (!mbar_try_wait(full0 + 8 * s, (u / NS) & 1u))
                     if (clock64() - t0 > wc.budget) break;
             }
         }
@@ -608,12 +619,12 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
             const uint16_t* x = s == 0 ? (a.x_in ? a.x_in : SD2_FIELD(x)) : st.x;
             const bool bulk = x && (K & 7) == 0 && (((uintptr_t)x) & 15) == 0 && Kr > 0;
             if (s > 0) {
-                // every CTA has written the previous stage's outputs (and has read its activations)
+                // this CTA's warps have left the previous stage, those without a tile in it among them ...
+                if (!wait_phase_warp(smem_u32(&sh->left), (uint32_t)(s - 1) & 1u, wc)) break;
+                // ... and every CTA has written its outputs (and has read its activations)
                 bool ok = true;
                 if (lane == 0) ok = grid_wait(a.gbar, (unsigned int)s * (unsigned int)G, wc);
                 if (!__all_sync(0xFFFFFFFFu, ok)) break;
-                // ... and this CTA's warps have left the stage, those without a tile in it among them
-                if (!wait_phase_warp(smem_u32(&sh->left), (uint32_t)(s - 1) & 1u, wc)) break;
                 __threadfence();
                 asm volatile("fence.proxy.async;" ::: "memory");     // ... written through the generic proxy, read by bulk copies
             }
