@@ -49,7 +49,6 @@ struct sd2_handle_s {
 struct CellNeeds {
     int pitch = 0;             // bytes of a staged activation row: the largest
     int max_chunk = 0;
-    int parts = 0;             // most contributions of a CTA to a tile
     int tiles_max = 0;         // most tiles of any stage
 };
 
@@ -586,7 +585,7 @@ sd2_status run_program(SArgs& a, int dev, int64_t N, const ProgramNeeds& needs, 
 // ------------------------------------------------------------------ programs over cells
 
 struct CellPlan {
-    int part_bytes, n_parts, xbuf_bytes, chunk_bytes, n_slots;
+    int n_parts, part_bytes, xbuf_bytes, chunk_bytes, n_slots;
 };
 
 constexpr int kCellFixedBytes = (int)((sizeof(CellShared) + 127) & ~127);
@@ -594,13 +593,13 @@ constexpr int kCellFixedBytes = (int)((sizeof(CellShared) + 127) & ~127);
 // Shared memory of a launch of n rows.  false: not even two chunks per group fit beside the staged rows.
 bool plan_cells(int n, const CellNeeds& needs, CellPlan* p)
 {
-    p->part_bytes = (needs.parts * n * kPartPitch + 127) & ~127;
     p->chunk_bytes = (needs.max_chunk + 127) & ~127;
     p->xbuf_bytes = (n * needs.pitch + 127) & ~127;
     // (n_parts: per finisher) the ring comes first: nine chunks in flight cover HBM's latency, then sums may wait, then more
-    static const int tries[][2] = {{4, 4}, {3, 2}, {3, 1}, {2, 1}};
+    static const int tries[][2] = {{4, 8}, {3, 8}, {3, 4}, {2, 4}};
     for (const int* t : tries) {
-        const int ring = kSmemMax - kCellFixedBytes - 2 * t[1] * p->part_bytes - p->xbuf_bytes;
+        p->part_bytes = 2 * t[1] * part_slot_bytes(n > 8 ? 16 : 8);
+        const int ring = kSmemMax - kCellFixedBytes - p->part_bytes - p->xbuf_bytes;
         p->n_parts = t[1];
         p->n_slots = ring > 0 ? ring / (kCellGroups * p->chunk_bytes) : 0;
         if (p->n_slots > kGroupSlots) p->n_slots = kGroupSlots;
@@ -675,9 +674,8 @@ struct CellBuilder {
             if (!pair || i == 0) st.V += m.T;
             if (hs[i]->max_chunk > needs.max_chunk) needs.max_chunk = hs[i]->max_chunk;
         }
-        const int pitch = cell_pitch(st.D), share = share_cells(st.D, 0), parts = share < kCellWarps ? share : kCellWarps;
+        const int pitch = cell_pitch(st.D);
         if (pitch > needs.pitch) needs.pitch = pitch;
-        if (parts > needs.parts) needs.parts = parts;
         if (st.V > needs.tiles_max) needs.tiles_max = st.V;
         st.rot = rot;
         rot = (int)(((int64_t)rot + st.V) % clusters);
@@ -704,12 +702,11 @@ sd2_status run_cell_panels(CArgs<kMaxStagesInline>& a, int64_t N, const CellNeed
         a.n0 = (int)n0;
         CellPlan p;
         if (!plan_cells(a.N, needs, &p)) return SD2_ERR_UNSUPPORTED;
-        a.part_bytes = p.part_bytes;
         a.part_mask = p.n_parts - 1;
         a.xbuf_bytes = p.xbuf_bytes;
         a.chunk_bytes = p.chunk_bytes;
         a.n_slots = p.n_slots;
-        const int smem = kCellFixedBytes + 2 * p.n_parts * p.part_bytes + p.xbuf_bytes + kCellGroups * p.n_slots * p.chunk_bytes;
+        const int smem = kCellFixedBytes + p.part_bytes + p.xbuf_bytes + kCellGroups * p.n_slots * p.chunk_bytes;
         sd2_status st;
         if (a.n_stages == 1) {
             static_cast<CArgsBase&>(one) = a;
@@ -753,7 +750,6 @@ bool use_cells(const sd2_handle* hs, int count, int64_t N)
         if (pitch > needs.pitch) needs.pitch = pitch;
         if (hs[i]->max_chunk > needs.max_chunk) needs.max_chunk = hs[i]->max_chunk;
     }
-    needs.parts = kCellWarps;
     return widest_cell_panel(needs) > 0;
 }
 

@@ -46,12 +46,14 @@ constexpr int kCellConsumers = kCellWarps * 32;
 constexpr int kProducerWarp = kCellWarps, kServiceWarp = kCellWarps + 1, kOwnWarp = kCellWarps + 2, kSendWarp = kCellWarps + 3;
 constexpr int kCellThreads = 32 * (kCellWarps + 4);
 constexpr int kGroupSlots = 4;              // chunks in flight per group, at most
-constexpr int kPartSlots = 4;               // tiles of a finisher whose partial sums may wait, at most
-constexpr int kRecvSlots = 4;               // sums from the other CTA that wait to be used
+constexpr int kPartSlots = 8;               // groups' partial sums that may wait for a finisher, at most (a power of two)
+constexpr int kRecvSlots = 8;               // sums from the other CTA that wait to be used
 constexpr int kPairSlots = 8;               // gate tiles whose results wait for the up tile's
 constexpr int kPanelRows = 16;              // activation rows of a launch, at most
-// A contribution to a tile is N rows of 16 fp32, 80 bytes apart: the lanes of a fragment store then hit 32 banks.
-constexpr int kPartPitch = 80;
+// A warp's contribution to a tile: for every eight activation rows 16 x 8 fp32, the activation row fastest.  A lane's
+// fragment goes there in 8-byte stores and a finisher reads 16 bytes a lane, both without bank conflicts.
+constexpr int kPartRowBytes = 32;
+__host__ __device__ constexpr int part_slot_bytes(int nr) { return kChunkCells * kTileRows * kPartRowBytes * (nr / 8); }
 
 struct CMat {
     const uint32_t* off;           // [T * D + 1], 32-byte units into `cells`
@@ -90,7 +92,7 @@ struct CArgsBase {
     int n_stages;
     int N;                          // activation rows of this launch
     int n0;                         // first activation row: every X / Y pointer is advanced by n0 rows
-    int part_bytes, part_mask;      // shared memory: one tile's partial sums, number of such slots per finisher - 1 (a power of two)
+    int part_mask;                  // slots of partial sums per finisher - 1 (a power of two)
     int xbuf_bytes;                 // staged activations
     int chunk_bytes, n_slots;       // a ring slot, slots per group
     int fold_any;                   // host side: launch the FOLD instance
@@ -110,12 +112,12 @@ struct CellShared {
     unsigned long long left;                            // consumers and finishers have left the stage: its descriptor and rows are free
     unsigned long long csync;                           // all consumers have come this far
     uint32_t cell[kCellGroups][kGroupSlots][kChunkCells]; // of each cell of the chunk: byte offset << 8 | H
-    unsigned long long pfull[2][kPartSlots];            // a tile's partial sums are complete: [0] to be sent, [1] to be finished here
+    unsigned long long pfull[2][kPartSlots];            // a group's partial sums are complete: [0] to be sent, [1] to be finished here
     unsigned long long rfull[kRecvSlots];               // sums from the other CTA have landed in recv[]
-    unsigned long long credit[kRecvSlots];              // ... the other CTA has taken ours out of its recv[]
+    unsigned long long credit[2];                       // the other CTA has taken ours out of this half of its recv[]
     unsigned int freed[2][kPartSlots];                  // how often the slot's sums have been read
-    uint16_t gate[kPairSlots][kPanelRows][kTileRows];   // bf16 results of gate tiles
-    float4 recv[kRecvSlots][kPanelRows][kTileRows / 4];
+    uint2 gate[kPairSlots][kPanelRows / 8][32];         // bf16 results of gate tiles, as the finisher's lanes hold them
+    float4 recv[kRecvSlots][kPanelRows / 8][32];
     int abort_flag;                                     // any warp: a bounded wait ran out
     float red[2][kCellWarps];                           // FOLD: per-warp partial sums of squares of two rows
     CStage stage[2];                                    // descriptors of the current and the next stage
@@ -148,19 +150,12 @@ __device__ __forceinline__ bool wait_count(const unsigned int* p, unsigned int w
     return ok;
 }
 
-__device__ __forceinline__ unsigned int ld_relaxed_gpu(const unsigned int* p)
-{
-    unsigned int v;
-    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
 // Until `target` arrivals have been counted.  false: the wait budget is out.
 __device__ __forceinline__ bool grid_wait(const unsigned int* gbar, unsigned int target, const WaitCtx& w)
 {
     const long long t0 = clock64();
     uint32_t it = 0;
-    while ((int)(ld_relaxed_gpu(gbar) - target) < 0) {           // (the caller fences once it is through)
+    while ((int)(ld_acquire_gpu(gbar) - target) < 0) {
         if ((++it & 15u) == 0u) {
             if (*w.abort_flag) return false;
             if (clock64() - t0 > w.budget) { *w.abort_flag = 1; return false; }
@@ -223,6 +218,33 @@ struct TileRuns {
         nt = min(end, base + T) - v;
         v += nt;
         return true;
+    }
+};
+
+// How a run's cells (nt tiles of Dr each, in order) are dealt to the groups.  Up to kSplitCells cells per tile a group
+// takes whole tiles: four contributions per tile for a finisher to add, not twelve.  Longer tiles are few and would leave
+// groups idle at the end of a stage: there the chunks go round and each group brings a third of a tile.
+constexpr int kSplitCells = 16;
+struct RunDeal {
+    bool split;
+    int tiles;         // per turn of a group
+    int cells;         // of a turn (the last one may be shorter)
+    int per;           // chunks of a turn
+    int turns;         // split: chunks
+    int chunks;        // of the run
+    __device__ __forceinline__ RunDeal(int Dr, int nt)
+    {
+        split = Dr > kSplitCells;
+        tiles = split ? nt : Dr < kChunkCells ? kChunkCells : (Dr & (kChunkCells - 1)) && Dr < 2 * kChunkCells ? 2 : 1;
+        cells = tiles * Dr;
+        per = (cells + kChunkCells - 1) / kChunkCells;
+        if (split) {
+            turns = chunks = per;
+            return;
+        }
+        const int sh = tiles == 4 ? 2 : tiles - 1, whole = nt >> sh, rest = nt - (whole << sh);
+        turns = Dr > 0 ? whole + (rest ? 1 : 0) : 0;
+        chunks = whole * per + (rest * Dr + kChunkCells - 1) / kChunkCells;
     }
 };
 
@@ -412,31 +434,23 @@ __device__ __noinline__ bool fold_norm(const XRows& r, const SFold& f, const uin
 // ---- finishing a tile ---------------------------------------------------------------------
 
 // A finisher shares its scheduler with busy warps and gets an instruction in every few cycles, so what counts here is the
-// number of instructions per tile.  Lane 4 n + t holds weight rows 4 t .. 4 t + 3 of panel rows n and n + 8.
+// number of instructions per tile.  Lane 2 r + t holds activation rows 4 t .. 4 t + 3 (and those + 8) of weight row r.
 
-// The sum of a tile's C contributions: four running sums, then one tree, an order that depends neither on N nor on the CTA.
-__device__ __forceinline__ void sum_parts(const unsigned char* p, int C, uint32_t part_row, float (&r)[4])
+// The sum of the C <= 4 contributions of a group, in one order.  p: the lane's place in the first.
+template <int NR>
+__device__ __forceinline__ void sum_parts(const unsigned char* p, int C, float (&r)[NR / 8][4])
 {
-    float acc[4][4];
+    constexpr uint32_t kStep = kTileRows * kPartRowBytes * (NR / 8);
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
+    for (int h = 0; h < NR / 8; ++h) {
+        float4 v[kChunkCells];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[k][j] = 0.f;
-    for (int c = 0; c < C; c += 4) {
-        float4 v[4];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = *(const float4*)(p + (uint32_t)min(c + k, C - 1) * part_row);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const bool there = c + k < C;
-            acc[k][0] += there ? v[k].x : 0.f;
-            acc[k][1] += there ? v[k].y : 0.f;
-            acc[k][2] += there ? v[k].z : 0.f;
-            acc[k][3] += there ? v[k].w : 0.f;
-        }
+        for (int k = 0; k < kChunkCells; ++k) v[k] = k < C ? *(const float4*)(p + (uint32_t)k * kStep + 512u * h) : make_float4(0.f, 0.f, 0.f, 0.f);
+        r[h][0] = (v[0].x + v[1].x) + (v[2].x + v[3].x);
+        r[h][1] = (v[0].y + v[1].y) + (v[2].y + v[3].y);
+        r[h][2] = (v[0].z + v[1].z) + (v[2].z + v[3].z);
+        r[h][3] = (v[0].w + v[1].w) + (v[2].w + v[3].w);
     }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) r[j] = (acc[0][j] + acc[1][j]) + (acc[2][j] + acc[3][j]);
 }
 
 __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi)
@@ -446,17 +460,13 @@ __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi)
     return d;
 }
 
-// four consecutive bf16 values to p, of which `n` exist; vec: p is aligned to eight bytes
-__device__ __forceinline__ void store_bf16(uint16_t* p, uint2 v, int n, bool vec)
+// bf16 values of up to four activation rows, `ld` elements apart
+__device__ __forceinline__ void store_bf16(uint16_t* p, uint2 v, int rows, size_t ld)
 {
-    if (vec && n >= 4) {
-        *(uint2*)p = v;
-        return;
-    }
-    if (n > 0) p[0] = (uint16_t)v.x;
-    if (n > 1) p[1] = (uint16_t)(v.x >> 16);
-    if (n > 2) p[2] = (uint16_t)v.y;
-    if (n > 3) p[3] = (uint16_t)(v.y >> 16);
+    if (rows > 0) p[0] = (uint16_t)v.x;
+    if (rows > 1) p[ld] = (uint16_t)(v.x >> 16);
+    if (rows > 2) p[2 * ld] = (uint16_t)v.y;
+    if (rows > 3) p[3 * ld] = (uint16_t)(v.y >> 16);
 }
 
 // ---- the kernel ---------------------------------------------------------------------------
@@ -467,7 +477,8 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr uint32_t kPartOff = (uint32_t)((sizeof(CellShared) + 127) & ~127);
     CellShared* sh = (CellShared*)smem;
-    const uint32_t xoff = kPartOff + (uint32_t)(2 * (a.part_mask + 1) * a.part_bytes);
+    constexpr uint32_t kSlotBytes = (uint32_t)part_slot_bytes(NR);
+    const uint32_t xoff = kPartOff + 2u * (uint32_t)(a.part_mask + 1) * kSlotBytes;
     const uint32_t ring_off = xoff + (uint32_t)a.xbuf_bytes;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rank = blockIdx.x & 1, cluster = blockIdx.x >> 1, clusters = gridDim.x >> 1;
@@ -486,12 +497,12 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         sh->abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     } else if (tid >= 64 && tid < 64 + 2 * kPartSlots) {
-        mbar_init(smem_u32(&sh->pfull[0][0]) + 8 * (tid - 64), kCellWarps);
+        mbar_init(smem_u32(&sh->pfull[0][0]) + 8 * (tid - 64), kChunkCells);
         (&sh->freed[0][0])[tid - 64] = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     } else if (tid >= 96 && tid < 96 + kRecvSlots) {
         mbar_init(smem_u32(&sh->rfull[tid - 96]), 1);
-        mbar_init(smem_u32(&sh->credit[tid - 96]), 1);
+        if (tid < 98) mbar_init(smem_u32(&sh->credit[tid - 96]), 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
@@ -506,16 +517,18 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
 #define SD2_FIELD(f) (a.ext ? a.ext[sa].f : a.inl[MAXS == 1 ? 0 : sa].f)
     if (warp == kProducerWarp) {
         // ---------------------------------------------------------------------- producer
-        // The chunks of all stages, numbered through, go to the groups in turn.  Directory entries come in batches of eight
+        // The chunks of all stages, numbered through.  Directory entries come in batches of eight
         // chunks (lane 4 k + j: cell j of the batch's chunk k), loaded a batch ahead, so their latency and a stage's fields'
         // stay off the ring's critical path.  (Like the finishers this warp gets an instruction in every few cycles only.)
         constexpr int kBatch = 32 / kChunkCells;
         struct PBatch {
             uint32_t o0, o1;                 // directory entries of the lane's cell; equal: none
             const unsigned char* cells;      // NULL: the end has come
+            int grp;                         // whose chunk it is
         };
         const int bk = lane / kChunkCells, bj = lane - bk * kChunkCells;
-        int sa = 0, run0 = 0, n = 0, n_chunks = 0;               // stage; first chunk of the run of tiles, its cells and chunks
+        int sa = 0, run0 = 0, n = 0, gb = 0;                     // stage; first chunk of the run of tiles, its cells, its first group
+        RunDeal deal(0, 0);
         const uint32_t* off = nullptr;
         const unsigned char* cells = nullptr;
         TileRuns runs(cluster, clusters, SD2_FIELD(rot), SD2_FIELD(tiles_div), SD2_FIELD(tiles_rem));
@@ -523,24 +536,29 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
             PBatch c;
             c.o0 = c.o1 = 0u;
             c.cells = nullptr;
+            c.grp = 0;
             while (true) {
                 const int q = first + bk - run0;
-                if (q >= 0 && q < n_chunks) {
-                    const int i = q * kChunkCells + bj;
-                    if (i < n) {
+                if (q >= 0 && q < deal.chunks) {
+                    const int turn = deal.split ? q : q / deal.per, i0 = deal.split ? 0 : turn * deal.cells;
+                    const int i = i0 + (deal.split ? q : q - turn * deal.per) * kChunkCells + bj;
+                    if (i < n && (deal.split || i < i0 + deal.cells)) {
                         c.o0 = __ldg(off + i);
                         c.o1 = __ldg(off + i + 1);
                     }
                     c.cells = cells;
+                    c.grp = (gb + turn) % kCellGroups;
                 }
-                if (run0 + n_chunks >= first + kBatch || sa >= a.n_stages) return c;
-                run0 += n_chunks;            // on to the next run of tiles, the next stage
-                n = n_chunks = 0;
+                if (run0 + deal.chunks >= first + kBatch || sa >= a.n_stages) return c;
+                run0 += deal.chunks;         // on to the next run of tiles, the next stage
+                gb = (gb + deal.turns) % kCellGroups;
+                n = 0;
+                deal = RunDeal(0, 0);
                 int mat, t0, nt;
                 if (runs.next(SD2_FIELD(pair), SD2_FIELD(count), SD2_FIELD(mat[0].T), SD2_FIELD(mat[1].T), SD2_FIELD(mat[2].T), mat, t0, nt)) {
                     const int D = SD2_FIELD(D), Dr = share_cells(D, rank);
                     n = nt * Dr;
-                    n_chunks = (n + kChunkCells - 1) / kChunkCells;
+                    deal = RunDeal(Dr, nt);
                     cells = SD2_FIELD(mat[mat].cells);
                     off = SD2_FIELD(mat[mat].off) + (rank ? (size_t)SD2_FIELD(mat[mat].T) * share_cells(D, 0) : 0) + (size_t)t0 * Dr;
                 } else if (++sa < a.n_stages) {
@@ -553,8 +571,7 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         const uint64_t policy = l2_evict_first();
         const bool hinted = a.n_stages > 1;
         const uint32_t full0 = smem_u32(&sh->full[0][0]), empty0 = smem_u32(&sh->empty[0][0]), ring = smem_u32(smem) + ring_off;
-        uint32_t slot = 0, phase = 1, issued = 0;
-        int grp = 0;
+        uint32_t next_slot = 0x101010u;      // of each group (a byte each): its next slot, 16 times the parity of the wait for it
         bool ok = true;
         PBatch cur = load_batch(0);
         for (int first = 0; ok; first += kBatch) {
@@ -568,8 +585,10 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
             const unsigned there = __ballot_sync(0xFFFFFFFFu, cur.cells != nullptr);
             for (int k = 0; k < kBatch; ++k) {
                 if (!(there >> (k * kChunkCells) & 1u)) break;
+                const int grp = __shfl_sync(0xFFFFFFFFu, cur.grp, k * kChunkCells);
+                const uint32_t at = next_slot >> (8 * grp) & 0xFFu, slot = at & 15u;
                 const uint32_t s = (uint32_t)(grp * kGroupSlots) + slot;
-                if (!wait_phase_warp(empty0 + 8 * s, phase, wc)) { ok = false; break; }
+                if (!wait_phase_warp(empty0 + 8 * s, at >> 4, wc)) { ok = false; break; }
                 if (bk == k && cur.o1 != cur.o0) (&sh->cell[0][0][0])[s * kChunkCells + bj] = mine;
                 __syncwarp();
                 if (lane == k * kChunkCells) {
@@ -579,23 +598,20 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                     else bulk_g2s(dst, cur.cells + (size_t)start * 32, bytes, full0 + 8 * s);
                 }
                 __syncwarp();
-                ++issued;
-                if (++grp == kCellGroups) {
-                    grp = 0;
-                    if (++slot == NS) { slot = 0; phase ^= 1u; }
-                }
+                next_slot ^= (at ^ (slot + 1 == NS ? (at ^ 16u) & 16u : at + 1u)) << (8 * grp);
             }
             if (there != 0xFFFFFFFFu) break;
             cur = next;
         }
         if (!ok && lane == 0) {
             // give the copies already issued time to land before this CTA's memory is released
-            for (uint32_t c = issued > kCellGroups * NS ? issued - kCellGroups * NS : 0u; c != issued; ++c) {
-                const uint32_t u = c / kCellGroups, s = (c % kCellGroups) * kGroupSlots + u % NS;
-                const long long t0 = clock64();
-                while (!mbar_try_wait(full0 + 8 * s, (u / NS) & 1u))
-                    if (clock64() - t0 > wc.budget) break;
-            }
+            for (int g = 0; g < kCellGroups; ++g)
+                for (uint32_t u = 0; u < NS; ++u) {
+                    const uint32_t at = next_slot >> (8 * g) & 0xFFu;
+                    const long long t0 = clock64();
+                    while (!mbar_try_wait(full0 + 8 * (g * kGroupSlots + u), (at >> 4) ^ (u < (at & 15u) ? 1u : 0u)))
+                        if (clock64() - t0 > wc.budget) break;
+                }
         }
         __syncwarp();
         asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
@@ -625,8 +641,7 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                 bool ok = true;
                 if (lane == 0) ok = grid_wait(a.gbar, (unsigned int)s * (unsigned int)G, wc);
                 if (!__all_sync(0xFFFFFFFFu, ok)) break;
-                __threadfence();
-                asm volatile("fence.proxy.async;" ::: "memory");     // ... written through the generic proxy, read by bulk copies
+                asm volatile("fence.proxy.async.global;" ::: "memory");     // ... written through the generic proxy, read by bulk copies
             }
             if (bulk && lane < N) {
                 int n = lane + cluster;                          // (not all CTAs ask for the same row first)
@@ -657,9 +672,9 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         const int own = warp == kOwnWarp ? 1 : 0;
         const uint32_t PM = (uint32_t)a.part_mask;
         const uint32_t pfull0 = smem_u32(&sh->pfull[own][0]);
-        const unsigned char* parts = smem + kPartOff + (uint32_t)own * (PM + 1u) * (uint32_t)a.part_bytes;
-        const int n0 = lane >> 2, r0 = (lane & 3) * 4;
-        const uint32_t part_row = (uint32_t)(N * kPartPitch), recv_off = (uint32_t)lane * 16u;
+        const uint32_t recv_off = (uint32_t)lane * 16u;
+        const unsigned char* parts = smem + kPartOff + (uint32_t)own * (PM + 1u) * kSlotBytes + recv_off;
+        const int n0 = (lane & 1) * 4, r0 = lane >> 1;
         const uint32_t peer_recv = peer_addr(&sh->recv[0][0][0], (uint32_t)(rank ^ 1)) + recv_off;
         const uint32_t peer_rfull = peer_addr(&sh->rfull[0], (uint32_t)(rank ^ 1)), peer_credit = peer_addr(&sh->credit[0], (uint32_t)(rank ^ 1));
         const uint32_t rfull0 = smem_u32(&sh->rfull[0]), credit0 = smem_u32(&sh->credit[0]);
@@ -670,7 +685,8 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         for (int s = 0; s < a.n_stages && ok; ++s) {
             if (!wait_phase_warp(smem_u32(&sh->xfull), (uint32_t)s & 1u, wc)) break;
             const CStage& st = sh->stage[s & 1];
-            const int D = st.D, Dr = share_cells(D, rank), C = Dr < kCellWarps ? Dr : kCellWarps;
+            const int D = st.D, Dr = share_cells(D, rank), C = Dr < kChunkCells ? Dr : kChunkCells;
+            const int n_parts = Dr > kSplitCells ? kCellGroups : 1;
             const bool alone = D == 1, pair = st.pair != 0;
             TileRuns runs(cluster, clusters, st.rot, st.tiles_div, st.tiles_rem);
             int mat, t0, nt;
@@ -678,28 +694,39 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                 if (alone && (rank || !own)) continue;           // CTA 0 has all the cells and finishes all the tiles
                 const CMat& md = st.mat[mat];
                 const int M = md.M;
-                const bool f32 = md.y_f32 != 0, vec = (M & 3) == 0;
+                const bool f32 = md.y_f32 != 0;
                 unsigned char* y = (unsigned char*)(s == a.n_stages - 1 && a.y_out && mat == 0 ? a.y_out : md.y);
-                const bool yvec = vec && (((uintptr_t)y) & 15) == 0;
                 for (int j = alone ? 0 : own ? rank : rank ^ 1; j < nt; j += alone ? 1 : 2) {
-                    if (!(ok = wait_phase_warp(pfull0 + 8 * ps, use & 1u, wc))) break;
                     float r[NR / 8][4];
+                    for (int part = 0; part < n_parts; ++part) {
+                        if (!(ok = wait_phase_warp(pfull0 + 8 * ps, use & 1u, wc))) break;
+                        if (part == 0) {
+                            sum_parts<NR>(parts + ps * kSlotBytes, C, r);
+                        } else {
+                            float q[NR / 8][4];
+                            sum_parts<NR>(parts + ps * kSlotBytes, C, q);
 #pragma unroll
-                    for (int h = 0; h < NR / 8; ++h)
-                        sum_parts(parts + ps * (uint32_t)a.part_bytes + (uint32_t)(min(n0 + 8 * h, N - 1) * kPartPitch + r0 * 4), C, part_row, r[h]);
-                    __syncwarp();
-                    if (lane == 0) *(volatile unsigned int*)&sh->freed[own][ps] = use + 1u;
-                    if (++ps > PM) { ps = 0; ++use; }
+                            for (int h = 0; h < NR / 8; ++h)
+#pragma unroll
+                                for (int k = 0; k < 4; ++k) r[h][k] += q[h][k];
+                        }
+                        __syncwarp();
+                        if (lane == 0) *(volatile unsigned int*)&sh->freed[own][ps] = use + 1u;
+                        if (++ps > PM) { ps = 0; ++use; }
+                    }
+                    if (!ok) break;
+                    // (the other CTA is told of every half of recv[] that has been used up: an arrival there that releases
+                    // takes some 700 cycles)
+                    const uint32_t half = rs / (kRecvSlots / 2);
                     if (!own) {
-                        if (ru > 0 && !(ok = wait_phase_warp(credit0 + 8 * rs, (ru - 1u) & 1u, wc))) break;
+                        if (ru > 0 && rs % (kRecvSlots / 2) == 0 && !(ok = wait_phase_warp(credit0 + 8 * half, (ru - 1u) & 1u, wc))) break;
 #pragma unroll
-                        for (int h = 0; h < NR / 8; ++h)
-                            if (n0 + 8 * h < N) st_async(peer_recv + rs * kRecvBytes + 512u * h, r[h], peer_rfull + 8 * rs);
+                        for (int h = 0; h < NR / 8; ++h) st_async(peer_recv + rs * kRecvBytes + 512u * h, r[h], peer_rfull + 8 * rs);
                         if (++rs == kRecvSlots) { rs = 0; ++ru; }
                         continue;
                     }
                     if (!alone) {
-                        if (lane == 0) mbar_expect_tx(rfull0 + 8 * rs, (uint32_t)N * 64u);
+                        if (lane == 0) mbar_expect_tx(rfull0 + 8 * rs, 512u * (NR / 8));
                         if (!(ok = wait_phase_warp(rfull0 + 8 * rs, ru & 1u, wc))) break;
 #pragma unroll
                         for (int h = 0; h < NR / 8; ++h) {
@@ -710,45 +737,36 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                             r[h][3] += v.w;
                         }
                         __syncwarp();
-                        if (lane == 0) mbar_arrive_remote(peer_credit + 8 * rs);
+                        if ((rs + 1) % (kRecvSlots / 2) == 0 && lane == 0) mbar_arrive_remote(peer_credit + 8 * half);
                         if (++rs == kRecvSlots) { rs = 0; ++ru; }
                     }
-                    const int left = M - (t0 + j) * kTileRows - r0;          // rows of the lane that exist
+                    const int row = (t0 + j) * kTileRows + r0;
+                    if (row >= M) continue;
 #pragma unroll
                     for (int h = 0; h < NR / 8; ++h) {
-                        const int n = n0 + 8 * h;
-                        if (n >= N || left <= 0) continue;
-                        const size_t at = (size_t)(a.n0 + n) * M + (size_t)(t0 + j) * kTileRows + r0;
+                        const int n = n0 + 8 * h, rows = N - n;      // activation rows of the lane that exist
+                        const size_t at = (size_t)(a.n0 + n) * M + row;
                         if (f32) {
-                            if (yvec && left >= 4) {
-                                *(float4*)((float*)y + at) = make_float4(r[h][0], r[h][1], r[h][2], r[h][3]);
-                            } else {
 #pragma unroll
-                                for (int k = 0; k < 4; ++k)
-                                    if (k < left) ((float*)y)[at + k] = r[h][k];
-                            }
+                            for (int k = 0; k < 4; ++k)
+                                if (k < rows) ((float*)y)[at + (size_t)k * M] = r[h][k];
                             continue;
                         }
                         const uint2 b = make_uint2(bf16_pair(r[h][0], r[h][1]), bf16_pair(r[h][2], r[h][3]));
-                        if (y) store_bf16((uint16_t*)y + at, b, left, yvec);
+                        if (y) store_bf16((uint16_t*)y + at, b, rows, (size_t)M);
                         if (pair) {
                             // gate tiles of a run wait for the up tiles of the run that follows, written and read by the same lane
-                            uint2* gt = (uint2*)&sh->gate[j % kPairSlots][n][r0];
+                            uint2* gt = &sh->gate[j % kPairSlots][h][lane];
                             if (mat == 0) *gt = b;
-                            else if (st.t_out) store_bf16(st.t_out + at, make_uint2(silu_mul_pair(gt->x, b.x), silu_mul_pair(gt->y, b.y)), left, vec && (((uintptr_t)st.t_out) & 15) == 0);
+                            else if (st.t_out) store_bf16(st.t_out + at, make_uint2(silu_mul_pair(gt->x, b.x), silu_mul_pair(gt->y, b.y)), rows, (size_t)M);
                         }
                     }
                 }
             }
             __syncwarp();
-            if (own && ok && s + 1 < a.n_stages) {
-                __threadfence();                                 // this CTA's outputs are visible before the grid barrier counts it
-                __syncwarp();
-                if (lane == 0) {
-                    __threadfence();
-                    atomicAdd(a.gbar, 1u);
-                }
-            }
+            // this CTA's outputs are visible before the grid barrier counts it (the warp's stores are ordered before this
+            // lane's release by the __syncwarp above)
+            if (own && ok && s + 1 < a.n_stages && lane == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.gbar) : "memory");
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&sh->left));
         }
@@ -797,23 +815,30 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                 }
                 if (!sync(wc, lane)) break;
             }
-            const uint32_t C = (uint32_t)(Dr < kCellWarps ? Dr : kCellWarps);
+            const uint32_t C = (uint32_t)(Dr < kChunkCells ? Dr : kChunkCells);
             const bool alone = D == 1;
             const uint32_t xl = sbase + xoff + (uint32_t)(xrow * pitch) + 16u * (lane & 3), xl8 = sbase + xoff + (uint32_t)(xrow8 * pitch) + 16u * (lane & 3);
             TileRuns runs(cluster, clusters, st.rot, st.tiles_div, st.tiles_rem);
             int mat, t0, nt;
             while (!failed && runs.next(st.pair, st.count, st.mat[0].T, st.mat[1].T, st.mat[2].T, mat, t0, nt)) {
-                const int n = nt * Dr, n_chunks = (n + kChunkCells - 1) / kChunkCells;
-                int q = grp - gb;
+                const RunDeal deal(Dr, nt);
+                const uint32_t n_parts = deal.split ? kCellGroups : 1;
+                const int step = deal.split ? kCellWarps : kChunkCells;
+                int q = grp - gb;                                // the group's first turn
                 if (q < 0) q += kCellGroups;
-                int i = q * kChunkCells + cj;
-                int tl = Dr > 0 ? i / Dr : 0, d = i - tl * Dr, c0 = d;
                 float acc[NR / 4][4];
 #pragma unroll
                 for (int m = 0; m < NR / 4; ++m)
 #pragma unroll
                     for (int k = 0; k < 4; ++k) acc[m][k] = 0.f;
-                for (; q < n_chunks; q += kCellGroups, i += kCellWarps) {
+                for (int turn = deal.split ? 0 : q; turn < (deal.split ? 1 : deal.turns) && !failed; turn += kCellGroups) {
+                int tl = turn * deal.tiles;                      // the warp's tile, its cell in the turn, in the tile
+                const int n = min(deal.tiles, nt - tl) * Dr;
+                int i = cj + (deal.split ? q * kChunkCells : 0);
+                int d = i;
+                while (d >= Dr && i < n) { d -= Dr; ++tl; }
+                int c0 = d;
+                for (int i0 = i - cj; i0 < n; i0 += step, i += step) {
                     if (!wait_phase_warp(full0 + 8 * slot, phase, wc)) { failed = true; break; }
                     if (i < n) {
                         const uint32_t where = sh->cell[grp][slot][cj];
@@ -827,43 +852,40 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                     if (lane == 0) mbar_arrive(empty0 + 8 * slot);
                     if (++slot == NS) { slot = 0; phase ^= 1u; }
                     if (i >= n) continue;
-                    d += kCellWarps;
+                    d += step;
                     if (d < Dr) continue;                        // the next cell belongs to the same tile
                     // the tile's sums go to the finisher in charge
                     {
                         const int own = alone || (tl & 1) == rank ? 1 : 0;
-                        const uint32_t k = (own ? cnt[1] : cnt[0]) + (uint32_t)(alone ? tl : tl >> 1);
+                        const uint32_t k = (own ? cnt[1] : cnt[0]) + (uint32_t)(alone ? tl : tl >> 1) * n_parts + (uint32_t)(c0 / kChunkCells);
                         const uint32_t ps = k & (uint32_t)a.part_mask, use = k / ((uint32_t)a.part_mask + 1u);
                         if (use > 0 && !wait_count(&sh->freed[own][ps], use, wc)) { failed = true; break; }
-                        float* p = (float*)(smem + kPartOff + ((uint32_t)own * ((uint32_t)a.part_mask + 1u) + ps) * (uint32_t)a.part_bytes +
-                                            (uint32_t)(c0 * N * kPartPitch)) + g;
+                        const uint32_t entry = (uint32_t)(c0 % kChunkCells);
+                        unsigned char* p = smem + kPartOff + ((uint32_t)own * ((uint32_t)a.part_mask + 1u) + ps) * kSlotBytes +
+                                           entry * (kSlotBytes / kChunkCells) + 8u * lane;       // (row g, activation rows 2 t and 2 t + 1)
 #pragma unroll
-                        for (int h = 0; h < NR / 8; ++h)
-#pragma unroll
-                            for (int k = 0; k < 2; ++k) {
-                                const int n = (lane & 3) * 2 + k + 8 * h;
-                                if (n < N) {
-                                    p[n * (kPartPitch / 4)] = acc[2 * h][k] + acc[2 * h + 1][k];
-                                    p[n * (kPartPitch / 4) + 8] = acc[2 * h][k + 2] + acc[2 * h + 1][k + 2];
-                                }
-                            }
+                        for (int h = 0; h < NR / 8; ++h) {
+                            *(float2*)(p + 512 * h) = make_float2(acc[2 * h][0] + acc[2 * h + 1][0], acc[2 * h][1] + acc[2 * h + 1][1]);
+                            *(float2*)(p + 512 * h + 256) = make_float2(acc[2 * h][2] + acc[2 * h + 1][2], acc[2 * h][3] + acc[2 * h + 1][3]);
+                        }
 #pragma unroll
                         for (int m = 0; m < NR / 4; ++m)
 #pragma unroll
                             for (int k = 0; k < 4; ++k) acc[m][k] = 0.f;
                         __syncwarp();
-                        // the C contributions make 12 arrivals between them
-                        if (lane == 0) mbar_arrive_n(smem_u32(&sh->pfull[own][ps]), c0 == 0 ? kCellWarps + 1u - C : 1u);
+                        // the C contributions make four arrivals between them
+                        if (lane == 0) mbar_arrive_n(smem_u32(&sh->pfull[own][ps]), entry == 0 ? kChunkCells + 1u - C : 1u);
                     }
                     do { d -= Dr; ++tl; } while (d >= Dr);
                     c0 = d;
                 }
-                gb = (gb + n_chunks) % kCellGroups;
+                }
+                gb = (gb + deal.turns) % kCellGroups;
                 if (alone) {
                     cnt[1] += rank ? 0u : (uint32_t)nt;
                 } else {                                         // tile j is finished by CTA j & 1
-                    cnt[1] += (uint32_t)(nt + 1 - rank) >> 1;
-                    cnt[0] += (uint32_t)(nt + rank) >> 1;
+                    cnt[1] += ((uint32_t)(nt + 1 - rank) >> 1) * n_parts;
+                    cnt[0] += ((uint32_t)(nt + rank) >> 1) * n_parts;
                 }
             }
             __syncwarp();
