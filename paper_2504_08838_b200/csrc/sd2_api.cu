@@ -72,6 +72,7 @@ struct sd2_drafter_s {
     int xs_need[4];            // bytes of staged activations at panel widths 1, 2, 4, 8
     // the same blocks as a program over cells, with barrier words of its own; NULL: a handle has no cells
     CStage* d_cstages;
+    CStage first_cstage;
     unsigned int* d_cbar;
     int n_cstages;
     CellNeeds cell_needs;
@@ -693,7 +694,8 @@ sd2_status run_cell_panels(CArgs<kMaxStagesInline>& a, int64_t N, const CellNeed
     const int64_t panels = (N + cap - 1) / cap;
     const int64_t rows = (N + panels - 1) / panels;
     CArgs<1> one;
-    if (a.n_stages == 1) {
+    const bool small = a.n_stages == 1 || a.ext;             // one inline stage is all that the launch reads
+    if (small) {
         one.inl[0] = a.inl[0];
         one.fold[0] = a.fold[0];
     }
@@ -708,7 +710,7 @@ sd2_status run_cell_panels(CArgs<kMaxStagesInline>& a, int64_t N, const CellNeed
         a.n_slots = p.n_slots;
         const int smem = kCellFixedBytes + p.part_bytes + p.xbuf_bytes + kCellGroups * p.n_slots * p.chunk_bytes;
         sd2_status st;
-        if (a.n_stages == 1) {
+        if (small) {
             static_cast<CArgsBase&>(one) = a;
             st = a.N > 8 ? launch_cells<1, 16>(one, grid, smem, s) : launch_cells<1, 8>(one, grid, smem, s);
         } else {
@@ -1882,6 +1884,7 @@ sd2_status sd2_drafter_create(const sd2_handle* h, int32_t L, int64_t n_max, sd2
                                base + wo[7], b + 1 < L);
         }
         d->n_cstages = bld.n;
+        d->first_cstage = cstages[0];
         d->cell_needs = bld.needs;
         ok = dev_malloc((void**)&d->d_cstages, sizeof(CStage) * (size_t)bld.n) == cudaSuccess &&
              cudaMemcpy(d->d_cstages, cstages.data(), sizeof(CStage) * (size_t)bld.n, cudaMemcpyHostToDevice) == cudaSuccess &&
@@ -1936,6 +1939,7 @@ sd2_status sd2_drafter_step(sd2_drafter d, const void* x, void* y, int64_t N, vo
     if (drafter_uses_cells(d, N)) {
         CArgs<kMaxStagesInline> c = {};
         c.ext = d->d_cstages;
+        c.inl[0] = d->first_cstage;
         c.n_stages = d->n_cstages;
         c.x_in = (const uint16_t*)x;
         c.y_out = y;

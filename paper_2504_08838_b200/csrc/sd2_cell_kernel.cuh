@@ -83,7 +83,7 @@ struct CStage {
 static_assert(sizeof(CStage) % 8 == 0, "stage descriptors are arrays of 8-byte fields");
 
 struct CArgsBase {
-    const CStage* ext;              // device array of stages, or NULL: the inline ones
+    const CStage* ext;              // device array of stages, or NULL: the inline ones (stage 0 is always inline)
     const uint16_t* x_in;           // replaces stage 0's x when not NULL
     void* y_out;                    // replaces the last stage's mat[0].y when not NULL
     unsigned int* gbar;             // grid barrier: [0] arrivals, [32] exits (two cache lines)
@@ -98,7 +98,8 @@ struct CArgsBase {
     int fold_any;                   // host side: launch the FOLD instance
 };
 
-// MAXS: inline stages the argument block has room for (a single-stage launch passes 0.4 KB of arguments, not 3 KB)
+// MAXS: inline stages the argument block has room for (a launch of one stage, or of stages in device memory, passes 0.4 KB
+// of arguments, not 3 KB)
 template <int MAXS>
 struct CArgs : CArgsBase {
     CStage inl[MAXS];
@@ -108,7 +109,8 @@ struct CArgs : CArgsBase {
 struct CellShared {
     unsigned long long full[kCellGroups][kGroupSlots];    // a chunk landed
     unsigned long long empty[kCellGroups][kGroupSlots];   // ... and has been consumed
-    unsigned long long xfull;                           // the stage's activations have landed, its descriptor is there
+    unsigned long long dfull;                           // the stage's descriptor is there
+    unsigned long long xfull;                           // the stage's activations have landed
     unsigned long long left;                            // consumers and finishers have left the stage: its descriptor and rows are free
     unsigned long long csync;                           // all consumers have come this far
     uint32_t cell[kCellGroups][kGroupSlots][kChunkCells]; // of each cell of the chunk: byte offset << 8 | H
@@ -491,6 +493,7 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         mbar_init(smem_u32(&sh->empty[0][0]) + 8 * tid, kChunkCells);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     } else if (tid == 32) {
+        mbar_init(smem_u32(&sh->dfull), 1);
         mbar_init(smem_u32(&sh->xfull), 1);
         mbar_init(smem_u32(&sh->left), kCellWarps + 2);
         mbar_init(smem_u32(&sh->csync), kCellWarps);
@@ -513,8 +516,39 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
     wc.abort_flag = &sh->abort_flag;
     wc.budget = a.wait_cycles;
 
-    // field f of stage sa (one by one, so that inline descriptors are read as kernel arguments, not through a generic pointer)
-#define SD2_FIELD(f) (a.ext ? a.ext[sa].f : a.inl[MAXS == 1 ? 0 : sa].f)
+    // word i of a stage's descriptor
+    auto stage_word = [&](int s, int i) {
+        return a.ext && s > 0 ? ((const uint32_t*)(a.ext + s))[i] : ((const uint32_t*)&a.inl[MAXS == 1 ? 0 : s])[i];
+    };
+    // Starts the copies of every second activation row of stage s (the service warp's and the sending finisher's halves;
+    // a copy takes a warp some 90 cycles to start).  bytes: of all the rows; 0: the consumers fetch them.
+    auto start_rows = [&](int s, int part, uint32_t& bytes) {
+        const uint32_t xfull = smem_u32(&sh->xfull);
+        const CStage& st = sh->stage[s & 1];
+        // (the first stage's rows are on their way before its descriptor has been copied to shared memory)
+        const int D = s == 0 ? a.inl[0].D : st.D, K = s == 0 ? a.inl[0].K : st.K;
+        const int Dr = share_cells(D, rank), xb = rank ? share_cells(D, 0) * kCellCols : 0;
+        const int Kr = min(K - xb, Dr * kCellCols);
+        const uint16_t* x = s == 0 ? (a.x_in ? a.x_in : a.inl[0].x) : st.x;
+        bytes = x && (K & 7) == 0 && (((uintptr_t)x) & 15) == 0 && Kr > 0 ? (uint32_t)(N * Kr * 2) : 0u;
+        if (s > 0) {
+            // this CTA's warps have left the previous stage, those without a tile in it among them ...
+            if (!wait_phase_warp(smem_u32(&sh->left), (uint32_t)(s - 1) & 1u, wc)) return false;
+            // ... and every CTA has written its outputs (and has read its activations)
+            bool ok = true;
+            if (lane == 0) ok = grid_wait(a.gbar, (unsigned int)s * (unsigned int)G, wc);
+            if (!__all_sync(0xFFFFFFFFu, ok)) return false;
+            asm volatile("fence.proxy.async.global;" ::: "memory");      // ... written through the generic proxy, read by bulk copies
+        }
+        int n = 2 * lane + part;
+        if (bytes && n < N) {
+            n += cluster;                                        // (not all CTAs ask for the same row first)
+            n -= n / N * N;
+            bulk_g2s(smem_u32(smem) + xoff + (uint32_t)(n * (2 * Dr * kCellCols + 64)), x + (size_t)(a.n0 + n) * K + xb, (uint32_t)(Kr * 2), xfull);
+        }
+        __syncwarp();
+        return true;
+    };
     if (warp == kProducerWarp) {
         // ---------------------------------------------------------------------- producer
         // The chunks of all stages, numbered through.  Directory entries come in batches of eight
@@ -527,11 +561,37 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
             int grp;                         // whose chunk it is
         };
         const int bk = lane / kChunkCells, bj = lane - bk * kChunkCells;
+        // A stage's descriptor is spread over the lanes, and the next stage's is loaded when the stage begins: its latency
+        // (and a chain of dependent loads, 3000 cycles at every run of tiles when they were made one by one) is hidden.
+        constexpr int kWords = (int)(sizeof(CStage) / 4);
+        static_assert(kWords <= 64, "two words a lane");
+        uint32_t w0 = stage_word(0, lane), w1 = 32 + lane < kWords ? stage_word(0, 32 + lane) : 0u, next_w0 = 0, next_w1 = 0;
+        auto word = [&](int i) { return __shfl_sync(0xFFFFFFFFu, i < 32 ? w0 : w1, i & 31); };
+        auto pointer = [&](int i) {
+            const uint32_t lo = word(i), hi = word(i + 1);
+            return (const unsigned char*)((unsigned long long)hi << 32 | lo);
+        };
+#define SD2_WORD(f) ((int)(offsetof(CStage, f) / 4))
         int sa = 0, run0 = 0, n = 0, gb = 0;                     // stage; first chunk of the run of tiles, its cells, its first group
         RunDeal deal(0, 0);
         const uint32_t* off = nullptr;
         const unsigned char* cells = nullptr;
-        TileRuns runs(cluster, clusters, SD2_FIELD(rot), SD2_FIELD(tiles_div), SD2_FIELD(tiles_rem));
+        TileRuns runs(0, 0, 0, 0, 0);
+        int D = 0, pair = 0, count = 0, T0 = 0, T1 = 0, T2 = 0;
+        auto begin_stage = [&]() {
+            if (sa + 1 < a.n_stages) {
+                next_w0 = stage_word(sa + 1, lane);
+                next_w1 = 32 + lane < kWords ? stage_word(sa + 1, 32 + lane) : 0u;
+            }
+            runs = TileRuns(cluster, clusters, (int)word(SD2_WORD(rot)), (int)word(SD2_WORD(tiles_div)), (int)word(SD2_WORD(tiles_rem)));
+            D = (int)word(SD2_WORD(D));
+            pair = (int)word(SD2_WORD(pair));
+            count = (int)word(SD2_WORD(count));
+            T0 = (int)word(SD2_WORD(mat[0].T));
+            T1 = (int)word(SD2_WORD(mat[1].T));
+            T2 = (int)word(SD2_WORD(mat[2].T));
+        };
+        begin_stage();
         auto load_batch = [&](int first) {
             PBatch c;
             c.o0 = c.o1 = 0u;
@@ -555,14 +615,17 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                 n = 0;
                 deal = RunDeal(0, 0);
                 int mat, t0, nt;
-                if (runs.next(SD2_FIELD(pair), SD2_FIELD(count), SD2_FIELD(mat[0].T), SD2_FIELD(mat[1].T), SD2_FIELD(mat[2].T), mat, t0, nt)) {
-                    const int D = SD2_FIELD(D), Dr = share_cells(D, rank);
+                if (runs.next(pair, count, T0, T1, T2, mat, t0, nt)) {
+                    const int Dr = share_cells(D, rank), w = mat * (int)(sizeof(CMat) / 4);
                     n = nt * Dr;
                     deal = RunDeal(Dr, nt);
-                    cells = SD2_FIELD(mat[mat].cells);
-                    off = SD2_FIELD(mat[mat].off) + (rank ? (size_t)SD2_FIELD(mat[mat].T) * share_cells(D, 0) : 0) + (size_t)t0 * Dr;
+                    cells = pointer(w + SD2_WORD(mat[0].cells));
+                    off = (const uint32_t*)pointer(w + SD2_WORD(mat[0].off)) +
+                          (rank ? (size_t)word(w + SD2_WORD(mat[0].T)) * share_cells(D, 0) : 0) + (size_t)t0 * Dr;
                 } else if (++sa < a.n_stages) {
-                    runs = TileRuns(cluster, clusters, SD2_FIELD(rot), SD2_FIELD(tiles_div), SD2_FIELD(tiles_rem));
+                    w0 = next_w0;
+                    w1 = next_w1;
+                    begin_stage();
                 }
             }
         };
@@ -620,46 +683,22 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         const uint32_t xfull = smem_u32(&sh->xfull);
         auto fetch_stage = [&](int s) {
             uint32_t* dst = (uint32_t*)&sh->stage[s & 1];
-            for (int i = lane; i < (int)(sizeof(CStage) / 4); i += 32)
-                dst[i] = a.ext ? ((const uint32_t*)(a.ext + s))[i] : ((const uint32_t*)&a.inl[s])[i];
+            for (int i = lane; i < (int)(sizeof(CStage) / 4); i += 32) dst[i] = stage_word(s, i);
             __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&sh->dfull));
         };
         bool landed = true;
         for (int s = 0; s < a.n_stages; ++s) {
-            // (the first stage's rows are on their way before its descriptor has been copied to shared memory)
-            const int sa = s;
-            const CStage& st = sh->stage[s & 1];
-            const int D = s == 0 ? SD2_FIELD(D) : st.D, K = s == 0 ? SD2_FIELD(K) : st.K;
-            const int Dr = share_cells(D, rank), xb = rank ? share_cells(D, 0) * kCellCols : 0;
-            const int Kr = min(K - xb, Dr * kCellCols);
-            const uint16_t* x = s == 0 ? (a.x_in ? a.x_in : SD2_FIELD(x)) : st.x;
-            const bool bulk = x && (K & 7) == 0 && (((uintptr_t)x) & 15) == 0 && Kr > 0;
-            if (s > 0) {
-                // this CTA's warps have left the previous stage, those without a tile in it among them ...
-                if (!wait_phase_warp(smem_u32(&sh->left), (uint32_t)(s - 1) & 1u, wc)) break;
-                // ... and every CTA has written its outputs (and has read its activations)
-                bool ok = true;
-                if (lane == 0) ok = grid_wait(a.gbar, (unsigned int)s * (unsigned int)G, wc);
-                if (!__all_sync(0xFFFFFFFFu, ok)) break;
-                asm volatile("fence.proxy.async.global;" ::: "memory");     // ... written through the generic proxy, read by bulk copies
-            }
-            if (bulk && lane < N) {
-                int n = lane + cluster;                          // (not all CTAs ask for the same row first)
-                n -= n / N * N;
-                bulk_g2s(smem_u32(smem) + xoff + (uint32_t)(n * (2 * Dr * kCellCols + 64)), x + (size_t)(a.n0 + n) * K + xb, (uint32_t)(Kr * 2), xfull);
-            }
-            __syncwarp();
-            if (s == 0) fetch_stage(0);
+            uint32_t bytes;
+            if (!start_rows(s, 0, bytes)) { landed = false; break; }
             if (lane == 0) {
-                if (bulk) mbar_expect_tx(xfull, (uint32_t)(N * Kr * 2));
+                if (bytes) mbar_expect_tx(xfull, bytes);
                 else mbar_arrive(xfull);
             }
-            landed = !bulk;
-            if (s + 1 < a.n_stages) {
-                fetch_stage(s + 1);
-            } else if (bulk) {
-                landed = wait_phase_warp(xfull, (uint32_t)s & 1u, wc);
-            }
+            landed = !bytes;
+            if (s == 0) fetch_stage(0);
+            if (s + 1 < a.n_stages) fetch_stage(s + 1);
+            else if (bytes) landed = wait_phase_warp(xfull, (uint32_t)s & 1u, wc);
         }
         if (!landed) {                                           // a wait ran out: give the rows in flight time to land
             const long long t0 = clock64();
@@ -681,9 +720,13 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         constexpr uint32_t kRecvBytes = (uint32_t)sizeof(sh->recv[0]);
         uint32_t ps = 0, use = 0, rs = 0, ru = 0;                // slot of partial sums and its use, the same for exchanged sums
         bool ok = true;
+        uint32_t bytes;
+        if (!own) start_rows(0, 1, bytes);
         asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-        for (int s = 0; s < a.n_stages && ok; ++s) {
-            if (!wait_phase_warp(smem_u32(&sh->xfull), (uint32_t)s & 1u, wc)) break;
+        const uint32_t dfull = smem_u32(&sh->dfull);
+        bool ready = wait_phase_warp(dfull, 0u, wc);
+        for (int s = 0; s < a.n_stages && ok && ready; ++s) {
+            if (!own && s > 0 && !start_rows(s, 1, bytes)) break;
             const CStage& st = sh->stage[s & 1];
             const int D = st.D, Dr = share_cells(D, rank), C = Dr < kChunkCells ? Dr : kChunkCells;
             const int n_parts = Dr > kSplitCells ? kCellGroups : 1;
@@ -768,6 +811,8 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
             // lane's release by the __syncwarp above)
             if (own && ok && s + 1 < a.n_stages && lane == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.gbar) : "memory");
             __syncwarp();
+            // (nobody counts as gone from a stage before it has seen the next one's descriptor: dfull never runs two ahead)
+            if (s + 1 < a.n_stages) ready = wait_phase_warp(dfull, (uint32_t)(s + 1) & 1u, wc);
             if (lane == 0) mbar_arrive(smem_u32(&sh->left));
         }
     } else {
@@ -786,9 +831,9 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         uint32_t slot = 0, phase = 0;
         uint32_t cnt[2] = {0, 0};                                // tiles of each finisher before this run
         int gb = 0;                                              // the group that gets the run's first chunk
-        bool failed = false;
+        const uint32_t dfull = smem_u32(&sh->dfull);
+        bool failed = !wait_phase_warp(dfull, 0u, wc);
         for (int s = 0; s < a.n_stages && !failed; ++s) {
-            if (!wait_phase_warp(xfull, (uint32_t)s & 1u, wc)) break;
             const CStage& st = sh->stage[s & 1];
             const int D = st.D, K = st.K, Dr = share_cells(D, rank), xb = rank ? share_cells(D, 0) * kCellCols : 0;
             const int Kp = Dr * kCellCols, Kr = min(K - xb, Kp);
@@ -796,6 +841,12 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                                                                  // 128-bit read fall into different banks
             const uint16_t* x = (s == 0 && a.x_in) ? a.x_in : st.x;
             const bool bulk = x && (K & 7) == 0 && (((uintptr_t)x) & 15) == 0;
+            TileRuns runs(cluster, clusters, st.rot, st.tiles_div, st.tiles_rem);
+            const int pair = st.pair, count = st.count, T0 = st.mat[0].T, T1 = st.mat[1].T, T2 = st.mat[2].T;
+            int mat, t0, nt;
+            bool more = runs.next(pair, count, T0, T1, T2, mat, t0, nt);
+            RunDeal deal(Dr, more ? nt : 0);
+            if (!wait_phase_warp(xfull, (uint32_t)s & 1u, wc)) break;    // (all that the descriptor decides is known by now)
             const bool norm = FOLD && a.fold[MAXS == 1 ? 0 : s].norm_w;
             if ((!bulk || Kr < Kp || norm) && Kr > 0) {
                 XRows xr;
@@ -818,10 +869,7 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
             const uint32_t C = (uint32_t)(Dr < kChunkCells ? Dr : kChunkCells);
             const bool alone = D == 1;
             const uint32_t xl = sbase + xoff + (uint32_t)(xrow * pitch) + 16u * (lane & 3), xl8 = sbase + xoff + (uint32_t)(xrow8 * pitch) + 16u * (lane & 3);
-            TileRuns runs(cluster, clusters, st.rot, st.tiles_div, st.tiles_rem);
-            int mat, t0, nt;
-            while (!failed && runs.next(st.pair, st.count, st.mat[0].T, st.mat[1].T, st.mat[2].T, mat, t0, nt)) {
-                const RunDeal deal(Dr, nt);
+            while (!failed && more) {
                 const uint32_t n_parts = deal.split ? kCellGroups : 1;
                 const int step = deal.split ? kCellWarps : kChunkCells;
                 int q = grp - gb;                                // the group's first turn
@@ -887,8 +935,11 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                     cnt[1] += ((uint32_t)(nt + 1 - rank) >> 1) * n_parts;
                     cnt[0] += ((uint32_t)(nt + rank) >> 1) * n_parts;
                 }
+                more = runs.next(pair, count, T0, T1, T2, mat, t0, nt);
+                if (more) deal = RunDeal(Dr, nt);
             }
             __syncwarp();
+            if (s + 1 < a.n_stages && !failed) failed = !wait_phase_warp(dfull, (uint32_t)(s + 1) & 1u, wc);
             if (lane == 0) mbar_arrive(smem_u32(&sh->left));
         }
         __syncwarp();
