@@ -807,6 +807,8 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                 }
             }
             __syncwarp();
+            // (a CTA without a tile must not be counted before the stage has begun: the barrier counts arrivals, not stages)
+            if (own && ok && s + 1 < a.n_stages) ok = wait_phase_warp(smem_u32(&sh->xfull), (uint32_t)s & 1u, wc);
             // this CTA's outputs are visible before the grid barrier counts it (the warp's stores are ordered before this
             // lane's release by the __syncwarp above)
             if (own && ok && s + 1 < a.n_stages && lane == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.gbar) : "memory");
