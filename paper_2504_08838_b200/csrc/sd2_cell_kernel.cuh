@@ -129,8 +129,14 @@ struct CellShared {
 // together and with one answer: mma.sync and other warp-wide instructions need it whole.
 __device__ __forceinline__ bool wait_phase_warp(uint32_t bar, uint32_t parity, const WaitCtx& w)
 {
+#ifdef SD2_ELECT
+    int ok = 1;
+    if ((threadIdx.x & 31) == 0) ok = wait_phase(bar, parity, w);
+    return __shfl_sync(0xFFFFFFFFu, ok, 0);
+#else
     const bool ok = wait_phase(bar, parity, w);
     return __all_sync(0xFFFFFFFFu, ok);
+#endif
 }
 
 // Until the shared counter at p has reached `want` (one warp, together).
@@ -482,7 +488,8 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
     constexpr uint32_t kSlotBytes = (uint32_t)part_slot_bytes(NR);
     const uint32_t xoff = kPartOff + 2u * (uint32_t)(a.part_mask + 1) * kSlotBytes;
     const uint32_t ring_off = xoff + (uint32_t)a.xbuf_bytes;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);      // (known to be the same in all lanes)
     const int rank = blockIdx.x & 1, cluster = blockIdx.x >> 1, clusters = gridDim.x >> 1;
     const int G = gridDim.x;
     const int N = a.N;
