@@ -125,37 +125,44 @@ struct CellShared {
     CStage stage[2];                                    // descriptors of the current and the next stage
 };
 
-// The lanes of a warp come back from wait_phase one by one, with answers of their own.  This one brings the warp back
-// together and with one answer: mma.sync and other warp-wide instructions need it whole.
+// wait_phase for a whole warp: its lanes get one answer, and every branch is on a vote.  (mma.sync and other warp-wide
+// instructions need the warp whole, and lanes that come back from a wait one by one cost hundreds of cycles to bring together:
+// an eight-row drafter step took 76 us with a wait per lane, 127 us with one lane waiting for the others.)
 __device__ __forceinline__ bool wait_phase_warp(uint32_t bar, uint32_t parity, const WaitCtx& w)
 {
-#ifdef SD2_ELECT
-    int ok = 1;
-    if ((threadIdx.x & 31) == 0) ok = wait_phase(bar, parity, w);
-    return __shfl_sync(0xFFFFFFFFu, ok, 0);
-#else
-    const bool ok = wait_phase(bar, parity, w);
-    return __all_sync(0xFFFFFFFFu, ok);
-#endif
+    if (__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity))) return true;
+    const long long t0 = clock64();
+    uint32_t it = 0;
+    while (!__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity))) {
+        if ((++it & 15u) == 0u) {
+            if (__any_sync(0xFFFFFFFFu, *w.abort_flag != 0)) return false;
+            if (__any_sync(0xFFFFFFFFu, clock64() - t0 > w.budget)) {
+                *w.abort_flag = 1;
+                return false;
+            }
+        }
+    }
+    return true;
 }
 
 // Until the shared counter at p has reached `want` (one warp, together).
 __device__ __forceinline__ bool wait_count(const unsigned int* p, unsigned int want, const WaitCtx& w)
 {
-    bool ok = true;
-    if ((int)(*(const volatile unsigned int*)p - want) < 0) {
+    if (__any_sync(0xFFFFFFFFu, (int)(*(const volatile unsigned int*)p - want) < 0)) {
         const long long t0 = clock64();
         uint32_t it = 0;
-        while ((int)(*(const volatile unsigned int*)p - want) < 0) {
+        while (__any_sync(0xFFFFFFFFu, (int)(*(const volatile unsigned int*)p - want) < 0)) {
             if ((++it & 15u) == 0u) {
-                if (*w.abort_flag) { ok = false; break; }
-                if (clock64() - t0 > w.budget) { *w.abort_flag = 1; ok = false; break; }
+                if (__any_sync(0xFFFFFFFFu, *w.abort_flag != 0)) return false;
+                if (__any_sync(0xFFFFFFFFu, clock64() - t0 > w.budget)) {
+                    *w.abort_flag = 1;
+                    return false;
+                }
             }
         }
     }
-    ok = __all_sync(0xFFFFFFFFu, ok);
     __threadfence_block();
-    return ok;
+    return true;
 }
 
 // Until `target` arrivals have been counted.  false: the wait budget is out.
@@ -188,9 +195,25 @@ __device__ __forceinline__ void mbar_arrive_remote(uint32_t bar)
 {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t n)
+// one lane's arrival, predicated: a branch around it splits the warp
+__device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t n, bool lead)
 {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(n) : "memory");
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0], %1;\n\t}" ::"r"(bar), "r"(n), "r"((int)lead) : "memory");
+}
+// ... that also announces a bulk copy, and the copy (with or without an L2 policy)
+__device__ __forceinline__ void bulk_chunk(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar, bool lead)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t@p mbarrier.arrive.expect_tx.shared::cta.b64 _, [%3], %2;\n\t"
+                 "@p cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n\t}" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(bar), "r"((int)lead)
+                 : "memory");
+}
+__device__ __forceinline__ void bulk_chunk(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar, bool lead, uint64_t policy)
+{
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t@p mbarrier.arrive.expect_tx.shared::cta.b64 _, [%3], %2;\n\t"
+                 "@p cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %5;\n\t}" ::"r"(dst),
+                 "l"(src), "r"(bytes), "r"(bar), "r"((int)lead), "l"(policy)
+                 : "memory");
 }
 
 // The runs of consecutive tiles of one weight that a cluster works through in a stage, in order.
@@ -661,13 +684,10 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                 if (!wait_phase_warp(empty0 + 8 * s, at >> 4, wc)) { ok = false; break; }
                 if (bk == k && cur.o1 != cur.o0) (&sh->cell[0][0][0])[s * kChunkCells + bj] = mine;
                 __syncwarp();
-                if (lane == k * kChunkCells) {
-                    const uint32_t bytes = (end - start) * 32u, dst = ring + ((uint32_t)grp * NS + slot) * (uint32_t)a.chunk_bytes;
-                    mbar_expect_tx(full0 + 8 * s, bytes);
-                    if (hinted) bulk_g2s(dst, cur.cells + (size_t)start * 32, bytes, full0 + 8 * s, policy);
-                    else bulk_g2s(dst, cur.cells + (size_t)start * 32, bytes, full0 + 8 * s);
-                }
-                __syncwarp();
+                // (by lane 4 k: the values are its own)
+                const uint32_t bytes = (end - start) * 32u, dst = ring + ((uint32_t)grp * NS + slot) * (uint32_t)a.chunk_bytes;
+                if (hinted) bulk_chunk(dst, cur.cells + (size_t)start * 32, bytes, full0 + 8 * s, lane == k * kChunkCells, policy);
+                else bulk_chunk(dst, cur.cells + (size_t)start * 32, bytes, full0 + 8 * s, lane == k * kChunkCells);
                 next_slot ^= (at ^ (slot + 1 == NS ? (at ^ 16u) & 16u : at + 1u)) << (8 * grp);
             }
             if (there != 0xFFFFFFFFu) break;
@@ -906,7 +926,7 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                         multiply_cell<NR>(m, v0 + 4u * lane, v0 + (H - 1u) * 128u + pi, xl + xd, xl8 + xd, acc);
                     }
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(empty0 + 8 * slot);
+                    mbar_arrive_n(empty0 + 8 * slot, 1u, lane == 0);
                     if (++slot == NS) { slot = 0; phase ^= 1u; }
                     if (i >= n) continue;
                     d += step;
@@ -931,7 +951,7 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                             for (int k = 0; k < 4; ++k) acc[m][k] = 0.f;
                         __syncwarp();
                         // the C contributions make four arrivals between them
-                        if (lane == 0) mbar_arrive_n(smem_u32(&sh->pfull[own][ps]), entry == 0 ? kChunkCells + 1u - C : 1u);
+                        mbar_arrive_n(smem_u32(&sh->pfull[own][ps]), entry == 0 ? kChunkCells + 1u - C : 1u, lane == 0);
                     }
                     do { d -= Dr; ++tl; } while (d >= Dr);
                     c0 = d;
