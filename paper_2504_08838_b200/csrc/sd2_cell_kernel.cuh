@@ -113,7 +113,6 @@ struct CellShared {
     unsigned long long xfull;                           // the stage's activations have landed
     unsigned long long left;                            // consumers and finishers have left the stage: its descriptor and rows are free
     unsigned long long csync;                           // all consumers have come this far
-    uint32_t cell[kCellGroups][kGroupSlots][kChunkCells]; // of each cell of the chunk: byte offset << 8 | H
     unsigned long long pfull[2][kPartSlots];            // a group's partial sums are complete: [0] to be sent, [1] to be finished here
     unsigned long long rfull[kRecvSlots];               // sums from the other CTA have landed in recv[]
     unsigned long long credit[2];                       // the other CTA has taken ours out of this half of its recv[]
@@ -581,16 +580,9 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
     };
     if (warp == kProducerWarp) {
         // ---------------------------------------------------------------------- producer
-        // The chunks of all stages, numbered through.  Directory entries come in batches of eight
-        // chunks (lane 4 k + j: cell j of the batch's chunk k), loaded a batch ahead, so their latency and a stage's fields'
-        // stay off the ring's critical path.  (Like the finishers this warp gets an instruction in every few cycles only.)
-        constexpr int kBatch = 32 / kChunkCells;
-        struct PBatch {
-            uint32_t o0, o1;                 // directory entries of the lane's cell; equal: none
-            const unsigned char* cells;      // NULL: the end has come
-            int grp;                         // whose chunk it is
-        };
-        const int bk = lane / kChunkCells, bj = lane - bk * kChunkCells;
+        // Directory entries come in batches of up to 32 chunks of a stage, a chunk to a lane.  (Like the finishers this warp
+        // gets an instruction in every few cycles only, and with single cells' entries to look up and to pass on it spent 600
+        // cycles per chunk where a chunk's share of HBM's bandwidth is 540.)
         // A stage's descriptor is spread over the lanes, and the next stage's is loaded when the stage begins: its latency
         // (and a chain of dependent loads, 3000 cycles at every run of tiles when they were made one by one) is hidden.
         constexpr int kWords = (int)(sizeof(CStage) / 4);
@@ -602,7 +594,7 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
             return (const unsigned char*)((unsigned long long)hi << 32 | lo);
         };
 #define SD2_WORD(f) ((int)(offsetof(CStage, f) / 4))
-        int sa = 0, run0 = 0, n = 0, gb = 0;                     // stage; first chunk of the run of tiles, its cells, its first group
+        int sa = 0, q0 = 0, n = 0, gb = 0;                       // stage; of the run of tiles: next chunk, cells, first group
         RunDeal deal(0, 0);
         const uint32_t* off = nullptr;
         const unsigned char* cells = nullptr;
@@ -622,28 +614,30 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
             T2 = (int)word(SD2_WORD(mat[2].T));
         };
         begin_stage();
-        auto load_batch = [&](int first) {
-            PBatch c;
-            c.o0 = c.o1 = 0u;
-            c.cells = nullptr;
-            c.grp = 0;
-            while (true) {
-                const int q = first + bk - run0;
-                if (q >= 0 && q < deal.chunks) {
-                    const int turn = deal.split ? q : q / deal.per, i0 = deal.split ? 0 : turn * deal.cells;
-                    const int i = i0 + (deal.split ? q : q - turn * deal.per) * kChunkCells + bj;
-                    if (i < n && (deal.split || i < i0 + deal.cells)) {
-                        c.o0 = __ldg(off + i);
-                        c.o1 = __ldg(off + i + 1);
+        uint32_t o0 = 0, o1 = 0;             // the lane's chunk: directory entries of its first cell and past its last
+        const unsigned char* from = nullptr;
+        int from_grp = 0;                    // whose chunk it is
+        auto load_batch = [&]() {            // returns the number of chunks; 0: the end
+            int got = 0;
+            while (got < 32 && sa < a.n_stages) {
+                if (q0 < deal.chunks) {
+                    const int q = q0 + lane - got;
+                    if (lane >= got && q < deal.chunks) {
+                        const int turn = deal.split ? q : q / deal.per, i0 = deal.split ? 0 : turn * deal.cells;
+                        const int i = i0 + (deal.split ? q : q - turn * deal.per) * kChunkCells;
+                        o0 = __ldg(off + i);
+                        o1 = __ldg(off + min(i + kChunkCells, deal.split ? n : min(i0 + deal.cells, n)));
+                        from = cells;
+                        from_grp = (gb + turn) % kCellGroups;
                     }
-                    c.cells = cells;
-                    c.grp = (gb + turn) % kCellGroups;
+                    const int take = min(32 - got, deal.chunks - q0);
+                    q0 += take;
+                    got += take;
+                    continue;
                 }
-                if (run0 + deal.chunks >= first + kBatch || sa >= a.n_stages) return c;
-                run0 += deal.chunks;         // on to the next run of tiles, the next stage
-                gb = (gb + deal.turns) % kCellGroups;
-                n = 0;
+                gb = (gb + deal.turns) % kCellGroups;            // on to the next run of tiles, the next stage
                 deal = RunDeal(0, 0);
+                q0 = 0;
                 int mat, t0, nt;
                 if (runs.next(pair, count, T0, T1, T2, mat, t0, nt)) {
                     const int Dr = share_cells(D, rank), w = mat * (int)(sizeof(CMat) / 4);
@@ -652,12 +646,16 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                     cells = pointer(w + SD2_WORD(mat[0].cells));
                     off = (const uint32_t*)pointer(w + SD2_WORD(mat[0].off)) +
                           (rank ? (size_t)word(w + SD2_WORD(mat[0].T)) * share_cells(D, 0) : 0) + (size_t)t0 * Dr;
-                } else if (++sa < a.n_stages) {
-                    w0 = next_w0;
-                    w1 = next_w1;
-                    begin_stage();
+                } else {
+                    if (++sa < a.n_stages) {
+                        w0 = next_w0;
+                        w1 = next_w1;
+                        begin_stage();
+                    }
+                    if (got > 0) break;      // (the next descriptor may still be on its way)
                 }
             }
+            return got;
         };
         // weights are read once: with several stages their lines leave L2 first, so that the stream does not push out
         // the small, shared, re-read activations
@@ -666,32 +664,17 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         const uint32_t full0 = smem_u32(&sh->full[0][0]), empty0 = smem_u32(&sh->empty[0][0]), ring = smem_u32(smem) + ring_off;
         uint32_t next_slot = 0x101010u;      // of each group (a byte each): its next slot, 16 times the parity of the wait for it
         bool ok = true;
-        PBatch cur = load_batch(0);
-        for (int first = 0; ok; first += kBatch) {
-            const PBatch next = load_batch(first + kBatch);
-            // first and last directory entry of the lane's chunk
-            const uint32_t start = __shfl_sync(0xFFFFFFFFu, cur.o0, lane & ~(kChunkCells - 1));
-            uint32_t end = cur.o1;
-#pragma unroll
-            for (int k = 1; k < kChunkCells; k <<= 1) end = max(end, __shfl_xor_sync(0xFFFFFFFFu, end, k));
-            const uint32_t mine = ((cur.o0 - start) << 13) | (((cur.o1 - cur.o0) * 32u - kCellHeaderBytes) >> 7);
-            const unsigned there = __ballot_sync(0xFFFFFFFFu, cur.cells != nullptr);
-            for (int k = 0; k < kBatch; ++k) {
-                if (!(there >> (k * kChunkCells) & 1u)) break;
-                const int grp = __shfl_sync(0xFFFFFFFFu, cur.grp, k * kChunkCells);
+        for (int got; ok && (got = load_batch()) > 0;) {
+            const uint32_t bytes = (o1 - o0) * 32u;
+            for (int k = 0; k < got; ++k) {
+                const int grp = __shfl_sync(0xFFFFFFFFu, from_grp, k);
                 const uint32_t at = next_slot >> (8 * grp) & 0xFFu, slot = at & 15u;
-                const uint32_t s = (uint32_t)(grp * kGroupSlots) + slot;
+                const uint32_t s = (uint32_t)(grp * kGroupSlots) + slot, dst = ring + ((uint32_t)grp * NS + slot) * (uint32_t)a.chunk_bytes;
                 if (!wait_phase_warp(empty0 + 8 * s, at >> 4, wc)) { ok = false; break; }
-                if (bk == k && cur.o1 != cur.o0) (&sh->cell[0][0][0])[s * kChunkCells + bj] = mine;
-                __syncwarp();
-                // (by lane 4 k: the values are its own)
-                const uint32_t bytes = (end - start) * 32u, dst = ring + ((uint32_t)grp * NS + slot) * (uint32_t)a.chunk_bytes;
-                if (hinted) bulk_chunk(dst, cur.cells + (size_t)start * 32, bytes, full0 + 8 * s, lane == k * kChunkCells, policy);
-                else bulk_chunk(dst, cur.cells + (size_t)start * 32, bytes, full0 + 8 * s, lane == k * kChunkCells);
+                if (hinted) bulk_chunk(dst, from + (size_t)o0 * 32, bytes, full0 + 8 * s, lane == k, policy);
+                else bulk_chunk(dst, from + (size_t)o0 * 32, bytes, full0 + 8 * s, lane == k);
                 next_slot ^= (at ^ (slot + 1 == NS ? (at ^ 16u) & 16u : at + 1u)) << (8 * grp);
             }
-            if (there != 0xFFFFFFFFu) break;
-            cur = next;
         }
         if (!ok && lane == 0) {
             // give the copies already issued time to land before this CTA's memory is released
@@ -918,10 +901,16 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                 for (int i0 = i - cj; i0 < n; i0 += step, i += step) {
                     if (!wait_phase_warp(full0 + 8 * slot, phase, wc)) { failed = true; break; }
                     if (i < n) {
-                        const uint32_t where = sh->cell[grp][slot][cj];
-                        const uint32_t cell = ring + slot * (uint32_t)a.chunk_bytes + (where >> 8), H = where & 0xFFu;
+                        // where the chunk's cells start: the first one's header tells the heights of all four
+                        const uint32_t first = ring + slot * (uint32_t)a.chunk_bytes;
+                        const uint32_t heights = __ballot_sync(0xFFFFFFFFu, (lds_u8(first + 128u + lane) & 0x80u) != 0);
+                        uint32_t H = heights & 63u, before = 0;
+#pragma unroll
+                        for (int k = 1; k < kChunkCells; ++k)
+                            if (k <= cj) { before += H; H = heights >> (6 * k) & 63u; }
+                        const uint32_t cell = first + (uint32_t)cj * kCellHeaderBytes + before * 128u;
                         const uint32_t m = lds_u32(cell + 4 * lane), v0 = cell + kCellHeaderBytes;
-                        const uint32_t pi = *(smem + (cell - sbase) + 128 + lane);
+                        const uint32_t pi = lds_u8(cell + 128u + lane) & 0x7Fu;
                         const uint32_t xd = (uint32_t)d * (2 * kCellCols);
                         multiply_cell<NR>(m, v0 + 4u * lane, v0 + (H - 1u) * 128u + pi, xl + xd, xl8 + xd, acc);
                     }

@@ -20,7 +20,8 @@
 // Two CTAs share a tile: one takes the first ceil(D / 2) cells of its columns, the other the rest.  The cells of each
 // share stand together, tile by tile, so that a CTA's run of tiles is one run of bytes.
 //
-//   cell    u32 mask[32], u8 pi[32] (4 x column), u32 words[H][32]
+//   cell    u32 mask[32], u8 pi[32] (4 x column), u32 words[H][32].  Bit 7 of pi[6 k + i] is bit i of the height H of the
+//           k-th cell from this one on, k = 0..3: a reader of four consecutive cells finds them from the first one.
 //   sec0    u32 cell_off[T * D + 1] (32-byte units into sec1), in order of share, then tile, then column
 //   sec1    cells
 
@@ -151,7 +152,17 @@ inline CellImage pack_cells(const uint16_t* W, const uint8_t* mask, int64_t M, i
     for (int64_t i = 0; i < g.T; ++i)
         for (int r = 0; r < 2; ++r) {
             const std::vector<uint8_t>& src = tiles[(size_t)(r * g.T + i)];
-            if (!src.empty()) std::memcpy(im.data + sec1_off + (size_t)off[(size_t)(first_cell[r] + i * share_cells(g.D, r))] * 32, src.data(), src.size());
+            if (src.empty()) continue;
+            const int64_t c0 = first_cell[r] + i * share_cells(g.D, r);
+            uint8_t* dst = im.data + sec1_off + (size_t)off[(size_t)c0] * 32;
+            std::memcpy(dst, src.data(), src.size());
+            for (int64_t c = c0; c < c0 + share_cells(g.D, r); ++c) {
+                uint32_t heights = 0;                     // of this cell and the three that follow it
+                for (int64_t k = 0; k < kChunkCells && c + k < n_cells; ++k)
+                    heights |= ((off[(size_t)(c + k + 1)] - off[(size_t)(c + k)]) * 32u - kCellHeaderBytes) / 128u << (6 * k);
+                uint8_t* pi = im.data + sec1_off + (size_t)off[(size_t)c] * 32 + 128;
+                for (int l = 0; l < 6 * kChunkCells; ++l) pi[l] |= (uint8_t)((heights >> l & 1u) << 7);
+            }
         }
     im.sec1_off = sec1_off;
     im.bytes = sec1_off + (size_t)units * 32;
