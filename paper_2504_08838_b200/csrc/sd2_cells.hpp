@@ -64,41 +64,57 @@ struct CellImage {
 inline void pack_cell(const uint16_t* W, const uint8_t* mask, int64_t M, int64_t K, int64_t m0, int64_t k0, std::vector<uint8_t>& out)
 {
     uint32_t bits[32];
-    uint32_t words[2][32][16];
+    uint32_t words[2][32][17];
     uint8_t n_words[2][32];
     std::memset(bits, 0, sizeof bits);
     std::memset(n_words, 0, sizeof n_words);
+    const int64_t left = K - k0;
+    const int cols = left < kCellCols ? (int)left : kCellCols;
+    uint16_t wv[kCellCols] = {};
     for (int row = 0; row < kTileRows && m0 + row < M; ++row) {
-        const uint16_t* wr = W + (m0 + row) * K;
-        const uint8_t* mr = mask ? mask + (m0 + row) * K : nullptr;
+        // the row's kept values, zero elsewhere, and which of them are kept (no branch on a single one: those are coin tosses)
+        const uint16_t* wr = W + (m0 + row) * K + k0;
+        uint8_t kept[kCellCols] = {};
+        if (mask) {
+            const uint8_t* mr = mask + (m0 + row) * K + k0;
+            for (int c = 0; c < cols; ++c) kept[c] = mr[c] != 0;
+        } else {
+            for (int c = 0; c < cols; ++c) kept[c] = (wr[c] & 0x7FFF) != 0;
+        }
+        for (int c = 0; c < cols; ++c) wv[c] = (uint16_t)(wr[c] & -(int)kept[c]);
         const int r = row >> 3;
-        const int64_t left = K - k0;
-        const int cols = left < kCellCols ? (int)left : kCellCols;
-        for (int c = 0; c < cols; c += 2) {
-            const int l = 4 * (row & 7) + ((c >> 3) & 3);
-            const bool two = c + 1 < cols;
-            const uint32_t lo = wr[k0 + c], hi = two ? wr[k0 + c + 1] : 0u;
-            const bool klo = mr ? mr[k0 + c] != 0 : (lo & 0x7FFF) != 0;
-            const bool khi = two && (mr ? mr[k0 + c + 1] != 0 : (hi & 0x7FFF) != 0);
-            if (!klo && !khi) continue;
-            bits[l] |= 1u << (16 * r + 4 * (c >> 5) + ((c >> 1) & 3));
-            words[r][l][n_words[r][l]++] = (klo ? lo : 0u) | (khi ? hi << 16 : 0u);
+        for (int t = 0; t < 4; ++t) {
+            const int l = 4 * (row & 7) + t;
+            uint32_t n = 0, b = 0;
+            for (int u = 0; u < 4; ++u)
+                for (int i = 0; i < 4; ++i) {
+                    const int c = 32 * u + 8 * t + 2 * i;
+                    const uint32_t any = kept[c] | kept[c + 1];
+                    words[r][l][n] = (uint32_t)wv[c] | (uint32_t)wv[c + 1] << 16;
+                    n += any;
+                    b |= any << (4 * u + i);
+                }
+            bits[l] |= b << (16 * r);
+            n_words[r][l] = (uint8_t)n;
         }
     }
     // lanes by the words of their first row, most first, and by those of their second, fewest first; equal ranks share a column
-    int col_of_rank[32], k = 0, H = 0;
-    for (int n = 16; n >= 0; --n)
-        for (int l = 0; l < 32; ++l)
-            if (n_words[0][l] == n) col_of_rank[k++] = l;
+    int place[2][18] = {}, col_of_rank[32], H = 0;
+    for (int l = 0; l < 32; ++l) {
+        ++place[0][17 - n_words[0][l]];
+        ++place[1][n_words[1][l] + 1];
+    }
+    for (int n = 1; n < 18; ++n) {
+        place[0][n] += place[0][n - 1];
+        place[1][n] += place[1][n - 1];
+    }
     uint8_t pi[32];
-    k = 0;
-    for (int n = 0; n <= 16; ++n)
-        for (int l = 0; l < 32; ++l)
-            if (n_words[1][l] == n) {
-                const int c = col_of_rank[k++];
-                pi[l] = (uint8_t)(4 * c);
-                if (n_words[0][c] + n > H) H = n_words[0][c] + n;
-            }
+    for (int l = 0; l < 32; ++l) col_of_rank[place[0][16 - n_words[0][l]]++] = l;
+    for (int l = 0; l < 32; ++l) {
+        const int c = col_of_rank[place[1][n_words[1][l]]++];
+        pi[l] = (uint8_t)(4 * c);
+        if (n_words[0][c] + n_words[1][l] > H) H = n_words[0][c] + n_words[1][l];
+    }
     const size_t at = out.size();
     out.resize(at + kCellHeaderBytes + (size_t)H * 128, 0);
     uint8_t* p = out.data() + at;

@@ -343,11 +343,27 @@ inline int gap4_run_entries(const int32_t* cols, int n)
     return e;
 }
 
-inline void gap4_row_cols(const uint16_t* W, const uint8_t* mask, int64_t m, int64_t K, std::vector<int32_t>& cols)
+// The kept columns of row m to the front of `cols` (a scratch that only grows); returns how many.
+inline int gap4_row_cols(const uint16_t* W, const uint8_t* mask, int64_t m, int64_t K, std::vector<int32_t>& cols)
 {
-    cols.clear();
-    for (int64_t k = 0; k < K; ++k)
-        if (is_kept(W, mask, m * K + k)) cols.push_back((int32_t)k);
+    // (no branch on a column's fate: it is a coin toss, and mispredicted ones were most of the packing time)
+    if ((int64_t)cols.size() < K + 1) cols.resize((size_t)K + 1);
+    int32_t* c = cols.data();
+    size_t n = 0;
+    if (mask) {
+        const uint8_t* mr = mask + m * K;
+        for (int64_t k = 0; k < K; ++k) {
+            c[n] = (int32_t)k;
+            n += mr[k] != 0;
+        }
+    } else {
+        const uint16_t* wr = W + m * K;
+        for (int64_t k = 0; k < K; ++k) {
+            c[n] = (int32_t)k;
+            n += (wr[k] & 0x7FFF) != 0;
+        }
+    }
+    return (int)n;
 }
 
 inline PackResult pack_gap4(const uint16_t* W, const uint8_t* mask, int64_t M, int64_t K, int y_dtype, bool pair_rows = false)
@@ -367,8 +383,8 @@ inline PackResult pack_gap4(const uint16_t* W, const uint8_t* mask, int64_t M, i
         std::vector<int> f((size_t)S + 1);
 #pragma omp for schedule(static)
         for (int64_t m = 0; m < M; ++m) {
-            gap4_row_cols(W, mask, m, K, cols);
-            gap4_deal_row(cols.data(), (int)cols.size(), S, B, V, f.data());
+            const int n_cols = gap4_row_cols(W, mask, m, K, cols);
+            gap4_deal_row(cols.data(), n_cols, S, B, V, f.data());
             int64_t tot = 0;
             for (int l = 0; l < S; ++l) {
                 first[(size_t)m * (S + 1) + l] = f[(size_t)l];
@@ -378,7 +394,7 @@ inline PackResult pack_gap4(const uint16_t* W, const uint8_t* mask, int64_t M, i
             }
             first[(size_t)m * (S + 1) + S] = f[(size_t)S];
             row_chunks[(size_t)m] = tot;
-            row_kept[(size_t)m] = (int64_t)cols.size();
+            row_kept[(size_t)m] = n_cols;
         }
     }
     // rows by chunk count, most first, ties by index
@@ -470,17 +486,20 @@ inline PackResult pack_gap4(const uint16_t* W, const uint8_t* mask, int64_t M, i
                     // the cursor starts on the run's first column, given relative to the lane's window
                     start[l] = (uint16_t)(cols[(size_t)e0] - ((int64_t)s * B - V));
                     int64_t cursor = cols[(size_t)e0];
+                    uint8_t* gap = eg[l].data();
+                    uint16_t* val = ev[l].data();
+                    const uint16_t* wr = W + m * K;
                     size_t e = 0;
                     for (int x = e0; x < e1; ++x) {
                         const int64_t k = cols[(size_t)x];
                         while (k - cursor > 15) {  // filler 15 columns ahead
-                            eg[l][e] = 15;
-                            ev[l][e] = 0;
+                            gap[e] = 15;
+                            val[e] = 0;
                             ++e;
                             cursor += 16;
                         }
-                        eg[l][e] = (uint8_t)(k - cursor);
-                        ev[l][e] = W[m * K + k];
+                        gap[e] = (uint8_t)(k - cursor);
+                        val[e] = wr[k];
                         ++e;
                         cursor = k + 1;
                     }
@@ -497,11 +516,10 @@ inline PackResult pack_gap4(const uint16_t* W, const uint8_t* mask, int64_t M, i
             for (int j = 0; j < maxc; ++j) {
                 for (int l = 0; l < 32; ++l) {
                     if (cnt[l] <= j) continue;
+                    const uint8_t* gaps = eg[l].data() + (size_t)j * 8;
                     uint32_t code = 0;
-                    for (int i = 0; i < 8; ++i) {
-                        code |= (uint32_t)eg[l][(size_t)j * 8 + i] << (4 * i);
-                        vals[slot * 8 + i] = ev[l][(size_t)j * 8 + i];
-                    }
+                    for (int i = 0; i < 8; ++i) code |= (uint32_t)gaps[i] << (4 * i);
+                    std::memcpy(vals + slot * 8, ev[l].data() + (size_t)j * 8, 16);
                     codes[slot] = code;
                     ++slot;
                 }
