@@ -69,7 +69,7 @@ struct sd2_drafter_s {
     int64_t tags_bytes;
     int K_max, max_tile;       // what decides the shared-memory split
     int free_tiles;            // every stage has enough tiles per CTA for free tile assignment
-    int xs_need[4];            // bytes of staged activations at panel widths 1, 2, 4, 8
+    int xs_need[3];            // bytes of staged activations at panel widths 1, 2, 4
     // the same blocks as a program over cells, with barrier words of its own; NULL: a handle has no cells
     CStage* d_cstages;
     CStage first_cstage;
@@ -174,10 +174,13 @@ sd2_status ensure_device(int* dev_out)
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev) != cudaSuccess) { cudaGetLastError(); return SD2_ERR_CUDA; }
         if (set_smem_attr<1>() != cudaSuccess || set_smem_attr<2>() != cudaSuccess || set_smem_attr<4>() != cudaSuccess ||
-            set_smem_attr<8>() != cudaSuccess || set_cell_attr<1, 8>() != cudaSuccess || set_cell_attr<1, 16>() != cudaSuccess ||
+            set_cell_attr<1, 8>() != cudaSuccess || set_cell_attr<1, 16>() != cudaSuccess ||
             set_cell_attr<kMaxStagesInline, 8>() != cudaSuccess || set_cell_attr<kMaxStagesInline, 16>() != cudaSuccess ||
             cudaFuncSetAttribute(mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
-            cudaFuncSetAttribute(lm_head_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess) {
+            cudaFuncSetAttribute(lm_head_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
+            cudaFuncSetAttribute(lm_head_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
+            cudaFuncSetAttribute(lm_head_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
+            cudaFuncSetAttribute(lm_head_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess) {
             cudaGetLastError();
             return SD2_ERR_CUDA;
         }
@@ -452,8 +455,7 @@ sd2_status launch_stream(int nt, SArgs& a, int grid, bool cooperative, cudaStrea
     switch (nt) {
         case 1: return launch_stream_nt<1>(a, grid, smem, cooperative, s);
         case 2: return launch_stream_nt<2>(a, grid, smem, cooperative, s);
-        case 4: return launch_stream_nt<4>(a, grid, smem, cooperative, s);
-        default: return launch_stream_nt<8>(a, grid, smem, cooperative, s);
+        default: return launch_stream_nt<4>(a, grid, smem, cooperative, s);
     }
 }
 
@@ -510,7 +512,7 @@ long long wait_budget(int dev)
 struct ProgramNeeds {
     int K_max = 0, max_tile = 0, tiles_max = 0;
     int tiles_min = 0x7FFFFFFF;   // fewest tiles of any stage
-    int xs_need[4] = {0, 0, 0, 0};   // staged activations at panel widths 1, 2, 4, 8: the largest over all stages
+    int xs_need[3] = {0, 0, 0};   // staged activations at panel widths 1, 2, 4: the largest over all stages
     // Free tile assignment pays where every stage gives a CTA about as many tiles as it has consumer
     // warps, or more; with fewer, the fixed deal is faster (see the consumer loop of stream_kernel).
     int free_tiles(int grid) const { return tiles_min >= 12 * grid ? 1 : 0; }
@@ -522,7 +524,7 @@ struct ProgramNeeds {
             const int lin = hs[i]->S * hs[i]->B + 2 * hs[i]->V + 64;
             if (lin > K_max) K_max = lin;
             if (hs[i]->max_tile_bytes > max_tile) max_tile = hs[i]->max_tile_bytes;
-            for (int w = 0; w < 4; ++w) {
+            for (int w = 0; w < 3; ++w) {
                 const int need = xs_bytes_for(hs[i]->S, hs[i]->B, hs[i]->V, 1 << w);
                 if (need > xs_need[w]) xs_need[w] = need;
             }
@@ -533,23 +535,23 @@ struct ProgramNeeds {
     }
 };
 
-int nt_index(int nt) { return nt == 1 ? 0 : nt == 2 ? 1 : nt == 4 ? 2 : 3; }
+int nt_index(int nt) { return nt == 1 ? 0 : nt == 2 ? 1 : 2; }
 
-// Widest panel (8, 4, 2, 1 rows) whose staged activations still leave room for the ring; 0 if none.
-int widest_panel(const int xs_need[4], int K_max, int max_tile)
+// Widest panel (4, 2, 1 rows; four and more take the cells) whose staged activations still leave room for the ring; 0 if none.
+int widest_panel(const int xs_need[3], int K_max, int max_tile)
 {
     // a wide panel whose activations crowd out the ring cannot stream: ask for a ring of at
     // least 96 KB first, and settle for whatever fits only if no width leaves that much
     SmemPlan p;
-    for (int nt = 8; nt >= 1; nt >>= 1)
+    for (int nt = 4; nt >= 1; nt >>= 1)
         if (plan_smem(nt, xs_need[nt_index(nt)], K_max, max_tile, &p) && p.ring_bytes >= 96 * 1024) return nt;
-    for (int nt = 8; nt >= 1; nt >>= 1)
+    for (int nt = 4; nt >= 1; nt >>= 1)
         if (plan_smem(nt, xs_need[nt_index(nt)], K_max, max_tile, &p)) return nt;
     return 0;
 }
 
 // Launches a program over all N rows, in panels of at most `nt_cap` rows (rows are independent).
-sd2_status run_panels(SArgs& a, int64_t N, const int xs_need[4], int K_max, int max_tile, int grid, cudaStream_t s)
+sd2_status run_panels(SArgs& a, int64_t N, const int xs_need[3], int K_max, int max_tile, int grid, cudaStream_t s)
 {
     const int nt_cap = widest_panel(xs_need, K_max, max_tile);
     if (nt_cap == 0) return SD2_ERR_UNSUPPORTED;
@@ -738,13 +740,41 @@ sd2_status run_cell_program(CArgs<kMaxStagesInline>& a, const CellBuilder& b, in
     return run_cell_panels(a, N, b.needs, grid, s);
 }
 
-// Whether a call of N rows over these GAP4 handles takes their cells.
-#ifndef SD2_CELLS_MIN
-#define SD2_CELLS_MIN 4
-#endif
+// An LM head of NT activation rows at most.
+template <int NT>
+sd2_status launch_lm_head(const uint16_t* x, const uint16_t* w, float* logits, int n, int V, int H, int sms, cudaStream_t s)
+{
+    const size_t smem = (size_t)NT * (size_t)H * 2;
+    int per_sm = (int)((size_t)(200 * 1024) / smem);
+    per_sm = per_sm < 1 ? 1 : per_sm > head_ctas(NT) ? head_ctas(NT) : per_sm;
+    int64_t grid = ((int64_t)V + kGlueThreads / 32 - 1) / (kGlueThreads / 32);
+    if (grid > (int64_t)sms * per_sm) grid = (int64_t)sms * per_sm;
+    lm_head_kernel<NT><<<(unsigned)grid, kGlueThreads, smem, s>>>(x, w, logits, n, V, H);
+    return cudaGetLastError() == cudaSuccess ? SD2_OK : SD2_ERR_CUDA;
+}
+
+// Whether N rows over these GAP4 handles are faster by their cells.  Cells bring 1.3 times the strips' bytes but expand them
+// once for all rows, the strips gather row by row.  Measured (us, cold caches, strips / cells): 2048 x 8192 at 50 %: N = 1
+// 14.4 / 16.4, N = 2 18.4 / 16.4, N = 3 24.6 / 16.4; the same at 30 %: 12.3 / 14.5, 15.4 / 16.4, 20.5 / 16.3; two blocks of
+// 2048/512/8192 at 50 %: 60 / 70, 75 / 70, 116 / 72.  Below a million slots both take the time of a launch for N <= 3, and
+// there the rows of small steps keep the sums of a one-row step.
+bool cells_pay(const sd2_handle* hs, int count, int64_t N)
+{
+    if (N >= 4) return true;
+    if (N < 2) return false;
+    int64_t slots = 0, kept = 0, largest = 0;
+    for (int i = 0; i < count; ++i) {
+        const int64_t n = hs[i]->M * hs[i]->K;
+        slots += n;
+        kept += hs[i]->nnz;
+        if (n > largest) largest = n;
+    }
+    return largest >= (1 << 20) && (N > 2 || 5 * kept >= 2 * slots);
+}
+
+// ... and whether the call can take them.
 bool use_cells(const sd2_handle* hs, int count, int64_t N)
 {
-    if (N < SD2_CELLS_MIN) return false;
     CellNeeds needs;
     for (int i = 0; i < count; ++i) {
         if (!hs[i]->d_image) return false;
@@ -752,7 +782,7 @@ bool use_cells(const sd2_handle* hs, int count, int64_t N)
         if (pitch > needs.pitch) needs.pitch = pitch;
         if (hs[i]->max_chunk > needs.max_chunk) needs.max_chunk = hs[i]->max_chunk;
     }
-    return widest_cell_panel(needs) > 0;
+    return cells_pay(hs, count, N) && widest_cell_panel(needs) > 0;
 }
 
 // Shared by sd2_spmm and sd2_spmm_fused (and by block steps that mix formats).
@@ -1402,19 +1432,17 @@ sd2_status sd2_lm_head(const void* x, const void* w_out, float* logits, int32_t*
     cudaStream_t s = (cudaStream_t)cuda_stream;
     for (int64_t n0 = 0; n0 < N; n0 += kHeadMaxRows) {
         const int n = (int)((N - n0) < kHeadMaxRows ? (N - n0) : kHeadMaxRows);
-        const size_t smem = (size_t)n * (size_t)H * 4;
-        int64_t grid = (V + kGlueThreads / 32 - 1) / (kGlueThreads / 32);
-        // as many CTAs per SM as the staged rows allow (8 x 256 threads fill an SM): the stream needs many loads in flight
-        int per_sm = smem ? (int)((200 * 1024) / smem) : 8;
-        per_sm = per_sm < 1 ? 1 : per_sm > 8 ? 8 : per_sm;
-        const int64_t cap = (int64_t)g_dev[dev].sms * per_sm;
-        if (grid > cap) grid = cap;
-        lm_head_kernel<<<(unsigned)grid, kGlueThreads, smem, s>>>((const uint16_t*)x + n0 * H, (const uint16_t*)w_out, logits + n0 * V, n, (int)V, (int)H);
-        if (cudaGetLastError() != cudaSuccess) return SD2_ERR_CUDA;
+        const uint16_t* xp = (const uint16_t*)x + n0 * H;
+        float* lp = logits + n0 * V;
+        st = n == 1 ? launch_lm_head<1>(xp, (const uint16_t*)w_out, lp, n, (int)V, (int)H, g_dev[dev].sms, s)
+           : n == 2 ? launch_lm_head<2>(xp, (const uint16_t*)w_out, lp, n, (int)V, (int)H, g_dev[dev].sms, s)
+           : n <= 4 ? launch_lm_head<4>(xp, (const uint16_t*)w_out, lp, n, (int)V, (int)H, g_dev[dev].sms, s)
+                    : launch_lm_head<8>(xp, (const uint16_t*)w_out, lp, n, (int)V, (int)H, g_dev[dev].sms, s);
+        if (st != SD2_OK) return st;
     }
     if (tokens && N > 0) {
         const int vec = ((V & 3) == 0 && (((uintptr_t)logits) & 15) == 0) ? 1 : 0;
-        argmax_kernel<<<(unsigned)N, 1024, 0, s>>>(logits, tokens, (int)V, vec);
+        argmax_kernel<<<(unsigned)(N * kArgmaxCtas), 512, 0, s>>>(logits, tokens, (int)V, vec);
         if (cudaGetLastError() != cudaSuccess) return SD2_ERR_CUDA;
     }
     return SD2_OK;
@@ -1871,7 +1899,7 @@ sd2_status sd2_drafter_create(const sd2_handle* h, int32_t L, int64_t n_max, sd2
     bool cells = true;
     for (const sd2_handle hh : d->handles)
         if (!hh->d_image) cells = false;
-    if (ok && cells && n_max >= SD2_CELLS_MIN) {
+    if (ok && cells && n_max >= 2) {
         // the same blocks over cells, for steps of several rows
         std::vector<CStage> cstages((size_t)L * 4);
         CellBuilder bld(cstages.data(), g_dev[dev].sms);
@@ -1910,7 +1938,7 @@ sd2_status sd2_drafter_create(const sd2_handle* h, int32_t L, int64_t n_max, sd2
     d->K_max = needs.K_max;
     d->free_tiles = needs.free_tiles(g_dev[dev].sms);
     d->max_tile = needs.max_tile;
-    for (int w = 0; w < 4; ++w) d->xs_need[w] = needs.xs_need[w];
+    for (int w = 0; w < 3; ++w) d->xs_need[w] = needs.xs_need[w];
     {
         std::lock_guard<std::mutex> lk(g_mu);
         g_live_drafters.insert(d);
@@ -1922,7 +1950,7 @@ sd2_status sd2_drafter_create(const sd2_handle* h, int32_t L, int64_t n_max, sd2
 namespace {
 bool drafter_uses_cells(sd2_drafter d, int64_t N)
 {
-    return N >= SD2_CELLS_MIN && d->d_cstages && widest_cell_panel(d->cell_needs) > 0;
+    return d->d_cstages && cells_pay(d->handles.data(), 7 * d->L, N) && widest_cell_panel(d->cell_needs) > 0;
 }
 }  // namespace
 

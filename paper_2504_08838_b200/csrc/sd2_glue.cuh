@@ -397,84 +397,86 @@ __global__ void __launch_bounds__(kGlueThreads) embedding_kernel(const int32_t* 
 }
 
 // logits[n, v] = sum_h W[v, h] x[n, h]: a warp takes kHeadRowsPerWarp vocabulary rows at a time (as many independent
-// 128-bit loads in flight per lane), the N <= 8 activation rows sit in shared memory as fp32.  H a multiple of 8.
+// 128-bit loads in flight per lane) of its share of the table, the activation rows sit in shared memory as bf16.  HBM bounds
+// it.  Shares are runs of rows of (almost) equal length: with steps of four rows dealt out in turn, 3.4 of them per warp for
+// 128256 rows, some warps worked while others were done.  Four rows share what is read of the activations; with one row per
+// step and fp32 activations a row took as long as a pass of its own (a step of one row 257 us, of four rows 1033 us).
 constexpr int kHeadRowsPerWarp = 4;
-__global__ void __launch_bounds__(kGlueThreads) lm_head_kernel(const uint16_t* x, const uint16_t* W, float* logits, int N, int V, int H)
+// CTAs per SM of an instance for NT rows, as many as its registers allow
+constexpr int head_ctas(int NT) { return NT <= 1 ? 5 : NT <= 2 ? 3 : 2; }
+template <int NT>
+__global__ void __launch_bounds__(kGlueThreads, head_ctas(NT)) lm_head_kernel(const uint16_t* x, const uint16_t* W, float* logits, int N, int V, int H)
 {
-    extern __shared__ float xs[];            // [N][H]
-    for (int i = threadIdx.x; i < N * H; i += blockDim.x) xs[i] = bf16_to_f32(x[i]);
+    extern __shared__ uint4 head_x[];        // [NT][H / 8]: zero beyond row N
+    const int groups = H / 8;
+    for (int i = threadIdx.x; i < NT * H; i += blockDim.x) ((uint16_t*)head_x)[i] = i < N * H ? x[i] : (uint16_t)0;
     __syncthreads();
     const int lane = threadIdx.x & 31;
-    const int warps = (gridDim.x * blockDim.x) >> 5;
-    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (N == 1) {
-        // the draft-token case: four rows per warp step
-        for (int v0 = gw * kHeadRowsPerWarp; v0 < V; v0 += warps * kHeadRowsPerWarp) {
-            float acc[kHeadRowsPerWarp] = {0.f, 0.f, 0.f, 0.f};
-            for (int c = lane; c < H / 8; c += 32) {
-                uint4 w4[kHeadRowsPerWarp];
+    const long long warps = (gridDim.x * blockDim.x) >> 5, gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int end = (int)(V * (gw + 1) / warps);
+    for (int v0 = (int)(V * gw / warps); v0 < end; v0 += kHeadRowsPerWarp) {
+        float acc[NT][kHeadRowsPerWarp];
 #pragma unroll
-                for (int r = 0; r < kHeadRowsPerWarp; ++r)
-                    w4[r] = v0 + r < V ? __ldg((const uint4*)(W + (size_t)(v0 + r) * H) + c) : make_uint4(0u, 0u, 0u, 0u);
-                const float* xr = xs + c * 8;
+        for (int n = 0; n < NT; ++n)
+#pragma unroll
+            for (int r = 0; r < kHeadRowsPerWarp; ++r) acc[n][r] = 0.f;
+#pragma unroll(NT < 8 ? 2 : 1)
+        for (int c = lane; c < groups; c += 32) {
+            uint4 w4[kHeadRowsPerWarp];
+#pragma unroll
+            for (int r = 0; r < kHeadRowsPerWarp; ++r)
+                w4[r] = v0 + r < end ? __ldg((const uint4*)(W + (size_t)(v0 + r) * H) + c) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+            for (int n = 0; n < NT; ++n) {
+                const uint4 xv = head_x[n * groups + c];
+                const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w};
 #pragma unroll
                 for (int r = 0; r < kHeadRowsPerWarp; ++r) {
                     const uint32_t ww[4] = {w4[r].x, w4[r].y, w4[r].z, w4[r].w};
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[r] += bf16_lo(ww[j]) * xr[2 * j] + bf16_hi(ww[j]) * xr[2 * j + 1];
+                    for (int j = 0; j < 4; ++j) acc[n][r] += bf16_lo(ww[j]) * bf16_lo(xw[j]) + bf16_hi(ww[j]) * bf16_hi(xw[j]);
                 }
             }
+        }
+#pragma unroll
+        for (int n = 0; n < NT; ++n)
 #pragma unroll
             for (int r = 0; r < kHeadRowsPerWarp; ++r) {
-                float s = acc[r];
-                for (int dd = 16; dd > 0; dd >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, dd);
-                if (lane == 0 && v0 + r < V) logits[v0 + r] = s;
+                const float s = warp_sum(acc[n][r]);
+                if (lane == 0 && n < N && v0 + r < end) logits[(size_t)n * V + v0 + r] = s;
             }
-        }
-        return;
-    }
-    for (int v = gw; v < V; v += warps) {
-        const uint4* wr = (const uint4*)(W + (size_t)v * H);
-        float acc[kHeadMaxRows];
-#pragma unroll
-        for (int n = 0; n < kHeadMaxRows; ++n) acc[n] = 0.f;
-#pragma unroll 4
-        for (int c = lane; c < H / 8; c += 32) {
-            const uint4 w4 = __ldg(wr + c);
-            const uint32_t ww[4] = {w4.x, w4.y, w4.z, w4.w};
-#pragma unroll
-            for (int n = 0; n < kHeadMaxRows; ++n) {
-                if (n < N) {
-                    const float* xr = xs + n * H + c * 8;
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[n] += bf16_lo(ww[j]) * xr[2 * j] + bf16_hi(ww[j]) * xr[2 * j + 1];
-                }
-            }
-        }
-#pragma unroll
-        for (int n = 0; n < kHeadMaxRows; ++n) {
-            if (n < N) {
-                float s = acc[n];
-                for (int dd = 16; dd > 0; dd >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, dd);
-                if (lane == 0) logits[(size_t)n * V + v] = s;
-            }
-        }
     }
 }
 
-// token[n] = index of the largest logit of row n, the lowest index among equals; one CTA per row.
-// vec: V is a multiple of 4 and the row is 16-byte aligned (four logits per load, eight loads in flight).
-__global__ void __launch_bounds__(1024) argmax_kernel(const float* logits, int32_t* token, int V, int vec)
+// token[n] = index of the largest logit of row n, the lowest index among equals; a cluster of kArgmaxCtas per row (one CTA
+// reads 513 KB of logits in 9 us).  vec: V is a multiple of 4 and the row is 16-byte aligned (four logits per load).
+constexpr int kArgmaxCtas = 8;
+__device__ __forceinline__ void argmax_merge(float& best, int& at, float v, int i)
+{
+    if (v > best || (v == best && i < at)) { best = v; at = i; }
+}
+__device__ __forceinline__ void argmax_warp(float& best, int& at)
+{
+    for (int d = 16; d > 0; d >>= 1) {
+        const float ov = __shfl_xor_sync(0xFFFFFFFFu, best, d);
+        const int oi = __shfl_xor_sync(0xFFFFFFFFu, at, d);
+        argmax_merge(best, at, ov, oi);
+    }
+}
+__global__ void __cluster_dims__(kArgmaxCtas, 1, 1) __launch_bounds__(512) argmax_kernel(const float* logits, int32_t* token, int V, int vec)
 {
     __shared__ float bv[32];
     __shared__ int bi[32];
-    const float* r = logits + (size_t)blockIdx.x * V;
+    __shared__ uint2 found[kArgmaxCtas];     // of rank 0: every CTA's best, as bits, and its index
+    const int row = blockIdx.x / kArgmaxCtas, rank = blockIdx.x % kArgmaxCtas;
+    const float* r = logits + (size_t)row * V;
     float best = -INFINITY;
     int at = 0x7FFFFFFF;
+    const int first = rank * blockDim.x + threadIdx.x, step = kArgmaxCtas * blockDim.x;
     if (vec) {
         const float4* r4 = (const float4*)r;
 #pragma unroll 8
-        for (int i = threadIdx.x; i < V / 4; i += blockDim.x) {
+        for (int i = first; i < V / 4; i += step) {
             const float4 v = r4[i];
             const float c[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
@@ -482,27 +484,32 @@ __global__ void __launch_bounds__(1024) argmax_kernel(const float* logits, int32
                 if (c[j] > best) { best = c[j]; at = 4 * i + j; }      // a thread meets its indices in ascending order
         }
     } else {
-        for (int i = threadIdx.x; i < V; i += blockDim.x) {
+        for (int i = first; i < V; i += step) {
             const float v = r[i];
             if (v > best) { best = v; at = i; }
         }
     }
-    for (int d = 16; d > 0; d >>= 1) {
-        const float ov = __shfl_xor_sync(0xFFFFFFFFu, best, d);
-        const int oi = __shfl_xor_sync(0xFFFFFFFFu, at, d);
-        if (ov > best || (ov == best && oi < at)) { best = ov; at = oi; }
-    }
+    argmax_warp(best, at);
     if ((threadIdx.x & 31) == 0) { bv[threadIdx.x >> 5] = best; bi[threadIdx.x >> 5] = at; }
-    __syncthreads();
+    // (both CTAs of a remote store have to be running, and rank 0 may leave only when all stores are there)
+    asm volatile("barrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory");
     if (threadIdx.x < 32) {
         best = threadIdx.x < (blockDim.x >> 5) ? bv[threadIdx.x] : -INFINITY;
         at = threadIdx.x < (blockDim.x >> 5) ? bi[threadIdx.x] : 0x7FFFFFFF;
-        for (int d = 16; d > 0; d >>= 1) {
-            const float ov = __shfl_xor_sync(0xFFFFFFFFu, best, d);
-            const int oi = __shfl_xor_sync(0xFFFFFFFFu, at, d);
-            if (ov > best || (ov == best && oi < at)) { best = ov; at = oi; }
+        argmax_warp(best, at);
+        if (threadIdx.x == 0) {
+            uint32_t to;
+            asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(to) : "r"(smem_u32(&found[rank])));
+            asm volatile("st.shared::cluster.v2.b32 [%0], {%1, %2};" ::"r"(to), "r"(__float_as_uint(best)), "r"((uint32_t)at) : "memory");
         }
-        if (threadIdx.x == 0) token[blockIdx.x] = at == 0x7FFFFFFF ? 0 : at;
+    }
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive;\n\tbarrier.cluster.wait;" ::: "memory");
+    if (rank == 0 && threadIdx.x < 32) {
+        best = threadIdx.x < kArgmaxCtas ? __uint_as_float(found[threadIdx.x].x) : -INFINITY;
+        at = threadIdx.x < kArgmaxCtas ? (int)found[threadIdx.x].y : 0x7FFFFFFF;
+        argmax_warp(best, at);
+        if (threadIdx.x == 0) token[row] = at == 0x7FFFFFFF ? 0 : at;
     }
 }
 
