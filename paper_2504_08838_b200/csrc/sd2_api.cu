@@ -100,6 +100,28 @@ std::mutex g_mu;
 std::unordered_set<sd2_handle> g_live;
 std::unordered_set<sd2_drafter> g_live_drafters;
 
+// A launch that may start while the kernel before it in the stream ends (see pdl_wait).
+cudaLaunchAttribute pdl_attribute()
+{
+    cudaLaunchAttribute a;
+    a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    a.val.programmaticStreamSerializationAllowed = 1;
+    return a;
+}
+template <class... P, class... A>
+cudaError_t launch_pdl(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr = pdl_attribute();
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 constexpr int kMaxDevices = 64;
 constexpr int kBarrierPool = 64;             // grid-barrier word pairs handed out round-robin
 constexpr int kBarrierStrideWords = 64;      // 256 bytes apart
@@ -343,7 +365,7 @@ int bitmask_grid(int64_t rows_total, int sms)
 template <int NT>
 sd2_status launch_bitmask_nt(const LaunchGroup& grp, int grid, cudaStream_t s)
 {
-    bitmask_kernel<NT><<<grid, kThreads, 0, s>>>(grp);
+    launch_pdl(bitmask_kernel<NT>, grid, kThreads, 0, s, grp);
     if (cudaGetLastError() != cudaSuccess) return SD2_ERR_CUDA;
     return SD2_OK;
 }
@@ -440,8 +462,9 @@ sd2_status launch_stream_nt(const SArgs& a, int grid, int smem, bool cooperative
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeCooperative;
     attr[0].val.cooperative = 1;
+    if (!cooperative) attr[0] = pdl_attribute();
     cfg.attrs = attr;
-    cfg.numAttrs = cooperative ? 1 : 0;
+    cfg.numAttrs = 1;
     const cudaError_t e = a.fold_any ? cudaLaunchKernelEx(&cfg, stream_kernel<NT, true>, a) : cudaLaunchKernelEx(&cfg, stream_kernel<NT, false>, a);
     if (e != cudaSuccess) { cudaGetLastError(); return SD2_ERR_CUDA; }
     if (cudaGetLastError() != cudaSuccess) return SD2_ERR_CUDA;
@@ -636,8 +659,9 @@ sd2_status launch_cells(const CArgs<MAXS>& a, int grid, int smem, cudaStream_t s
     attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeCooperative;
     attr[1].val.cooperative = 1;
+    if (a.n_stages == 1) attr[1] = pdl_attribute();
     cfg.attrs = attr;
-    cfg.numAttrs = a.n_stages > 1 ? 2 : 1;
+    cfg.numAttrs = 2;
     const cudaError_t e = a.fold_any ? cudaLaunchKernelEx(&cfg, cell_kernel<MAXS, NR, true>, a) : cudaLaunchKernelEx(&cfg, cell_kernel<MAXS, NR, false>, a);
     if (e != cudaSuccess) { cudaGetLastError(); return SD2_ERR_CUDA; }
     return SD2_OK;
@@ -749,7 +773,7 @@ sd2_status launch_lm_head(const uint16_t* x, const uint16_t* w, float* logits, i
     per_sm = per_sm < 1 ? 1 : per_sm > head_ctas(NT) ? head_ctas(NT) : per_sm;
     int64_t grid = ((int64_t)V + kGlueThreads / 32 - 1) / (kGlueThreads / 32);
     if (grid > (int64_t)sms * per_sm) grid = (int64_t)sms * per_sm;
-    lm_head_kernel<NT><<<(unsigned)grid, kGlueThreads, smem, s>>>(x, w, logits, n, V, H);
+    launch_pdl(lm_head_kernel<NT>, (unsigned)grid, kGlueThreads, smem, s, x, w, logits, n, V, H);
     return cudaGetLastError() == cudaSuccess ? SD2_OK : SD2_ERR_CUDA;
 }
 
@@ -873,7 +897,7 @@ sd2_status run_mma(sd2_handle h, const uint16_t* x, void* Y, int64_t N, bool y_f
         a.slot_bytes = batch * rec_bytes;
         a.n_slots = slots;
         const int smem = fixed + slots * a.slot_bytes;
-        mma_kernel<<<grid, kMmaThreads, smem, s>>>(a, xmap);
+        launch_pdl(mma_kernel, grid, kMmaThreads, smem, s, a, xmap);
         if (cudaGetLastError() != cudaSuccess) return SD2_ERR_CUDA;
     }
     return SD2_OK;
@@ -1315,7 +1339,7 @@ sd2_status sd2_rmsnorm(const void* x, const void* w, void* y, int64_t N, int64_t
     if (N < 0 || H < 1 || N > 0x7FFFFFFF || H > 0x7FFFFFFF) return SD2_ERR_SHAPE;
     if (N == 0) return SD2_OK;
     const int vec = ((H & 7) == 0 && ((((uintptr_t)x) | ((uintptr_t)w) | ((uintptr_t)y)) & 15) == 0) ? 1 : 0;
-    rmsnorm_kernel<<<(unsigned)N, kGlueThreads, 0, (cudaStream_t)cuda_stream>>>((const uint16_t*)x, (const uint16_t*)w, (uint16_t*)y, (int)H, eps, vec);
+    launch_pdl(rmsnorm_kernel, (unsigned)N, kGlueThreads, 0, (cudaStream_t)cuda_stream, (const uint16_t*)x, (const uint16_t*)w, (uint16_t*)y, (int)H, eps, vec);
     return cudaGetLastError() == cudaSuccess ? SD2_OK : SD2_ERR_CUDA;
 }
 
@@ -1340,7 +1364,7 @@ sd2_status sd2_add_rmsnorm(const void* a, const void* b, void* sum, const void* 
     if (!a || !b || !sum || !w || !y) return SD2_ERR_INVALID_ARG;
     if (N < 0 || H < 1 || N > 0x7FFFFFFF || H > 0x7FFFFFFF) return SD2_ERR_SHAPE;
     if (N == 0) return SD2_OK;
-    add_rmsnorm_kernel<<<(unsigned)N, kGlueThreads, 0, (cudaStream_t)cuda_stream>>>((const uint16_t*)a, (const uint16_t*)b, (uint16_t*)sum,
+    launch_pdl(add_rmsnorm_kernel, (unsigned)N, kGlueThreads, 0, (cudaStream_t)cuda_stream, (const uint16_t*)a, (const uint16_t*)b, (uint16_t*)sum,
                                                                                      (const uint16_t*)w, (uint16_t*)y, (int)H, eps);
     return cudaGetLastError() == cudaSuccess ? SD2_OK : SD2_ERR_CUDA;
 }
@@ -1354,7 +1378,7 @@ sd2_status sd2_rope_cache(void* q, const void* k, const void* v, void* k_cache, 
         return SD2_ERR_SHAPE;
     if (N == 0) return SD2_OK;
     if (head_dim > 2 * kRopeMaxHalf) return SD2_ERR_UNSUPPORTED;
-    rope_cache_kernel<<<(unsigned)N, kGlueThreads, 0, (cudaStream_t)cuda_stream>>>((uint16_t*)q, (const uint16_t*)k, (const uint16_t*)v,
+    launch_pdl(rope_cache_kernel, (unsigned)N, kGlueThreads, 0, (cudaStream_t)cuda_stream, (uint16_t*)q, (const uint16_t*)k, (const uint16_t*)v,
                                                                                     (uint16_t*)k_cache, (uint16_t*)v_cache, (int)heads_q,
                                                                                     (int)heads_kv, (int)head_dim, (int)pos, (int)T_max,
                                                                                     rope_table(head_dim, pos, theta));
@@ -1373,7 +1397,7 @@ sd2_status sd2_attention_decode(const void* q, const void* k_cache, const void* 
     if (N == 0) return SD2_OK;
     const bool pow2 = (head_dim & (head_dim - 1)) == 0;
     const int vec = (pow2 && head_dim >= 8 && ((((uintptr_t)k_cache) | ((uintptr_t)v_cache)) & 15) == 0) ? 1 : 0;
-    attention_decode_kernel<<<(unsigned)(N * heads_q), kAttnThreads, (size_t)T * 4, (cudaStream_t)cuda_stream>>>(
+    launch_pdl(attention_decode_kernel, (unsigned)(N * heads_q), kAttnThreads, (size_t)T * 4, (cudaStream_t)cuda_stream, 
         (const uint16_t*)q, (const uint16_t*)k_cache, (const uint16_t*)v_cache, (uint16_t*)out, (int)heads_q, (int)heads_kv, (int)head_dim,
         (int)T, (int)T_max, vec);
     return cudaGetLastError() == cudaSuccess ? SD2_OK : SD2_ERR_CUDA;
@@ -1392,7 +1416,7 @@ sd2_status sd2_rope_attention(void* q, const void* k, const void* v, void* k_cac
     if (N == 0) return SD2_OK;
     const bool pow2 = (head_dim & (head_dim - 1)) == 0;
     const int vec = (pow2 && head_dim >= 8 && ((((uintptr_t)k_cache) | ((uintptr_t)v_cache)) & 15) == 0) ? 1 : 0;
-    rope_attention_kernel<<<(unsigned)(N * heads_q), kAttnThreads, (size_t)(pos + 1) * 4, (cudaStream_t)cuda_stream>>>(
+    launch_pdl(rope_attention_kernel, (unsigned)(N * heads_q), kAttnThreads, (size_t)(pos + 1) * 4, (cudaStream_t)cuda_stream, 
         (uint16_t*)q, (const uint16_t*)k, (const uint16_t*)v, (uint16_t*)k_cache, (uint16_t*)v_cache, (uint16_t*)out, (int)heads_q,
         (int)heads_kv, (int)head_dim, (int)pos, (int)T_max, rope_table(head_dim, pos, theta), vec);
     return cudaGetLastError() == cudaSuccess ? SD2_OK : SD2_ERR_CUDA;
@@ -1405,7 +1429,7 @@ sd2_status sd2_add(const void* a, const void* b, void* y, int64_t count, void* c
     if (count == 0) return SD2_OK;
     int64_t grid = (count + kGlueThreads - 1) / kGlueThreads;
     if (grid > 148 * 8) grid = 148 * 8;
-    add_kernel<<<(unsigned)grid, kGlueThreads, 0, (cudaStream_t)cuda_stream>>>((const uint16_t*)a, (const uint16_t*)b, (uint16_t*)y, (long long)count);
+    launch_pdl(add_kernel, (unsigned)grid, kGlueThreads, 0, (cudaStream_t)cuda_stream, (const uint16_t*)a, (const uint16_t*)b, (uint16_t*)y, (long long)count);
     return cudaGetLastError() == cudaSuccess ? SD2_OK : SD2_ERR_CUDA;
 }
 
@@ -1414,7 +1438,7 @@ sd2_status sd2_embedding(const int32_t* tokens, const void* table, void* x, int6
     if (!tokens || !table || !x) return SD2_ERR_INVALID_ARG;
     if (N < 0 || V < 1 || H < 1 || N > 0x7FFFFFFF || V > 0x7FFFFFFF || H > 0x7FFFFFFF) return SD2_ERR_SHAPE;
     if (N == 0) return SD2_OK;
-    embedding_kernel<<<(unsigned)N, kGlueThreads, 0, (cudaStream_t)cuda_stream>>>(tokens, (const uint16_t*)table, (uint16_t*)x, (int)H, (int)V);
+    launch_pdl(embedding_kernel, (unsigned)N, kGlueThreads, 0, (cudaStream_t)cuda_stream, tokens, (const uint16_t*)table, (uint16_t*)x, (int)H, (int)V);
     return cudaGetLastError() == cudaSuccess ? SD2_OK : SD2_ERR_CUDA;
 }
 
@@ -1442,7 +1466,7 @@ sd2_status sd2_lm_head(const void* x, const void* w_out, float* logits, int32_t*
     }
     if (tokens && N > 0) {
         const int vec = ((V & 3) == 0 && (((uintptr_t)logits) & 15) == 0) ? 1 : 0;
-        argmax_kernel<<<(unsigned)(N * kArgmaxCtas), 512, 0, s>>>(logits, tokens, (int)V, vec);
+        launch_pdl(argmax_kernel, (unsigned)(N * kArgmaxCtas), 512, 0, s, logits, tokens, (int)V, vec);
         if (cudaGetLastError() != cudaSuccess) return SD2_ERR_CUDA;
     }
     return SD2_OK;

@@ -517,6 +517,7 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
     const int N = a.N;
     const uint32_t NS = (uint32_t)a.n_slots;
 
+    pdl_let_next_start();
     if (tid < kCellGroups * kGroupSlots) {
         mbar_init(smem_u32(&sh->full[0][0]) + 8 * tid, 1);
         mbar_init(smem_u32(&sh->empty[0][0]) + 8 * tid, kChunkCells);
@@ -578,6 +579,7 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         __syncwarp();
         return true;
     };
+    if (warp != kProducerWarp) pdl_wait();       // (the producer streams weights already)
     if (warp == kProducerWarp) {
         // ---------------------------------------------------------------------- producer
         // Directory entries come in batches of up to 32 chunks of a stage, a chunk to a lane.  (Like the finishers this warp

@@ -58,6 +58,8 @@ __device__ __forceinline__ float block_max(float v, float* red)
 // 16-byte aligned, so a thread moves eight values per load (the second pass finds the row in L1)
 __global__ void __launch_bounds__(kGlueThreads) rmsnorm_kernel(const uint16_t* x, const uint16_t* w, uint16_t* y, int H, float eps, int vec)
 {
+    pdl_let_next_start();
+    pdl_wait();
     __shared__ float red[32];
     const uint16_t* xr = x + (size_t)blockIdx.x * H;
     uint16_t* yr = y + (size_t)blockIdx.x * H;
@@ -99,6 +101,8 @@ __global__ void __launch_bounds__(kGlueThreads) rmsnorm_kernel(const uint16_t* x
 __global__ void __launch_bounds__(kGlueThreads) add_rmsnorm_kernel(const uint16_t* a, const uint16_t* b, uint16_t* sum, const uint16_t* w,
                                                                   uint16_t* y, int H, float eps)
 {
+    pdl_let_next_start();
+    pdl_wait();
     __shared__ float red[32];
     const size_t r0 = (size_t)blockIdx.x * H;
     float ss = 0.f;
@@ -118,6 +122,8 @@ __global__ void __launch_bounds__(kGlueThreads) rope_cache_kernel(uint16_t* q, c
                                                                  uint16_t* vc, int Hq, int Hkv, int d, int pos, int T_max,
                                                                  const RopeTable tab)
 {
+    pdl_let_next_start();
+    pdl_wait();
     const int n = blockIdx.x, half = d / 2;
     uint16_t* qr = q + (size_t)n * Hq * d;
     const uint16_t* kr = k + (size_t)n * Hkv * d;
@@ -146,6 +152,8 @@ __global__ void __launch_bounds__(kGlueThreads) rope_cache_kernel(uint16_t* q, c
 __global__ void __launch_bounds__(kAttnThreads) attention_decode_kernel(const uint16_t* q, const uint16_t* kc, const uint16_t* vc,
                                                                        uint16_t* out, int Hq, int Hkv, int d, int T, int T_max, int vec)
 {
+    pdl_let_next_start();
+    pdl_wait();
     extern __shared__ float sc[];            // T scores, then the weights
     __shared__ float red[32];
     __shared__ float qs[128];
@@ -253,6 +261,8 @@ __global__ void __launch_bounds__(kAttnThreads) rope_attention_kernel(uint16_t* 
                                                                      uint16_t* vc, uint16_t* out, int Hq, int Hkv, int d, int pos,
                                                                      int T_max, const RopeTable tab, int vec)
 {
+    pdl_let_next_start();
+    pdl_wait();
     extern __shared__ float sc[];            // pos + 1 scores, then the weights
     __shared__ float red[32];
     __shared__ float qs[128], ks[128];
@@ -384,6 +394,8 @@ __global__ void __launch_bounds__(kAttnThreads) rope_attention_kernel(uint16_t* 
 // y = a + b, element by element
 __global__ void __launch_bounds__(kGlueThreads) add_kernel(const uint16_t* a, const uint16_t* b, uint16_t* y, long long count)
 {
+    pdl_let_next_start();
+    pdl_wait();
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += (long long)gridDim.x * blockDim.x)
         y[i] = f32_to_bf16_rne(bf16_to_f32(a[i]) + bf16_to_f32(b[i]));
 }
@@ -391,6 +403,8 @@ __global__ void __launch_bounds__(kGlueThreads) add_kernel(const uint16_t* a, co
 // x[n, :] = table[token[n], :]
 __global__ void __launch_bounds__(kGlueThreads) embedding_kernel(const int32_t* tokens, const uint16_t* table, uint16_t* x, int H, int V)
 {
+    pdl_let_next_start();
+    pdl_wait();
     const int tok = tokens[blockIdx.x];
     for (int i = threadIdx.x; i < H; i += blockDim.x)
         x[(size_t)blockIdx.x * H + i] = (tok >= 0 && tok < V) ? table[(size_t)tok * H + i] : (uint16_t)0;
@@ -407,6 +421,8 @@ constexpr int head_ctas(int NT) { return NT <= 1 ? 5 : NT <= 2 ? 3 : 2; }
 template <int NT>
 __global__ void __launch_bounds__(kGlueThreads, head_ctas(NT)) lm_head_kernel(const uint16_t* x, const uint16_t* W, float* logits, int N, int V, int H)
 {
+    pdl_let_next_start();
+    pdl_wait();
     extern __shared__ uint4 head_x[];        // [NT][H / 8]: zero beyond row N
     const int groups = H / 8;
     for (int i = threadIdx.x; i < NT * H; i += blockDim.x) ((uint16_t*)head_x)[i] = i < N * H ? x[i] : (uint16_t)0;
@@ -465,6 +481,8 @@ __device__ __forceinline__ void argmax_warp(float& best, int& at)
 }
 __global__ void __cluster_dims__(kArgmaxCtas, 1, 1) __launch_bounds__(512) argmax_kernel(const float* logits, int32_t* token, int V, int vec)
 {
+    pdl_let_next_start();
+    pdl_wait();
     __shared__ float bv[32];
     __shared__ int bi[32];
     __shared__ uint2 found[kArgmaxCtas];     // of rank 0: every CTA's best, as bits, and its index

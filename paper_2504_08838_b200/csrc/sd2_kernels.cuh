@@ -178,6 +178,14 @@ struct SArgs {
     int fold_any;                   // host side: launch the FOLD instance
 };
 
+// Launches without a grid barrier are programmatic dependents (launch_pdl): a CTA may start when every CTA of the kernel
+// before it in the stream has started, and gets its SM as soon as that one's CTA leaves.  pdl_wait holds it until the kernel
+// before is through and its results are visible; what a launch reads before (weights, their directories, its arguments) no
+// kernel writes.  Every CTA waits before it ends, so the launches of a stream still finish in order.  Without this the
+// boundary between two launches cost 2 us and more: it is most of a small call.
+__device__ __forceinline__ void pdl_let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
@@ -727,6 +735,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const __grid_
     const uint32_t empty0 = smem_u32(&sh->empty[0]);
     const uint32_t ring0 = smem_u32(ring);
 
+    pdl_let_next_start();
     if (tid == 0) {
         for (int i = 0; i < kSlots; ++i) {
             mbar_init(full0 + 8 * i, 1);
@@ -898,6 +907,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const __grid_
     // the current one is computed; the barrier at the end of the stage makes it visible.
     constexpr int kGroups = 32 / xs_words(NT);
     constexpr int kStageWords = (int)(sizeof(SStage) / 4);
+    pdl_wait();             // (the producer warp streams weights already)
     const int ctid = tid;   // consumer threads are 0 .. kConsumerThreads - 1
     const int N = a.N;
     const int xlin_row = NT <= 2 ? 0 : a.xlin_bytes >> 2;   // elements between the two linear buffers of a pass
@@ -1202,6 +1212,8 @@ __device__ __forceinline__ void store_row(const MatDesc& md, int row, const floa
 template <int NT>
 __global__ void __launch_bounds__(kThreads) bitmask_kernel(const __grid_constant__ LaunchGroup grp)
 {
+    pdl_let_next_start();
+    pdl_wait();
     int mi = 0;
 #pragma unroll
     for (int i = 1; i < kMaxFused; ++i)

@@ -179,6 +179,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) mma_kernel(const MmaArgs a, co
     const int nblk = (int)(b1 - b0);
     const WaitCtx wc = {&sh->abort_flag, a.budget};
 
+    pdl_let_next_start();
     if (tid == 0) {
         for (int i = 0; i < kMmaSlots; ++i) {
             mbar_init(smem_u32(&sh->full[i]), 1);
@@ -211,6 +212,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) mma_kernel(const MmaArgs a, co
     tc_fence_after();
     const uint32_t tmem = *(volatile uint32_t*)&sh->tmem_base;
 
+    if (warp != kMmaProducerWarp) pdl_wait();    // (the producer streams block records already)
     if (warp == kMmaProducerWarp) {
         // ---------------------------------------------------------------- producer: block records, a batch per copy
         int issued = 0;                                      // batches
