@@ -124,15 +124,28 @@ def _ptr(t):
     if t is None:
         return None
     if isinstance(t, np.ndarray):
-        return t.ctypes.data_as(ctypes.c_void_p)
-    return ctypes.c_void_p(t.data_ptr())
+        return t.ctypes.data
+    return t.data_ptr()
+
+
+_raw_stream = None
 
 
 def _stream(stream):
-    if stream is None:
+    """``stream``, or torch's current one: by its raw handle, since a Stream object costs half of a small call."""
+    if stream is not None:
+        return int(stream)
+    global _raw_stream
+    if _raw_stream is None:
         import torch
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
-    return ctypes.c_void_p(int(stream))
+        by_device = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        device = getattr(torch._C, "_cuda_getDevice", None)
+        torch.cuda.init()
+        if by_device and device:
+            _raw_stream = lambda: by_device(device())
+        else:
+            _raw_stream = lambda: torch.cuda.current_stream().cuda_stream
+    return _raw_stream()
 
 
 # ---- host format builder ---------------------------------------------------------------

@@ -167,12 +167,12 @@ sd2_status from_pack(int s)
 
 constexpr int kFoldStaticBytes = 256;   // static shared memory of the kernel instances that fold a norm into staging
 
-template <int NT>
+template <int MAXS, int NT>
 cudaError_t set_smem_attr()
 {
-    cudaError_t e = cudaFuncSetAttribute(stream_kernel<NT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+    cudaError_t e = cudaFuncSetAttribute(stream_kernel<MAXS, NT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(stream_kernel<NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - kFoldStaticBytes);
+    return cudaFuncSetAttribute(stream_kernel<MAXS, NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - kFoldStaticBytes);
 }
 
 template <int MAXS, int NR>
@@ -195,9 +195,11 @@ sd2_status ensure_device(int* dev_out)
         int sms = 0, khz = 0;
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
             cudaDeviceGetAttribute(&khz, cudaDevAttrClockRate, dev) != cudaSuccess) { cudaGetLastError(); return SD2_ERR_CUDA; }
-        if (set_smem_attr<1>() != cudaSuccess || set_smem_attr<2>() != cudaSuccess || set_smem_attr<4>() != cudaSuccess ||
+        constexpr int kMany = kMaxStagesInline;
+        if (set_smem_attr<1, 1>() != cudaSuccess || set_smem_attr<1, 2>() != cudaSuccess || set_smem_attr<1, 4>() != cudaSuccess ||
+            set_smem_attr<kMany, 1>() != cudaSuccess || set_smem_attr<kMany, 2>() != cudaSuccess || set_smem_attr<kMany, 4>() != cudaSuccess ||
             set_cell_attr<1, 8>() != cudaSuccess || set_cell_attr<1, 16>() != cudaSuccess ||
-            set_cell_attr<kMaxStagesInline, 8>() != cudaSuccess || set_cell_attr<kMaxStagesInline, 16>() != cudaSuccess ||
+            set_cell_attr<kMany, 8>() != cudaSuccess || set_cell_attr<kMany, 16>() != cudaSuccess ||
             cudaFuncSetAttribute(mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
             cudaFuncSetAttribute(lm_head_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
             cudaFuncSetAttribute(lm_head_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
@@ -451,8 +453,8 @@ bool plan_smem(int nt, int xs_max, int K_max, int max_tile, SmemPlan* p)
     return true;
 }
 
-template <int NT>
-sd2_status launch_stream_nt(const SArgs& a, int grid, int smem, bool cooperative, cudaStream_t s)
+template <int MAXS, int NT>
+sd2_status launch_stream_nt(const SArgsT<MAXS>& a, int grid, int smem, bool cooperative, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
@@ -465,20 +467,20 @@ sd2_status launch_stream_nt(const SArgs& a, int grid, int smem, bool cooperative
     if (!cooperative) attr[0] = pdl_attribute();
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = a.fold_any ? cudaLaunchKernelEx(&cfg, stream_kernel<NT, true>, a) : cudaLaunchKernelEx(&cfg, stream_kernel<NT, false>, a);
+    const cudaError_t e = a.fold_any ? cudaLaunchKernelEx(&cfg, stream_kernel<MAXS, NT, true>, a) : cudaLaunchKernelEx(&cfg, stream_kernel<MAXS, NT, false>, a);
     if (e != cudaSuccess) { cudaGetLastError(); return SD2_ERR_CUDA; }
     if (cudaGetLastError() != cudaSuccess) return SD2_ERR_CUDA;
     return SD2_OK;
 }
 
-sd2_status launch_stream(int nt, SArgs& a, int grid, bool cooperative, cudaStream_t s)
+template <int MAXS>
+sd2_status launch_stream(int nt, const SArgsT<MAXS>& a, int grid, bool cooperative, cudaStream_t s)
 {
-    if (a.fold_any) a.ring_bytes -= kFoldStaticBytes;   // those instances keep a little static shared memory (the ring still holds two tiles)
     const int smem = a.xs_bytes + a.xlin_bytes + (int)((sizeof(StreamShared) + 127) & ~127) + a.ring_bytes;
     switch (nt) {
-        case 1: return launch_stream_nt<1>(a, grid, smem, cooperative, s);
-        case 2: return launch_stream_nt<2>(a, grid, smem, cooperative, s);
-        default: return launch_stream_nt<4>(a, grid, smem, cooperative, s);
+        case 1: return launch_stream_nt<MAXS, 1>(a, grid, smem, cooperative, s);
+        case 2: return launch_stream_nt<MAXS, 2>(a, grid, smem, cooperative, s);
+        default: return launch_stream_nt<MAXS, 4>(a, grid, smem, cooperative, s);
     }
 }
 
@@ -578,6 +580,12 @@ sd2_status run_panels(SArgs& a, int64_t N, const int xs_need[3], int K_max, int 
 {
     const int nt_cap = widest_panel(xs_need, K_max, max_tile);
     if (nt_cap == 0) return SD2_ERR_UNSUPPORTED;
+    const bool small = a.n_stages == 1 || a.ext;             // one inline stage at most is all that the launch reads
+    SArgsT<1> one;
+    if (small) {
+        one.inl[0] = a.inl[0];
+        one.fold[0] = a.fold[0];
+    }
     for (int64_t n0 = 0; n0 < N; n0 += nt_cap) {
         const int n = (int)((N - n0) < nt_cap ? (N - n0) : nt_cap);
         const int nt = round_nt(n, nt_cap);
@@ -588,7 +596,14 @@ sd2_status run_panels(SArgs& a, int64_t N, const int xs_need[3], int K_max, int 
         a.xs_bytes = p.xs_bytes;
         a.xlin_bytes = p.xlin_bytes;
         a.ring_bytes = p.ring_bytes;
-        sd2_status st = launch_stream(nt, a, grid, a.n_stages > 1, s);
+        if (a.fold_any) a.ring_bytes -= kFoldStaticBytes;   // those instances keep a little static shared memory (the ring still holds two tiles)
+        sd2_status st;
+        if (small) {
+            static_cast<SArgsBase&>(one) = a;
+            st = launch_stream(nt, one, grid, a.n_stages > 1, s);
+        } else {
+            st = launch_stream(nt, a, grid, a.n_stages > 1, s);
+        }
         if (st != SD2_OK) return st;
     }
     return SD2_OK;

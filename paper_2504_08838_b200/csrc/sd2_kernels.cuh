@@ -154,8 +154,7 @@ struct SFold {
     int reserved;
 };
 
-struct SArgs {
-    SStage inl[kMaxStagesInline];   // used when ext == NULL
+struct SArgsBase {
     const SStage* ext;              // device array of stages (programs longer than four stages)
     const uint16_t* x_in;           // replaces stage 0's x when not NULL
     void* y_out;                    // replaces the last stage's mat[0].y when not NULL
@@ -174,9 +173,17 @@ struct SArgs {
     int free_tiles;                 // 1: a consumer warp that is done draws the next tile from a shared counter;
                                     // 0: tile k of a stage goes to warp k % 16 (see the consumer loop)
     long long* reserved_ptr;
-    SFold fold[kMaxStagesInline];   // per inline stage; read by FOLD instances only
     int fold_any;                   // host side: launch the FOLD instance
 };
+
+// MAXS: inline stages the argument block has room for.  A launch of one stage, or of stages in device memory, passes 0.5 KB
+// of arguments, not 3.5 KB.
+template <int MAXS>
+struct SArgsT : SArgsBase {
+    SStage inl[MAXS];               // used when ext == NULL
+    SFold fold[MAXS];               // per inline stage; read by FOLD instances only
+};
+using SArgs = SArgsT<kMaxStagesInline>;
 
 // Launches without a grid barrier are programmatic dependents (launch_pdl): a CTA may start when every CTA of the kernel
 // before it in the stream has started, and gets its SM as soon as that one's CTA leaves.  pdl_wait holds it until the kernel
@@ -718,8 +725,8 @@ __device__ __forceinline__ void stage_x(const SStage& st, int N, const uint16_t*
     }
 }
 
-template <int NT, bool FOLD = false>
-__global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const __grid_constant__ SArgs a)
+template <int MAXS, int NT, bool FOLD>
+__global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const __grid_constant__ SArgsT<MAXS> a)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     float* xs = (float*)smem;
@@ -775,7 +782,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const __grid_
         };
         auto load_stage = [&](int s) {
             PStage p;
-            const SStage* st = a.ext ? a.ext + s : &a.inl[s];
+            const SStage* st = a.ext ? a.ext + s : &a.inl[MAXS == 1 ? 0 : s];
             p.count = st->count;
             p.n_cta = st->tiles_div + (cta < st->tiles_rem ? 1 : 0);
 #pragma unroll
@@ -968,14 +975,14 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const __grid_
                 __shared__ float fold_red[2][kConsumerWarps];   // per-warp partial sums of squares of the rows being normalised
                 stage_x<NT, true>(st, N, x_src ? x_src + xw : nullptr, st.g ? st.g + xw : nullptr, st.u ? st.u + xw : nullptr,
                                   st.t_out ? st.t_out + xoff : nullptr, xs, xlin, xlin_row, ctid, tag_in, tagb, wc, a.n0, fold_red,
-                                  (!a.ext && s < kMaxStagesInline) ? &a.fold[s] : nullptr);
+                                  (!a.ext && s < MAXS) ? &a.fold[MAXS == 1 ? 0 : s] : nullptr);
             } else {
                 stage_x<NT>(st, N, x_src ? x_src + xw : nullptr, st.g ? st.g + xw : nullptr, st.u ? st.u + xw : nullptr,
                             st.t_out ? st.t_out + xoff : nullptr, xs, xlin, xlin_row, ctid, tag_in, tagb, wc);
             }
         }
         if (warp == 1 && s + 1 < a.n_stages) {
-            const uint32_t* src = (const uint32_t*)(a.ext ? a.ext + (s + 1) : &a.inl[s + 1]);
+            const uint32_t* src = (const uint32_t*)(a.ext ? a.ext + (s + 1) : &a.inl[MAXS == 1 ? 0 : s + 1]);
             for (int i = lane; i < kStageWords; i += 32) ((uint32_t*)&sh->stage[(s + 1) & 1])[i] = src[i];
         }
 
