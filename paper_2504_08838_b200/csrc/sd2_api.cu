@@ -779,6 +779,31 @@ sd2_status run_cell_program(CArgs<kMaxStagesInline>& a, const CellBuilder& b, in
     return run_cell_panels(a, N, b.needs, grid, s);
 }
 
+// Attention by attention_kernel.  A head's positions are split over CTAs while each keeps more than 128 and the SMs are not
+// yet taken twice.
+template <bool ROPE>
+sd2_status launch_attention(uint16_t* q, const uint16_t* k, const uint16_t* v, uint16_t* kc, uint16_t* vc, uint16_t* out, int64_t N,
+                            int64_t Hq, int64_t Hkv, int64_t d, int64_t T, int64_t T_max, const RopeTable& tab, int sms, cudaStream_t s)
+{
+    int64_t S = 1;
+    while (S < kAttnMaxCluster && T > 128 * S && N * Hq * 2 * S <= 2 * sms) S *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(N * Hq * S));
+    cfg.blockDim = dim3(kAttnThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0] = pdl_attribute();
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = (unsigned)S;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, attention_kernel<ROPE>, q, k, v, kc, vc, out, (int)Hq, (int)Hkv, (int)d, (int)T, (int)T_max,
+                                             (int)S, tab);
+    if (e != cudaSuccess) { cudaGetLastError(); return SD2_ERR_CUDA; }
+    return SD2_OK;
+}
+
 // An LM head of NT activation rows at most.
 template <int NT>
 sd2_status launch_lm_head(const uint16_t* x, const uint16_t* w, float* logits, int n, int V, int H, int sms, cudaStream_t s)
@@ -1410,11 +1435,17 @@ sd2_status sd2_attention_decode(const void* q, const void* k_cache, const void* 
         return SD2_ERR_SHAPE;
     if (head_dim > 128 || T > kAttnMaxT) return SD2_ERR_UNSUPPORTED;
     if (N == 0) return SD2_OK;
+    int dev = 0;
+    const sd2_status st = ensure_device(&dev);
+    if (st != SD2_OK) return st;
     const bool pow2 = (head_dim & (head_dim - 1)) == 0;
     const int vec = (pow2 && head_dim >= 8 && ((((uintptr_t)k_cache) | ((uintptr_t)v_cache)) & 15) == 0) ? 1 : 0;
-    launch_pdl(attention_decode_kernel, (unsigned)(N * heads_q), kAttnThreads, (size_t)T * 4, (cudaStream_t)cuda_stream, 
-        (const uint16_t*)q, (const uint16_t*)k_cache, (const uint16_t*)v_cache, (uint16_t*)out, (int)heads_q, (int)heads_kv, (int)head_dim,
-        (int)T, (int)T_max, vec);
+    if (vec)
+        return launch_attention<false>((uint16_t*)q, nullptr, nullptr, (uint16_t*)k_cache, (uint16_t*)v_cache, (uint16_t*)out, N, heads_q,
+                                       heads_kv, head_dim, T, T_max, RopeTable{}, g_dev[dev].sms, (cudaStream_t)cuda_stream);
+    launch_pdl(attention_any_kernel, (unsigned)(N * heads_q), kAttnThreads, (size_t)T * 4, (cudaStream_t)cuda_stream,
+               (const uint16_t*)q, (const uint16_t*)k_cache, (const uint16_t*)v_cache, (uint16_t*)out, (int)heads_q, (int)heads_kv,
+               (int)head_dim, (int)T, (int)T_max);
     return cudaGetLastError() == cudaSuccess ? SD2_OK : SD2_ERR_CUDA;
 }
 
@@ -1429,11 +1460,18 @@ sd2_status sd2_rope_attention(void* q, const void* k, const void* v, void* k_cac
         return SD2_ERR_SHAPE;
     if (head_dim > 128 || pos + 1 > kAttnMaxT) return SD2_ERR_UNSUPPORTED;
     if (N == 0) return SD2_OK;
+    int dev = 0;
+    const sd2_status st = ensure_device(&dev);
+    if (st != SD2_OK) return st;
     const bool pow2 = (head_dim & (head_dim - 1)) == 0;
     const int vec = (pow2 && head_dim >= 8 && ((((uintptr_t)k_cache) | ((uintptr_t)v_cache)) & 15) == 0) ? 1 : 0;
-    launch_pdl(rope_attention_kernel, (unsigned)(N * heads_q), kAttnThreads, (size_t)(pos + 1) * 4, (cudaStream_t)cuda_stream, 
-        (uint16_t*)q, (const uint16_t*)k, (const uint16_t*)v, (uint16_t*)k_cache, (uint16_t*)v_cache, (uint16_t*)out, (int)heads_q,
-        (int)heads_kv, (int)head_dim, (int)pos, (int)T_max, rope_table(head_dim, pos, theta), vec);
+    if (vec)
+        return launch_attention<true>((uint16_t*)q, (const uint16_t*)k, (const uint16_t*)v, (uint16_t*)k_cache, (uint16_t*)v_cache,
+                                      (uint16_t*)out, N, heads_q, heads_kv, head_dim, pos, T_max, rope_table(head_dim, pos, theta),
+                                      g_dev[dev].sms, (cudaStream_t)cuda_stream);
+    launch_pdl(rope_attention_any_kernel, (unsigned)(N * heads_q), kAttnThreads, (size_t)(pos + 1) * 4, (cudaStream_t)cuda_stream,
+               (uint16_t*)q, (const uint16_t*)k, (const uint16_t*)v, (uint16_t*)k_cache, (uint16_t*)v_cache, (uint16_t*)out, (int)heads_q,
+               (int)heads_kv, (int)head_dim, (int)pos, (int)T_max, rope_table(head_dim, pos, theta));
     return cudaGetLastError() == cudaSuccess ? SD2_OK : SD2_ERR_CUDA;
 }
 

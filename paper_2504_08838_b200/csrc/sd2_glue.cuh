@@ -146,11 +146,184 @@ __global__ void __launch_bounds__(kGlueThreads) rope_cache_kernel(uint16_t* q, c
     for (int i = threadIdx.x; i < Hkv * d; i += blockDim.x) vdst[i] = v[(size_t)n * Hkv * d + i];
 }
 
+// Attention of one new token per row over T cached positions, by clusters of one to eight CTAs per (row, query head), each
+// with its share of the positions.  d is 8, 16, 32, 64 or 128 and the caches are 16-byte aligned: d / 8 lanes share a position,
+// a lane holds eight dimensions (one 128-bit load), a warp takes 256 / d positions per step and four steps at a time.
+// Latency bounds it (300 positions of 64 dimensions are 38 KB a head), so keys and values are asked for together, and before
+// the query is there, and a running maximum takes the place of a pass over the scores with its barriers: with three passes
+// (scores, weights, values) by one CTA per head such a step took 19.5 us.
+// ROPE: also rotates the query (and writes it back) and the new key, attends over the new token from registers and shared
+// memory, and appends it to the caches (the first query head of every group does).
+constexpr int kAttnSteps = 4;
+constexpr int kAttnMaxCluster = 8;
+template <bool ROPE>
+__global__ void __launch_bounds__(kAttnThreads) attention_kernel(uint16_t* q, const uint16_t* k, const uint16_t* v, uint16_t* kc, uint16_t* vc,
+                                                                 uint16_t* out, int Hq, int Hkv, int d, int T, int T_max, int S,
+                                                                 const __grid_constant__ RopeTable tab)
+{
+    constexpr int kWarps = kAttnThreads / 32;
+    __shared__ float qs[128], ks[128];
+    __shared__ float part[kWarps + 1][128], pm[kWarps + 1], pl[kWarps + 1];
+    __shared__ float cacc[kAttnMaxCluster][128], cm[kAttnMaxCluster], cl[kAttnMaxCluster];   // of rank 0: every CTA's share
+    pdl_let_next_start();
+    pdl_wait();
+    const int rank = blockIdx.x % S, row = blockIdx.x / S;
+    const int n = row / Hq, h = row - n * Hq, group = Hq / Hkv, g = h / group;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const size_t pitch = (size_t)Hkv * d, first = (size_t)n * T_max * pitch + (size_t)g * d;
+    const int lpp = d >> 3, ppw = 32 / lpp, dl = (lane % lpp) * 8;
+    const int begin = (int)((long long)T * rank / S), end = (int)((long long)T * (rank + 1) / S);
+    const int w0 = begin + warp * ppw, t0 = w0 + lane / lpp, step = kWarps * ppw;
+    const uint16_t* kb = kc + first + (size_t)t0 * pitch + dl;
+    const uint16_t* vb = vc + first + (size_t)t0 * pitch + dl;
+    uint4 kv[kAttnSteps], vv[kAttnSteps];
+    auto load = [&](int at) {                // the four steps from position t0 + at on
+#pragma unroll
+        for (int i = 0; i < kAttnSteps; ++i) {
+            const bool there = t0 + at + i * step < end;
+            kv[i] = there ? *(const uint4*)(kb + (size_t)(at + i * step) * pitch) : make_uint4(0u, 0u, 0u, 0u);
+            vv[i] = there ? *(const uint4*)(vb + (size_t)(at + i * step) * pitch) : make_uint4(0u, 0u, 0u, 0u);
+        }
+    };
+    load(0);
+    uint16_t* qr = q + (size_t)row * d;
+    const int half = d / 2;
+    uint16_t q0 = 0, q1 = 0, k0 = 0, k1 = 0;
+    if (ROPE) {
+        if (tid < half) {
+            const float c = tab.c[tid], sn = tab.s[tid];
+            const uint16_t* kr = k + ((size_t)n * Hkv + g) * d;
+            const float a = bf16_to_f32(qr[tid]), b = bf16_to_f32(qr[tid + half]);
+            q0 = f32_to_bf16_rne(a * c - b * sn);
+            q1 = f32_to_bf16_rne(b * c + a * sn);
+            const float ka = bf16_to_f32(kr[tid]), kb2 = bf16_to_f32(kr[tid + half]);
+            k0 = f32_to_bf16_rne(ka * c - kb2 * sn);
+            k1 = f32_to_bf16_rne(kb2 * c + ka * sn);
+            qs[tid] = bf16_to_f32(q0);
+            qs[tid + half] = bf16_to_f32(q1);
+            ks[tid] = bf16_to_f32(k0);
+            ks[tid + half] = bf16_to_f32(k1);
+        }
+    } else if (tid < d) {
+        qs[tid] = bf16_to_f32(qr[tid]);
+    }
+    __syncthreads();
+    if (S > 1) asm volatile("barrier.cluster.arrive.release;" ::: "memory");     // this CTA runs, and has read q
+    float qv[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) qv[j] = qs[dl + j];
+    const float scale = rsqrtf((float)d);
+    float m = -INFINITY, l = 0.f, acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (int at = 0; w0 + at < end; at += kAttnSteps * step) {                   // (the same for the whole warp)
+        if (at > 0) load(at);
+        float s[kAttnSteps], top = m;
+#pragma unroll
+        for (int i = 0; i < kAttnSteps; ++i) {
+            const uint32_t u[4] = {kv[i].x, kv[i].y, kv[i].z, kv[i].w};
+            s[i] = 0.f;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) s[i] += qv[2 * j] * bf16_lo(u[j]) + qv[2 * j + 1] * bf16_hi(u[j]);
+            for (int dd = 1; dd < lpp; dd <<= 1) s[i] += __shfl_xor_sync(0xFFFFFFFFu, s[i], dd);
+            s[i] = t0 + at + i * step < end ? s[i] * scale : -INFINITY;
+            top = fmaxf(top, s[i]);
+        }
+        const float base = top == -INFINITY ? 0.f : top;                         // (a lane may have no position yet)
+        const float keep = expf(m - base);
+        m = top;
+        l *= keep;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[j] *= keep;
+#pragma unroll
+        for (int i = 0; i < kAttnSteps; ++i) {
+            const float p = expf(s[i] - base);
+            const uint32_t u[4] = {vv[i].x, vv[i].y, vv[i].z, vv[i].w};
+            l += p;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                acc[2 * j] += p * bf16_lo(u[j]);
+                acc[2 * j + 1] += p * bf16_hi(u[j]);
+            }
+        }
+    }
+    // the warp's lanes, the CTA's warps, the cluster's CTAs
+    float top = m;
+    for (int dd = lpp; dd < 32; dd <<= 1) top = fmaxf(top, __shfl_xor_sync(0xFFFFFFFFu, top, dd));
+    const float f = m == -INFINITY ? 0.f : expf(m - top);
+    l *= f;
+    for (int dd = lpp; dd < 32; dd <<= 1) l += __shfl_xor_sync(0xFFFFFFFFu, l, dd);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        float a = acc[j] * f;
+        for (int dd = lpp; dd < 32; dd <<= 1) a += __shfl_xor_sync(0xFFFFFFFFu, a, dd);
+        if (lane < lpp) part[warp][dl + j] = a;
+    }
+    if (lane == 0) { pm[warp] = top; pl[warp] = l; }
+    const uint16_t* vnew = ROPE ? v + ((size_t)n * Hkv + g) * d : nullptr;
+    const int parts = kWarps + (ROPE && rank == 0 ? 1 : 0);                      // rank 0 has the new token
+    if (ROPE && rank == 0 && warp == kWarps - 1) {
+        float s = 0.f;
+        for (int i = lane; i < d; i += 32) {
+            s += qs[i] * ks[i];
+            part[kWarps][i] = bf16_to_f32(vnew[i]);
+        }
+        s = warp_sum(s);
+        if (lane == 0) { pm[kWarps] = s * scale; pl[kWarps] = 1.f; }
+    }
+    __syncthreads();
+    if (S > 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");       // the others run; all have read q
+    float A = 0.f, L = 0.f, M = -INFINITY;
+    if (tid < d) {
+        for (int w = 0; w < parts; ++w) M = fmaxf(M, pm[w]);
+        for (int w = 0; w < parts; ++w) {
+            const float e = pm[w] == -INFINITY ? 0.f : expf(pm[w] - M);
+            L += pl[w] * e;
+            A += part[w][tid] * e;
+        }
+        if (S > 1) {
+            uint32_t to_a, to_m, to_l;
+            asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(to_a) : "r"(smem_u32(&cacc[rank][tid])));
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(to_a), "f"(A) : "memory");
+            if (tid == 0) {
+                asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(to_m) : "r"(smem_u32(&cm[rank])));
+                asm("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(to_l) : "r"(smem_u32(&cl[rank])));
+                asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(to_m), "f"(M) : "memory");
+                asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(to_l), "f"(L) : "memory");
+            }
+        }
+    }
+    if (S > 1) {
+        asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+        if (rank != 0) return;
+        if (tid < d) {
+            M = -INFINITY;
+            for (int c = 0; c < S; ++c) M = fmaxf(M, cm[c]);
+            A = L = 0.f;
+            for (int c = 0; c < S; ++c) {
+                const float e = cm[c] == -INFINITY ? 0.f : expf(cm[c] - M);
+                L += cl[c] * e;
+                A += cacc[c][tid] * e;
+            }
+        }
+    }
+    if (tid < d) out[(size_t)row * d + tid] = f32_to_bf16_rne(A / L);
+    if (ROPE) {
+        uint16_t* kdst = kc + first + (size_t)T * pitch;
+        uint16_t* vdst = vc + first + (size_t)T * pitch;
+        const bool writer = h - g * group == 0;
+        if (tid < half) {
+            qr[tid] = q0;
+            qr[tid + half] = q1;
+            if (writer) { kdst[tid] = k0; kdst[tid + half] = k1; }
+        }
+        if (writer && tid < d) vdst[tid] = vnew[tid];
+    }
+}
+
 // One new token per row over T cached positions; one CTA per (row, query head); d <= 128.
-// vec: d is 8, 16, 32, 64 or 128 and the caches are 16-byte aligned: d / 8 lanes share a position, a lane holds eight
-// dimensions (one 128-bit load), so a warp takes 256 / d positions per step and all its loads are independent.
-__global__ void __launch_bounds__(kAttnThreads) attention_decode_kernel(const uint16_t* q, const uint16_t* kc, const uint16_t* vc,
-                                                                       uint16_t* out, int Hq, int Hkv, int d, int T, int T_max, int vec)
+// For head widths and caches that attention_kernel cannot read in 128-bit words.
+__global__ void __launch_bounds__(kAttnThreads) attention_any_kernel(const uint16_t* q, const uint16_t* kc, const uint16_t* vc,
+                                                                       uint16_t* out, int Hq, int Hkv, int d, int T, int T_max)
 {
     pdl_let_next_start();
     pdl_wait();
@@ -166,34 +339,12 @@ __global__ void __launch_bounds__(kAttnThreads) attention_decode_kernel(const ui
     const uint16_t* vb = vc + (size_t)n * T_max * Hkv * d + (size_t)g * d;
     const size_t pitch = (size_t)Hkv * d;
     const float scale = rsqrtf((float)d);
-    const int lpp = d >> 3;                  // lanes per position (vec)
-    const int ppw = vec ? 32 / lpp : 1;      // positions per warp step
-    const int sub = vec ? lane / lpp : 0, dl = vec ? (lane % lpp) * 8 : 0;
-    if (vec) {
-        float qv[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) qv[j] = qs[dl + j];
 #pragma unroll 4
-        for (int t0 = warp * ppw; t0 < T; t0 += nw * ppw) {
-            const int t = t0 + sub;
-            float s = 0.f;
-            if (t < T) {
-                const uint4 kv = *(const uint4*)(kb + (size_t)t * pitch + dl);
-                const uint32_t u[4] = {kv.x, kv.y, kv.z, kv.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j) s += qv[2 * j] * bf16_lo(u[j]) + qv[2 * j + 1] * bf16_hi(u[j]);
-            }
-            for (int dd = 1; dd < lpp; dd <<= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, dd);
-            if (t < T && (lane % lpp) == 0) sc[t] = s * scale;
-        }
-    } else {
-#pragma unroll 4
-        for (int t = warp; t < T; t += nw) {
-            float s = 0.f;
-            for (int i = lane; i < d; i += 32) s += qs[i] * bf16_to_f32(kb[(size_t)t * pitch + i]);
-            for (int dd = 16; dd > 0; dd >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, dd);
-            if (lane == 0) sc[t] = s * scale;
-        }
+    for (int t = warp; t < T; t += nw) {
+        float s = 0.f;
+        for (int i = lane; i < d; i += 32) s += qs[i] * bf16_to_f32(kb[(size_t)t * pitch + i]);
+        for (int dd = 16; dd > 0; dd >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, dd);
+        if (lane == 0) sc[t] = s * scale;
     }
     __syncthreads();
     float m = -INFINITY;
@@ -208,43 +359,18 @@ __global__ void __launch_bounds__(kAttnThreads) attention_decode_kernel(const ui
     z = block_sum(z, red);
     __syncthreads();
     // weights times values; the warps' partial sums meet in shared memory
-    if (vec) {
-        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 4
-        for (int t0 = warp * ppw; t0 < T; t0 += nw * ppw) {
-            const int t = t0 + sub;
-            if (t < T) {
-                const float p = sc[t];
-                const uint4 vv = *(const uint4*)(vb + (size_t)t * pitch + dl);
-                const uint32_t u[4] = {vv.x, vv.y, vv.z, vv.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    acc[2 * j] += p * bf16_lo(u[j]);
-                    acc[2 * j + 1] += p * bf16_hi(u[j]);
-                }
-            }
-        }
-        // the 32 / lpp position groups of the warp add up
-        for (int dd = lpp; dd < 32; dd <<= 1)
-#pragma unroll
-            for (int j = 0; j < 8; ++j) acc[j] += __shfl_xor_sync(0xFFFFFFFFu, acc[j], dd);
-        if (lane < lpp)
-#pragma unroll
-            for (int j = 0; j < 8; ++j) part[warp * 128 + dl + j] = acc[j];
-    } else {
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-        for (int t = warp; t < T; t += nw) {
-            const float p = sc[t];
-            const uint16_t* vr = vb + (size_t)t * pitch;
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (lane + 32 * j < d) acc[j] += p * bf16_to_f32(vr[lane + 32 * j]);
-        }
+    for (int t = warp; t < T; t += nw) {
+        const float p = sc[t];
+        const uint16_t* vr = vb + (size_t)t * pitch;
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-            if (lane + 32 * j < d) part[warp * 128 + lane + 32 * j] = acc[j];
+            if (lane + 32 * j < d) acc[j] += p * bf16_to_f32(vr[lane + 32 * j]);
     }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (lane + 32 * j < d) part[warp * 128 + lane + 32 * j] = acc[j];
     __syncthreads();
     if (threadIdx.x < d) {
         float a = 0.f;
@@ -257,9 +383,9 @@ __global__ void __launch_bounds__(kAttnThreads) attention_decode_kernel(const ui
 // (and writes it back), rotates the key head of its group for itself, and attends over the cached positions 0..pos-1
 // plus the new token, whose key and value it takes from its own shared memory and from `v`, not from the cache; the
 // first head of every group also appends the rotated key and the value to the caches.  No CTA reads what another writes.
-__global__ void __launch_bounds__(kAttnThreads) rope_attention_kernel(uint16_t* q, const uint16_t* k, const uint16_t* v, uint16_t* kc,
+__global__ void __launch_bounds__(kAttnThreads) rope_attention_any_kernel(uint16_t* q, const uint16_t* k, const uint16_t* v, uint16_t* kc,
                                                                      uint16_t* vc, uint16_t* out, int Hq, int Hkv, int d, int pos,
-                                                                     int T_max, const RopeTable tab, int vec)
+                                                                     int T_max, const __grid_constant__ RopeTable tab)
 {
     pdl_let_next_start();
     pdl_wait();
@@ -300,34 +426,12 @@ __global__ void __launch_bounds__(kAttnThreads) rope_attention_kernel(uint16_t* 
     const uint16_t* kb = kc + (size_t)n * T_max * pitch + (size_t)g * d;
     const uint16_t* vb = vc + (size_t)n * T_max * pitch + (size_t)g * d;
     const float scale = rsqrtf((float)d);
-    const int lpp = d >> 3;
-    const int ppw = vec ? 32 / lpp : 1;
-    const int sub = vec ? lane / lpp : 0, dl = vec ? (lane % lpp) * 8 : 0;
-    if (vec) {
-        float qv[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) qv[j] = qs[dl + j];
 #pragma unroll 4
-        for (int t0 = warp * ppw; t0 < T; t0 += nw * ppw) {
-            const int t = t0 + sub;
-            float s = 0.f;
-            if (t < T) {
-                const uint4 kv = *(const uint4*)(kb + (size_t)t * pitch + dl);
-                const uint32_t u[4] = {kv.x, kv.y, kv.z, kv.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j) s += qv[2 * j] * bf16_lo(u[j]) + qv[2 * j + 1] * bf16_hi(u[j]);
-            }
-            for (int dd = 1; dd < lpp; dd <<= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, dd);
-            if (t < T && (lane % lpp) == 0) sc[t] = s * scale;
-        }
-    } else {
-#pragma unroll 4
-        for (int t = warp; t < T; t += nw) {
-            float s = 0.f;
-            for (int i = lane; i < d; i += 32) s += qs[i] * bf16_to_f32(kb[(size_t)t * pitch + i]);
-            for (int dd = 16; dd > 0; dd >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, dd);
-            if (lane == 0) sc[t] = s * scale;
-        }
+    for (int t = warp; t < T; t += nw) {
+        float s = 0.f;
+        for (int i = lane; i < d; i += 32) s += qs[i] * bf16_to_f32(kb[(size_t)t * pitch + i]);
+        for (int dd = 16; dd > 0; dd >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, dd);
+        if (lane == 0) sc[t] = s * scale;
     }
     if (warp == 0) {                         // the new token's own score
         float s = 0.f;
@@ -347,42 +451,18 @@ __global__ void __launch_bounds__(kAttnThreads) rope_attention_kernel(uint16_t* 
     }
     z = block_sum(z, red);
     __syncthreads();
-    if (vec) {
-        float acc[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 4
-        for (int t0 = warp * ppw; t0 < T; t0 += nw * ppw) {
-            const int t = t0 + sub;
-            if (t < T) {
-                const float p = sc[t];
-                const uint4 vv = *(const uint4*)(vb + (size_t)t * pitch + dl);
-                const uint32_t u[4] = {vv.x, vv.y, vv.z, vv.w};
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    acc[2 * j] += p * bf16_lo(u[j]);
-                    acc[2 * j + 1] += p * bf16_hi(u[j]);
-                }
-            }
-        }
-        for (int dd = lpp; dd < 32; dd <<= 1)
-#pragma unroll
-            for (int j = 0; j < 8; ++j) acc[j] += __shfl_xor_sync(0xFFFFFFFFu, acc[j], dd);
-        if (lane < lpp)
-#pragma unroll
-            for (int j = 0; j < 8; ++j) part[warp * 128 + dl + j] = acc[j];
-    } else {
-        float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-        for (int t = warp; t < T; t += nw) {
-            const float p = sc[t];
-            const uint16_t* vr = vb + (size_t)t * pitch;
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                if (lane + 32 * j < d) acc[j] += p * bf16_to_f32(vr[lane + 32 * j]);
-        }
+    for (int t = warp; t < T; t += nw) {
+        const float p = sc[t];
+        const uint16_t* vr = vb + (size_t)t * pitch;
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-            if (lane + 32 * j < d) part[warp * 128 + lane + 32 * j] = acc[j];
+            if (lane + 32 * j < d) acc[j] += p * bf16_to_f32(vr[lane + 32 * j]);
     }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (lane + 32 * j < d) part[warp * 128 + lane + 32 * j] = acc[j];
     __syncthreads();
     if (threadIdx.x < d) {
         float a = sc[T] * bf16_to_f32(vnew[threadIdx.x]);
