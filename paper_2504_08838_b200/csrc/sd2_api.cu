@@ -46,10 +46,18 @@ struct sd2_handle_s {
 };
 
 // What a program over cells needs from shared memory.
+int cell_pitch(int D) { return 2 * share_cells(D, 0) * kCellCols + 64; }
+
 struct CellNeeds {
     int pitch = 0;             // bytes of a staged activation row: the largest
     int max_chunk = 0;
     int tiles_max = 0;         // most tiles of any stage
+    void add(sd2_handle h)
+    {
+        const int p = cell_pitch(h->cell_D);
+        if (p > pitch) pitch = p;
+        if (h->max_chunk > max_chunk) max_chunk = h->max_chunk;
+    }
 };
 
 struct sd2_drafter_s {
@@ -72,7 +80,8 @@ struct sd2_drafter_s {
     int xs_need[3];            // bytes of staged activations at panel widths 1, 2, 4
     // the same blocks as a program over cells, with barrier words of its own; NULL: a handle has no cells
     CStage* d_cstages;
-    CStage first_cstage;
+    CStage first_cstage;       // the first stages of both programs go along with a launch
+    SStage first_stage;
     unsigned int* d_cbar;
     int n_cstages;
     CellNeeds cell_needs;
@@ -658,7 +667,6 @@ int widest_cell_panel(const CellNeeds& needs)
     return 0;
 }
 
-int cell_pitch(int D) { return 2 * share_cells(D, 0) * kCellCols + 64; }
 
 template <int MAXS, int NR>
 sd2_status launch_cells(const CArgs<MAXS>& a, int grid, int smem, cudaStream_t s)
@@ -714,10 +722,8 @@ struct CellBuilder {
             m.T = hs[i]->cell_T;
             m.y_f32 = (!y_force_bf16 && hs[i]->y_dtype == SD2_DTYPE_F32) ? 1 : 0;
             if (!pair || i == 0) st.V += m.T;
-            if (hs[i]->max_chunk > needs.max_chunk) needs.max_chunk = hs[i]->max_chunk;
+            needs.add(hs[i]);
         }
-        const int pitch = cell_pitch(st.D);
-        if (pitch > needs.pitch) needs.pitch = pitch;
         if (st.V > needs.tiles_max) needs.tiles_max = st.V;
         st.rot = rot;
         rot = (int)(((int64_t)rot + st.V) % clusters);
@@ -842,9 +848,7 @@ bool use_cells(const sd2_handle* hs, int count, int64_t N)
     CellNeeds needs;
     for (int i = 0; i < count; ++i) {
         if (!hs[i]->d_image) return false;
-        const int pitch = cell_pitch(hs[i]->cell_D);
-        if (pitch > needs.pitch) needs.pitch = pitch;
-        if (hs[i]->max_chunk > needs.max_chunk) needs.max_chunk = hs[i]->max_chunk;
+        needs.add(hs[i]);
     }
     return cells_pay(hs, count, N) && widest_cell_panel(needs) > 0;
 }
@@ -1135,6 +1139,30 @@ void append_block_cells(CellBuilder& b, const sd2_handle* h, const uint16_t* x, 
     b.add(h + 3, 1, q, y_o, true);
     b.add(h + 4, 2, hdn, y_gu, true, true).t_out = t;
     b.add(h + 6, 1, t, y_d, y_force_bf16);
+}
+
+// A block step over cells.  gbar: barrier words of the caller's, or NULL.
+// One program of four stages where its panels are no narrower than the rest of the block needs them.  Where the down
+// projection's long rows of activations fill shared memory, it goes apart, in panels of its own: sixteen rows of
+// 3072/1024/8192 at 50 % took 94 us as two panels of eight through all stages.
+sd2_status run_block_cells(const sd2_handle* h, const uint16_t* x, uint16_t* q, uint16_t* k, uint16_t* v, uint16_t* hdn, uint16_t* g, uint16_t* u,
+                           uint16_t* t, void* y, unsigned int* gbar, int dev, int64_t N, cudaStream_t s)
+{
+    CArgs<kMaxStagesInline> a = {};
+    CellBuilder b(a.inl, g_dev[dev].sms);
+    append_block_cells(b, h, x, q, k, v, hdn, g, u, t, y, false);
+    a.gbar = gbar;
+    CArgs<kMaxStagesInline> d = {};
+    CellBuilder down(d.inl, g_dev[dev].sms), rest(a.inl, g_dev[dev].sms);
+    void* y_d[1] = {y};
+    down.add(h + 6, 1, t, y_d, false);
+    for (int i = 0; i < 6; ++i) rest.needs.add(h[i]);
+    rest.needs.tiles_max = b.needs.tiles_max;
+    rest.n = b.n - 1;
+    const int64_t all = widest_cell_panel(b.needs), most = widest_cell_panel(rest.needs);
+    if ((N + most - 1) / most >= (N + all - 1) / all) return run_cell_program(a, b, dev, N, s);
+    const sd2_status st = run_cell_program(a, rest, dev, N, s);
+    return st != SD2_OK ? st : run_cell_program(d, down, dev, N, s);
 }
 
 // Builds the paired stack of a block's gate and up (row 2i = gate row i, row 2i+1 = up row i)
@@ -1774,10 +1802,7 @@ sd2_status sd2_block_step(const sd2_handle* h, const void* x, void* y, int64_t N
         for (int i = 0; i < 7; ++i)
             if (h[i]->device != dev) return SD2_ERR_INVALID_ARG;
         if (use_cells(h, 7, N)) {
-            CArgs<kMaxStagesInline> a = {};
-            CellBuilder b(a.inl, g_dev[dev].sms);
-            append_block_cells(b, h, (const uint16_t*)x, q, k, v, hdn, g, u, t, y, false);
-            return run_cell_program(a, b, dev, N, s);
+            return run_block_cells(h, (const uint16_t*)x, q, k, v, hdn, g, u, t, y, nullptr, dev, N, s);
         }
         SArgs a;
         std::memset(&a, 0, sizeof a);
@@ -1844,12 +1869,9 @@ sd2_status sd2_block_step_static(const sd2_handle* h, const void* x, void* y, in
     if (cudaMemsetAsync(base, 0, 256, s) != cudaSuccess) { cudaGetLastError(); return SD2_ERR_CUDA; }
     char* ws = (char*)base + 256;
     if (use_cells(h, 7, N)) {
-        CArgs<kMaxStagesInline> a = {};
-        CellBuilder b(a.inl, g_dev[dev].sms);
-        append_block_cells(b, h, (const uint16_t*)x, (uint16_t*)(ws + off[0]), (uint16_t*)(ws + off[1]), (uint16_t*)(ws + off[2]),
-                           (uint16_t*)(ws + off[3]), (uint16_t*)(ws + off[4]), (uint16_t*)(ws + off[5]), (uint16_t*)(ws + off[6]), y, false);
-        a.gbar = (unsigned int*)base;
-        return run_cell_program(a, b, dev, N, s);
+        return run_block_cells(h, (const uint16_t*)x, (uint16_t*)(ws + off[0]), (uint16_t*)(ws + off[1]), (uint16_t*)(ws + off[2]),
+                               (uint16_t*)(ws + off[3]), (uint16_t*)(ws + off[4]), (uint16_t*)(ws + off[5]), (uint16_t*)(ws + off[6]), y,
+                               (unsigned int*)base, dev, N, s);
     }
     SArgs a;
     std::memset(&a, 0, sizeof a);
@@ -1969,6 +1991,7 @@ sd2_status sd2_drafter_create(const sd2_handle* h, int32_t L, int64_t n_max, sd2
                                      tagged ? &tg : nullptr, pairs[(size_t)b]);
         }
         d->n_stages = n;
+        d->first_stage = stages[0];
         ok = dev_malloc((void**)&d->d_stages, sizeof(SStage) * (size_t)n) == cudaSuccess &&
              cudaMemcpy(d->d_stages, stages.data(), sizeof(SStage) * (size_t)n, cudaMemcpyHostToDevice) == cudaSuccess &&
              dev_malloc((void**)&d->d_gbar, kDrafterWordsBytes) == cudaSuccess && cudaMemset(d->d_gbar, 0, kDrafterWordsBytes) == cudaSuccess;
@@ -2056,6 +2079,7 @@ sd2_status sd2_drafter_step(sd2_drafter d, const void* x, void* y, int64_t N, vo
     SArgs a;
     std::memset(&a, 0, sizeof a);
     a.ext = d->d_stages;
+    a.inl[0] = d->first_stage;
     a.n_stages = d->n_stages;
     a.x_in = (const uint16_t*)x;
     a.y_out = y;

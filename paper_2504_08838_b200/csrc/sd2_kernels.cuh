@@ -180,7 +180,7 @@ struct SArgsBase {
 // of arguments, not 3.5 KB.
 template <int MAXS>
 struct SArgsT : SArgsBase {
-    SStage inl[MAXS];               // used when ext == NULL
+    SStage inl[MAXS];               // the first stage; all of them when ext == NULL
     SFold fold[MAXS];               // per inline stage; read by FOLD instances only
 };
 using SArgs = SArgsT<kMaxStagesInline>;
@@ -782,7 +782,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const __grid_
         };
         auto load_stage = [&](int s) {
             PStage p;
-            const SStage* st = a.ext ? a.ext + s : &a.inl[MAXS == 1 ? 0 : s];
+            const SStage* st = a.ext && s > 0 ? a.ext + s : &a.inl[MAXS == 1 ? 0 : s];
             p.count = st->count;
             p.n_cta = st->tiles_div + (cta < st->tiles_rem ? 1 : 0);
 #pragma unroll
@@ -928,7 +928,7 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const __grid_
     uint32_t q_mine = (uint32_t)warp;
     bool failed = false;
     if (warp == 1) {
-        const uint32_t* src = (const uint32_t*)(a.ext ? a.ext : &a.inl[0]);
+        const uint32_t* src = (const uint32_t*)&a.inl[0];
         for (int i = lane; i < kStageWords; i += 32) ((uint32_t*)&sh->stage[0])[i] = src[i];
     }
     if (ctid < 8) sh->tag_base[ctid] = (a.tagged && ctid < a.N) ? ((*(volatile unsigned int*)(a.rowseq + a.n0 + ctid)) & 0xFFu) << 8 : 0u;
