@@ -1,0 +1,142 @@
+"""The kernels for several rows at the sizes where they change: edges of tiles, cells, chunks and panels.
+
+Linears over cells: fp32 sums of exact products.  A row's K products are added one after the other at worst, each
+addition rounds or truncates by at most 2^-23 of a partial sum that S = sum |w x| bounds, so |y - ref| <= (K + 32) 2^-23 S;
+bf16 outputs add their rounding, 2^-8 |y|.
+"""
+
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from oracle import decoder_oracle as do
+from oracle import oracle
+from paper_2504_08838_b200 import binding as sd2
+from paper_2504_08838_b200 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+def dev(bits):
+    return torch.from_numpy(np.ascontiguousarray(bits).view(np.int16).copy()).cuda().view(torch.bfloat16)
+
+
+def bits_of(t):
+    return t.view(torch.int16).cpu().numpy().view(np.uint16)
+
+
+def values(bits):
+    return synth.bf16_bits_to_f32(bits).astype(np.float64)
+
+
+def linear_close(y, W, mask, x, f32):
+    ref, S = oracle.masked_linear(W, mask, x)
+    tol = (W.shape[1] + 32) * 2.0 ** -23 * S
+    assert np.all(np.abs(y - ref) <= tol + (0.0 if f32 else 2.0 ** -8 * (np.abs(ref) + tol)))
+
+
+@pytest.mark.parametrize("M,K,N,density,shift", [
+    (1, 8, 4, 0.5, 0), (15, 40, 5, 0.5, 0),                          # one cell: one CTA of a cluster has it all
+    (17, 129, 8, 0.5, 0), (16, 256, 9, 0.5, 0), (100, 257, 16, 0.5, 0),   # a column, a cell for the second CTA; both panel widths
+    (333, 1000, 17, 0.3, 0), (64, 1536, 33, 0.7, 0),                 # two and three launches
+    (3000, 640, 4, 0.5, 0), (2500, 1152, 12, 0.1, 0),                # five and nine cells a tile: turns of two tiles, of one and a rest
+    (200, 4096, 8, 0.5, 0), (200, 4100, 8, 0.5, 0), (1531, 8192, 16, 0.5, 0),  # whole tiles to a group, thirds of tiles
+    (77, 3001, 5, 0.5, 0), (77, 3000, 7, 0.5, 1), (40, 1003, 16, 0.9, 3), (9, 5, 6, 1.0, 1),   # rows that do not start on 16 bytes
+    (320, 2048, 8, 0.0, 0), (320, 2048, 8, 1.0, 0),                  # nothing kept, everything kept
+    (512, 2048, 2, 0.5, 0), (512, 2048, 3, 0.5, 0),                  # the smallest panels of large weights
+])
+def test_linear_over_cells(M, K, N, density, shift):
+    W = synth.normal_bf16(M + K, (M, K), 0.02)
+    mask = synth.bernoulli_mask(M + K + 1, (M, K), density) if 0.0 < density < 1.0 else np.full((M, K), int(density), np.uint8)
+    x = synth.normal_bf16(M + K + 2, (N, K), 1.0)
+    f32 = N % 2 == 0
+    h = sd2.sd2_compress(W, mask, sd2.SD2_FORMAT_GAP4, sd2.SD2_DTYPE_F32 if f32 else sd2.SD2_DTYPE_BF16)
+    store = torch.zeros(N * K + shift, dtype=torch.bfloat16, device="cuda")
+    store[shift:] = dev(x).view(-1)
+    guard = 40
+    buf = torch.full((N * M + 2 * guard,), float("nan"), dtype=torch.float32 if f32 else torch.bfloat16, device="cuda")
+    sd2.sd2_spmm(h, store[shift:].view(N, K), buf[guard:guard + N * M].view(N, M))
+    sd2.sd2_stream_check()
+    out = buf.float().cpu().numpy().astype(np.float64)
+    assert np.isnan(out[:guard]).all() and np.isnan(out[-guard:]).all() and not np.isnan(out[guard:-guard]).any()
+    linear_close(out[guard:-guard].reshape(N, M), W, mask, x, f32)
+    sd2.sd2_free(h)
+
+
+@pytest.mark.parametrize("hidden,kv,inter,N", [(160, 48, 9600, 5),      # more gate tiles per cluster than wait for their up tiles at once
+                                               (256, 64, 8192, 16)])    # the down projection in panels of its own
+def test_block_over_cells(hidden, kv, inter, N):
+    shape = synth.DrafterShape("tiny", hidden, kv, inter, 1)
+    lin = synth.make_block(3, 0, shape, 0.5)
+    hs = [sd2.sd2_compress(W, m, sd2.SD2_FORMAT_GAP4, sd2.SD2_DTYPE_F32 if i == 6 else sd2.SD2_DTYPE_BF16) for i, (W, m) in enumerate(lin)]
+    x = synth.make_activations(3, 0, 0, N, hidden)
+    ws = torch.full((sd2.sd2_block_workspace_bytes(hs, N) // 2,), float("nan"), dtype=torch.bfloat16, device="cuda")
+    y = torch.full((N, hidden), float("nan"), dtype=torch.float32, device="cuda")
+    for _ in range(2):                                                  # twice: the barrier words have to come back clean
+        sd2.sd2_block_step(hs, dev(x), y, ws)
+        sd2.sd2_stream_check()
+    wsb = bits_of(ws)
+    dims = [hidden, kv, kv, hidden, inter, inter, inter]
+    q, k, v, hdn, g, u, t = [wsb[o // 2:o // 2 + N * d].reshape(N, d) for o, d in zip(sd2.sd2_block_workspace_layout(hs, N), dims)]
+    for i, (inp, out) in enumerate([(x, q), (x, k), (x, v), (q, hdn), (hdn, g), (hdn, u)]):
+        linear_close(values(out), lin[i][0], lin[i][1], inp, False)
+    t_ref = values(np.array([oracle.f64_to_bf16_rne(float(z)) for z in oracle.silu_mul(g, u)], np.uint16)).reshape(N, -1)
+    assert np.all(np.abs(values(t) - t_ref) <= 2.0 ** -6 * np.abs(t_ref))      # two ulp of bf16
+    linear_close(y.double().cpu().numpy(), lin[6][0], lin[6][1], t, True)
+    for h in hs:
+        sd2.sd2_free(h)
+
+
+@pytest.mark.parametrize("T,d", [(128, 64), (129, 64), (257, 128), (513, 8), (1100, 16)])     # clusters of one to eight
+def test_attention_split_over_a_cluster(T, d):
+    Hq, Hkv = 4, 2
+    q = synth.normal_bf16(T, (1, Hq * d), 1.0)
+    kc = synth.normal_bf16(T + 1, (1, T + 3, Hkv * d), 1.0)
+    vc = synth.normal_bf16(T + 2, (1, T + 3, Hkv * d), 1.0)
+    out = torch.full((1, Hq * d), float("nan"), dtype=torch.bfloat16, device="cuda")
+    sd2.sd2_attention_decode(dev(q), dev(kc), dev(vc), out, Hq, Hkv, T)
+    torch.cuda.synchronize()
+    f64 = do.bf16_to_f64
+    V = f64(vc[0, :T]).reshape(T, Hkv, d)
+    ref = do.attention_decode(f64(q[0]).reshape(Hq, d), f64(kc[0, :T]).reshape(T, Hkv, d), V)
+    # bf16 rounding, and fp32 arithmetic on weights that sum to one
+    assert np.all(np.abs(f64(bits_of(out)).reshape(Hq, d) - ref) <= 2.0 ** -8 * np.abs(ref) + 2e-4 * np.abs(V).max())
+
+
+@pytest.mark.parametrize("N,V,H", [(2, 1003, 72), (4, 5000, 264), (5, 50, 8), (1, 3, 8)])     # every width, shares of a few rows
+def test_lm_head_widths(N, V, H):
+    W = synth.normal_bf16(V, (V, H), 0.02)
+    x = synth.normal_bf16(V + 1, (N, H), 1.0)
+    logits = torch.full((N, V), float("nan"), dtype=torch.float32, device="cuda")
+    toks = torch.full((N,), -1, dtype=torch.int32, device="cuda")
+    sd2.sd2_lm_head(dev(x), dev(W), logits, toks)
+    torch.cuda.synchronize()
+    got = logits.double().cpu().numpy()
+    linear_close(got, W, np.ones((V, H), np.uint8), x, True)
+    assert [int(t) for t in toks] == [int(np.argmax(row)) for row in got]
+
+
+@pytest.mark.parametrize("N", [1, 8])
+def test_launches_that_overlap_still_run_in_order(N):
+    # each product reads what the one before it wrote, and writes what the one before that read
+    K = 1024
+    W = synth.normal_bf16(7, (K, K), 0.045)
+    h = sd2.sd2_compress(W, synth.bernoulli_mask(8, (K, K), 0.5))
+    x = dev(synth.normal_bf16(9, (N, K), 1.0))
+
+    def chain(wait):
+        a, b = x.clone(), torch.zeros_like(x)
+        for _ in range(40):
+            sd2.sd2_spmm(h, a, b)
+            if wait:
+                torch.cuda.synchronize()
+            a, b = b, a
+        torch.cuda.synchronize()
+        return a
+
+    want = chain(True)
+    assert torch.isfinite(want).all() and want.abs().max() > 0
+    for _ in range(5):
+        assert torch.equal(chain(False), want)
+    sd2.sd2_free(h)
