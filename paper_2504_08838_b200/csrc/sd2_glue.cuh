@@ -491,13 +491,27 @@ __global__ void __launch_bounds__(kGlueThreads) embedding_kernel(const int32_t* 
 }
 
 // logits[n, v] = sum_h W[v, h] x[n, h]: a warp takes kHeadRowsPerWarp vocabulary rows at a time (as many independent
-// 128-bit loads in flight per lane) of its share of the table, the activation rows sit in shared memory as bf16.  HBM bounds
-// it.  Shares are runs of rows of (almost) equal length: with steps of four rows dealt out in turn, 3.4 of them per warp for
-// 128256 rows, some warps worked while others were done.  Four rows share what is read of the activations; with one row per
-// step and fp32 activations a row took as long as a pass of its own (a step of one row 257 us, of four rows 1033 us).
+// 128-bit loads in flight per lane and column step) of its share of the table, the activation rows sit in shared memory as
+// bf16.  HBM bounds it: 128256 x 2048 takes 80 us for one and two rows (6.5 TB/s), from 102.  What that took:
+//   - even shares of rows per warp; steps of four rows dealt out in turn, 3.4 of them per warp, left warps idle: 94 us;
+//   - 256-byte requests that pass L1 by and four column steps in flight, on three CTAs per SM: 80 us;
+//   - four rows that share what is read of the activations, and fma.rn.f32x2 (the same fp32 sums, even and odd columns
+//     apart): with one row per step every activation row took as long as a pass of its own, four of them 520 us.
 constexpr int kHeadRowsPerWarp = 4;
 // CTAs per SM of an instance for NT rows, as many as its registers allow
-constexpr int head_ctas(int NT) { return NT <= 1 ? 5 : NT <= 2 ? 3 : 2; }
+constexpr int head_ctas(int NT) { return NT <= 1 ? 3 : 2; }
+__device__ __forceinline__ uint4 ldg_stream(const uint4* p)
+{
+    uint4 v;
+    asm volatile("ld.global.nc.L1::no_allocate.L2::256B.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+// two bf16 values as a pair of fp32, two fp32 multiply-adds
+__device__ __forceinline__ unsigned long long f32_pair(uint32_t w) { return (unsigned long long)(w & 0xFFFF0000u) << 32 | (w << 16); }
+__device__ __forceinline__ void fma_pair(unsigned long long& acc, unsigned long long a, unsigned long long b)
+{
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
 template <int NT>
 __global__ void __launch_bounds__(kGlueThreads, head_ctas(NT)) lm_head_kernel(const uint16_t* x, const uint16_t* W, float* logits, int N, int V, int H)
 {
@@ -511,26 +525,26 @@ __global__ void __launch_bounds__(kGlueThreads, head_ctas(NT)) lm_head_kernel(co
     const long long warps = (gridDim.x * blockDim.x) >> 5, gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int end = (int)(V * (gw + 1) / warps);
     for (int v0 = (int)(V * gw / warps); v0 < end; v0 += kHeadRowsPerWarp) {
-        float acc[NT][kHeadRowsPerWarp];
+        unsigned long long acc[NT][kHeadRowsPerWarp];
 #pragma unroll
         for (int n = 0; n < NT; ++n)
 #pragma unroll
-            for (int r = 0; r < kHeadRowsPerWarp; ++r) acc[n][r] = 0.f;
-#pragma unroll(NT < 8 ? 2 : 1)
+            for (int r = 0; r < kHeadRowsPerWarp; ++r) acc[n][r] = 0ull;
+#pragma unroll(NT <= 2 ? 4 : NT <= 4 ? 2 : 1)
         for (int c = lane; c < groups; c += 32) {
             uint4 w4[kHeadRowsPerWarp];
 #pragma unroll
             for (int r = 0; r < kHeadRowsPerWarp; ++r)
-                w4[r] = v0 + r < end ? __ldg((const uint4*)(W + (size_t)(v0 + r) * H) + c) : make_uint4(0u, 0u, 0u, 0u);
+                w4[r] = v0 + r < end ? ldg_stream((const uint4*)(W + (size_t)(v0 + r) * H) + c) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
             for (int n = 0; n < NT; ++n) {
                 const uint4 xv = head_x[n * groups + c];
-                const uint32_t xw[4] = {xv.x, xv.y, xv.z, xv.w};
+                const unsigned long long xw[4] = {f32_pair(xv.x), f32_pair(xv.y), f32_pair(xv.z), f32_pair(xv.w)};
 #pragma unroll
                 for (int r = 0; r < kHeadRowsPerWarp; ++r) {
                     const uint32_t ww[4] = {w4[r].x, w4[r].y, w4[r].z, w4[r].w};
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[n][r] += bf16_lo(ww[j]) * bf16_lo(xw[j]) + bf16_hi(ww[j]) * bf16_hi(xw[j]);
+                    for (int j = 0; j < 4; ++j) fma_pair(acc[n][r], f32_pair(ww[j]), xw[j]);
                 }
             }
         }
@@ -538,7 +552,7 @@ __global__ void __launch_bounds__(kGlueThreads, head_ctas(NT)) lm_head_kernel(co
         for (int n = 0; n < NT; ++n)
 #pragma unroll
             for (int r = 0; r < kHeadRowsPerWarp; ++r) {
-                const float s = warp_sum(acc[n][r]);
+                const float s = warp_sum(__uint_as_float((uint32_t)acc[n][r]) + __uint_as_float((uint32_t)(acc[n][r] >> 32)));
                 if (lane == 0 && n < N && v0 + r < end) logits[(size_t)n * V + v0 + r] = s;
             }
     }
