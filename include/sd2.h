@@ -61,7 +61,10 @@ enum {
     SD2_FORMAT_BITMASK = 1, /* 1 bit per dense slot + packed kept values + row offsets    */
     SD2_FORMAT_GAP4 = 2,    /* 4-bit column gaps + packed kept values in 8-entry chunks,  */
                             /* rows cut into column strips, 32 strips to a tile (the fast */
-                            /* path; column strips wider than 496 are not supported)      */
+                            /* path; column strips wider than 496 are not supported).     */
+                            /* The handle also keeps the weights as cells in the order of */
+                            /* a tensor-core operand (about 1.3 times the strips' bytes), */
+                            /* which calls of several rows read instead.                  */
     SD2_FORMAT_GAP4_PAIRED = 3,/* as an option of sd2_pack_host / sd2_compress only: GAP4 */
                             /* whose rows 2i and 2i+1 stay next to each other in a tile   */
                             /* (for a stack that interleaves gate row i and up row i; M   */
@@ -158,12 +161,13 @@ sd2_status sd2_spmm_fused(const sd2_handle* h, int32_t count, const void* X, voi
  * x: device bf16 [N*hidden]; y: device [N*M_down] in h[6]'s y_dtype.
  * workspace: device, sd2_block_workspace_bytes bytes, 256-byte aligned; after the call it
  * holds, in this order and each [N*dim] bf16, 256-byte aligned: q, k, v, hdn, g, u, t.
- * With seven GAP4 weights the block is ONE launch: a persistent CTA per SM runs the stages
+ * With seven GAP4 weights the block is ONE launch per panel of rows (the down projection goes
+ * apart where its long rows would narrow the panel): a persistent CTA per SM runs the stages
  * one after another, separated by grid-wide barriers, while a producer warp keeps copying the
  * coming stages' weights into shared memory.  Such launches take every SM; two of them should
  * not be put on different streams in the hope of overlap.
  * Errors: SHAPE if the seven shapes do not chain, or N outside [0, 65536].  Any N in that range
- * is served: rows are independent and go through the block in panels of at most 8. */
+ * is served: rows are independent and go through the block in panels of at most 16. */
 sd2_status sd2_block_step(const sd2_handle* h, const void* x, void* y, int64_t N,
                           void* workspace, void* cuda_stream);
 

@@ -52,11 +52,13 @@ struct CellNeeds {
     int pitch = 0;             // bytes of a staged activation row: the largest
     int max_chunk = 0;
     int tiles_max = 0;         // most tiles of any stage
+    bool split = false;        // a stage's tiles are split over the groups
     void add(sd2_handle h)
     {
         const int p = cell_pitch(h->cell_D);
         if (p > pitch) pitch = p;
         if (h->max_chunk > max_chunk) max_chunk = h->max_chunk;
+        if (share_cells(h->cell_D, 0) > kSplitCells) split = true;
     }
 };
 
@@ -209,6 +211,7 @@ sd2_status ensure_device(int* dev_out)
             set_smem_attr<kMany, 1>() != cudaSuccess || set_smem_attr<kMany, 2>() != cudaSuccess || set_smem_attr<kMany, 4>() != cudaSuccess ||
             set_cell_attr<1, 8>() != cudaSuccess || set_cell_attr<1, 16>() != cudaSuccess ||
             set_cell_attr<kMany, 8>() != cudaSuccess || set_cell_attr<kMany, 16>() != cudaSuccess ||
+            cudaFuncSetAttribute(cell_kernel<1, kWidePanelRows, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
             cudaFuncSetAttribute(mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
             cudaFuncSetAttribute(lm_head_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
             cudaFuncSetAttribute(lm_head_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
@@ -635,21 +638,28 @@ sd2_status run_program(SArgs& a, int dev, int64_t N, const ProgramNeeds& needs, 
 // ------------------------------------------------------------------ programs over cells
 
 struct CellPlan {
-    int n_parts, part_bytes, xbuf_bytes, chunk_bytes, n_slots;
+    int fixed_bytes, n_parts, part_bytes, xbuf_bytes, chunk_bytes, n_slots;
 };
 
-constexpr int kCellFixedBytes = (int)((sizeof(CellShared) + 127) & ~127);
+template <int NR>
+constexpr int cell_fixed_bytes() { return (int)((sizeof(CellShared<NR>) + 127) & ~127); }
+
+int cell_instance(int n) { return n <= 8 ? 8 : n <= 16 ? 16 : 32; }
 
 // Shared memory of a launch of n rows.  false: not even two chunks per group fit beside the staged rows.
 bool plan_cells(int n, const CellNeeds& needs, CellPlan* p)
 {
     p->chunk_bytes = (needs.max_chunk + 127) & ~127;
     p->xbuf_bytes = (n * needs.pitch + 127) & ~127;
-    // (n_parts: per finisher) the ring comes first: nine chunks in flight cover HBM's latency, then sums may wait, then more
-    static const int tries[][2] = {{4, 8}, {3, 8}, {3, 4}, {2, 4}};
+    // (n_parts: per finisher) the ring comes first: nine chunks in flight cover HBM's latency, then sums may wait, then more.
+    // A tile of split stages takes three of the slots for sums.
+    const int nr = cell_instance(n);
+    p->fixed_bytes = nr == 8 ? cell_fixed_bytes<8>() : nr == 16 ? cell_fixed_bytes<16>() : cell_fixed_bytes<32>();
+    static const int tries[][2] = {{4, 8}, {3, 8}, {3, 4}, {2, 4}, {2, 2}};
     for (const int* t : tries) {
-        p->part_bytes = 2 * t[1] * part_slot_bytes(n > 8 ? 16 : 8);
-        const int ring = kSmemMax - kCellFixedBytes - p->part_bytes - p->xbuf_bytes;
+        if (t[1] < 4 && needs.split) break;
+        p->part_bytes = 2 * t[1] * part_slot_bytes(nr);
+        const int ring = kSmemMax - p->fixed_bytes - p->part_bytes - p->xbuf_bytes;
         p->n_parts = t[1];
         p->n_slots = ring > 0 ? ring / (kCellGroups * p->chunk_bytes) : 0;
         if (p->n_slots > kGroupSlots) p->n_slots = kGroupSlots;
@@ -658,18 +668,18 @@ bool plan_cells(int n, const CellNeeds& needs, CellPlan* p)
     return false;
 }
 
-// Most rows a launch of the program can take (at most 16); 0 if none.
-int widest_cell_panel(const CellNeeds& needs)
+// Most rows a launch of the program can take; 0 if none.
+int widest_cell_panel(const CellNeeds& needs, int most = kPanelRows)
 {
     CellPlan p;
-    for (int n = kPanelRows; n >= 1; --n)
+    for (int n = most; n >= 1; --n)
         if (plan_cells(n, needs, &p)) return n;
     return 0;
 }
 
 
-template <int MAXS, int NR>
-sd2_status launch_cells(const CArgs<MAXS>& a, int grid, int smem, cudaStream_t s)
+template <int MAXS>
+sd2_status launch_cell_kernel(void (*kernel)(CArgs<MAXS>), const CArgs<MAXS>& a, int grid, int smem, cudaStream_t s)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
@@ -685,9 +695,19 @@ sd2_status launch_cells(const CArgs<MAXS>& a, int grid, int smem, cudaStream_t s
     if (a.n_stages == 1) attr[1] = pdl_attribute();
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    const cudaError_t e = a.fold_any ? cudaLaunchKernelEx(&cfg, cell_kernel<MAXS, NR, true>, a) : cudaLaunchKernelEx(&cfg, cell_kernel<MAXS, NR, false>, a);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, a);
     if (e != cudaSuccess) { cudaGetLastError(); return SD2_ERR_CUDA; }
     return SD2_OK;
+}
+
+template <int MAXS, int NR>
+sd2_status launch_cells(const CArgs<MAXS>& a, int grid, int smem, cudaStream_t s)
+{
+    return launch_cell_kernel<MAXS>(a.fold_any ? cell_kernel<MAXS, NR, true> : cell_kernel<MAXS, NR, false>, a, grid, smem, s);
+}
+sd2_status launch_wide_cells(const CArgs<1>& a, int grid, int smem, cudaStream_t s)
+{
+    return launch_cell_kernel<1>(cell_kernel<1, kWidePanelRows, false>, a, grid, smem, s);
 }
 
 void set_stage_clusters(CStage& st, int clusters)
@@ -736,7 +756,7 @@ struct CellBuilder {
 // Launches a program over all N rows, in panels of equal size (rows are independent).
 sd2_status run_cell_panels(CArgs<kMaxStagesInline>& a, int64_t N, const CellNeeds& needs, int grid, cudaStream_t s)
 {
-    const int cap = widest_cell_panel(needs);
+    const int cap = widest_cell_panel(needs, a.n_stages == 1 && !a.fold_any ? kWidePanelRows : kPanelRows);
     if (cap == 0) return SD2_ERR_UNSUPPORTED;
     const int64_t panels = (N + cap - 1) / cap;
     const int64_t rows = (N + panels - 1) / panels;
@@ -755,11 +775,11 @@ sd2_status run_cell_panels(CArgs<kMaxStagesInline>& a, int64_t N, const CellNeed
         a.xbuf_bytes = p.xbuf_bytes;
         a.chunk_bytes = p.chunk_bytes;
         a.n_slots = p.n_slots;
-        const int smem = kCellFixedBytes + p.part_bytes + p.xbuf_bytes + kCellGroups * p.n_slots * p.chunk_bytes;
+        const int smem = p.fixed_bytes + p.part_bytes + p.xbuf_bytes + kCellGroups * p.n_slots * p.chunk_bytes;
         sd2_status st;
         if (small) {
             static_cast<CArgsBase&>(one) = a;
-            st = a.N > 8 ? launch_cells<1, 16>(one, grid, smem, s) : launch_cells<1, 8>(one, grid, smem, s);
+            st = a.N > 16 ? launch_wide_cells(one, grid, smem, s) : a.N > 8 ? launch_cells<1, 16>(one, grid, smem, s) : launch_cells<1, 8>(one, grid, smem, s);
         } else {
             st = a.N > 8 ? launch_cells<kMaxStagesInline, 16>(a, grid, smem, s) : launch_cells<kMaxStagesInline, 8>(a, grid, smem, s);
         }

@@ -31,7 +31,7 @@
 // What bounds it: HBM for large matrices (15 slots per clock and SM at 50 % density against 33 that twelve warps expand, 29
 // for sixteen rows); between stages some 2.8 us: from the last output to the barrier's release 1.2, to the activations 0.6, to
 // the first cell 0.9.  One launch with its start and its last sums is 8 us at least, and launches of a stream overlap there.
-// Against the strips, which gather row by row (us): 5 rows of 1531 x 3001 18.5 -> 8.3, 48 rows of 8192 x 2048 111 -> 29, two
+// Against the strips, which gather row by row (us): 5 rows of 1531 x 3001 18.5 -> 8.3, 48 rows of 8192 x 2048 111 -> 24, two
 // blocks of 2048/512/8192 for 8 rows 230 -> 68, a block of 3072/1024/8192 for 16 rows 342 -> 59.
 //
 // Every wait (ring barriers, counters, grid barrier) is bounded by a cycle budget: when it runs out the CTA raises the
@@ -54,7 +54,9 @@ constexpr int kGroupSlots = 4;              // chunks in flight per group, at mo
 constexpr int kPartSlots = 8;               // groups' partial sums that may wait for a finisher, at most (a power of two)
 constexpr int kRecvSlots = 8;               // sums from the other CTA that wait to be used
 constexpr int kPairSlots = 8;               // gate tiles whose results wait for the up tile's
-constexpr int kPanelRows = 16;              // activation rows of a launch, at most
+constexpr int kPanelRows = 16;              // activation rows of a launch of several stages, at most
+constexpr int kWidePanelRows = 32;          // ... of a single stage: a cell is expanded once for all of them (us, in panels of
+                                            // 16 / of 32: 24 rows of 8192 x 2048 at 50 % 19.5 / 12.0, 48 rows 29.3 / 24.0)
 // A warp's contribution to a tile: for every eight activation rows 16 x 8 fp32, the activation row fastest.  A lane's
 // fragment goes there in 8-byte stores and a finisher reads 16 bytes a lane, both without bank conflicts.
 constexpr int kPartRowBytes = 32;
@@ -111,6 +113,7 @@ struct CArgs : CArgsBase {
     SFold fold[MAXS];               // read by FOLD instances only
 };
 
+template <int NR>
 struct CellShared {
     unsigned long long full[kCellGroups][kGroupSlots];    // a chunk landed
     unsigned long long empty[kCellGroups][kGroupSlots];   // ... and has been consumed
@@ -122,8 +125,8 @@ struct CellShared {
     unsigned long long rfull[kRecvSlots];               // sums from the other CTA have landed in recv[]
     unsigned long long credit[2];                       // the other CTA has taken ours out of this half of its recv[]
     unsigned int freed[2][kPartSlots];                  // how often the slot's sums have been read
-    uint2 gate[kPairSlots][kPanelRows / 8][32];         // bf16 results of gate tiles, as the finisher's lanes hold them
-    float4 recv[kRecvSlots][kPanelRows / 8][32];
+    uint2 gate[kPairSlots][NR / 8][32];         // bf16 results of gate tiles, as the finisher's lanes hold them
+    float4 recv[kRecvSlots][NR / 8][32];
     int abort_flag;                                     // any warp: a bounded wait ran out
     float red[2][kCellWarps];                           // FOLD: per-warp partial sums of squares of two rows
     CStage stage[2];                                    // descriptors of the current and the next stage
@@ -322,24 +325,26 @@ __device__ __forceinline__ void load_pairs(uint32_t nib, uint32_t& at, uint32_t 
     at = byte_times_128<SGN, 3>(upto, at);
 }
 
+// Sets of sums per eight activation rows: two keep two chains of mma in flight where one or two column tiles would not.
+__host__ __device__ constexpr int sum_sets(int NR) { return NR <= 16 ? 2 : 1; }
+
 // One cell: eight mma steps for each eight activation rows.  m: the lane's mask; lo, hi: shared addresses of the first
-// words of its rows g and g + 8; xo, xo8: of the first eight activations of panel rows g and g + 8.
-// Two sets of sums per eight rows keep two chains of mma in flight.
+// words of its rows g and g + 8; xo[h]: of the first eight activations of panel row g + 8 h.
 template <int NR>
-__device__ __forceinline__ void multiply_cell(uint32_t m, uint32_t lo, uint32_t hi, uint32_t xo, uint32_t xo8, float (&c)[NR / 4][4])
+__device__ __forceinline__ void multiply_cell(uint32_t m, uint32_t lo, uint32_t hi, const uint32_t (&xo)[NR / 8], uint32_t xd,
+                                              float (&c)[NR / 8 * sum_sets(NR)][4])
 {
+    constexpr int kSets = sum_sets(NR);
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         uint32_t a[4], b[4];
         load_pairs<1>((m >> (4 * u)) & 0xFu, lo, a);
         load_pairs<-1>((m >> (16 + 4 * u)) & 0xFu, hi, b);
-        const uint4 x = lds_v4(xo + 64u * u);
-        mma_rows(c[0], a[0], b[0], a[1], b[1], x.x, x.y);
-        mma_rows(c[1], a[2], b[2], a[3], b[3], x.z, x.w);
-        if (NR > 8) {
-            const uint4 y = lds_v4(xo8 + 64u * u);
-            mma_rows(c[NR / 4 - 2], a[0], b[0], a[1], b[1], y.x, y.y);
-            mma_rows(c[NR / 4 - 1], a[2], b[2], a[3], b[3], y.z, y.w);
+#pragma unroll
+        for (int h = 0; h < NR / 8; ++h) {
+            const uint4 x = lds_v4(xo[h] + xd + 64u * u);
+            mma_rows(c[kSets * h], a[0], b[0], a[1], b[1], x.x, x.y);
+            mma_rows(c[kSets * h + kSets - 1], a[2], b[2], a[3], b[3], x.z, x.w);
         }
     }
 }
@@ -560,8 +565,8 @@ template <int MAXS, int NR, bool FOLD>
 __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_constant__ CArgs<MAXS> a)
 {
     extern __shared__ __align__(128) unsigned char smem[];
-    constexpr uint32_t kPartOff = (uint32_t)((sizeof(CellShared) + 127) & ~127);
-    CellShared* sh = (CellShared*)smem;
+    constexpr uint32_t kPartOff = (uint32_t)((sizeof(CellShared<NR>) + 127) & ~127);
+    CellShared<NR>* sh = (CellShared<NR>*)smem;
     constexpr uint32_t kSlotBytes = (uint32_t)part_slot_bytes(NR);
     const uint32_t xoff = kPartOff + 2u * (uint32_t)(a.part_mask + 1) * kSlotBytes;
     const uint32_t ring_off = xoff + (uint32_t)a.xbuf_bytes;
@@ -893,7 +898,6 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         const uint32_t sbase = smem_u32(smem);
         const uint32_t ring = sbase + ring_off + (uint32_t)grp * NS * (uint32_t)a.chunk_bytes;
         const int g = lane >> 2;
-        const int xrow = g < N ? g : 0, xrow8 = g + 8 < N ? g + 8 : 0;   // rows beyond N repeat row 0; their sums are never read
         ConsumerSync sync;
         sync.bar = smem_u32(&sh->csync);
         sync.phase = 0;
@@ -937,15 +941,18 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
             }
             const uint32_t C = (uint32_t)(Dr < kChunkCells ? Dr : kChunkCells);
             const bool alone = D == 1;
-            const uint32_t xl = sbase + xoff + (uint32_t)(xrow * pitch) + 16u * (lane & 3), xl8 = sbase + xoff + (uint32_t)(xrow8 * pitch) + 16u * (lane & 3);
+            uint32_t xl[NR / 8];                                 // rows beyond N repeat row 0; their sums are never read
+#pragma unroll
+            for (int h = 0; h < NR / 8; ++h) xl[h] = sbase + xoff + (uint32_t)((g + 8 * h < N ? g + 8 * h : 0) * pitch) + 16u * (lane & 3);
             while (!failed && more) {
                 const uint32_t n_parts = deal.split ? kCellGroups : 1;
                 const int step = deal.split ? kCellWarps : kChunkCells;
                 int q = grp - gb;                                // the group's first turn
                 if (q < 0) q += kCellGroups;
-                float acc[NR / 4][4];
+                constexpr int kSets = sum_sets(NR);
+                float acc[NR / 8 * kSets][4];
 #pragma unroll
-                for (int m = 0; m < NR / 4; ++m)
+                for (int m = 0; m < NR / 8 * kSets; ++m)
 #pragma unroll
                     for (int k = 0; k < 4; ++k) acc[m][k] = 0.f;
                 for (int turn = deal.split ? 0 : q; turn < (deal.split ? 1 : deal.turns) && !failed; turn += kCellGroups) {
@@ -969,7 +976,7 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                         const uint32_t m = lds_u32(cell + 4 * lane), v0 = cell + kCellHeaderBytes;
                         const uint32_t pi = lds_u8(cell + 128u + lane) & 0x7Fu;
                         const uint32_t xd = (uint32_t)d * (2 * kCellCols);
-                        multiply_cell<NR>(m, v0 + 4u * lane, v0 + (H - 1u) * 128u + pi, xl + xd, xl8 + xd, acc);
+                        multiply_cell<NR>(m, v0 + 4u * lane, v0 + (H - 1u) * 128u + pi, xl, xd, acc);
                     }
                     __syncwarp();
                     mbar_arrive_n(empty0 + 8 * slot, 1u, lane == 0);
@@ -988,11 +995,15 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                                            entry * (kSlotBytes / kChunkCells) + 8u * lane;       // (row g, activation rows 2 t and 2 t + 1)
 #pragma unroll
                         for (int h = 0; h < NR / 8; ++h) {
-                            *(float2*)(p + 512 * h) = make_float2(acc[2 * h][0] + acc[2 * h + 1][0], acc[2 * h][1] + acc[2 * h + 1][1]);
-                            *(float2*)(p + 512 * h + 256) = make_float2(acc[2 * h][2] + acc[2 * h + 1][2], acc[2 * h][3] + acc[2 * h + 1][3]);
+                            float* s0 = acc[kSets * h];
+                            if (kSets == 2)
+#pragma unroll
+                                for (int k = 0; k < 4; ++k) s0[k] += acc[kSets * h + kSets - 1][k];
+                            *(float2*)(p + 512 * h) = make_float2(s0[0], s0[1]);
+                            *(float2*)(p + 512 * h + 256) = make_float2(s0[2], s0[3]);
                         }
 #pragma unroll
-                        for (int m = 0; m < NR / 4; ++m)
+                        for (int m = 0; m < NR / 8 * kSets; ++m)
 #pragma unroll
                             for (int k = 0; k < 4; ++k) acc[m][k] = 0.f;
                         __syncwarp();

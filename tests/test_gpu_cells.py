@@ -39,7 +39,7 @@ def linear_close(y, W, mask, x, f32):
 @pytest.mark.parametrize("M,K,N,density,shift", [
     (1, 8, 4, 0.5, 0), (15, 40, 5, 0.5, 0),                          # one cell: one CTA of a cluster has it all
     (17, 129, 8, 0.5, 0), (16, 256, 9, 0.5, 0), (100, 257, 16, 0.5, 0),   # a column, a cell for the second CTA; both panel widths
-    (333, 1000, 17, 0.3, 0), (64, 1536, 33, 0.7, 0),                 # two and three launches
+    (333, 1000, 17, 0.3, 0), (200, 2048, 32, 0.5, 0), (64, 1536, 33, 0.7, 0), (50, 4608, 20, 0.5, 0),   # wide panels, two launches
     (3000, 640, 4, 0.5, 0), (2500, 1152, 12, 0.1, 0),                # five and nine cells a tile: turns of two tiles, of one and a rest
     (200, 4096, 8, 0.5, 0), (200, 4100, 8, 0.5, 0), (1531, 8192, 16, 0.5, 0),  # whole tiles to a group, thirds of tiles
     (77, 3001, 5, 0.5, 0), (77, 3000, 7, 0.5, 1), (40, 1003, 16, 0.9, 3), (9, 5, 6, 1.0, 1),   # rows that do not start on 16 bytes
