@@ -19,6 +19,7 @@
 #include "sd2_format_mma.hpp"
 #include "sd2_kernels.cuh"
 #include "sd2_cell_kernel.cuh"
+#include "sd2_cells_pack.cuh"
 #include "sd2_mma_kernel.cuh"
 #include "sd2_glue.cuh"
 
@@ -329,43 +330,90 @@ sd2_status upload(const uint8_t* blob, int64_t bytes, const BlobHeader& hd, sd2_
     return SD2_OK;
 }
 
-// Gives a fresh GAP4 handle its cells.  On failure the handle is freed.
-sd2_status add_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask)
-{
-    CellImage im;
-    sd2_status st = SD2_OK;
-    try {
-        im = pack_cells(W, mask, h->M, h->K);
-        st = from_pack(im.status);
-    } catch (const std::bad_alloc&) {
-        st = SD2_ERR_ALLOC;
-    }
-    void* d = nullptr;
-    if (st == SD2_OK && dev_malloc(&d, im.bytes) != cudaSuccess) { cudaGetLastError(); st = SD2_ERR_ALLOC; }
-    if (st == SD2_OK && cudaMemcpy(d, im.data, im.bytes, cudaMemcpyHostToDevice) != cudaSuccess) { cudaGetLastError(); st = SD2_ERR_CUDA; }
-    std::free(im.data);
-    if (st != SD2_OK) {
-        if (d) cudaFree(d);
-        sd2_free(h);
-        return st;
-    }
-    const CellGeom g = cell_geometry(h->M, h->K);
-    h->d_image = (uint8_t*)d;
-    h->d_cells = h->d_image + im.sec1_off;
-    h->image_bytes = (int64_t)im.bytes;
-    h->cell_bytes = (g.T * g.D + 1) * 4 + (int64_t)(im.bytes - im.sec1_off);
-    h->cell_T = (int)g.T;
-    h->cell_D = g.D;
-    h->max_chunk = im.max_chunk;
-    return SD2_OK;
-}
-
 bool is_device_ptr(const void* p)
 {
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) { cudaGetLastError(); return false; }
     return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
+
+// Gives a fresh GAP4 handle its cells, from dense weights (and a mask, or NULL) in device memory.
+sd2_status pack_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask)
+{
+    const CellGeom g = cell_geometry(h->M, h->K);
+    const int64_t n_cells = g.T * g.D;
+    if (n_cells > 0x3FFFFFFF) return SD2_ERR_UNSUPPORTED;
+    const size_t dir_bytes = align256((size_t)(n_cells + 1) * 4);
+    std::vector<uint32_t> off((size_t)n_cells + 1);          // first the cells' heights, then their places
+    uint32_t* d_height = nullptr;
+    if (dev_malloc(&d_height, (size_t)n_cells * 4) != cudaSuccess) return SD2_ERR_ALLOC;
+    const unsigned grid = (unsigned)((n_cells + kPackWarps - 1) / kPackWarps);
+    pack_cells_kernel<<<grid, 32 * kPackWarps>>>(W, mask, h->M, h->K, (int)g.T, g.D, d_height, nullptr, nullptr);
+    cudaError_t e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpy(off.data(), d_height, (size_t)n_cells * 4, cudaMemcpyDeviceToHost);
+    cudaFree(d_height);
+    if (e != cudaSuccess) return SD2_ERR_CUDA;
+    uint64_t units = 0;
+    uint32_t max_run = 0;
+    for (int64_t c = 0; c < n_cells; ++c) {
+        const uint32_t n = (kCellHeaderBytes + off[(size_t)c] * 128u) / 32u;
+        off[(size_t)c] = (uint32_t)units;
+        units += n;
+        const uint32_t from = c >= kChunkCells - 1 ? off[(size_t)(c - (kChunkCells - 1))] : 0u;
+        if ((uint32_t)units - from > max_run) max_run = (uint32_t)units - from;
+    }
+    if (units > 0xFFFFFFF0ull) return SD2_ERR_UNSUPPORTED;
+    off[(size_t)n_cells] = (uint32_t)units;
+    uint8_t* image = nullptr;
+    const size_t bytes = dir_bytes + (size_t)units * 32;
+    if (dev_malloc(&image, bytes) != cudaSuccess) return SD2_ERR_ALLOC;
+    h->d_image = image;                                       // (sd2_free has it from here on)
+    h->d_cells = image + dir_bytes;
+    e = cudaMemset(image, 0, bytes);
+    if (e == cudaSuccess) e = cudaMemcpy(image, off.data(), off.size() * 4, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) {
+        pack_cells_kernel<<<grid, 32 * kPackWarps>>>(W, mask, h->M, h->K, (int)g.T, g.D, nullptr, (const uint32_t*)image, image + dir_bytes);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(0);       // W and mask may go away now
+    if (e != cudaSuccess) return SD2_ERR_CUDA;
+    h->image_bytes = (int64_t)bytes;
+    h->cell_bytes = (n_cells + 1) * 4 + (int64_t)units * 32;
+    h->cell_T = (int)g.T;
+    h->cell_D = g.D;
+    h->max_chunk = (int)(max_run * 32u);
+    return SD2_OK;
+}
+
+// The same from weights and mask of either kind of memory.  On failure the handle is freed.
+sd2_status add_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask)
+{
+    const size_t n = (size_t)(h->M * h->K);
+    uint16_t* w_dev = nullptr;
+    uint8_t* m_dev = nullptr;
+    sd2_status st = SD2_OK;
+    if (!is_device_ptr(W)) {
+        if (dev_malloc(&w_dev, n * 2) != cudaSuccess) st = SD2_ERR_ALLOC;
+        else if (cudaMemcpy(w_dev, W, n * 2, cudaMemcpyHostToDevice) != cudaSuccess) st = SD2_ERR_CUDA;
+    }
+    if (st == SD2_OK && mask && !is_device_ptr(mask)) {
+        if (dev_malloc(&m_dev, n) != cudaSuccess) st = SD2_ERR_ALLOC;
+        else if (cudaMemcpy(m_dev, mask, n, cudaMemcpyHostToDevice) != cudaSuccess) st = SD2_ERR_CUDA;
+    }
+    try {
+        if (st == SD2_OK) st = pack_cells(h, w_dev ? w_dev : W, m_dev ? m_dev : mask);
+    } catch (const std::bad_alloc&) {
+        st = SD2_ERR_ALLOC;
+    }
+    cudaFree(w_dev);
+    cudaFree(m_dev);
+    if (st != SD2_OK) {
+        cudaGetLastError();
+        sd2_free(h);
+    }
+    return st;
+}
+
 
 // ------------------------------------------------------------------ BITMASK launches
 
@@ -1287,6 +1335,7 @@ sd2_status sd2_compress(const void* weight_bf16, const uint8_t* mask, int64_t M,
     if (!weight_bf16 || !out) return SD2_ERR_INVALID_ARG;
     if (M < 1 || K < 1 || M * K > (1ll << 40)) return SD2_ERR_SHAPE;
     const uint16_t* W = (const uint16_t*)weight_bf16;
+    const uint8_t* mask_in = mask;
     uint16_t* w_tmp = nullptr;
     uint8_t* m_tmp = nullptr;
     sd2_status st = SD2_OK;
@@ -1311,7 +1360,7 @@ sd2_status sd2_compress(const void* weight_bf16, const uint8_t* mask, int64_t M,
         sd2_handle h = nullptr;
         st = upload(blob, bytes, hd, &h);
         std::free(blob);
-        if (st == SD2_OK && h->format == SD2_FORMAT_GAP4) st = add_cells(h, W, mask);
+        if (st == SD2_OK && h->format == SD2_FORMAT_GAP4) st = add_cells(h, (const uint16_t*)weight_bf16, mask_in);
         if (st == SD2_OK) *out = h;
     }
     std::free(w_tmp);
