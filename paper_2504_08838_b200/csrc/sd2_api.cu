@@ -288,7 +288,11 @@ sd2_status upload(const uint8_t* blob, int64_t bytes, const BlobHeader& hd, sd2_
     sd2_handle h = lib_alloc_fails() ? nullptr : new (std::nothrow) sd2_handle_s();
     if (!h) return SD2_ERR_ALLOC;
     void* d = nullptr;
-    if (dev_malloc(&d, (size_t)bytes) != cudaSuccess) { cudaGetLastError(); delete h; return SD2_ERR_ALLOC; }
+    // (with room behind a GAP4 blob for the heights of its cells while they are packed: an allocation of their own took
+    // longer than the packing)
+    const CellGeom cells = cell_geometry(hd.M, hd.K);
+    const size_t heights = hd.format == (uint32_t)kFormatGap4 ? (size_t)(cells.T * cells.D) * 4 : 0;
+    if (dev_malloc(&d, align256((size_t)bytes) + heights) != cudaSuccess) { cudaGetLastError(); delete h; return SD2_ERR_ALLOC; }
     if (cudaMemcpy(d, blob, (size_t)bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(d);
@@ -345,13 +349,11 @@ sd2_status pack_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask)
     if (n_cells > 0x3FFFFFFF) return SD2_ERR_UNSUPPORTED;
     const size_t dir_bytes = align256((size_t)(n_cells + 1) * 4);
     std::vector<uint32_t> off((size_t)n_cells + 1);          // first the cells' heights, then their places
-    uint32_t* d_height = nullptr;
-    if (dev_malloc(&d_height, (size_t)n_cells * 4) != cudaSuccess) return SD2_ERR_ALLOC;
+    uint32_t* d_height = (uint32_t*)(h->d_blob + align256((size_t)h->blob_bytes));
     const unsigned grid = (unsigned)((n_cells + kPackWarps - 1) / kPackWarps);
     pack_cells_kernel<<<grid, 32 * kPackWarps>>>(W, mask, h->M, h->K, (int)g.T, g.D, d_height, nullptr, nullptr);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpy(off.data(), d_height, (size_t)n_cells * 4, cudaMemcpyDeviceToHost);
-    cudaFree(d_height);
     if (e != cudaSuccess) return SD2_ERR_CUDA;
     uint64_t units = 0;
     uint32_t max_run = 0;
