@@ -570,7 +570,7 @@ __device__ __forceinline__ void publish_t_slice(int K, int N, const uint32_t* g,
 // x_src, g, u, t_out already point at the launch's first activation row.
 // `tag` != 0: x_src / g / u point at tagged 32-bit words (see stage_linear_tagged); row n's words carry
 // tag | tagb[n].
-// Panels of four and eight rows go two rows at a time: both rows are fetched into their own linear
+// Panels of four rows go two rows at a time: both rows are fetched into their own linear
 // buffer (xlin holds two, `xlin_row` elements apart), then one scatter writes the packed words.
 // (Panels of two keep one buffer and take a pass per row: the second buffer would come out of the
 // weight ring, which costs them more than the extra pass.)
