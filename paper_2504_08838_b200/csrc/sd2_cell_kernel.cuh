@@ -15,10 +15,11 @@
 //              eight (twice eight) activation rows the B operand, so the expanded weights never pass through shared
 //              memory.  At the end of a tile a warp leaves its 16 x N partial sums in shared memory and goes on.
 //   2 finishers: one takes the tiles this CTA finishes, one those it sends, each in order.  They add a tile's partial sums
-//              up in one fixed order (so a row's result depends neither on the launch nor on N).  The sums for the other
-//              CTA travel as asynchronous stores that count bytes on its mbarrier.  (When the consumer that brought a
-//              tile's last contribution finished it, with flags and fences, it was away for 2400 to 7000 cycles per
-//              tile: 80 us for 48 rows of an 8192 x 2048 matrix.)
+//              up in one fixed order (so a row's result depends neither on the launch nor on how many rows are with it, as
+//              long as they go over cells; the strips add up in another order).  The sums for the other CTA travel as
+//              asynchronous stores that count bytes on its mbarrier.  (When the consumer that brought a tile's last
+//              contribution finished it, with flags and fences, it was away for 2400 to 7000 cycles per tile: 80 us for 48
+//              rows of an 8192 x 2048 matrix.)
 //   1 producer: one bulk asynchronous copy per chunk (13 KB at 50 % density) into the group's own ring slots.  Copies of
 //              13 KB reach 7 TB/s with 118 KB in flight per SM, 6.5 TB/s with 52 KB; copies of single cells of 2.7 KB
 //              1.6 TB/s from one thread (measured).  Nothing waits for a stage boundary: while the previous stage
@@ -31,8 +32,8 @@
 // What bounds it: HBM for large matrices (15 slots per clock and SM at 50 % density against 33 that twelve warps expand, 29
 // for sixteen rows); between stages some 2.8 us: from the last output to the barrier's release 1.2, to the activations 0.6, to
 // the first cell 0.9.  One launch with its start and its last sums is 8 us at least, and launches of a stream overlap there.
-// Against the strips, which gather row by row (us): 5 rows of 1531 x 3001 18.5 -> 8.3, 48 rows of 8192 x 2048 111 -> 24, two
-// blocks of 2048/512/8192 for 8 rows 230 -> 68, a block of 3072/1024/8192 for 16 rows 342 -> 59.
+// Against the strips, which gather row by row (us): 5 rows of 1531 x 3001 18.5 -> 8.3, 48 rows of 8192 x 2048 111 -> 25, two
+// blocks of 2048/512/8192 for 8 rows 230 -> 68, a block of 3072/1024/8192 for 16 rows 342 -> 61.
 //
 // Every wait (ring barriers, counters, grid barrier) is bounded by a cycle budget: when it runs out the CTA raises the
 // error word and winds down instead of hanging.
@@ -56,7 +57,7 @@ constexpr int kRecvSlots = 8;               // sums from the other CTA that wait
 constexpr int kPairSlots = 8;               // gate tiles whose results wait for the up tile's
 constexpr int kPanelRows = 16;              // activation rows of a launch of several stages, at most
 constexpr int kWidePanelRows = 32;          // ... of a single stage: a cell is expanded once for all of them (us, in panels of
-                                            // 16 / of 32: 24 rows of 8192 x 2048 at 50 % 19.5 / 12.0, 48 rows 29.3 / 24.0)
+                                            // 16 / of 32: 24 rows of 8192 x 2048 at 50 % 19.5 / 12.5, 48 rows 29.3 / 25.3)
 // A warp's contribution to a tile: for every eight activation rows 16 x 8 fp32, the activation row fastest.  A lane's
 // fragment goes there in 8-byte stores and a finisher reads 16 bytes a lane, both without bank conflicts.
 constexpr int kPartRowBytes = 32;
@@ -299,11 +300,19 @@ __device__ __forceinline__ uint32_t byte_times_128(uint32_t p, uint32_t c)
     return d;
 }
 
+// d = A B, from zero
 __device__ __forceinline__ void mma_rows(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
 {
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%10,%10,%10};"
+        : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(0.f));
+}
+// d += s, two sums to an instruction
+__device__ __forceinline__ void add_rows(float (&d)[4], const float (&s)[4])
+{
+    asm("{\n\t.reg .b64 p, q;\n\tmov.b64 p, {%0, %1};\n\tmov.b64 q, {%4, %5};\n\tadd.rn.f32x2 p, p, q;\n\tmov.b64 {%0, %1}, p;\n\t"
+        "mov.b64 p, {%2, %3};\n\tmov.b64 q, {%6, %7};\n\tadd.rn.f32x2 p, p, q;\n\tmov.b64 {%2, %3}, p;\n\t}"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "f"(s[0]), "f"(s[1]), "f"(s[2]), "f"(s[3]));
 }
 
 // One unit of a row: its four pairs' words, zero where a pair has none.  nib: the unit's mask bits; at: shared address of
@@ -325,16 +334,18 @@ __device__ __forceinline__ void load_pairs(uint32_t nib, uint32_t& at, uint32_t 
     at = byte_times_128<SGN, 3>(upto, at);
 }
 
-// Sets of sums per eight activation rows: two keep two chains of mma in flight where one or two column tiles would not.
-__host__ __device__ constexpr int sum_sets(int NR) { return NR <= 16 ? 2 : 1; }
-
 // One cell: eight mma steps for each eight activation rows.  m: the lane's mask; lo, hi: shared addresses of the first
 // words of its rows g and g + 8; xo[h]: of the first eight activations of panel row g + 8 h.
+// Every mma starts from zero and its sums are added up in fp32, pair by pair: the tensor core truncates the sum that it
+// carries on, so chains of mma drift towards zero.  Relative error of a row of 2048 at 50 % density against 64 bits: chains over
+// a warp's cells 9.4e-8 (of one set of sums for 32 activation rows 15.2e-8), chains of a cell 7.5e-8, single steps 6.8e-8, which
+// is what the strips' fused multiply-adds have; at 11008 columns 14.9e-8, 8.7e-8, 8.2e-8 (strips 8.9e-8).  The order of the
+// sums is that of every instance, so a row has the same sums in every panel.
 template <int NR>
 __device__ __forceinline__ void multiply_cell(uint32_t m, uint32_t lo, uint32_t hi, const uint32_t (&xo)[NR / 8], uint32_t xd,
-                                              float (&c)[NR / 8 * sum_sets(NR)][4])
+                                              float (&c)[NR / 8][4])
 {
-    constexpr int kSets = sum_sets(NR);
+    float two[NR / 8][4], four[NR / 8][4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         uint32_t a[4], b[4];
@@ -343,8 +354,21 @@ __device__ __forceinline__ void multiply_cell(uint32_t m, uint32_t lo, uint32_t 
 #pragma unroll
         for (int h = 0; h < NR / 8; ++h) {
             const uint4 x = lds_v4(xo[h] + xd + 64u * u);
-            mma_rows(c[kSets * h], a[0], b[0], a[1], b[1], x.x, x.y);
-            mma_rows(c[kSets * h + kSets - 1], a[2], b[2], a[3], b[3], x.z, x.w);
+            float s[4], t[4];
+            mma_rows(s, a[0], b[0], a[1], b[1], x.x, x.y);
+            mma_rows(t, a[2], b[2], a[3], b[3], x.z, x.w);
+            add_rows(s, t);
+            float (&to)[4] = u < 2 ? two[h] : four[h];
+            if (u & 1) {
+                add_rows(to, s);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) to[k] = s[k];
+            }
+            if (u == 3) {
+                add_rows(two[h], four[h]);
+                add_rows(c[h], two[h]);
+            }
         }
     }
 }
@@ -949,10 +973,9 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                 const int step = deal.split ? kCellWarps : kChunkCells;
                 int q = grp - gb;                                // the group's first turn
                 if (q < 0) q += kCellGroups;
-                constexpr int kSets = sum_sets(NR);
-                float acc[NR / 8 * kSets][4];
+                float acc[NR / 8][4];
 #pragma unroll
-                for (int m = 0; m < NR / 8 * kSets; ++m)
+                for (int m = 0; m < NR / 8; ++m)
 #pragma unroll
                     for (int k = 0; k < 4; ++k) acc[m][k] = 0.f;
                 for (int turn = deal.split ? 0 : q; turn < (deal.split ? 1 : deal.turns) && !failed; turn += kCellGroups) {
@@ -995,15 +1018,11 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                                            entry * (kSlotBytes / kChunkCells) + 8u * lane;       // (row g, activation rows 2 t and 2 t + 1)
 #pragma unroll
                         for (int h = 0; h < NR / 8; ++h) {
-                            float* s0 = acc[kSets * h];
-                            if (kSets == 2)
-#pragma unroll
-                                for (int k = 0; k < 4; ++k) s0[k] += acc[kSets * h + kSets - 1][k];
-                            *(float2*)(p + 512 * h) = make_float2(s0[0], s0[1]);
-                            *(float2*)(p + 512 * h + 256) = make_float2(s0[2], s0[3]);
+                            *(float2*)(p + 512 * h) = make_float2(acc[h][0], acc[h][1]);
+                            *(float2*)(p + 512 * h + 256) = make_float2(acc[h][2], acc[h][3]);
                         }
 #pragma unroll
-                        for (int m = 0; m < NR / 8 * kSets; ++m)
+                        for (int m = 0; m < NR / 8; ++m)
 #pragma unroll
                             for (int k = 0; k < 4; ++k) acc[m][k] = 0.f;
                         __syncwarp();
