@@ -961,6 +961,8 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                 if constexpr (FOLD) {
                     if (norm && !fold_norm(xr, a.fold[MAXS == 1 ? 0 : s], x + (size_t)a.n0 * K, a.n0, xb, pub, sh->red, sync, wc, ctid)) break;
                 }
+                // (the next stage's rows come here by bulk copies, which do not see these stores in the order of `left` alone)
+                fence_async_smem();
                 if (!sync(wc, lane)) break;
             }
             const uint32_t C = (uint32_t)(Dr < kChunkCells ? Dr : kChunkCells);
