@@ -334,11 +334,25 @@ sd2_status upload(const uint8_t* blob, int64_t bytes, const BlobHeader& hd, sd2_
     return SD2_OK;
 }
 
-bool is_device_ptr(const void* p)
+MemoryPlace place_of(const void* p, int* owner)
 {
     cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) { cudaGetLastError(); return false; }
-    return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) { cudaGetLastError(); return kPlaceHost; }
+    *owner = a.device;
+    return a.type == cudaMemoryTypeManaged ? kPlaceManaged : a.type == cudaMemoryTypeDevice ? kPlaceDevice : kPlaceHost;
+}
+
+bool is_device_ptr(const void* p)
+{
+    int owner = 0;
+    return place_of(p, &owner) != kPlaceHost;
+}
+
+bool kernel_reads(const void* p, size_t size, int device)
+{
+    int owner = -1;
+    const MemoryPlace place = place_of(p, &owner);
+    return readable_in_place(place, owner, device, p, size);
 }
 
 // Gives a fresh GAP4 handle its cells, from dense weights (and a mask, or NULL) in device memory.
@@ -387,18 +401,18 @@ sd2_status pack_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask)
     return SD2_OK;
 }
 
-// The same from weights and mask of either kind of memory.  On failure the handle is freed.
+// The same from weights and mask in host memory or where the handle's GPU can read them.  On failure the handle is freed.
 sd2_status add_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask)
 {
     const size_t n = (size_t)(h->M * h->K);
     uint16_t* w_dev = nullptr;
     uint8_t* m_dev = nullptr;
     sd2_status st = SD2_OK;
-    if (!is_device_ptr(W)) {
+    if (!kernel_reads(W, sizeof *W, h->device)) {
         if (dev_malloc(&w_dev, n * 2) != cudaSuccess) st = SD2_ERR_ALLOC;
         else if (cudaMemcpy(w_dev, W, n * 2, cudaMemcpyHostToDevice) != cudaSuccess) st = SD2_ERR_CUDA;
     }
-    if (st == SD2_OK && mask && !is_device_ptr(mask)) {
+    if (st == SD2_OK && mask && !kernel_reads(mask, sizeof *mask, h->device)) {
         if (dev_malloc(&m_dev, n) != cudaSuccess) st = SD2_ERR_ALLOC;
         else if (cudaMemcpy(m_dev, mask, n, cudaMemcpyHostToDevice) != cudaSuccess) st = SD2_ERR_CUDA;
     }
@@ -1337,7 +1351,7 @@ sd2_status sd2_compress(const void* weight_bf16, const uint8_t* mask, int64_t M,
     if (!weight_bf16 || !out) return SD2_ERR_INVALID_ARG;
     if (M < 1 || K < 1 || M * K > (1ll << 40)) return SD2_ERR_SHAPE;
     const uint16_t* W = (const uint16_t*)weight_bf16;
-    const uint8_t* mask_in = mask;
+    const uint8_t* const mask_in = mask;
     uint16_t* w_tmp = nullptr;
     uint8_t* m_tmp = nullptr;
     sd2_status st = SD2_OK;
@@ -1362,7 +1376,9 @@ sd2_status sd2_compress(const void* weight_bf16, const uint8_t* mask, int64_t M,
         sd2_handle h = nullptr;
         st = upload(blob, bytes, hd, &h);
         std::free(blob);
-        if (st == SD2_OK && h->format == SD2_FORMAT_GAP4) st = add_cells(h, (const uint16_t*)weight_bf16, mask_in);
+        if (st == SD2_OK && h->format == SD2_FORMAT_GAP4)    // (from the host's copies of what lies on another GPU)
+            st = add_cells(h, kernel_reads(weight_bf16, sizeof *W, h->device) ? (const uint16_t*)weight_bf16 : W,
+                           mask_in && kernel_reads(mask_in, sizeof *mask_in, h->device) ? mask_in : mask);
         if (st == SD2_OK) *out = h;
     }
     std::free(w_tmp);

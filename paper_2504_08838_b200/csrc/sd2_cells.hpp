@@ -45,6 +45,15 @@ struct CellGeom {
 // cells of share r (0, 1) of a tile
 SD2_HD int share_cells(int D, int r) { return r == 0 ? (D + 1) / 2 : D / 2; }
 
+// Whether a kernel on GPU `device` can read weights or a mask (elements of `size` bytes) where they lie.  Memory of another GPU
+// is out of its reach unless peer access happens to be on, and host memory takes a copy of its own.
+enum MemoryPlace { kPlaceHost, kPlaceDevice, kPlaceManaged };
+inline bool readable_in_place(MemoryPlace place, int owner, int device, const void* p, size_t size)
+{
+    if ((uintptr_t)p % size != 0) return false;
+    return place == kPlaceManaged || (place == kPlaceDevice && owner == device);
+}
+
 inline CellGeom cell_geometry(int64_t M, int64_t K)
 {
     CellGeom g;
