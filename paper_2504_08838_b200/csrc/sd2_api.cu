@@ -1391,9 +1391,13 @@ sd2_status sd2_load_blob(const void* blob, int64_t blob_bytes, sd2_handle* out)
     if (!blob || !out) return SD2_ERR_INVALID_ARG;
     BlobHeader hd;
     if (check_header((const uint8_t*)blob, blob_bytes, hd, true) != 0) return SD2_ERR_CORRUPT;
-    // full structural validation before anything reaches a kernel
+    // M and K are believed once the directory bears them out (the checksum does not cover the header); full structural
+    // validation before anything reaches a kernel
     uint16_t* dense = nullptr;
-    if (hd.format == (uint32_t)kFormatGap4 && !(dense = (uint16_t*)lib_malloc((size_t)(hd.M * hd.K) * 2))) return SD2_ERR_ALLOC;
+    if (hd.format == (uint32_t)kFormatGap4) {
+        if (check_gap4(hd, (const uint8_t*)blob) != 0) return SD2_ERR_CORRUPT;
+        if (!(dense = (uint16_t*)lib_malloc((size_t)(hd.M * hd.K) * 2))) return SD2_ERR_ALLOC;
+    }
     int rc;
     try {
         rc = unpack_any(hd, (const uint8_t*)blob, dense);

@@ -533,31 +533,43 @@ inline PackResult pack_gap4(const uint16_t* W, const uint8_t* mask, int64_t M, i
     return r;
 }
 
-// Validates every tile record (so that a kernel can trust it) and, if `dense` is given, decodes.
-inline int unpack_gap4(const BlobHeader& h, const uint8_t* blob, uint16_t* dense)
+// Validates the header against the tile directory.  What passes has a tile record in the blob for every 32 / S rows, so M and K
+// are no larger than the blob can answer for.
+inline int check_gap4(const BlobHeader& h, const uint8_t* blob)
 {
     const int64_t M = h.M, K = h.K;
     if (h.pairing > 1) return -6;
+    if (M > 0x7FFFFFF0ll || K > 0x7FFFFFF0ll) return -6;
     const Gap4Geom g = gap4_geometry(M, K, h.pairing == 1);
     if (g.S == 0 || h.strips != (uint32_t)g.S || h.strip_cols != (uint32_t)g.B || h.overlap != (uint32_t)g.V) return -6;
-    const int S = g.S, B = g.B, R = g.R, V = g.V;
+    const int R = g.R;
     const int64_t T = (M + R - 1) / R;
-    if (h.pairing > 1 || (h.pairing == 1 && ((M & 1) || R < 2))) return -6;
+    if (h.pairing == 1 && ((M & 1) || R < 2)) return -6;
     if (h.n_tiles != (uint64_t)T || h.sec_bytes[0] != (uint64_t)(T + 1) * 4 || h.sec_bytes[2] != 0) return -6;
     if (h.sec_bytes[1] % 16) return -6;
     const uint32_t* toff = (const uint32_t*)(blob + h.sec_off[0]);
+    if (toff[0] != 0 || toff[T] != h.sec_bytes[1] / 16) return -6;
+    for (int64_t t = 0; t < T; ++t)
+        if (toff[t + 1] <= toff[t] || (uint64_t)(toff[t + 1] - toff[t]) * 16 < (uint64_t)gap4_tile_header_bytes(R)) return -6;
+    return 0;
+}
+
+// Validates every tile record (so that a kernel can trust it) and, if `dense` is given, decodes.
+inline int unpack_gap4(const BlobHeader& h, const uint8_t* blob, uint16_t* dense)
+{
+    if (check_gap4(h, blob) != 0) return -6;
+    const int64_t M = h.M, K = h.K;
+    const Gap4Geom g = gap4_geometry(M, K, h.pairing == 1);
+    const int S = g.S, B = g.B, R = g.R, V = g.V;
+    const int64_t T = (M + R - 1) / R;
+    const uint32_t* toff = (const uint32_t*)(blob + h.sec_off[0]);
     const uint8_t* tiles = blob + h.sec_off[1];
-    const uint64_t units = h.sec_bytes[1] / 16;
     const int hdr = gap4_tile_header_bytes(R);
     const int window = B + 2 * V;   // columns a lane may touch, before the slack
-    if (toff[0] != 0 || toff[T] != units) return -6;
-    for (int64_t t = 0; t < T; ++t)
-        if (toff[t + 1] <= toff[t]) return -6;
     std::vector<uint8_t> seen((size_t)M, 0);
     int bad = 0;
     int64_t chunks = 0;
     for (int64_t t = 0; t < T; ++t) {  // row ids: a permutation of 0..M-1, checked serially
-        if ((uint64_t)(toff[t + 1] - toff[t]) * 16 < (uint64_t)hdr) return -6;
         const uint32_t* rows = (const uint32_t*)(tiles + (size_t)toff[t] * 16 + 144);
         for (int rr = 0; rr < R; ++rr) {
             const int64_t i = t * R + rr;

@@ -313,3 +313,16 @@ def test_a_failed_blob_allocation_is_reported_not_fatal(fmt):
         sd2.sd2_debug_fail_allocations(0, 0)
     dense, _ = sd2.sd2_unpack_host(sd2.sd2_pack_host(W, mask, fmt))      # and the next call works
     assert np.array_equal(dense, oracle.roundtrip_ref(W, mask))
+
+
+@pytest.mark.parametrize("fmt", FORMATS + [sd2.SD2_FORMAT_GAP4_MMA])
+@pytest.mark.parametrize("field,value", [(24, 1 << 40), (24, 1 << 62), (32, 1 << 40), (32, 300 * 1024), (24, 4000)])
+def test_loading_believes_no_size_that_the_directory_does_not_bear_out(fmt, field, value):
+    # M and K (bytes 24 and 32 of the header, which the checksum does not cover) decide how much is allocated
+    W, mask = _case(4343, 40, 300, 0.5)
+    blob = bytearray(sd2.sd2_pack_host(W, mask, fmt))
+    assert struct.unpack_from("<qq", blob, 24) == (40, 300)
+    struct.pack_into("<q", blob, field, value)
+    with pytest.raises(sd2.Sd2Error) as e:
+        sd2.sd2_load_blob(bytes(blob))
+    assert e.value.status == sd2.SD2_ERR_CORRUPT
