@@ -401,7 +401,9 @@ sd2_status pack_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask)
     return SD2_OK;
 }
 
-// The same from weights and mask in host memory or where the handle's GPU can read them.  On failure the handle is freed.
+// The same from weights and mask in host memory or where the handle's GPU can read them.  Cells are a second image of the
+// weights: where there is no memory for them, or for the dense weights that they are made from, the handle goes without, and
+// calls of several rows read its strips.  On any other failure the handle is freed.
 sd2_status add_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask)
 {
     const size_t n = (size_t)(h->M * h->K);
@@ -423,10 +425,10 @@ sd2_status add_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask)
     }
     cudaFree(w_dev);
     cudaFree(m_dev);
-    if (st != SD2_OK) {
-        cudaGetLastError();
-        sd2_free(h);
-    }
+    if (st == SD2_OK) return st;
+    cudaGetLastError();
+    if (st == SD2_ERR_ALLOC || st == SD2_ERR_UNSUPPORTED) return SD2_OK;
+    sd2_free(h);
     return st;
 }
 
@@ -1396,11 +1398,16 @@ sd2_status sd2_load_blob(const void* blob, int64_t blob_bytes, sd2_handle* out)
     uint16_t* dense = nullptr;
     if (hd.format == (uint32_t)kFormatGap4) {
         if (check_gap4(hd, (const uint8_t*)blob) != 0) return SD2_ERR_CORRUPT;
-        if (!(dense = (uint16_t*)lib_malloc((size_t)(hd.M * hd.K) * 2))) return SD2_ERR_ALLOC;
+        dense = (uint16_t*)lib_malloc((size_t)(hd.M * hd.K) * 2);     // for the cells; NULL: the handle goes without
     }
     int rc;
     try {
         rc = unpack_any(hd, (const uint8_t*)blob, dense);
+        if (rc != 0 && dense) {              // a column that two lanes share has a sum in strips, but no dense form
+            std::free(dense);
+            dense = nullptr;
+            rc = unpack_any(hd, (const uint8_t*)blob, nullptr);
+        }
     } catch (const std::bad_alloc&) {
         std::free(dense);
         return SD2_ERR_ALLOC;
@@ -2105,9 +2112,15 @@ sd2_status sd2_drafter_create(const sd2_handle* h, int32_t L, int64_t n_max, sd2
         d->n_cstages = bld.n;
         d->first_cstage = cstages[0];
         d->cell_needs = bld.needs;
-        ok = dev_malloc((void**)&d->d_cstages, sizeof(CStage) * (size_t)bld.n) == cudaSuccess &&
-             cudaMemcpy(d->d_cstages, cstages.data(), sizeof(CStage) * (size_t)bld.n, cudaMemcpyHostToDevice) == cudaSuccess &&
-             dev_malloc((void**)&d->d_cbar, kDrafterWordsBytes) == cudaSuccess && cudaMemset(d->d_cbar, 0, kDrafterWordsBytes) == cudaSuccess;
+        if (dev_malloc((void**)&d->d_cstages, sizeof(CStage) * (size_t)bld.n) == cudaSuccess && dev_malloc((void**)&d->d_cbar, kDrafterWordsBytes) == cudaSuccess) {
+            ok = cudaMemcpy(d->d_cstages, cstages.data(), sizeof(CStage) * (size_t)bld.n, cudaMemcpyHostToDevice) == cudaSuccess &&
+                 cudaMemset(d->d_cbar, 0, kDrafterWordsBytes) == cudaSuccess;
+        } else {                                             // no memory: steps of several rows go through the strips
+            cudaGetLastError();
+            cudaFree(d->d_cstages);
+            d->d_cstages = nullptr;
+            d->n_cstages = 0;
+        }
     }
     auto drop = [&]() {
         cudaGetLastError();

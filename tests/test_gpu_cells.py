@@ -14,6 +14,7 @@ from oracle import decoder_oracle as do
 from oracle import oracle
 from paper_2504_08838_b200 import binding as sd2
 from paper_2504_08838_b200 import synth
+from tests.test_gpu_parity import _read_u16
 
 pytestmark = pytest.mark.gpu
 
@@ -90,6 +91,76 @@ def test_panels_add_up_like_each_other_and_as_well_as_single_rows(M, K):
     # a tenth more is left to the draw of 64 M sums
     assert error(panels) <= 1.1 * error(rows(1))
     sd2.sd2_free(h)
+
+
+def test_without_memory_for_cells_the_strips_answer():
+    M, K = 600, 2048
+    W = synth.normal_bf16(31, (M, K), 0.02)
+    mask = synth.bernoulli_mask(32, (M, K), 0.5)
+    x = synth.normal_bf16(33, (8, K), 1.0)
+    blob = sd2.sd2_pack_host(W, mask, sd2.SD2_FORMAT_GAP4, sd2.SD2_DTYPE_F32)
+    sd2.sd2_free(sd2.sd2_load_blob(blob))                               # device set-up is done before counting
+    free0 = torch.cuda.mem_get_info()[0]
+
+    def product(h, n):                                                  # all rows in calls of n
+        y = torch.full((8, M), float("nan"), dtype=torch.float32, device="cuda")
+        for i in range(0, 8, n):
+            sd2.sd2_spmm(h, dev(x[i:i + n]), y[i:i + n])
+        sd2.sd2_stream_check()
+        return y
+
+    def served_by_strips(make, skip):
+        sd2.sd2_debug_fail_allocations(skip, 1)
+        try:
+            h = make()
+        except sd2.Sd2Error as e:
+            assert e.status == sd2.SD2_ERR_ALLOC
+            assert torch.cuda.mem_get_info()[0] == free0
+            return "refused"
+        finally:
+            sd2.sd2_debug_fail_allocations(0, 0)
+        y = product(h, 8)
+        linear_close(y.double().cpu().numpy(), W, mask, x, True)
+        same = torch.equal(y, product(h, 1))                            # the strips add up alike for any number of rows
+        sd2.sd2_free(h)
+        assert torch.cuda.mem_get_info()[0] == free0
+        return "strips" if same else "cells"
+
+    # (packing, the handle, its strips; then the dense weights on the device, the mask there, the cells)
+    compress = lambda: sd2.sd2_compress(W, mask, sd2.SD2_FORMAT_GAP4, sd2.SD2_DTYPE_F32)
+    assert [served_by_strips(compress, k) for k in range(7)] == ["refused"] * 3 + ["strips"] * 3 + ["cells"]
+    # (the dense weights on the host; the handle, its strips; the dense weights on the device, the cells)
+    load = lambda: sd2.sd2_load_blob(blob, sd2.SD2_DTYPE_F32)
+    assert [served_by_strips(load, k) for k in range(6)] == ["strips", "refused", "refused", "strips", "strips", "cells"]
+
+
+def test_a_drafter_without_memory_for_its_cells_steps_through_the_strips():
+    shape = synth.DrafterShape("small", 512, 128, 2048, 1)
+    lin = synth.make_block(5, 0, shape, 0.5)
+    hs = [sd2.sd2_compress(W, m, sd2.SD2_FORMAT_GAP4, sd2.SD2_DTYPE_F32 if i == 6 else sd2.SD2_DTYPE_BF16) for i, (W, m) in enumerate(lin)]
+    x = dev(synth.make_activations(5, 0, 0, 8, shape.hidden))
+    kinds = []
+    for skip in range(24):
+        sd2.sd2_debug_fail_allocations(skip, 1)
+        try:
+            d = sd2.sd2_drafter_create([hs], n_max=8)
+        except sd2.Sd2Error as e:
+            assert e.status == sd2.SD2_ERR_ALLOC
+            kinds.append("refused")
+            continue
+        finally:
+            sd2.sd2_debug_fail_allocations(0, 0)
+        y = torch.full((8, shape.hidden), float("nan"), dtype=torch.float32, device="cuda")
+        sd2.sd2_drafter_step(d, x, y)
+        sd2.sd2_stream_check()
+        t = _read_u16(sd2.sd2_drafter_buffers(d, 0)[6], 8 * shape.inter).reshape(8, -1)
+        linear_close(y.double().cpu().numpy(), lin[6][0], lin[6][1], t, True)
+        kinds.append("strips" if sd2.sd2_drafter_query(d, 8)["panel_rows"] == 4 else "cells")
+        sd2.sd2_drafter_free(d)
+    n = kinds.index("strips")
+    assert kinds == ["refused"] * n + ["strips"] * 2 + ["cells"] * (22 - n)
+    for h in hs:
+        sd2.sd2_free(h)
 
 
 @pytest.mark.parametrize("hidden,kv,inter,N", [(160, 48, 9600, 5),      # more gate tiles per cluster than wait for their up tiles at once
