@@ -242,6 +242,18 @@ sd2_status ensure_device(int* dev_out)
     return SD2_OK;
 }
 
+// The SM count alone, for calls that need nothing else of a device: they allocate nothing, so that the first call of a program may
+// be one that is captured.
+sd2_status device_sms(int* sms)
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return SD2_ERR_CUDA;
+    }
+    return SD2_OK;
+}
+
 int resolve_format(const sd2_options* opt, int64_t M, int64_t K)
 {
     int f = opt ? opt->format : SD2_FORMAT_AUTO;
@@ -1561,14 +1573,14 @@ sd2_status sd2_attention_decode(const void* q, const void* k_cache, const void* 
         return SD2_ERR_SHAPE;
     if (head_dim > 128 || T > kAttnMaxT) return SD2_ERR_UNSUPPORTED;
     if (N == 0) return SD2_OK;
-    int dev = 0;
-    const sd2_status st = ensure_device(&dev);
+    int sms = 0;
+    const sd2_status st = device_sms(&sms);
     if (st != SD2_OK) return st;
     const bool pow2 = (head_dim & (head_dim - 1)) == 0;
     const int vec = (pow2 && head_dim >= 8 && ((((uintptr_t)k_cache) | ((uintptr_t)v_cache)) & 15) == 0) ? 1 : 0;
     if (vec)
         return launch_attention<false>((uint16_t*)q, nullptr, nullptr, (uint16_t*)k_cache, (uint16_t*)v_cache, (uint16_t*)out, N, heads_q,
-                                       heads_kv, head_dim, T, T_max, RopeTable{}, g_dev[dev].sms, (cudaStream_t)cuda_stream);
+                                       heads_kv, head_dim, T, T_max, RopeTable{}, sms, (cudaStream_t)cuda_stream);
     launch_pdl(attention_any_kernel, (unsigned)(N * heads_q), kAttnThreads, (size_t)T * 4, (cudaStream_t)cuda_stream,
                (const uint16_t*)q, (const uint16_t*)k_cache, (const uint16_t*)v_cache, (uint16_t*)out, (int)heads_q, (int)heads_kv,
                (int)head_dim, (int)T, (int)T_max);
@@ -1586,15 +1598,15 @@ sd2_status sd2_rope_attention(void* q, const void* k, const void* v, void* k_cac
         return SD2_ERR_SHAPE;
     if (head_dim > 128 || pos + 1 > kAttnMaxT) return SD2_ERR_UNSUPPORTED;
     if (N == 0) return SD2_OK;
-    int dev = 0;
-    const sd2_status st = ensure_device(&dev);
+    int sms = 0;
+    const sd2_status st = device_sms(&sms);
     if (st != SD2_OK) return st;
     const bool pow2 = (head_dim & (head_dim - 1)) == 0;
     const int vec = (pow2 && head_dim >= 8 && ((((uintptr_t)k_cache) | ((uintptr_t)v_cache)) & 15) == 0) ? 1 : 0;
     if (vec)
         return launch_attention<true>((uint16_t*)q, (const uint16_t*)k, (const uint16_t*)v, (uint16_t*)k_cache, (uint16_t*)v_cache,
                                       (uint16_t*)out, N, heads_q, heads_kv, head_dim, pos, T_max, rope_table(head_dim, pos, theta),
-                                      g_dev[dev].sms, (cudaStream_t)cuda_stream);
+                                      sms, (cudaStream_t)cuda_stream);
     launch_pdl(rope_attention_any_kernel, (unsigned)(N * heads_q), kAttnThreads, (size_t)(pos + 1) * 4, (cudaStream_t)cuda_stream,
                (uint16_t*)q, (const uint16_t*)k, (const uint16_t*)v, (uint16_t*)k_cache, (uint16_t*)v_cache, (uint16_t*)out, (int)heads_q,
                (int)heads_kv, (int)head_dim, (int)pos, (int)T_max, rope_table(head_dim, pos, theta));

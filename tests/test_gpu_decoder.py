@@ -6,6 +6,10 @@ outputs: |y - ref| <= 2^-8 |ref| (the rounding of the output) + an absolute slac
 fp32 arithmetic on the operation's scale; fp32 logits: the 1e-3 * sum |w x| rule of the linears.
 """
 
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -279,6 +283,39 @@ def test_decoder_block_over_cells(shape, Hq, Hkv, N):
         assert torch.equal(y, first)
     for h in hs:
         sd2.sd2_free(h)
+
+
+FIRST_CALL = """
+import torch
+from paper_2504_08838_b200 import binding as sd2
+gen = torch.Generator(device="cuda")
+gen.manual_seed(1)
+normal = lambda *shape: torch.empty(shape, dtype=torch.bfloat16, device="cuda").normal_(0.0, 1.0, generator=gen)
+q, k, v, kc, vc = normal(1, 256), normal(1, 128), normal(1, 128), normal(1, 300, 128), normal(1, 300, 128)
+out, out2 = torch.zeros_like(q), torch.zeros_like(q)
+calls = {
+    "attention": lambda o: sd2.sd2_attention_decode(q, kc, vc, o, 4, 2, 290),
+    "rope": lambda o: sd2.sd2_rope_attention(q.clone(), k, v, kc, vc, o, 4, 2, 290, 1e4),
+}
+run = calls["%s"]
+sd2.lib()
+torch.cuda.synchronize()
+graph = torch.cuda.CUDAGraph()
+with torch.cuda.graph(graph):
+    run(out)
+graph.replay()
+run(out2)
+torch.cuda.synchronize()
+assert torch.isfinite(out).all() and out.abs().max() > 0 and torch.equal(out, out2)
+print("same")
+"""
+
+
+@pytest.mark.parametrize("call", ["attention", "rope"])
+def test_the_first_call_of_a_program_may_be_captured(call):
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", FIRST_CALL % call], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and r.stdout.strip() == "same", r.stderr[-2000:]
 
 
 def test_argument_checks_of_the_glue_calls():
