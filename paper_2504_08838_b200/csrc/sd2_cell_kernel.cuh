@@ -153,6 +153,15 @@ __device__ __forceinline__ bool wait_phase_warp(uint32_t bar, uint32_t parity, c
     return true;
 }
 
+// Until the copies counted by a phase have landed.  For a warp that is about to leave: the abort flag does not cut this short,
+// since memory that copies are on their way to must not be given up.
+__device__ __forceinline__ void wait_landed(uint32_t bar, uint32_t parity, long long budget)
+{
+    const long long t0 = clock64();
+    while (!__all_sync(0xFFFFFFFFu, mbar_try_wait(bar, parity)))
+        if (__any_sync(0xFFFFFFFFu, clock64() - t0 > budget)) return;
+}
+
 // Until the shared counter at p has reached `want` (one warp, together).
 __device__ __forceinline__ bool wait_count(const unsigned int* p, unsigned int want, const WaitCtx& w)
 {
@@ -762,16 +771,12 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                 next_slot ^= (at ^ (slot + 1 == NS ? (at ^ 16u) & 16u : at + 1u)) << (8 * grp);
             }
         }
-        if (!ok && lane == 0) {
-            // give the copies already issued time to land before this CTA's memory is released
-            for (int g = 0; g < kCellGroups; ++g)
-                for (uint32_t u = 0; u < NS; ++u) {
-                    const uint32_t at = next_slot >> (8 * g) & 0xFFu;
-                    const long long t0 = clock64();
-                    while (!mbar_try_wait(full0 + 8 * (g * kGroupSlots + u), (at >> 4) ^ (u < (at & 15u) ? 1u : 0u)))
-                        if (clock64() - t0 > wc.budget) break;
-                }
-        }
+        // (consumers that gave up have left chunks on their way; where they did not, these have landed)
+        for (int g = 0; g < kCellGroups; ++g)
+            for (uint32_t u = 0; u < NS; ++u) {
+                const uint32_t at = next_slot >> (8 * g) & 0xFFu;
+                wait_landed(full0 + 8 * (g * kGroupSlots + u), (at >> 4) ^ (u < (at & 15u) ? 1u : 0u), wc.budget);
+            }
         __syncwarp();
         asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
     } else if (warp == kServiceWarp) {
@@ -783,23 +788,19 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&sh->dfull));
         };
-        bool landed = true;
+        int started = -1;                                        // the last stage whose rows are on their way
         for (int s = 0; s < a.n_stages; ++s) {
             uint32_t bytes;
-            if (!start_rows(s, 0, bytes)) { landed = false; break; }
+            if (!start_rows(s, 0, bytes)) break;
             if (lane == 0) {
                 if (bytes) mbar_expect_tx(xfull, bytes);
                 else mbar_arrive(xfull);
             }
-            landed = !bytes;
+            started = s;
             if (s == 0) fetch_stage(0);
             if (s + 1 < a.n_stages) fetch_stage(s + 1);
-            else if (bytes) landed = wait_phase_warp(xfull, (uint32_t)s & 1u, wc);
         }
-        if (!landed) {                                           // a wait ran out: give the rows in flight time to land
-            const long long t0 = clock64();
-            while (clock64() - t0 < 200000) {}
-        }
+        wait_landed(xfull, (uint32_t)started & 1u, wc.budget);   // (stage 0's at least; no phase is begun before the one before it is through)
         __syncwarp();
         asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
     } else if (warp > kServiceWarp) {
@@ -817,12 +818,16 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         uint32_t ps = 0, use = 0, rs = 0, ru = 0;                // slot of partial sums and its use, the same for exchanged sums
         bool ok = true;
         uint32_t bytes;
+        int started = 0;                                         // (the sending finisher) the last stage whose rows it has started
         if (!own) start_rows(0, 1, bytes);
         asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
         const uint32_t dfull = smem_u32(&sh->dfull);
         bool ready = wait_phase_warp(dfull, 0u, wc);
         for (int s = 0; s < a.n_stages && ok && ready; ++s) {
-            if (!own && s > 0 && !start_rows(s, 1, bytes)) break;
+            if (!own && s > 0) {
+                if (!start_rows(s, 1, bytes)) break;
+                started = s;
+            }
             const CStage& st = sh->stage[s & 1];
             const int D = st.D, Dr = share_cells(D, rank), C = Dr < kChunkCells ? Dr : kChunkCells;
             const int n_parts = Dr > kSplitCells ? kCellGroups : 1;
@@ -913,6 +918,7 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
             if (s + 1 < a.n_stages) ready = wait_phase_warp(dfull, (uint32_t)(s + 1) & 1u, wc);
             if (lane == 0) mbar_arrive(smem_u32(&sh->left));
         }
+        if (!own) wait_landed(smem_u32(&sh->xfull), (uint32_t)started & 1u, wc.budget);
     } else {
         // ---------------------------------------------------------------------- consumers
         const int ctid = tid;
