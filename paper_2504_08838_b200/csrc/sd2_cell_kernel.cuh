@@ -765,6 +765,8 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                 const int grp = __shfl_sync(0xFFFFFFFFu, from_grp, k);
                 const uint32_t at = next_slot >> (8 * grp) & 0xFFu, slot = at & 15u;
                 const uint32_t s = (uint32_t)(grp * kGroupSlots) + slot, dst = ring + ((uint32_t)grp * NS + slot) * (uint32_t)a.chunk_bytes;
+                // (slots are not given back before the consumers are let go, which the budget of a wait is not meant for)
+                if (at == 0u) pdl_wait();        // (a group's first slot that has to be given back)
                 if (!wait_phase_warp(empty0 + 8 * s, at >> 4, wc)) { ok = false; break; }
                 if (hinted) bulk_chunk(dst, from + (size_t)o0 * 32, bytes, full0 + 8 * s, lane == k, policy);
                 else bulk_chunk(dst, from + (size_t)o0 * 32, bytes, full0 + 8 * s, lane == k);

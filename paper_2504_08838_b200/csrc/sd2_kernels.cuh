@@ -188,7 +188,8 @@ using SArgs = SArgsT<kMaxStagesInline>;
 // Launches without a grid barrier are programmatic dependents (launch_pdl): a CTA may start when every CTA of the kernel
 // before it in the stream has started, and gets its SM as soon as that one's CTA leaves.  pdl_wait holds it until the kernel
 // before is through and its results are visible; what a launch reads before (weights, their directories, its arguments) no
-// kernel writes.  Every CTA waits before it ends, so the launches of a stream still finish in order.  Without this the
+// kernel writes.  A producer that streams weights before it waits for room only after pdl_wait, so that no bounded wait counts
+// the time that the kernel before still takes.  Every CTA waits before it ends, so the launches of a stream still finish in order.  Without this the
 // boundary between two launches cost 2 us and more: it is most of a small call.
 __device__ __forceinline__ void pdl_let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
@@ -881,6 +882,8 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const __grid_
                     }
                     // no room: wait until the oldest tile in the ring has been consumed, and take
                     // along every further tile that is already done
+                    // (none is consumed before the consumers are let go, which the wait's budget is not meant for)
+                    if (oldest == 0) pdl_wait();
                     if (!wait_phase(empty0 + 8 * (oldest % kSlots), (oldest / kSlots) & 1u, wc)) { ok = false; break; }
                     ++oldest;
                     while (oldest != q) {   // each lane looks at one of the next 32 tiles; the leading run of done ones goes

@@ -224,6 +224,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) mma_kernel(const MmaArgs a, co
                 const uint32_t o1 = j + a.batch >= 32 ? end32 : __shfl_sync(0xFFFFFFFFu, mine, (j + a.batch) & 31);
                 const int q = (i0 + j) / a.batch;
                 const int slot = q % a.n_slots;
+                if (q == a.n_slots) pdl_wait();              // (slots are given back by warps that have waited, too)
                 if (lane == 0 && !wait_phase(smem_u32(&sh->empty[slot]), ((uint32_t)(q / a.n_slots) & 1u) ^ 1u, wc)) ok = false;
                 ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
                 if (!ok) break;

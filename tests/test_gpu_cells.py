@@ -239,3 +239,37 @@ def test_launches_that_overlap_still_run_in_order(N):
     for _ in range(5):
         assert torch.equal(chain(False), want)
     sd2.sd2_free(h)
+
+
+@pytest.mark.parametrize("fmt,N", [(sd2.SD2_FORMAT_GAP4, 1), (sd2.SD2_FORMAT_GAP4, 8), (sd2.SD2_FORMAT_GAP4_MMA, 16)])
+def test_wait_budgets_do_not_count_the_kernel_before(fmt, N, monkeypatch):
+    # weights that do not fit the ring, behind a launch of one CTA that leaves the other SMs free and takes longer than the
+    # shortest budget: the launch streams weights ahead until its ring is full, and must then wait without a limit
+    K_slow = 1 << 24
+    slow = sd2.sd2_compress(np.full((1, K_slow), 0x3C00, np.uint16), np.ones((1, K_slow), np.uint8), sd2.SD2_FORMAT_BITMASK)
+    xs = torch.ones((1, K_slow), dtype=torch.bfloat16, device="cuda")
+    ys = torch.zeros((1, 1), dtype=torch.bfloat16, device="cuda")
+    M, K = 8192, 4096
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(3)
+    w = torch.empty((M, K), dtype=torch.bfloat16, device="cuda").normal_(0.0, 0.02, generator=gen)
+    h = sd2.sd2_compress(w, (torch.rand((M, K), device="cuda", generator=gen) < 0.5).to(torch.uint8), fmt)
+    x = torch.empty((N, K), dtype=torch.bfloat16, device="cuda").normal_(0.0, 1.0, generator=gen)
+    want, y = torch.zeros((N, M), dtype=torch.bfloat16, device="cuda"), torch.zeros((N, M), dtype=torch.bfloat16, device="cuda")
+    sd2.sd2_spmm(h, x, want)
+    sd2.sd2_spmm(slow, xs, ys)
+    start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    torch.cuda.synchronize()
+    start.record()
+    sd2.sd2_spmm(slow, xs, ys)
+    end.record()
+    torch.cuda.synchronize()
+    assert start.elapsed_time(end) > 3.0
+    monkeypatch.setenv("SD2_WAIT_MS", "1")
+    sd2.sd2_spmm(slow, xs, ys)
+    sd2.sd2_spmm(h, x, y)
+    sd2.sd2_stream_check()
+    close = {"rtol": 0.01, "atol": 0.01} if fmt == sd2.SD2_FORMAT_GAP4_MMA else {"rtol": 0.0, "atol": 0.0}   # (that one's order of sums varies)
+    torch.testing.assert_close(y, want, **close)
+    for hh in (slow, h):
+        sd2.sd2_free(hh)
