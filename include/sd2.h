@@ -135,12 +135,16 @@ sd2_status sd2_free(sd2_handle h);
 /* ---- the hot path -------------------------------------------------------------------- */
 
 /* Y = X (W.*mask)^T.   X: device bf16 [N*K].   Y: device [N*M], bf16 or fp32 per the
- * handle's y_dtype.  N = 0 is a no-op; more than 8 rows (GAP4: fewer where the staged rows of a
- * wide layer would crowd the weight ring out of shared memory, e.g. 4 for K = 8192) are processed
- * in panels of at most that many rows of X (the weight is re-read for each panel).  cuda_stream is a
- * cudaStream_t (NULL = default stream).  X and Y need only their natural alignment; all
- * activations are expected to be finite (a filler entry of the GAP4 format multiplies +0 by
- * the activation of a masked-out column). */
+ * handle's y_dtype.  N = 0 is a no-op; any other N is served in panels of rows, each of which reads
+ * the weight once: GAP4 up to 32 rows (fewer where the staged rows of a wide layer would crowd the
+ * weights out of shared memory; up to 4 on a handle without cells), BITMASK up to 8, GAP4_MMA up
+ * to 64.  cuda_stream is a cudaStream_t (NULL = default stream).  X and Y need only their natural
+ * alignment.  One row, and two or three of some weights, are summed in another order than more of
+ * them: the same activation row may come out differently rounded.  Among calls of four rows and
+ * more on a handle with cells its sums are the same whatever goes with it.
+ * Activations are expected to be finite.  What an infinite or undefined one does to outputs that
+ * drop the weight for it depends on the path: nothing over cells; NaN where a filler entry of the
+ * strips (value +0) falls on it, and everywhere with GAP4_MMA. */
 sd2_status sd2_spmm(sd2_handle h, const void* X, void* Y, int64_t N, void* cuda_stream);
 
 /* Same-input fusion (q|k|v, gate|up): count <= 4 weights with equal K share one staged X

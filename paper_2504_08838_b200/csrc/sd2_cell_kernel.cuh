@@ -32,7 +32,7 @@
 // What bounds it: HBM for large matrices (15 slots per clock and SM at 50 % density against 33 that twelve warps expand, 29
 // for sixteen rows); between stages some 2.8 us: from the last output to the barrier's release 1.2, to the activations 0.6, to
 // the first cell 0.9.  One launch with its start and its last sums is 8 us at least, and launches of a stream overlap there.
-// Against the strips, which gather row by row (us): 5 rows of 1531 x 3001 18.5 -> 8.3, 48 rows of 8192 x 2048 111 -> 25, two
+// Against the strips, which gather row by row (us): 5 rows of 1531 x 3001 18.5 -> 8.6, 48 rows of 8192 x 2048 111 -> 26, two
 // blocks of 2048/512/8192 for 8 rows 230 -> 68, a block of 3072/1024/8192 for 16 rows 342 -> 61.
 //
 // Every wait (ring barriers, counters, grid barrier) is bounded by a cycle budget: when it runs out the CTA raises the
@@ -57,7 +57,7 @@ constexpr int kRecvSlots = 8;               // sums from the other CTA that wait
 constexpr int kPairSlots = 8;               // gate tiles whose results wait for the up tile's
 constexpr int kPanelRows = 16;              // activation rows of a launch of several stages, at most
 constexpr int kWidePanelRows = 32;          // ... of a single stage: a cell is expanded once for all of them (us, in panels of
-                                            // 16 / of 32: 24 rows of 8192 x 2048 at 50 % 19.5 / 12.5, 48 rows 29.3 / 25.3)
+                                            // 16 / of 32: 24 rows of 8192 x 2048 at 50 % 19.5 / 12.8, 48 rows 29.3 / 25.8)
 // A warp's contribution to a tile: for every eight activation rows 16 x 8 fp32, the activation row fastest.  A lane's
 // fragment goes there in 8-byte stores and a finisher reads 16 bytes a lane, both without bank conflicts.
 constexpr int kPartRowBytes = 32;
@@ -66,7 +66,7 @@ __host__ __device__ constexpr int part_slot_bytes(int nr) { return kChunkCells *
 struct CMat {
     const uint32_t* off;           // [T * D + 1], 32-byte units into `cells`
     const unsigned char* cells;
-    void* y;                       // [N * M] (may be NULL in a gate|up stage)
+    void* y;                       // [N * M]
     int M;
     int T;
     int y_f32;                     // 1: fp32 output, 0: bf16
@@ -592,6 +592,96 @@ __device__ __forceinline__ void store_bf16(uint16_t* p, uint2 v, int rows, size_
     if (rows > 3) p[3 * ld] = (uint16_t)(v.y >> 16);
 }
 
+// ---- activations that are not finite --------------------------------------------------------
+
+// The products of an expanded cell take in the weights that were dropped, as zeros, and zero times an infinite or undefined
+// activation is NaN: it would reach every output of its row.  So the finishers keep an eye on their sums, and where a stage had
+// any that were not finite they form these again, from the kept weights alone.  (To look for such activations instead is a pass
+// over every stage's rows.)  What it costs where all is finite (us): five rows of 1531 x 3001 8.4 -> 8.6, 48 rows of 8192 x 2048
+// 25.4 -> 25.8, an eight-row step of two blocks of 2048/512/8192 67.8 -> 68.2, a block of 3072/1024/8192 for 16 rows 61.4 -> 61.5.
+// With a vote and the slow path in the loop over tiles these took 8.5, 26.4, 69.1, 61.9; a call in the loop over stages, the
+// arguments of which tie up the finishers' registers, 8.8, 26.7, 69.5, 63.5.
+
+// the largest magnitude of m, a, b; NaN if one of them is
+__device__ __forceinline__ float watch(float m, float a, float b)
+{
+    asm("max.NaN.abs.f32 %0, %0, %1, %2;" : "+f"(m) : "f"(a), "f"(b));
+    return m;
+}
+
+// The sum over the Dr cells of a share of a tile for one weight row and one activation row, kept weight by kept weight.  off: the
+// share's directory entries; x: the staged activations, in either CTA.  A kept zero counts as dropped.
+__device__ __forceinline__ float sum_kept(float sum, const uint32_t* off, const unsigned char* cells, int Dr, int row, const unsigned char* x)
+{
+    const int second = row >> 3;
+#pragma unroll 1
+    for (int d = 0; d < Dr; ++d) {
+        const unsigned char* cell = cells + (size_t)__ldg(off + d) * 32;
+        const int H = (int)((__ldg(off + d + 1) - __ldg(off + d)) * 32u - kCellHeaderBytes) / 128;
+        const uint32_t* words = (const uint32_t*)(cell + kCellHeaderBytes);
+#pragma unroll 1
+        for (int t = 0; t < 4; ++t) {
+            const int owner = 4 * (row & 7) + t;
+            const int column = second ? (__ldg(cell + 128 + owner) & 0x7F) >> 2 : owner;
+            int at = second ? H - 1 : 0;
+#pragma unroll 1
+            for (uint32_t left = __ldg((const uint32_t*)cell + owner) >> (16 * second) & 0xFFFFu; left; left &= left - 1u, at += second ? -1 : 1) {
+                const int e = __ffs((int)left) - 1;
+                const uint32_t w = __ldg(words + 32 * at + column);
+                const uint32_t xv = *(const uint32_t*)(x + 2 * (d * kCellCols + 32 * (e >> 2) + 8 * t + 2 * (e & 3)));
+                if (w & 0x7FFFu) sum = fmaf(bf16_lo(w), bf16_lo(xv), sum);
+                if (w & 0x7FFF0000u) sum = fmaf(bf16_hi(w), bf16_hi(xv), sum);
+            }
+        }
+    }
+    return sum;
+}
+
+// Every tile that this CTA has finished in the stage, once more: outputs that are not finite are replaced.  One warp, with the
+// lanes that stored them.  rows: this CTA's staged activations; the other CTA's stay where they are until the grid barrier, or
+// its end, for which this warp is still missing.
+__device__ __forceinline__ void repair_stage(const CStage& st, int rank, int cluster, int clusters, void* y_last, const unsigned char* rows, int N, int n0)
+{
+    const int lane = threadIdx.x & 31, D = st.D;
+    const bool alone = D == 1;
+    TileRuns runs(cluster, clusters, st.rot, st.tiles_div, st.tiles_rem);
+    int mat, t0, nt;
+    while (runs.next(st.pair, st.count, st.mat[0].T, st.mat[1].T, st.mat[2].T, mat, t0, nt)) {
+        const CMat& md = st.mat[mat];
+        unsigned char* y = (unsigned char*)(y_last && mat == 0 ? y_last : md.y);
+        for (int j = alone ? 0 : rank; j < nt; j += alone ? 1 : 2) {
+            const int row = (t0 + j) * kTileRows + (lane >> 1);
+#pragma unroll 1
+            for (int n = (lane & 1) * 4; n < N && row < md.M; n += (n & 3) == 3 ? 5 : 1) {
+                const size_t at = (size_t)(n0 + n) * md.M + row;
+                float* f = (float*)y + at;
+                uint16_t* b = (uint16_t*)y + at;
+                if (md.y_f32 ? !isfinite(*f) : (*b & 0x7F80u) == 0x7F80u) {
+                    float sum = 0.f;
+#pragma unroll 1
+                    for (int r = 0; r < 2; ++r) {
+                        uint64_t x;
+                        asm("mapa.u64 %0, %1, %2;" : "=l"(x) : "l"((uint64_t)rows), "r"(r));
+                        const int Dr = share_cells(D, r);
+                        const size_t first = (r ? (size_t)md.T * share_cells(D, 0) : 0) + (size_t)(t0 + j) * Dr;
+                        sum = sum_kept(sum, md.off + first, md.cells, Dr, lane >> 1, (const unsigned char*)x + (size_t)n * (2 * Dr * kCellCols + 64));
+                    }
+                    if (md.y_f32) *f = sum;
+                    else *b = (uint16_t)bf16_pair(sum, 0.f);
+                }
+                if (st.pair && mat == 1 && st.t_out) st.t_out[at] = (uint16_t)silu_mul_pair(((const uint16_t*)st.mat[0].y)[at], *b);
+            }
+        }
+        __syncwarp();
+    }
+}
+
+// ... out of line, for launches of one stage, which repair it on their way out
+__device__ __noinline__ void repair_call(const CStage& st, int rank, int cluster, int clusters, void* y_last, const unsigned char* rows, int N, int n0)
+{
+    repair_stage(st, rank, cluster, clusters, y_last, rows, N, n0);
+}
+
 // ---- the kernel ---------------------------------------------------------------------------
 
 template <int MAXS, int NR, bool FOLD>
@@ -672,6 +762,8 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
         __syncwarp();
         return true;
     };
+    constexpr bool kWide = NR > kPanelRows;      // (launches of one stage)
+    bool odd = false;                            // (finishers) sums of the stage were not finite
     if (warp != kProducerWarp) pdl_wait();       // (the producer streams weights already)
     if (warp == kProducerWarp) {
         // ---------------------------------------------------------------------- producer
@@ -834,6 +926,7 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
             const int D = st.D, Dr = share_cells(D, rank), C = Dr < kChunkCells ? Dr : kChunkCells;
             const int n_parts = Dr > kSplitCells ? kCellGroups : 1;
             const bool alone = D == 1, pair = st.pair != 0;
+            float seen = 0.f;                                    // largest magnitude of the lane's sums
             TileRuns runs(cluster, clusters, st.rot, st.tiles_div, st.tiles_rem);
             int mat, t0, nt;
             while (ok && runs.next(pair, st.count, st.mat[0].T, st.mat[1].T, st.mat[2].T, mat, t0, nt)) {
@@ -886,6 +979,8 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                         if ((rs + 1) % (kRecvSlots / 2) == 0 && lane == 0) mbar_arrive_remote(peer_credit + 8 * half);
                         if (++rs == kRecvSlots) { rs = 0; ++ru; }
                     }
+#pragma unroll
+                    for (int h = 0; h < NR / 8; ++h) seen = watch(watch(seen, r[h][0], r[h][1]), r[h][2], r[h][3]);
                     const int row = (t0 + j) * kTileRows + r0;
                     if (row >= M) continue;
 #pragma unroll
@@ -899,7 +994,7 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                             continue;
                         }
                         const uint2 b = make_uint2(bf16_pair(r[h][0], r[h][1]), bf16_pair(r[h][2], r[h][3]));
-                        if (y) store_bf16((uint16_t*)y + at, b, rows, (size_t)M);
+                        store_bf16((uint16_t*)y + at, b, rows, (size_t)M);
                         if (pair) {
                             // gate tiles of a run wait for the up tiles of the run that follows, written and read by the same lane
                             uint2* gt = &sh->gate[j % kPairSlots][h][lane];
@@ -911,7 +1006,11 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
             }
             __syncwarp();
             // (a CTA without a tile must not be counted before the stage has begun: the barrier counts arrivals, not stages)
-            if (own && ok && s + 1 < a.n_stages) ok = wait_phase_warp(smem_u32(&sh->xfull), (uint32_t)s & 1u, wc);
+            odd = own && ok && __any_sync(0xFFFFFFFFu, !(seen < INFINITY));
+            if (own && ok && ((odd && !kWide) || s + 1 < a.n_stages)) ok = wait_phase_warp(smem_u32(&sh->xfull), (uint32_t)s & 1u, wc);
+            if (!kWide && __builtin_expect(odd && ok, 0))
+                repair_stage(st, rank, cluster, clusters, s == a.n_stages - 1 ? a.y_out : nullptr, smem + xoff, N, a.n0);
+            __syncwarp();
             // this CTA's outputs are visible before the grid barrier counts it (the warp's stores are ordered before this
             // lane's release by the __syncwarp above)
             if (own && ok && s + 1 < a.n_stages && lane == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.gbar) : "memory");
@@ -1062,6 +1161,9 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
     }
 
     // ---- exit: every role comes here; nobody leaves while the other CTA may still write to this one's memory
+    __syncwarp();
+    if (kWide && odd && wait_phase_warp(smem_u32(&sh->xfull), 0u, wc))
+        repair_call(sh->stage[0], rank, cluster, clusters, a.y_out, smem + xoff, N, a.n0);
     __syncwarp();
     asm volatile("barrier.cluster.arrive.release;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire;" ::: "memory");

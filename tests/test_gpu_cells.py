@@ -93,6 +93,57 @@ def test_panels_add_up_like_each_other_and_as_well_as_single_rows(M, K):
     sd2.sd2_free(h)
 
 
+@pytest.mark.parametrize("M,K,N", [(40, 100, 4), (77, 3001, 5), (300, 2048, 8), (50, 8200, 16), (200, 2048, 24)])
+def test_dropped_weights_take_no_part_whatever_the_activations(M, K, N):
+    # infinite and undefined activations reach the rows that keep a weight for them, and no others
+    W = synth.normal_bf16(M + K, (M, K), 0.02)
+    mask = synth.bernoulli_mask(M + K + 1, (M, K), 0.5)
+    x = synth.normal_bf16(M + K + 2, (N, K), 1.0)
+    special = [(0, K // 2, 0xFF80), (1, 5, 0x7F80), (1, K - 2, 0x7F80), (2, K - 1, 0x7FC0), (N - 1, 0, 0x7F80), (N - 1, 1, 0xFF80)]
+    finite = x.copy()
+    for n, k, bits in special:
+        x[n, k] = bits
+        finite[n, k] = 0
+    h = sd2.sd2_compress(W, mask, sd2.SD2_FORMAT_GAP4, sd2.SD2_DTYPE_F32)
+    y = torch.full((N, M), 7.0, dtype=torch.float32, device="cuda")
+    sd2.sd2_spmm(h, dev(x), y)
+    sd2.sd2_stream_check()
+    got = y.double().cpu().numpy()
+    extra = np.zeros((N, M))
+    with np.errstate(invalid="ignore"):
+        for n, k, _ in special:
+            extra[n] += np.where(mask[:, k] != 0, values(W[:, k]) * values(x[n:n + 1, k]), 0.0)
+    assert np.array_equal(got[~np.isfinite(extra)], extra[~np.isfinite(extra)], equal_nan=True)
+    ref, S = oracle.masked_linear(W, mask, finite)
+    left = np.isfinite(extra)
+    assert left[:3].any() and not left[:3].all() and np.all(np.abs(got - ref)[left] <= 1e-5 * S[left])   # (one sum after the other)
+    sd2.sd2_free(h)
+
+
+def test_dropped_weights_take_no_part_in_a_normalised_row():
+    # an infinite column becomes NaN in the norm that is folded into staging: as far as BITMASK handles carry it, and no further
+    shape, N, pos = synth.DrafterShape("tiny", 256, 64, 1024, 1), 6, 3
+    lin = synth.make_block(2, 0, shape, 0.5)
+    x = synth.normal_bf16(70, (N, shape.hidden), 1.0)
+    x[2, 100] = 0x7F80
+    ones = dev(np.full(shape.hidden, 0x3F80, np.uint16))
+    seen = []
+    for fmt in (sd2.SD2_FORMAT_BITMASK, sd2.SD2_FORMAT_GAP4):
+        hs = [sd2.sd2_compress(W, m, fmt) for W, m in lin]
+        kc, vc = (torch.zeros((N, pos + 1, shape.kv), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        ws = torch.zeros(sd2.sd2_decoder_workspace_bytes(hs, N) // 2, dtype=torch.bfloat16, device="cuda")
+        y = torch.zeros((N, shape.hidden), dtype=torch.bfloat16, device="cuda")
+        sd2.sd2_decoder_block_step(hs, ones, ones, dev(x), y, kc, vc, 8, 2, pos, 1e-5, 1e4, ws)
+        sd2.sd2_stream_check()
+        seen.append((vc[:, pos].isnan(), y.isnan()))
+        for h in hs:
+            sd2.sd2_free(h)
+    for a, b in zip(*seen):
+        assert torch.equal(a, b)
+    nans = seen[1][0]
+    assert nans[2].any() and not nans[2].all() and not nans[[0, 1, 3, 4, 5]].any()
+
+
 def test_without_memory_for_cells_the_strips_answer():
     M, K = 600, 2048
     W = synth.normal_bf16(31, (M, K), 0.02)
