@@ -373,6 +373,14 @@ def time_full_step(torch, sd2, args, shape, handles, harr, N, stream):
                     "second norm folded into gate|up's staging pass); the last residual"}
 
 
+def kernel_name(sd2, path, rows):
+    """The kernel a launch of ``rows`` activation rows on this path is."""
+    return {sd2.SD2_PATH_BITMASK: "bitmask_kernel<%d>" % min(8, 1 << (rows - 1).bit_length()),
+            sd2.SD2_PATH_STRIPS: "stream_kernel<%d>" % min(4, 1 << (rows - 1).bit_length()),
+            sd2.SD2_PATH_CELLS: "cell_kernel<%d>" % (8 if rows <= 8 else 16 if rows <= 16 else 32),
+            sd2.SD2_PATH_MMA: "mma_kernel"}[path]
+
+
 def run_ours(args):
     import torch
     import torch.distributed as dist
@@ -628,6 +636,8 @@ def run_ours(args):
         t_launch = ms_step * 1e-3 / launches_per_step              # seconds per launch (one panel of the step)
         kept = facts["kept_weights"]
         streamed = facts["streamed_bytes"]                         # what one launch reads of the compressed drafter
+        in_cells = [sd2.sd2_spmm_query(h, 16) for hs in handles for h in hs]
+        over_cells = all(f["path"] == sd2.SD2_PATH_CELLS for f in in_cells) and streamed == sum(f["streamed_bytes"] for f in in_cells)
         useful = 2.5 * kept                                        # a bf16 value and a 4-bit column code per kept weight
         bitmask_eq = 2.0 * kept + dense_elems / 8.0                # values + one mask bit per position
         traffic = ncu_traffic_ratio()
@@ -638,7 +648,7 @@ def run_ours(args):
             "useful_is": "2.5 B per kept weight (bf16 value + 4-bit column code); padding = tile headers, filler entries, alignment",
             "achieved_streamed": streamed / t_launch / 1e9, "frac_streamed": streamed / t_launch / 1e9 / peak,
             "achieved_bitmask_equivalent": bitmask_eq / t_launch / 1e9, "frac_bitmask_equivalent": bitmask_eq / t_launch / 1e9 / peak,
-            "kernel": "stream_kernel<%d>" % (1 << max(0, (min(N, facts["panel_rows"]) - 1).bit_length())),
+            "kernel": kernel_name(sd2, sd2.SD2_PATH_CELLS if over_cells else sd2.SD2_PATH_STRIPS, min(N, facts["panel_rows"])),
             "launches_per_step": launches_per_step, "panel_rows": facts["panel_rows"],
             "avg_launch_us": t_launch * 1e6,
             "traffic": (traffic["dram_bytes_per_algorithmic_byte"] * streamed) if traffic else None,
@@ -771,8 +781,10 @@ def run_sweep(args):
 
                     us_s = time_graph_us(torch, sparse_all, 20) / len(hs)
                     best = us_s if best is None else min(best, us_s)
+                    facts = sd2.sd2_spmm_query(hs[0], N)
+                    read = facts["streamed_bytes"] * facts["launches"]        # every panel of rows reads the weights
                     print("| %dx%d | %d | %.2f | %s | %.3f | %.2f | %.0f | %.2f | %.2f |" % (
-                        M, K, N, sp, path, hs[0].compressed_bytes / max(hs[0].nnz, 1), us_s, hs[0].compressed_bytes / us_s / 1e3,
+                        M, K, N, sp, path, facts["streamed_bytes"] / max(hs[0].nnz, 1), us_s, read / us_s / 1e3,
                         us_d, us_d / us_s), flush=True)
                 cross[N].append((sp, best, us_d))
             for hs in loaded.values():
@@ -840,7 +852,8 @@ def run_config1(args):
         parity = {"max_abs_err_over_S": float((np.abs(y - Yr) / np.maximum(S, 1e-300)).max()), "bound_over_S": 2.0 ** -8 + 2e-3,
                   "against": "oracle, copy 0"}
     peak, peak_src = measured_peak()
-    comp = sum(h.compressed_bytes for h in hs) / R
+    facts = sd2.sd2_spmm_query(hs[0], N)
+    comp = sum(sd2.sd2_spmm_query(h, N)["streamed_bytes"] for h in hs) / R * facts["launches"]    # every panel reads the weights
     kept = sum(h.nnz for h in hs) / R
     line = {
         "metric": "single sparse linear us per launch at N=%d" % N, "value": cold, "unit": "us/launch", "n_gpus": 1,
@@ -851,13 +864,13 @@ def run_config1(args):
                                % (M, K, round(100 * args.sparsity), N, K, R, comp * R / 1e6),
                    "timing": "CUDA events around replays of a CUDA graph holding one sd2_spmm per copy"},
         "clocks": clocks, "gpu_launches": max(3, args.steps // R) * R,
-        "l2_warm_us_per_launch": warm, "l2_warm_note": "same copy every launch: the 4.7 MB matrix stays in L2; not an HBM figure",
+        "l2_warm_us_per_launch": warm, "l2_warm_note": "same copy every launch: the %.1f MB matrix stays in L2; not an HBM figure" % (comp / 1e6),
         "roofline": {"bound": "hbm", "achieved": 2.5 * kept / cold / 1e3, "peak": peak, "unit": "GB/s",
                      "frac": 2.5 * kept / cold / 1e3 / peak, "peak_source": peak_src, "useful_bytes": 2.5 * kept,
                      "padding_bytes": comp - 2.5 * kept, "achieved_streamed": comp / cold / 1e3,
-                     "frac_streamed": comp / cold / 1e3 / peak, "kernel": "stream_kernel<%d>" % max(1, min(8, 1 << max(0, (N - 1).bit_length()))),
+                     "frac_streamed": comp / cold / 1e3 / peak, "kernel": kernel_name(sd2, facts["path"], min(N, facts["panel_rows"])),
                      "avg_launch_us": cold, "traffic": None,
-                     "note": "a 4.7 MB launch lasts a few microseconds: launch and pipeline-fill latency, not bandwidth, bound it"},
+                     "note": "a %.1f MB launch lasts a few microseconds: launch and pipeline-fill latency, not bandwidth, bound it" % (comp / 1e6)},
         "cublas_dense": {"cold_us_per_launch": dcold, "l2_warm_us_per_launch": dwarm} if dense else None,
         "parity": parity,
     }

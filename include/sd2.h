@@ -147,6 +147,12 @@ sd2_status sd2_free(sd2_handle h);
  * strips (value +0) falls on it, and everywhere with GAP4_MMA. */
 sd2_status sd2_spmm(sd2_handle h, const void* X, void* Y, int64_t N, void* cuda_stream);
 
+/* What sd2_spmm does with N rows (N >= 1) on this handle, out[5]: out[0] kernel launches (one per panel of
+ * rows), out[1] rows of the widest panel, out[2] device bytes the handle owns, out[3] bytes of
+ * compressed weights one launch reads, out[4] SD2_PATH_*. */
+enum { SD2_PATH_BITMASK = 0, SD2_PATH_STRIPS = 1, SD2_PATH_CELLS = 2, SD2_PATH_MMA = 3 };
+sd2_status sd2_spmm_query(sd2_handle h, int64_t N, int64_t* out);
+
 /* Same-input fusion (q|k|v, gate|up): count <= 4 weights with equal K share one staged X
  * and one launch.  Y[i] is device [N*M_i] with handle i's y_dtype. */
 sd2_status sd2_spmm_fused(const sd2_handle* h, int32_t count, const void* X, void* const* Y,

@@ -20,10 +20,11 @@ SD2_ERR_INVALID_ARG, SD2_ERR_SHAPE, SD2_ERR_ALLOC, SD2_ERR_CUDA = -1, -2, -3, -4
 SD2_ERR_UNSUPPORTED, SD2_ERR_CORRUPT, SD2_ERR_TIMEOUT = -5, -6, -7
 SD2_FORMAT_AUTO, SD2_FORMAT_BITMASK, SD2_FORMAT_GAP4, SD2_FORMAT_GAP4_PAIRED, SD2_FORMAT_GAP4_MMA = 0, 1, 2, 3, 4
 SD2_DTYPE_BF16, SD2_DTYPE_F32 = 0, 1
+SD2_PATH_BITMASK, SD2_PATH_STRIPS, SD2_PATH_CELLS, SD2_PATH_MMA = 0, 1, 2, 3
 
 EXPORTS = [
     "sd2_pack_host", "sd2_unpack_host", "sd2_blob_free", "sd2_compress", "sd2_load_blob",
-    "sd2_decompress", "sd2_info", "sd2_free", "sd2_spmm", "sd2_spmm_fused", "sd2_block_step",
+    "sd2_decompress", "sd2_info", "sd2_free", "sd2_spmm", "sd2_spmm_query", "sd2_spmm_fused", "sd2_block_step",
     "sd2_block_workspace_bytes", "sd2_block_workspace_layout", "sd2_status_string", "sd2_stream_check",
     "sd2_drafter_create", "sd2_drafter_step", "sd2_drafter_buffers", "sd2_drafter_free",
     "sd2_block_step_static", "sd2_selftest_timeout", "sd2_drafter_query",
@@ -68,6 +69,7 @@ def lib():
             "sd2_info": [p, pi64, pi64, pi64, pi64, pi32],
             "sd2_free": [p],
             "sd2_spmm": [p, p, p, i64, p],
+            "sd2_spmm_query": [p, i64, pi64],
             "sd2_spmm_fused": [pp, i32, p, pp, i64, p],
             "sd2_block_step": [pp, p, p, i64, p, p],
             "sd2_block_workspace_bytes": [pp, i64, pi64],
@@ -252,6 +254,13 @@ def sd2_spmm(h: Handle, X, Y, stream=None):
     """``X``: device bf16 ``[N, K]``; ``Y``: device ``[N, M]`` (bf16 or fp32 per the handle)."""
     N = X.shape[0] if X.dim() == 2 else 1
     _check(lib().sd2_spmm(h.raw, _ptr(X), _ptr(Y), N, _stream(stream)), "sd2_spmm")
+
+
+def sd2_spmm_query(h: Handle, N: int) -> dict:
+    """Launches per call of N rows, widest panel, device bytes of the handle, weight bytes read per launch, SD2_PATH_*."""
+    out = (ctypes.c_int64 * 5)()
+    _check(lib().sd2_spmm_query(h.raw, N, out), "sd2_spmm_query")
+    return dict(zip(("launches", "panel_rows", "device_bytes", "streamed_bytes", "path"), (int(v) for v in out)))
 
 
 def _handle_array(hs):

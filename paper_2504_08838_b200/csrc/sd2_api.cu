@@ -38,7 +38,8 @@ struct sd2_handle_s {
     // GAP4: the same weights as cells (sd2_cells.hpp), for panels of rows (d_image NULL: none)
     uint8_t* d_image;
     const unsigned char* d_cells;
-    int64_t image_bytes, cell_bytes;   // device bytes; what a launch reads of them
+    int64_t cell_bytes;        // what a launch reads of them
+    int64_t device_bytes;      // all that the handle owns
     int cell_T, cell_D, max_chunk;
     // GAP4_MMA: fp32 partial sums [64][rows padded to 128] followed by one arrival count per row panel,
     // all zero between launches (the CTA that completes a panel writes Y and clears them)
@@ -330,6 +331,7 @@ sd2_status upload(const uint8_t* blob, int64_t bytes, const BlobHeader& hd, sd2_
     h->d_image = nullptr;
     h->d_partial = nullptr;
     h->partial_bytes = 0;
+    h->device_bytes = (int64_t)(align256((size_t)bytes) + heights);
     if (h->format == SD2_FORMAT_GAP4_MMA) {
         const int64_t panels = (hd.M + kMmaBlockRows - 1) / kMmaBlockRows;
         h->partial_bytes = (int64_t)kMmaMaxRows * panels * kMmaBlockRows * 4 + panels * 4;
@@ -337,6 +339,7 @@ sd2_status upload(const uint8_t* blob, int64_t bytes, const BlobHeader& hd, sd2_
         if (dev_malloc(&pp, (size_t)h->partial_bytes) != cudaSuccess) { cudaGetLastError(); cudaFree(d); delete h; return SD2_ERR_ALLOC; }
         if (cudaMemset(pp, 0, (size_t)h->partial_bytes) != cudaSuccess) { cudaGetLastError(); cudaFree(pp); cudaFree(d); delete h; return SD2_ERR_CUDA; }
         h->d_partial = (float*)pp;
+        h->device_bytes += h->partial_bytes;
     }
     {
         std::lock_guard<std::mutex> lk(g_mu);
@@ -405,7 +408,7 @@ sd2_status pack_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask)
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);       // W and mask may go away now
     if (e != cudaSuccess) return SD2_ERR_CUDA;
-    h->image_bytes = (int64_t)bytes;
+    h->device_bytes += (int64_t)bytes;
     h->cell_bytes = (n_cells + 1) * 4 + (int64_t)units * 32;
     h->cell_T = (int)g.T;
     h->cell_D = g.D;
@@ -1846,6 +1849,36 @@ sd2_status sd2_spmm(sd2_handle h, const void* X, void* Y, int64_t N, void* cuda_
     return run_group(&h, 1, (const uint16_t*)X, nullptr, nullptr, nullptr, ys, N, false, (cudaStream_t)cuda_stream);
 }
 
+sd2_status sd2_spmm_query(sd2_handle h, int64_t N, int64_t* out)
+{
+    if (!live(h) || !out) return SD2_ERR_INVALID_ARG;
+    if (N < 1) return SD2_ERR_SHAPE;
+    int path = SD2_PATH_STRIPS, cap = 0;
+    if (h->format == SD2_FORMAT_BITMASK) {
+        path = SD2_PATH_BITMASK;
+        cap = 8;
+    } else if (h->format == SD2_FORMAT_GAP4_MMA) {
+        path = SD2_PATH_MMA;
+        cap = kMmaMaxRows;
+    } else if (use_cells(&h, 1, N)) {
+        path = SD2_PATH_CELLS;
+        CellNeeds needs;
+        needs.add(h);
+        cap = widest_cell_panel(needs, kWidePanelRows);
+    } else {
+        ProgramNeeds needs;
+        needs.add(&h, 1);
+        cap = widest_panel(needs.xs_need, needs.K_max, needs.max_tile);
+    }
+    if (cap == 0) return SD2_ERR_UNSUPPORTED;
+    out[0] = (N + cap - 1) / cap;
+    out[1] = cap;
+    out[2] = h->device_bytes;
+    out[3] = path == SD2_PATH_CELLS ? h->cell_bytes : h->compressed_bytes;
+    out[4] = path;
+    return SD2_OK;
+}
+
 sd2_status sd2_spmm_fused(const sd2_handle* h, int32_t count, const void* X, void* const* Y, int64_t N,
                           void* cuda_stream)
 {
@@ -2227,7 +2260,7 @@ sd2_status sd2_drafter_query(sd2_drafter d, int64_t N, int64_t* out)
     // what a step streams: every handle once, except that a block's gate and up are read from the
     // drafter's own paired stack where it has one
     std::vector<char> paired((size_t)d->L, 0);
-    for (sd2_handle p : d->owned) { streamed += p->compressed_bytes; owned += p->blob_bytes; }
+    for (sd2_handle p : d->owned) { streamed += p->compressed_bytes; owned += p->device_bytes; }
     owned += (int64_t)sizeof(CStage) * d->n_cstages + (d->d_cbar ? kDrafterWordsBytes : 0);
     size_t oi = 0;
     for (int b = 0; b < d->L; ++b) {
@@ -2249,7 +2282,7 @@ sd2_status sd2_drafter_query(sd2_drafter d, int64_t N, int64_t* out)
     out[1] = cap;                                                  // rows of the widest panel
     out[2] = owned + d->ws_off.back() + d->tags_bytes + (int64_t)sizeof(SStage) * d->n_stages + kDrafterWordsBytes;
     out[3] = streamed;                                             // bytes of compressed weights read per launch
-    out[4] = d->n_stages;
+    out[4] = cells ? d->n_cstages : d->n_stages;
     out[5] = kept;
     return SD2_OK;
 }

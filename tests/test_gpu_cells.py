@@ -185,6 +185,30 @@ def test_without_memory_for_cells_the_strips_answer():
     assert [served_by_strips(load, k) for k in range(6)] == ["strips", "refused", "refused", "strips", "strips", "cells"]
 
 
+def test_a_handle_tells_what_it_owns_and_what_a_call_reads():
+    M, K = 1024, 2048
+    W = synth.normal_bf16(41, (M, K), 0.02)
+    mask = synth.bernoulli_mask(42, (M, K), 0.5)
+    h = sd2.sd2_compress(W, mask, sd2.SD2_FORMAT_GAP4)
+    one, many = sd2.sd2_spmm_query(h, 1), sd2.sd2_spmm_query(h, 40)
+    assert (one["launches"], one["path"], one["streamed_bytes"]) == (1, sd2.SD2_PATH_STRIPS, h.compressed_bytes)
+    assert (many["launches"], many["panel_rows"], many["path"]) == (2, 32, sd2.SD2_PATH_CELLS)
+    assert 1.6 < many["streamed_bytes"] / (M * K) < 1.7                  # (three of four pairs have a word, at 50 %)
+    assert one["device_bytes"] == many["device_bytes"] >= h.compressed_bytes + many["streamed_bytes"]
+    sd2.sd2_debug_fail_allocations(5, 1)                                 # no memory for the cells
+    try:
+        bare = sd2.sd2_compress(W, mask, sd2.SD2_FORMAT_GAP4)
+    finally:
+        sd2.sd2_debug_fail_allocations(0, 0)
+    facts = sd2.sd2_spmm_query(bare, 40)
+    assert (facts["launches"], facts["panel_rows"], facts["path"]) == (10, 4, sd2.SD2_PATH_STRIPS)
+    assert facts["device_bytes"] <= one["device_bytes"] - many["streamed_bytes"]
+    bits, mma = sd2.sd2_compress(W, mask, sd2.SD2_FORMAT_BITMASK), sd2.sd2_compress(W, mask, sd2.SD2_FORMAT_GAP4_MMA)
+    assert [sd2.sd2_spmm_query(x, 65)[k] for x in (bits, mma) for k in ("launches", "path")] == [9, sd2.SD2_PATH_BITMASK, 2, sd2.SD2_PATH_MMA]
+    for x in (h, bare, bits, mma):
+        sd2.sd2_free(x)
+
+
 def test_a_drafter_without_memory_for_its_cells_steps_through_the_strips():
     shape = synth.DrafterShape("small", 512, 128, 2048, 1)
     lin = synth.make_block(5, 0, shape, 0.5)
