@@ -64,12 +64,17 @@ enum {
                             /* path; column strips wider than 496 are not supported).     */
                             /* The handle also keeps the weights as cells in the order of */
                             /* a tensor-core operand (about 1.3 times the strips' bytes), */
-                            /* which calls of several rows read instead.                  */
+                            /* which calls of several rows read instead; where there is   */
+                            /* no memory for them it does without.                        */
     SD2_FORMAT_GAP4_PAIRED = 3,/* as an option of sd2_pack_host / sd2_compress only: GAP4 */
                             /* whose rows 2i and 2i+1 stay next to each other in a tile   */
                             /* (for a stack that interleaves gate row i and up row i; M   */
                             /* even and at least two rows per tile, else UNSUPPORTED).    */
                             /* The blob and the handle report SD2_FORMAT_GAP4.            */
+    SD2_FORMAT_GAP4_STRIPS = 5,/* as an option only: GAP4 whose handle keeps no cells, for */
+                            /* programs of one row at a time or short of device memory    */
+                            /* (0.44 of a GAP4 handle's).  Calls of several rows read the */
+                            /* strips.  The blob and the handle report SD2_FORMAT_GAP4.   */
     SD2_FORMAT_GAP4_MMA = 4 /* for panels of N >= 16 activation rows: 128 x 128 blocks    */
                             /* whose 4-bit gaps run in the order of a tensor-core operand */
                             /* tile; sd2_spmm expands each block in shared memory and     */

@@ -259,7 +259,8 @@ int resolve_format(const sd2_options* opt, int64_t M, int64_t K)
 {
     int f = opt ? opt->format : SD2_FORMAT_AUTO;
     if (f == SD2_FORMAT_AUTO) f = gap4_geometry(M, K).S > 0 ? SD2_FORMAT_GAP4 : SD2_FORMAT_BITMASK;
-    return f;   // SD2_FORMAT_GAP4_PAIRED stays as asked: only the packer tells it from GAP4
+    // SD2_FORMAT_GAP4_PAIRED stays as asked: only the packer tells it from GAP4.  SD2_FORMAT_GAP4_STRIPS is GAP4 to the packer.
+    return f == SD2_FORMAT_GAP4_STRIPS ? (int)SD2_FORMAT_GAP4 : f;
 }
 
 sd2_status pack_any(const uint16_t* W, const uint8_t* mask, int64_t M, int64_t K, const sd2_options* opt,
@@ -1393,7 +1394,8 @@ sd2_status sd2_compress(const void* weight_bf16, const uint8_t* mask, int64_t M,
         sd2_handle h = nullptr;
         st = upload(blob, bytes, hd, &h);
         std::free(blob);
-        if (st == SD2_OK && h->format == SD2_FORMAT_GAP4)    // (from the host's copies of what lies on another GPU)
+        const bool cells = h && h->format == SD2_FORMAT_GAP4 && !(opt && opt->format == SD2_FORMAT_GAP4_STRIPS);
+        if (st == SD2_OK && cells)    // (from the host's copies of what lies on another GPU)
             st = add_cells(h, kernel_reads(weight_bf16, sizeof *W, h->device) ? (const uint16_t*)weight_bf16 : W,
                            mask_in && kernel_reads(mask_in, sizeof *mask_in, h->device) ? mask_in : mask);
         if (st == SD2_OK) *out = h;

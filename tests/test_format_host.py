@@ -315,6 +315,11 @@ def test_a_failed_blob_allocation_is_reported_not_fatal(fmt):
     assert np.array_equal(dense, oracle.roundtrip_ref(W, mask))
 
 
+def test_strips_without_cells_are_the_same_blob():
+    W, mask = _case(4444, 40, 300, 0.5)
+    assert sd2.sd2_pack_host(W, mask, sd2.SD2_FORMAT_GAP4_STRIPS) == sd2.sd2_pack_host(W, mask, sd2.SD2_FORMAT_GAP4)
+
+
 @pytest.mark.parametrize("fmt", FORMATS + [sd2.SD2_FORMAT_GAP4_MMA])
 @pytest.mark.parametrize("field,value", [(24, 1 << 40), (24, 1 << 62), (32, 1 << 40), (32, 300 * 1024), (24, 4000)])
 def test_loading_believes_no_size_that_the_directory_does_not_bear_out(fmt, field, value):

@@ -203,6 +203,15 @@ def test_a_handle_tells_what_it_owns_and_what_a_call_reads():
     facts = sd2.sd2_spmm_query(bare, 40)
     assert (facts["launches"], facts["panel_rows"], facts["path"]) == (10, 4, sd2.SD2_PATH_STRIPS)
     assert facts["device_bytes"] <= one["device_bytes"] - many["streamed_bytes"]
+    asked = sd2.sd2_compress(W, mask, sd2.SD2_FORMAT_GAP4_STRIPS)        # the same, by choice
+    assert sd2.sd2_spmm_query(asked, 40) == facts and asked.format == sd2.SD2_FORMAT_GAP4
+    y = [torch.zeros((5, M), dtype=torch.bfloat16, device="cuda") for _ in range(2)]
+    x = dev(synth.normal_bf16(43, (5, K), 1.0))
+    sd2.sd2_spmm(bare, x, y[0])
+    sd2.sd2_spmm(asked, x, y[1])
+    sd2.sd2_stream_check()
+    assert torch.equal(*y) and y[0].abs().max() > 0
+    sd2.sd2_free(asked)
     bits, mma = sd2.sd2_compress(W, mask, sd2.SD2_FORMAT_BITMASK), sd2.sd2_compress(W, mask, sd2.SD2_FORMAT_GAP4_MMA)
     assert [sd2.sd2_spmm_query(x, 65)[k] for x in (bits, mma) for k in ("launches", "path")] == [9, sd2.SD2_PATH_BITMASK, 2, sd2.SD2_PATH_MMA]
     for x in (h, bare, bits, mma):
