@@ -521,7 +521,7 @@ sd2_status run_bitmask(const sd2_handle* hs, int count, const uint16_t* x, const
 
 // ------------------------------------------------------------------ GAP4 programs
 
-// Largest panel width (8, 4, 2, 1) whose staged activations leave room for a ring that holds
+// Largest panel width (4, 2, 1) whose staged activations leave room for a ring that holds
 // `max_tile` bytes at least twice; 0 if even one row does not fit.
 struct SmemPlan {
     int nt, xs_bytes, xlin_bytes, ring_bytes;
@@ -537,7 +537,7 @@ int xs_bytes_for(int S, int B, int V, int nt)
 bool plan_smem(int nt, int xs_max, int K_max, int max_tile, SmemPlan* p)
 {
     const int fixed = (int)((sizeof(StreamShared) + 127) & ~127);
-    const int xlin = ((2 * K_max + 127) & ~127) * (nt > 2 ? 2 : 1);   // panels of 4 and 8 go two rows at a time
+    const int xlin = ((2 * K_max + 127) & ~127) * (nt > 2 ? 2 : 1);   // panels of 4 go two rows at a time
     const int ring = (kSmemMax - fixed - xs_max - xlin) & ~127;
     if (ring < 2 * max_tile + 256) return false;
     p->nt = nt;
@@ -928,8 +928,11 @@ sd2_status launch_lm_head(const uint16_t* x, const uint16_t* w, float* logits, i
 // Whether N rows over these GAP4 handles are faster by their cells.  Cells bring 1.3 times the strips' bytes but expand them
 // once for all rows, the strips gather row by row.  Measured (us, cold caches, strips / cells): 2048 x 8192 at 50 %: N = 1
 // 14.4 / 16.4, N = 2 18.4 / 16.4, N = 3 24.6 / 16.4; the same at 30 %: 12.3 / 14.5, 15.4 / 16.4, 20.5 / 16.3; two blocks of
-// 2048/512/8192 at 50 %: 60 / 70, 75 / 70, 116 / 72.  Below a million slots both take the time of a launch for N <= 3, and
-// there the rows of small steps keep the sums of a one-row step.
+// 2048/512/8192 at 50 %: 60 / 70, 75 / 70, 116 / 72.  From four rows on cells are faster at every density, though the strips'
+// work shrinks with it: at 10 % 2048 x 2048 for N = 4 about 10 / 6, 640 x 640 9.4 / 5.7, 2048 x 11008 20.6 / 11.3, 1024 x 15360
+// (where a launch takes twelve rows) 22 / 10 and for N = 64 345 / 63.  Below a million slots three rows would gain too (640 x
+// 640: 8.8 / 5.7, two rows 6.5 / 5.7) and stay with the strips all the same, whose sums do not depend on how many rows a
+// call has: small steps give the bits of one-row steps.
 bool cells_pay(const sd2_handle* hs, int count, int64_t N)
 {
     if (N >= 4) return true;

@@ -29,8 +29,8 @@
 // The last four share their schedulers with three busy warps each and get an instruction in every four to eight cycles: what
 // counts for them is the number of instructions.
 //
-// What bounds it: HBM for large matrices (15 slots per clock and SM at 50 % density against 33 that twelve warps expand, 29
-// for sixteen rows); between stages some 2.8 us: from the last output to the barrier's release 1.2, to the activations 0.6, to
+// What bounds it: HBM for large matrices (15 slots per clock and SM at 50 % density against 33 that twelve warps expanded, 29
+// for sixteen rows, before the sums were added up in fp32); between stages some 2.8 us: from the last output to the barrier's release 1.2, to the activations 0.6, to
 // the first cell 0.9.  One launch with its start and its last sums is 8 us at least, and launches of a stream overlap there.
 // Against the strips, which gather row by row (us): 5 rows of 1531 x 3001 18.5 -> 8.6, 48 rows of 8192 x 2048 111 -> 26, two
 // blocks of 2048/512/8192 for 8 rows 230 -> 68, a block of 3072/1024/8192 for 16 rows 342 -> 61.

@@ -13,9 +13,9 @@
 //     those of row g + 8 in column pi(l), from row H - 1 down.  pi matches lanes with many words in one row to lanes
 //     with few in the other, which keeps H close to the mean.  Whatever rows 32 lanes read, they read 32 different banks.
 //
-// Bytes per dense slot at 50 % density: 1.61 (three of four pairs have a word; the strips take 1.28).  Packing the values
+// Bytes per dense slot at 50 % density: 1.65 (three of four pairs have a word; the strips take 1.28).  Packing the values
 // without the pairs' zeros takes 1.39, but its expansion by byte permutations ran at 18 slots per clock and SM; this
-// one, a predicated load per pair, runs at 33 (29 for sixteen activation rows), and HBM brings 15.
+// one, a predicated load per pair, ran at 33 (29 for sixteen activation rows) with chains of mma, and HBM brings 15.
 //
 // Two CTAs share a tile: one takes the first ceil(D / 2) cells of its columns, the other the rest.  The cells of each
 // share stand together, tile by tile, so that a CTA's run of tiles is one run of bytes.
