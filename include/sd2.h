@@ -75,15 +75,14 @@ enum {
                             /* programs of one row at a time or short of device memory    */
                             /* (0.44 of a GAP4 handle's).  Calls of several rows read the */
                             /* strips.  The blob and the handle report SD2_FORMAT_GAP4.   */
-    SD2_FORMAT_GAP4_MMA = 4 /* for panels of N >= 16 activation rows: 128 x 128 blocks    */
-                            /* whose 4-bit gaps run in the order of a tensor-core operand */
-                            /* tile; sd2_spmm expands each block in shared memory and     */
-                            /* multiplies it on the tensor cores (tcgen05.mma, fp32       */
-                            /* accumulators in tensor memory).  Any N is accepted (rows   */
-                            /* are taken 64 at a time, padded to a multiple of 16); never */
-                            /* picked by AUTO; not accepted by sd2_block_step or a        */
-                            /* drafter.  Calls on one handle must not overlap on the GPU: */
-                            /* they share the handle's partial-sum buffer.                */
+    SD2_FORMAT_GAP4_MMA = 4 /* for panels of N >= 16 activation rows: blocks of 128 x 64,  */
+                            /* as a blob 4-bit gaps in the order of a tensor-core operand  */
+                            /* tile, in a handle words of two neighbouring columns;        */
+                            /* sd2_spmm expands the blocks in registers and multiplies     */
+                            /* them on the tensor cores (tcgen05.mma, weights and fp32     */
+                            /* sums in tensor memory).  Any N is accepted (rows are taken  */
+                            /* 64 at a time, padded to a multiple of 16); never picked by  */
+                            /* AUTO; not accepted by sd2_block_step or a drafter.          */
 };
 
 enum { SD2_DTYPE_BF16 = 0, SD2_DTYPE_F32 = 1 };

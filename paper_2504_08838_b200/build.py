@@ -1,9 +1,9 @@
 """Builds ``libsd2.so`` (sm_100a) in-tree from ``csrc/``.
 
 ``python -m paper_2504_08838_b200.build`` or ``build.build()``.  ``SD2_CHECKED=1`` in the environment builds
-the checked variant: the tensor-core kernel verifies every record offset and store address it derives
-from compressed data, records a violation in the device error word (``sd2_stream_check`` then returns
-``SD2_ERR_CORRUPT``) and skips the access.  nvcc cross-compiles
+the checked variant: the tensor-core kernel verifies the offsets that it derives from a block's headers,
+records a violation in the device error word (``sd2_stream_check`` then returns ``SD2_ERR_CORRUPT``) and
+skips the block.  nvcc cross-compiles
 without a GPU; the shared object sits next to this file so that it travels with the
 source tree and is the one the binding loads.
 """

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdio>
@@ -35,16 +36,13 @@ struct sd2_handle_s {
     // GAP4 geometry
     int S, B, T, max_tile_bytes, V;
     int paired;   // GAP4: rows 2i, 2i+1 share a tile (header field `pairing`)
-    // GAP4: the same weights as cells (sd2_cells.hpp), for panels of rows (d_image NULL: none)
+    // GAP4: the same weights as cells (sd2_cells.hpp), for panels of rows (d_image NULL: none); GAP4_MMA: the weights as panel
+    // cells (and nothing else: d_blob has room for their heights)
     uint8_t* d_image;
     const unsigned char* d_cells;
     int64_t cell_bytes;        // what a launch reads of them
     int64_t device_bytes;      // all that the handle owns
     int cell_T, cell_D, max_chunk;
-    // GAP4_MMA: fp32 partial sums [64][rows padded to 128] followed by one arrival count per row panel,
-    // all zero between launches (the CTA that completes a panel writes Y and clears them)
-    float* d_partial;
-    int64_t partial_bytes;
 };
 
 // What a program over cells needs from shared memory.
@@ -148,6 +146,7 @@ struct DeviceState {
     int clock_khz;
     int* err_word;
     unsigned int* barriers;
+    int mma_clusters[kMmaMaxCluster + 1];    // how many clusters of so many CTAs of mma_kernel run at once
 };
 DeviceState g_dev[kMaxDevices];
 std::atomic<unsigned> g_next_barrier{0};
@@ -196,6 +195,8 @@ cudaError_t set_cell_attr()
     return cudaFuncSetAttribute(cell_kernel<MAXS, NR, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
 }
 
+sd2_status count_mma_clusters(int* room);
+
 // Once per device: SM count, shared-memory opt-in, the error word and the barrier pool.
 sd2_status ensure_device(int* dev_out)
 {
@@ -222,6 +223,8 @@ sd2_status ensure_device(int* dev_out)
             cudaGetLastError();
             return SD2_ERR_CUDA;
         }
+        const sd2_status counted = count_mma_clusters(ds.mma_clusters);
+        if (counted != SD2_OK) return counted;
         int* err = nullptr;
         unsigned int* bars = nullptr;
         const size_t bar_bytes = (size_t)kBarrierPool * kBarrierStrideWords * 4;
@@ -304,10 +307,12 @@ sd2_status upload(const uint8_t* blob, int64_t bytes, const BlobHeader& hd, sd2_
     void* d = nullptr;
     // (with room behind a GAP4 blob for the heights of its cells while they are packed: an allocation of their own took
     // longer than the packing)
-    const CellGeom cells = cell_geometry(hd.M, hd.K);
-    const size_t heights = hd.format == (uint32_t)kFormatGap4 ? (size_t)(cells.T * cells.D) * 4 : 0;
+    const bool mma = hd.format == (uint32_t)kFormatGap4Mma;
+    const size_t heights = hd.format == (uint32_t)kFormatGap4 ? (size_t)cell_geometry(hd.M, hd.K).cells() * 4
+                         : mma ? (size_t)panel_geometry(hd.M, hd.K).cells() * 4 : 0;
+    if (mma) bytes = 0;                       // (the GPU has no use for the records)
     if (dev_malloc(&d, align256((size_t)bytes) + heights) != cudaSuccess) { cudaGetLastError(); delete h; return SD2_ERR_ALLOC; }
-    if (cudaMemcpy(d, blob, (size_t)bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
+    if (bytes && cudaMemcpy(d, blob, (size_t)bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
         cudaGetLastError();
         cudaFree(d);
         delete h;
@@ -330,18 +335,7 @@ sd2_status upload(const uint8_t* blob, int64_t bytes, const BlobHeader& hd, sd2_
     h->V = (int)hd.overlap;
     h->paired = (int)hd.pairing;
     h->d_image = nullptr;
-    h->d_partial = nullptr;
-    h->partial_bytes = 0;
     h->device_bytes = (int64_t)(align256((size_t)bytes) + heights);
-    if (h->format == SD2_FORMAT_GAP4_MMA) {
-        const int64_t panels = (hd.M + kMmaBlockRows - 1) / kMmaBlockRows;
-        h->partial_bytes = (int64_t)kMmaMaxRows * panels * kMmaBlockRows * 4 + panels * 4;
-        void* pp = nullptr;
-        if (dev_malloc(&pp, (size_t)h->partial_bytes) != cudaSuccess) { cudaGetLastError(); cudaFree(d); delete h; return SD2_ERR_ALLOC; }
-        if (cudaMemset(pp, 0, (size_t)h->partial_bytes) != cudaSuccess) { cudaGetLastError(); cudaFree(pp); cudaFree(d); delete h; return SD2_ERR_CUDA; }
-        h->d_partial = (float*)pp;
-        h->device_bytes += h->partial_bytes;
-    }
     {
         std::lock_guard<std::mutex> lk(g_mu);
         g_live.insert(h);
@@ -371,17 +365,20 @@ bool kernel_reads(const void* p, size_t size, int device)
     return readable_in_place(place, owner, device, p, size);
 }
 
-// Gives a fresh GAP4 handle its cells, from dense weights (and a mask, or NULL) in device memory.
-sd2_status pack_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask)
+// Gives a fresh handle its cells (GAP4_MMA: panel cells), from dense weights (and a mask, or NULL: see pack_cells_kernel) in device
+// memory.
+sd2_status pack_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask, uint32_t nonzero)
 {
-    const CellGeom g = cell_geometry(h->M, h->K);
-    const int64_t n_cells = g.T * g.D;
+    const bool panel = h->format == SD2_FORMAT_GAP4_MMA;
+    const CellGeom g = panel ? panel_geometry(h->M, h->K) : cell_geometry(h->M, h->K);
+    const int64_t n_cells = g.cells();
+    auto* const kernel = panel ? pack_cells_kernel<true> : pack_cells_kernel<false>;
     if (n_cells > 0x3FFFFFFF) return SD2_ERR_UNSUPPORTED;
     const size_t dir_bytes = align256((size_t)(n_cells + 1) * 4);
     std::vector<uint32_t> off((size_t)n_cells + 1);          // first the cells' heights, then their places
     uint32_t* d_height = (uint32_t*)(h->d_blob + align256((size_t)h->blob_bytes));
     const unsigned grid = (unsigned)((n_cells + kPackWarps - 1) / kPackWarps);
-    pack_cells_kernel<<<grid, 32 * kPackWarps>>>(W, mask, h->M, h->K, (int)g.T, g.D, d_height, nullptr, nullptr);
+    kernel<<<grid, 32 * kPackWarps>>>(W, mask, nonzero, h->M, h->K, (int)g.T, g.D, d_height, nullptr, nullptr);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpy(off.data(), d_height, (size_t)n_cells * 4, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return SD2_ERR_CUDA;
@@ -404,7 +401,7 @@ sd2_status pack_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask)
     e = cudaMemset(image, 0, bytes);
     if (e == cudaSuccess) e = cudaMemcpy(image, off.data(), off.size() * 4, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) {
-        pack_cells_kernel<<<grid, 32 * kPackWarps>>>(W, mask, h->M, h->K, (int)g.T, g.D, nullptr, (const uint32_t*)image, image + dir_bytes);
+        kernel<<<grid, 32 * kPackWarps>>>(W, mask, nonzero, h->M, h->K, (int)g.T, g.D, nullptr, (const uint32_t*)image, image + dir_bytes);
         e = cudaGetLastError();
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(0);       // W and mask may go away now
@@ -417,10 +414,10 @@ sd2_status pack_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask)
     return SD2_OK;
 }
 
-// The same from weights and mask in host memory or where the handle's GPU can read them.  Cells are a second image of the
-// weights: where there is no memory for them, or for the dense weights that they are made from, the handle goes without, and
-// calls of several rows read its strips.  On any other failure the handle is freed.
-sd2_status add_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask)
+// The same from weights and mask in host memory or where the handle's GPU can read them.  The cells of a GAP4 handle are a second
+// image of the weights: where there is no memory for them, or for the dense weights that they are made from, the handle goes without,
+// and calls of several rows read its strips.  On any other failure the handle is freed.
+sd2_status add_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask, uint32_t nonzero = 0x7FFFu)
 {
     const size_t n = (size_t)(h->M * h->K);
     uint16_t* w_dev = nullptr;
@@ -435,7 +432,7 @@ sd2_status add_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask)
         else if (cudaMemcpy(m_dev, mask, n, cudaMemcpyHostToDevice) != cudaSuccess) st = SD2_ERR_CUDA;
     }
     try {
-        if (st == SD2_OK) st = pack_cells(h, w_dev ? w_dev : W, m_dev ? m_dev : mask);
+        if (st == SD2_OK) st = pack_cells(h, w_dev ? w_dev : W, m_dev ? m_dev : mask, nonzero);
     } catch (const std::bad_alloc&) {
         st = SD2_ERR_ALLOC;
     }
@@ -443,7 +440,7 @@ sd2_status add_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask)
     cudaFree(m_dev);
     if (st == SD2_OK) return st;
     cudaGetLastError();
-    if (st == SD2_ERR_ALLOC || st == SD2_ERR_UNSUPPORTED) return SD2_OK;
+    if (h->format == SD2_FORMAT_GAP4 && (st == SD2_ERR_ALLOC || st == SD2_ERR_UNSUPPORTED)) return SD2_OK;
     sd2_free(h);
     return st;
 }
@@ -995,26 +992,91 @@ bool make_x_map(CUtensorMap* map, const uint16_t* X, int64_t N, int64_t K, int n
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// GAP4_MMA: one launch per 64 activation rows; each expands the blocks in shared memory and multiplies on the
-// tensor cores.
+// Shared memory of a launch of mma_kernel.  false: not even one block for each team fits.
+bool plan_mma(const MmaArgs& a, int block_bytes, int* slot_bytes, int* n_slots, int* smem)
+{
+    const int fixed = 1024 + kMmaStages * a.npad * 128 + mma_recv_bytes(a.npad, a.shares) + (int)((sizeof(MmaShared) + 127) & ~127);
+    *slot_bytes = (block_bytes + 127) & ~127;
+    int slots = (kSmemMax - fixed) / *slot_bytes / kMmaTeams * kMmaTeams;
+    const int most = (((a.KB + a.shares - 1) / a.shares) + kMmaTeams - 1) / kMmaTeams * kMmaTeams;
+    if (slots > kMmaMaxSlots) slots = kMmaMaxSlots;
+    if (slots > most) slots = most;
+    if (slots < kMmaTeams) return false;
+    *n_slots = slots;
+    *smem = fixed + slots * *slot_bytes;
+    // all of an SM's tensor memory goes to one CTA: another one of the launch must not come to the SM, where it would wait for it
+    if (*smem < kSmemMax / 2 + 1024) *smem = kSmemMax / 2 + 1024;
+    return true;
+}
+
+// How many CTAs share a panel's columns: the fewest steps of a CTA, in blocks.  What a CTA does beside its blocks (start, last sums)
+// is worth about four of them, the exchange of sums three more.
+int mma_cluster(int64_t P, int KB, const int* room)
+{
+    int best = 1;
+    int64_t least = 0;
+    for (int c = 1; c <= kMmaMaxCluster && c <= KB; ++c) {
+        if (room[c] < 1) continue;
+        const int64_t waves = (P + room[c] - 1) / room[c];
+        const int64_t steps = waves * ((KB + c - 1) / c + 4) + (c > 1 ? 3 : 0);
+        if (c == 1 || steps < least) { best = c; least = steps; }
+    }
+    return best;
+}
+
+cudaError_t launch_mma(const MmaArgs& a, const CUtensorMap& xmap, int64_t P, int smem, cudaStream_t s, int* room = nullptr)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(P * a.shares));
+    cfg.blockDim = dim3(kMmaThreads);
+    cfg.dynamicSmemBytes = (size_t)smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)a.shares;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    attr[1] = pdl_attribute();
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    if (room) {                              // how many clusters of this size run at once
+        cfg.numAttrs = 1;
+        return cudaOccupancyMaxActiveClusters(room, mma_kernel, &cfg);
+    }
+    return cudaLaunchKernelEx(&cfg, mma_kernel, a, xmap);
+}
+
+sd2_status count_mma_clusters(int* room)
+{
+    room[0] = 0;
+    for (int c = 1; c <= kMmaMaxCluster; ++c) {
+        MmaArgs a;
+        std::memset(&a, 0, sizeof a);
+        a.shares = c;
+        room[c] = 0;
+        if (launch_mma(a, CUtensorMap{}, 1, kSmemMax, nullptr, &room[c]) != cudaSuccess) {
+            cudaGetLastError();
+            room[c] = 0;
+        }
+    }
+    return room[1] > 0 ? SD2_OK : SD2_ERR_CUDA;
+}
+
+// GAP4_MMA: one launch per 64 activation rows.
 sd2_status run_mma(sd2_handle h, const uint16_t* x, void* Y, int64_t N, bool y_force_bf16, int dev, cudaStream_t s)
 {
     MmaArgs a;
     std::memset(&a, 0, sizeof a);
-    a.dir = h->d_sec0;
-    a.recs = (const uint8_t*)h->d_sec1;
+    a.off = (const uint32_t*)h->d_image;
+    a.cells = h->d_cells;
     a.M = (int)h->M;
     a.K = (int)h->K;
-    a.P = (int)((h->M + kMmaBlockRows - 1) / kMmaBlockRows);
-    a.KC = (int)((h->K + kMmaBlockCols - 1) / kMmaBlockCols);
-    a.NB = (long long)a.P * a.KC;
-    a.partial = h->d_partial;
-    a.done = (unsigned int*)(h->d_partial + (size_t)kMmaMaxRows * a.P * kMmaBlockRows);
+    const int64_t P = h->cell_T;
+    a.KB = h->cell_D;
+    a.shares = mma_cluster(P, a.KB, g_dev[dev].mma_clusters);
     a.y_f32 = (!y_force_bf16 && h->y_dtype == SD2_DTYPE_F32) ? 1 : 0;
     a.err = g_dev[dev].err_word;
     a.budget = wait_budget(dev);
     const size_t esz = a.y_f32 ? 4 : 2;
-    const int grid = (int)(a.NB < g_dev[dev].sms ? a.NB : g_dev[dev].sms);
     for (int64_t n0 = 0; n0 < N; n0 += kMmaMaxRows) {
         a.N = (int)((N - n0) < kMmaMaxRows ? (N - n0) : kMmaMaxRows);
         a.npad = (a.N + 15) & ~15;
@@ -1024,30 +1086,9 @@ sd2_status run_mma(sd2_handle h, const uint16_t* x, void* Y, int64_t N, bool y_f
         std::memset(&xmap, 0, sizeof xmap);
         a.x_tma = make_x_map(&xmap, a.X, a.N, h->K, a.npad) ? 1 : 0;
         a.x_vec = ((h->K & 7) == 0 && (((uintptr_t)a.X) & 15) == 0) ? 1 : 0;
-        const int rec_bytes = (h->max_tile_bytes + 127) & ~127;
-        // six stages: with eight the ring is left with three slots and the producer starves (measured 24 us against
-        // 21.7 us on a 3072 x 8192 matrix at N = 16); four where six leave no room for a record
-        a.stages = 6;
-        int fixed = 0, ring = 0;
-        for (;;) {
-            fixed = 1024 + a.stages * (kMmaTileBytes + a.npad * 128) + (int)((sizeof(MmaShared) + 127) & ~127);
-            ring = kSmemMax - fixed;
-            if (a.stages == 4 || ring >= 2 * rec_bytes) break;
-            a.stages = 4;
-        }
-        // records per copy: about 32 KiB where three such slots fit, fewer otherwise
-        int batch = 1;
-        while (batch < kMmaMaxBatch && batch * rec_bytes < 32 * 1024) batch <<= 1;
-        while (batch > 1 && ring / (batch * rec_bytes) < 3) batch >>= 1;
-        int slots = ring / (batch * rec_bytes);
-        if (slots < 1) return SD2_ERR_UNSUPPORTED;
-        if (slots > kMmaSlots) slots = kMmaSlots;
-        a.batch = batch;
-        a.slot_bytes = batch * rec_bytes;
-        a.n_slots = slots;
-        const int smem = fixed + slots * a.slot_bytes;
-        launch_pdl(mma_kernel, grid, kMmaThreads, smem, s, a, xmap);
-        if (cudaGetLastError() != cudaSuccess) return SD2_ERR_CUDA;
+        int smem = 0;
+        if (!plan_mma(a, h->max_chunk, &a.slot_bytes, &a.n_slots, &smem)) return SD2_ERR_UNSUPPORTED;
+        if (launch_mma(a, xmap, P, smem, s) != cudaSuccess) { cudaGetLastError(); return SD2_ERR_CUDA; }
     }
     return SD2_OK;
 }
@@ -1397,7 +1438,7 @@ sd2_status sd2_compress(const void* weight_bf16, const uint8_t* mask, int64_t M,
         sd2_handle h = nullptr;
         st = upload(blob, bytes, hd, &h);
         std::free(blob);
-        const bool cells = h && h->format == SD2_FORMAT_GAP4 && !(opt && opt->format == SD2_FORMAT_GAP4_STRIPS);
+        const bool cells = h && (h->format == SD2_FORMAT_GAP4_MMA || (h->format == SD2_FORMAT_GAP4 && !(opt && opt->format == SD2_FORMAT_GAP4_STRIPS)));
         if (st == SD2_OK && cells)    // (from the host's copies of what lies on another GPU)
             st = add_cells(h, kernel_reads(weight_bf16, sizeof *W, h->device) ? (const uint16_t*)weight_bf16 : W,
                            mask_in && kernel_reads(mask_in, sizeof *mask_in, h->device) ? mask_in : mask);
@@ -1419,11 +1460,15 @@ sd2_status sd2_load_blob(const void* blob, int64_t blob_bytes, sd2_handle* out)
     if (hd.format == (uint32_t)kFormatGap4) {
         if (check_gap4(hd, (const uint8_t*)blob) != 0) return SD2_ERR_CORRUPT;
         dense = (uint16_t*)lib_malloc((size_t)(hd.M * hd.K) * 2);     // for the cells; NULL: the handle goes without
+    } else if (hd.format == (uint32_t)kFormatGap4Mma) {
+        if (unpack_any(hd, (const uint8_t*)blob, nullptr) != 0) return SD2_ERR_CORRUPT;
+        dense = (uint16_t*)lib_malloc((size_t)(hd.M * hd.K) * 2);
+        if (!dense) return SD2_ERR_ALLOC;
     }
     int rc;
     try {
         rc = unpack_any(hd, (const uint8_t*)blob, dense);
-        if (rc != 0 && dense) {              // a column that two lanes share has a sum in strips, but no dense form
+        if (rc != 0 && dense && hd.format == (uint32_t)kFormatGap4) {   // a column that two lanes share has a sum in strips, but no dense form
             std::free(dense);
             dense = nullptr;
             rc = unpack_any(hd, (const uint8_t*)blob, nullptr);
@@ -1434,8 +1479,9 @@ sd2_status sd2_load_blob(const void* blob, int64_t blob_bytes, sd2_handle* out)
     }
     sd2_handle h = nullptr;
     sd2_status st = rc != 0 ? SD2_ERR_CORRUPT : upload((const uint8_t*)blob, blob_bytes, hd, &h);
-    // for the cells what decoded to +0 or -0 was masked out, or was a kept zero, which adds nothing
-    if (st == SD2_OK && dense) st = add_cells(h, dense, nullptr);
+    // for the cells what decoded to +0 or -0 was masked out, or was a kept zero, which adds nothing (panel cells are what a handle
+    // is decompressed from: they keep a -0)
+    if (st == SD2_OK && dense) st = add_cells(h, dense, nullptr, hd.format == (uint32_t)kFormatGap4 ? 0x7FFFu : 0xFFFFu);
     std::free(dense);
     if (st == SD2_OK) *out = h;
     return st;
@@ -1444,15 +1490,30 @@ sd2_status sd2_load_blob(const void* blob, int64_t blob_bytes, sd2_handle* out)
 sd2_status sd2_decompress(sd2_handle h, void* dense_bf16_out)
 {
     if (!live(h) || !dense_bf16_out) return SD2_ERR_INVALID_ARG;
-    uint8_t* blob = (uint8_t*)lib_malloc((size_t)h->blob_bytes);
+    const bool panel = h->format == SD2_FORMAT_GAP4_MMA;
+    const CellGeom geom = panel_geometry(h->M, h->K);
+    const size_t dir_bytes = align256((size_t)(geom.cells() + 1) * 4);
+    const size_t image_bytes = panel ? dir_bytes + (size_t)h->cell_bytes - (size_t)(geom.cells() + 1) * 4 : (size_t)h->blob_bytes;
+    uint8_t* blob = (uint8_t*)lib_malloc(image_bytes);
     if (!blob) return SD2_ERR_ALLOC;
     sd2_status st = SD2_OK;
-    if (cudaMemcpy(blob, h->d_blob, (size_t)h->blob_bytes, cudaMemcpyDeviceToHost) != cudaSuccess) { cudaGetLastError(); st = SD2_ERR_CUDA; }
+    if (cudaMemcpy(blob, panel ? h->d_image : h->d_blob, image_bytes, cudaMemcpyDeviceToHost) != cudaSuccess) { cudaGetLastError(); st = SD2_ERR_CUDA; }
     const size_t dense_bytes = (size_t)(h->M * h->K) * 2;
     const bool to_dev = is_device_ptr(dense_bf16_out);
     uint16_t* host_out = to_dev ? (uint16_t*)lib_malloc(dense_bytes) : (uint16_t*)dense_bf16_out;
     if (!host_out) st = SD2_ERR_ALLOC;
-    if (st == SD2_OK) st = sd2_unpack_host(blob, h->blob_bytes, host_out, nullptr, nullptr, nullptr, nullptr, nullptr);
+    if (st == SD2_OK && !panel) st = sd2_unpack_host(blob, h->blob_bytes, host_out, nullptr, nullptr, nullptr, nullptr, nullptr);
+    if (st == SD2_OK && panel) {
+        const uint32_t* off = (const uint32_t*)blob;
+#pragma omp parallel for schedule(static)
+        for (int64_t p = 0; p < geom.T; ++p) {
+            const int64_t first = p * kPanelRowsOfBlock, rows = std::min<int64_t>(kPanelRowsOfBlock, h->M - first);
+            std::memset(host_out + first * h->K, 0, (size_t)(rows * h->K) * 2);
+            for (int64_t c = p * geom.D * geom.per; c < (p + 1) * geom.D * geom.per; ++c)
+                unpack_panel_cell(blob + dir_bytes + (size_t)off[c] * 32, (int)(((off[c + 1] - off[c]) * 32u - kCellHeaderBytes) / 128u),
+                                  first + 32 * (c % geom.per), (c / geom.per - p * geom.D) * kPanelBlockCols, h->M, h->K, host_out);
+        }
+    }
     if (st == SD2_OK && to_dev &&
         cudaMemcpy(dense_bf16_out, host_out, dense_bytes, cudaMemcpyHostToDevice) != cudaSuccess) { cudaGetLastError(); st = SD2_ERR_CUDA; }
     if (to_dev) std::free(host_out);
@@ -1481,7 +1542,6 @@ sd2_status sd2_free(sd2_handle h)
     sd2_status st = SD2_OK;
     if (cudaFree(h->d_blob) != cudaSuccess) { cudaGetLastError(); st = SD2_ERR_CUDA; }
     if (h->d_image && cudaFree(h->d_image) != cudaSuccess) { cudaGetLastError(); st = SD2_ERR_CUDA; }
-    if (h->d_partial && cudaFree(h->d_partial) != cudaSuccess) { cudaGetLastError(); st = SD2_ERR_CUDA; }
     delete h;
     return st;
 }
@@ -1507,8 +1567,6 @@ sd2_status sd2_stream_check(void* cuda_stream)
                     if (d->d_tags) cudaMemset(d->d_tags, 0, (size_t)d->tags_bytes);
                     if (d->d_cbar) cudaMemset(d->d_cbar, 0, kDrafterWordsBytes);
                 }
-            for (sd2_handle h : g_live)
-                if (h->device == dev && h->d_partial) cudaMemset(h->d_partial, 0, (size_t)h->partial_bytes);
         }
         cudaGetLastError();
         return flag == 2 ? SD2_ERR_CORRUPT : SD2_ERR_TIMEOUT;      // 2: an index check of a checked build failed
@@ -1879,7 +1937,7 @@ sd2_status sd2_spmm_query(sd2_handle h, int64_t N, int64_t* out)
     out[0] = (N + cap - 1) / cap;
     out[1] = cap;
     out[2] = h->device_bytes;
-    out[3] = path == SD2_PATH_CELLS ? h->cell_bytes : h->compressed_bytes;
+    out[3] = path == SD2_PATH_CELLS || path == SD2_PATH_MMA ? h->cell_bytes : h->compressed_bytes;
     out[4] = path;
     return SD2_OK;
 }

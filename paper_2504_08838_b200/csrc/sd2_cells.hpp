@@ -37,9 +37,17 @@ constexpr int kCellHeaderBytes = 128 + 32;
 
 constexpr int kChunkCells = 4;        // consecutive cells of a share that travel in one copy, at most
 
+// Panel cells: the same words and header for a tensor-memory operand.  A block of 128 rows x 64 columns is a chunk of four cells of
+// 32 rows; lane l holds row l of its cell, of which columns 0..31 count as row g above and columns 32..63 as row g + 8: bit
+// 16 r + e of mask[l] is pair e (columns 32 r + 2 e and the next).  Blocks stand panel by panel, ascending columns inside a panel.
+constexpr int kPanelRowsOfBlock = 128;
+constexpr int kPanelBlockCols = 64;
+
 struct CellGeom {
-    int64_t T;        // row tiles
-    int D;            // cells per tile
+    int64_t T;        // row tiles (panel cells: row panels)
+    int D;            // cells per tile (blocks per panel)
+    int per;          // cells of a place in this grid: 1 (a block's four)
+    int64_t cells() const { return T * D * per; }
 };
 
 // cells of share r (0, 1) of a tile
@@ -59,7 +67,38 @@ inline CellGeom cell_geometry(int64_t M, int64_t K)
     CellGeom g;
     g.T = (M + kTileRows - 1) / kTileRows;
     g.D = (int)((K + kCellCols - 1) / kCellCols);
+    g.per = 1;
     return g;
+}
+
+inline CellGeom panel_geometry(int64_t M, int64_t K)
+{
+    CellGeom g;
+    g.T = (M + kPanelRowsOfBlock - 1) / kPanelRowsOfBlock;
+    g.D = (int)((K + kPanelBlockCols - 1) / kPanelBlockCols);
+    g.per = kChunkCells;
+    return g;
+}
+
+// One cell of a panel's block back into dense weights.  cell: its header; H: its height; row0, col0: its place in W.
+inline void unpack_panel_cell(const uint8_t* cell, int H, int64_t row0, int64_t col0, int64_t M, int64_t K, uint16_t* W)
+{
+    const uint32_t* mask = (const uint32_t*)cell;
+    const uint32_t* words = (const uint32_t*)(cell + kCellHeaderBytes);
+    for (int l = 0; l < 32 && row0 + l < M; ++l)
+        for (int r = 0; r < 2; ++r) {
+            const int column = r ? (cell[128 + l] & 0x7F) / 4 : l;
+            int at = r ? H - 1 : 0;
+            for (int e = 0; e < 16; ++e) {
+                if (!(mask[l] >> (16 * r + e) & 1u)) continue;
+                const uint32_t w = words[32 * at + column];
+                const int64_t col = col0 + 32 * r + 2 * e;
+                uint16_t* to = W + (row0 + l) * K + col;
+                if (col < K) to[0] = (uint16_t)w;
+                if (col + 1 < K) to[1] = (uint16_t)(w >> 16);
+                at += r ? -1 : 1;
+            }
+        }
 }
 
 }  // namespace sd2

@@ -13,14 +13,17 @@ namespace sd2 {
 
 constexpr int kPackWarps = 8;
 
+// PANEL: panel cells (sd2_mma_kernel.cuh); T and D are then row panels and blocks of a panel.
 // height: [cells] (first pass), or NULL; off: directory (second pass).
-// mask: one byte per weight, not zero where it is kept; NULL: what is not +0 or -0 is kept.
-__global__ void __launch_bounds__(32 * kPackWarps) pack_cells_kernel(const uint16_t* W, const uint8_t* mask, long long M, long long K, int T, int D,
-                                                                    uint32_t* height, const uint32_t* off, unsigned char* cells)
+// mask: one byte per weight, not zero where it is kept; NULL: a weight that has one of the bits of `nonzero` is kept (0x7FFF: what is
+// not +0 or -0; 0xFFFF: what is not +0).
+template <bool PANEL>
+__global__ void __launch_bounds__(32 * kPackWarps) pack_cells_kernel(const uint16_t* W, const uint8_t* mask, uint32_t nonzero, long long M, long long K,
+                                                                    int T, int D, uint32_t* height, const uint32_t* off, unsigned char* cells)
 {
     __shared__ uint8_t lane_of_rank[kPackWarps][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const long long n_cells = (long long)T * D, in_first = (long long)T * share_cells(D, 0);
+    const long long n_cells = (long long)T * D * (PANEL ? kChunkCells : 1), in_first = (long long)T * share_cells(D, 0);
     const long long c = (long long)blockIdx.x * kPackWarps + warp;
     if (c >= n_cells) return;                // (whole warps)
     const int n0 = share_cells(D, 0), n1 = share_cells(D, 1);
@@ -28,17 +31,18 @@ __global__ void __launch_bounds__(32 * kPackWarps) pack_cells_kernel(const uint1
     const int d = c < in_first ? (int)(c - tile * n0) : n0 + (int)(c - in_first - tile * n1);
     const int g = lane >> 2, t = lane & 3;
     uint32_t bits = 0;
-    // pair i of unit u of row g + 8 r: its word, and whether there is one
+    const long long block = c / kChunkCells, panel = block / D;
+    // pair i of unit u of row g + 8 r (PANEL: pair 4 u + i of the row's r-th 32 columns): its word, and whether there is one
     auto pair = [&](int r, int u, int i, uint32_t& word) {
-        const long long row = tile * kTileRows + g + 8 * r;
+        const long long row = PANEL ? panel * kPanelRowsOfBlock + 32 * (c % kChunkCells) + lane : tile * kTileRows + g + 8 * r;
         uint32_t w = 0;
         bool any = false;
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
-            const long long col = (long long)d * kCellCols + 32 * u + 8 * t + 2 * i + k;
+            const long long col = PANEL ? (block - panel * D) * kPanelBlockCols + 32 * r + 8 * u + 2 * i + k : (long long)d * kCellCols + 32 * u + 8 * t + 2 * i + k;
             if (row >= M || col >= K) continue;
             const uint32_t v = W[row * K + col];
-            const bool kept = mask ? mask[row * K + col] != 0 : (v & 0x7FFFu) != 0;
+            const bool kept = mask ? mask[row * K + col] != 0 : (v & nonzero) != 0;
             if (kept) { w |= v << (16 * k); any = true; }
         }
         word = w;

@@ -1,4 +1,5 @@
-// GAP4_MMA: the compressed weight format of the tensor-core path (N >= 16 activation rows).
+// GAP4_MMA: the blob format of the tensor-core path (N >= 16 activation rows).  On the GPU a handle keeps the same weights as
+// panel cells (sd2_cells.hpp), which expand in registers; the order below is that of a shared-memory operand.
 //
 // With a panel of activation rows the product is a dense contraction once the weights are
 // dense again, so this format is built to be *expanded* fast rather than gathered from: a

@@ -1,119 +1,108 @@
 // Tensor-core path of libsd2 for panels of activation rows (GAP4_MMA handles).
 //
-// Y[n, m] = sum over kept k of W[m, k] X[n, k] for N <= 64 rows per launch.  With that many rows
-// the product is worth a dense contraction: the compressed weights still cross HBM once, but
-// instead of gathering activations entry by entry, a CTA expands each 128 x 64 block of W into
-// shared memory as a dense bf16 operand tile and lets tcgen05.mma multiply it with the matching
-// 64 columns of X; the fp32 sums live in tensor memory.  One persistent CTA per SM:
+// Y[n, m] = sum over kept k of W[m, k] X[n, k] for N <= 64 rows per launch.  With that many rows the product is worth a dense
+// contraction: the compressed weights still cross HBM once, a warp expands them in registers, and tcgen05.mma takes them from
+// tensor memory, so that the expanded weights pass through no shared memory.
 //
-//   warp 4        producer: per block one bulk asynchronous copy of its record (global -> ring)
-//   warp 22       per block one tensor-map copy of its X columns, which arrive in shared memory
-//                 in the swizzled K-major layout the B operand needs (rows beyond N and columns
-//                 beyond K are filled with zeros by the copy engine)
-//   warps 6..21   eight teams of two warps take the blocks in turn; a team zero-fills the operand
-//                 tile of the block's stage and scatters the block's values into it: lane w of
-//                 the team's warp h walks the 16-bit half h of word column w down the rows, row
-//                 offsets are running sums of 4-bit gaps, and the 32 lanes of a store always hit
-//                 32 different banks (see sd2_format_mma.hpp)
-//   warp 5        one thread issues the four K = 16 tcgen05.mma of a block, in block order, two
-//                 blocks per barrier wait, and commits them to the mbarriers that free the
-//                 stages and, at a row panel's end, hand the sums over
-//   warps 0..3    read the sums out of tensor memory (tcgen05.ld, one 32-lane quarter each)
+// On the device the weights of such a handle are *panel cells*: the cells of sd2_cells.hpp (a word per pair of columns of which
+// anything is kept, words of 32 lanes in 32 banks) cut for an operand in tensor memory.  A panel is 128 weight rows, a block of
+// it 64 columns: four cells of 32 rows, which stand together, block after block, so that a CTA's share is one run of bytes.
+// Lane l of cell q holds row 32 q + l: the words of columns 0..31 from the bottom of the cell up, those of columns 32..63 from
+// its top down.  That is the tensor memory layout of the A operand (a lane a row, a 32-bit column two elements of K).
 //
-// Six stages (operand tile + X columns) are in flight, one per working team, so a team never
-// waits for the MMAs of the block it has just expanded.  Blocks are dealt to the CTAs in contiguous runs, so a
-// row panel's K range is usually shared by several CTAs: each adds its part into the handle's
-// fp32 partial-sum buffer with red.add, and the CTA that brings the panel's block count to KC
-// rounds, writes Y and clears the buffer.  Every wait is bounded; a wait that runs out sets the
-// error word and the CTA leaves in order (copies drained, tensor memory returned).
+// A CTA has one panel and one share of its columns; the shares of a panel are a cluster (mma_cluster chooses how many).
+//
+//   warps 0..15   expand: team t = warp / 4 takes blocks t, t + 4, ...; warp q of a team has cell q, whose rows are the 32 lanes
+//                 of tensor memory that the warp can reach.  Then all of them read the sums.
+//   warp 16       weights: a bulk asynchronous copy per block (13 KB at 50 % density) into a ring
+//   warp 17       activations: a tensor-map copy per block (64 columns of all rows, in the swizzled K-major layout of the B
+//                 operand; rows beyond N and columns beyond K arrive as zeros)
+//   warps 18..21  issue the four K = 16 tcgen05.mma of a block, one warp for every team (one thread needs 560 cycles a block for its
+//                 waits, the products and the commit, whatever they multiply: alone it took twice as long as the expanding).  Every
+//                 team has sums of its own, so a chain of truncated sums is a quarter as long; they meet in fp32.
+//
+// The sums of a cluster meet by stores into the shared memory of the CTA that writes the activation row, in one order: results
+// do not depend on timing, and a handle has no state that launches share.
+//
+// What bounds it: HBM while blocks are expanded (24 of them in 6.4 us on each of 128 CTAs, 6.5 TB/s), then what stands between
+// launches: the last products, reading and exchanging the sums 2 us, the next start and its first block 2 us.  3072 x 8192 at 50 %
+// for 16 rows takes 11.5 us in a row of launches, 8192 x 3072 for 64 rows 13.1.  Before, 16-bit values were scattered into operand
+// tiles in shared memory (eight dependent steps of 340 cycles a block) and shares added up by red.add: 20.0 and 35.3.  Half-size
+// CTAs, two to an SM, whose successors fetch weights early: 11.2 for 16 rows, but 5.2 to 5.5 for 2048 x 2048 instead of 5.0, and sums
+// twice as far from 64 bits; not taken.
+//
+// Every wait is bounded; a wait that runs out sets the error word and the CTA leaves in order (copies drained, tensor memory
+// returned).
 
 #pragma once
 
 #include <cuda.h>
 
+#include "sd2_cell_kernel.cuh"
 #include "sd2_format_mma.hpp"
-#include "sd2_kernels.cuh"
 
 namespace sd2 {
 
 constexpr int kMmaMaxRows = 64;                     // activation rows of one launch
-constexpr int kMmaTeams = 8;                        // expanding teams of two warps (one per 16-bit side of the words)
-constexpr int kMmaStages = 8;                       // most operand tiles (and X column sets) in flight
-constexpr int kMmaEpiWarps = 4;
-constexpr int kMmaProducerWarp = 4;
-constexpr int kMmaIssueWarp = 5;
-constexpr int kMmaFirstGroupWarp = 6;
-constexpr int kMmaXWarp = kMmaFirstGroupWarp + kMmaTeams * kMmaSides;                 // 22: tensor-map copies of X
-constexpr int kMmaThreads = 32 * (kMmaXWarp + 1);                                     // 736
-constexpr int kMmaPairs = kMmaStages / 2;            // the MMA thread takes the stages two at a time
-constexpr int kMmaSlots = 8;                        // most ring slots
-constexpr int kMmaMaxBatch = 8;                     // most block records per bulk copy
-constexpr int kMmaTileBytes = kMmaBlockRows * kMmaBlockCols * 2;                       // 16 KiB
-constexpr int kMmaTmemCols = 2 * kMmaMaxRows;       // two accumulator stages of up to 64 columns
+constexpr int kMmaTeams = 4;                        // expanding teams
+constexpr int kMmaQuads = kMmaBlockRows / 32;       // cells of a block, warps of a team
+constexpr int kMmaExpandWarps = kMmaTeams * kMmaQuads;
+constexpr int kMmaWeightWarp = kMmaExpandWarps, kMmaXWarp = kMmaExpandWarps + 1, kMmaIssueWarp = kMmaExpandWarps + 2;
+constexpr int kMmaThreads = 32 * (kMmaExpandWarps + 2 + kMmaTeams);
+constexpr int kMmaStages = 2 * kMmaTeams;           // blocks expanded or being expanded; stage s belongs to team s % 4
+constexpr int kMmaMaxSlots = 16;                    // blocks in the ring, at most; always a multiple of the teams, so that a
+                                                    // slot is waited for by one team only, in order
+constexpr int kMmaStageCols = kMmaBlockCols / 2;    // tensor memory columns of an expanded block
+constexpr int kMmaTmemCols = 512;
+constexpr int kMmaSumCols = kMmaStages * kMmaStageCols;   // the sums stand behind the operands
+constexpr int kMmaMaxCluster = 8;
+static_assert(kMmaSumCols + kMmaTeams * kMmaMaxRows <= kMmaTmemCols, "operands and sums share tensor memory");
+static_assert(kMmaQuads == kChunkCells, "a block is a chunk of cells");
 
 struct MmaArgs {
-    const uint32_t* dir;     // block directory (16-byte units into recs)
-    const uint8_t* recs;     // block records
+    const uint32_t* off;     // [4 * blocks + 1] cells' places (32-byte units into `cells`)
+    const unsigned char* cells;
     const uint16_t* X;       // [N, K] bf16
     void* Y;                 // [N, M] bf16 or fp32
-    float* partial;          // [kMmaMaxRows, P * 128] fp32, zero on entry and on exit
-    unsigned int* done;      // [P] blocks of each row panel accounted for, zero on entry and on exit
     int M, K, N, npad;       // npad: N rounded up to a multiple of 16
-    int P, KC;               // row panels, blocks per panel
-    long long NB;            // P * KC
+    int KB;                  // blocks of a panel
+    int shares;              // CTAs of a cluster
     int y_f32;
-    int stages;              // operand tiles in flight: 6 or 8 (what shared memory allows)
-    int slot_bytes, n_slots; // ring geometry
-    int batch;               // block records per bulk copy and ring slot (1, 2, 4 or 8): a copy is worth issuing
-                             // only every few hundred cycles, so records travel several at a time
-    int x_tma;               // 1: the producer fetches X through the tensor map; 0: the groups fetch it
+    int slot_bytes, n_slots; // ring
+    int x_tma;               // 1: X comes through the tensor map; 0: the teams fetch it
     int x_vec;               // x_tma == 0: rows of X can be fetched in 16-byte pieces
     int* err;
     long long budget;        // clock cycles a wait may take
 };
 
 struct MmaShared {
-    unsigned long long full[kMmaSlots];       // a batch of block records landed
-    unsigned long long empty[kMmaSlots];      // ... and has been expanded
-    unsigned long long a_full[kMmaPairs];     // both operand tiles of a stage pair are ready and their X columns landed
-    unsigned long long st_empty[kMmaPairs];   // the MMAs that read the stage pair have completed
-    uint32_t boff[kMmaSlots][kMmaMaxBatch];   // byte offset of each record inside its slot
-    unsigned long long acc_full[2];           // a row panel's sums are complete in tensor memory
-    unsigned long long acc_empty[2];          // ... and have been read out
-    unsigned long long drain;                 // exit: nothing of ours is left in the tensor pipe
+    unsigned long long full[kMmaMaxSlots];    // a block landed
+    unsigned long long empty[kMmaMaxSlots];   // ... and has been expanded
+    unsigned long long xfull[kMmaStages];     // a block's activations have landed
+    unsigned long long afull[kMmaStages];     // a block is in tensor memory
+    unsigned long long aempty[kMmaStages];    // the products of a block are done
+    unsigned long long done;                  // all products are (one arrival per team)
+    unsigned long long rfull;                 // the other CTAs' sums have landed
     uint32_t tmem_base;
-    uint32_t issued;                          // batches whose copy has been issued: a team looks at a slot's barrier only
-                                              // once its batch is on the way, so that a parity always means one phase
     int abort_flag;
-    int last_flag;
     int never_flag;                           // stays 0: the exit waits must not be cut short by abort_flag
 };
+
+// activation rows are written by the CTAs of a cluster in turn, four at a time; how many such fours a CTA has at most
+__host__ __device__ constexpr int mma_own_fours(int npad, int shares) { return (npad / 4 + shares - 1) / shares; }
+// room for the others' sums: per CTA of the cluster and four rows 128 x 4 fp32
+__host__ __device__ constexpr int mma_recv_bytes(int npad, int shares) { return shares > 1 ? shares * mma_own_fours(npad, shares) * kMmaBlockRows * 16 : 0; }
 
 __device__ __forceinline__ void sts_u16(uint32_t a, uint32_t v)
 {
     asm volatile("st.shared.u16 [%0], %1;" ::"r"(a), "h"((uint16_t)v) : "memory");
 }
-__device__ __forceinline__ void sts_zero16(uint32_t a)
+__device__ __forceinline__ void sts_v4(uint32_t a, uint4 v)
 {
-    asm volatile("st.shared.v4.u32 [%0], {%1,%1,%1,%1};" ::"r"(a), "r"(0u) : "memory");
+    asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
-// 16 bytes global -> shared, of which only the first `src_bytes` are read (the rest is zero-filled)
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t src_bytes)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// c + 2 * byte K8 of p
-template <int K8>
-__device__ __forceinline__ uint32_t byte_times_2_plus(uint32_t p, uint32_t c)
-{
-    uint32_t d;
-    asm("dp4a.u32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(p), "r"(0x2u << (8 * K8)), "r"(c));
-    return d;
-}
 
 // Shared-memory matrix descriptor of a K-major bf16 tile under the 128-byte swizzle: rows of 128
 // bytes, groups of eight rows 1024 bytes apart.  Stepping K by 16 elements inside the 64-column
@@ -128,13 +117,13 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr)
     return d;
 }
 
-// D[128 x npad] (+)= A[128 x 16] B[npad x 16]^T, bf16 in, fp32 out, both operands K-major in shared memory
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
+// D[128 x npad] (+)= A[128 x 16] B[npad x 16]^T, bf16 in, fp32 out, A in tensor memory, B K-major in shared memory
+__device__ __forceinline__ void umma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc, uint32_t accumulate)
 {
     asm volatile(
         "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
+        ::"r"(d_tmem), "r"(a_tmem), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
 // the mbarrier gets one arrival when every tcgen05.mma issued so far by this thread has completed
@@ -142,16 +131,24 @@ __device__ __forceinline__ void umma_commit(uint32_t bar)
 {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16])
+// 32 columns of the warp's 32 lanes
+__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32])
 {
     asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr)
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,%20,%21,%22,%23,%24,"
+        "%25,%26,%27,%28,%29,%30,%31,%32};"
+        ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]),
+          "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]),
+          "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])
         : "memory");
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
 }
+// four columns (the values are there after tmem_ld_wait)
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, float (&r)[4])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];" : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]) : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // one box of the tensor map (64 columns x npad rows of X, swizzled) -> shared memory
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int c0, int c1, uint32_t bar)
@@ -161,46 +158,119 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
                  : "memory");
 }
 
-__global__ void __launch_bounds__(kMmaThreads, 1) mma_kernel(const MmaArgs a, const __grid_constant__ CUtensorMap xmap)
+// The word at shared address `at` if the mask has the bit, and on to the next word; else zero.  (Four instructions a pair.  The cell
+// kernel's load_pairs, which finds four addresses at once, takes five: it keeps fewer warps busy, and latency counts more there.)
+template <int SGN>
+__device__ __forceinline__ uint32_t take_word(uint32_t mask, uint32_t bit, uint32_t& at)
+{
+    uint32_t w;
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 t;\n\tand.b32 t, %2, %3;\n\tsetp.ne.u32 p, t, 0;\n\tmov.b32 %0, 0;\n\t"
+                 "@p ld.shared.u32 %0, [%1];\n\t@p add.u32 %1, %1, %4;\n\t}"
+                 : "=&r"(w), "+r"(at) : "r"(mask), "r"(bit), "r"(SGN > 0 ? 128u : 0xFFFFFF80u) : "memory");
+    return w;
+}
+
+// The cell `q` of a block at shared address `block`: the lane's row, as 32 words of two columns each.
+__device__ __forceinline__ void expand_row(uint32_t block, int q, int lane, uint32_t (&w)[32])
+{
+    // where the cells start: the first one's header tells the heights of all four
+    const uint32_t heights = __ballot_sync(0xFFFFFFFFu, (lds_u8(block + 128u + lane) & 0x80u) != 0);
+    uint32_t H = heights & 63u, before = 0;
+#pragma unroll
+    for (int k = 1; k < kMmaQuads; ++k)
+        if (k <= q) { before += H; H = heights >> (6 * k) & 63u; }
+    const uint32_t cell = block + (uint32_t)q * kCellHeaderBytes + before * 128u;
+    const uint32_t m = lds_u32(cell + 4 * lane), v0 = cell + kCellHeaderBytes;
+    const uint32_t pi = lds_u8(cell + 128u + lane) & 0x7Fu;
+    uint32_t lo = v0 + 4u * lane, hi = v0 + (H - 1u) * 128u + pi;
+#pragma unroll
+    for (int e = 0; e < 16; ++e) {
+        w[e] = take_word<1>(m, 1u << e, lo);
+        w[16 + e] = take_word<-1>(m, 0x10000u << e, hi);
+    }
+}
+
+#ifdef SD2_CHECKED
+__device__ __forceinline__ bool block_fits(uint32_t block, uint32_t bytes, int q, int lane)
+{
+    const uint32_t heights = __ballot_sync(0xFFFFFFFFu, (lds_u8(block + 128u + lane) & 0x80u) != 0);
+    uint32_t total = 0, before = 0;
+    for (int k = 0; k < kMmaQuads; ++k) {
+        if (k == q) before = total;
+        total += heights >> (6 * k) & 63u;
+    }
+    if (kMmaQuads * (uint32_t)kCellHeaderBytes + total * 128u > bytes) return false;
+    const uint32_t cell = block + (uint32_t)q * kCellHeaderBytes + before * 128u, H = heights >> (6 * q) & 63u, m = lds_u32(cell + 4 * lane);
+    return __all_sync(0xFFFFFFFFu, (uint32_t)__popc(m & 0xFFFFu) <= H && (uint32_t)__popc(m >> 16) <= H);
+}
+#endif
+
+// A block's 64 columns of X, rows below N, into the B operand's tile at `xt`, by a team's 128 threads.  (What stands in the
+// tile's other rows reaches only sums that nobody reads.)
+__device__ __forceinline__ void fetch_x(const MmaArgs& a, int k0, uint32_t xt, int t)
+{
+    if (a.x_vec) {
+        for (int i = t; i < a.N * 8; i += 32 * kMmaQuads) {
+            const int n = i >> 3, ch = i & 7;
+            const uint32_t dst = xt + (uint32_t)n * 128u + (uint32_t)((ch ^ (n & 7)) << 4);
+            sts_v4(dst, k0 + ch * 8 < a.K ? __ldcg((const uint4*)(a.X + (size_t)n * a.K + k0 + ch * 8)) : make_uint4(0u, 0u, 0u, 0u));   // K % 8 == 0
+        }
+    } else {
+        for (int i = t; i < a.N * kMmaBlockCols; i += 32 * kMmaQuads) {
+            const int n = i >> 6, c = i & 63;
+            const uint32_t v = k0 + c < a.K ? (uint32_t)__ldcg(a.X + (size_t)n * a.K + k0 + c) : 0u;
+            sts_u16(xt + (uint32_t)n * 128u + (uint32_t)((((c >> 3) ^ (n & 7)) << 4) | ((c & 7) << 1)), v);
+        }
+    }
+}
+
+// activation rows n .. n + 3 of a weight row
+__device__ __forceinline__ void store_four(const MmaArgs& a, int n, int row, const float (&v)[4])
+{
+    if (row >= a.M) return;
+    const size_t at = (size_t)n * a.M + row;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (n + j >= a.N) break;
+        if (a.y_f32) ((float*)a.Y)[at + (size_t)j * a.M] = v[j];
+        else ((uint16_t*)a.Y)[at + (size_t)j * a.M] = f32_to_bf16_rne(v[j]);
+    }
+}
+
+__global__ void __launch_bounds__(kMmaThreads, 1) mma_kernel(const __grid_constant__ MmaArgs a, const __grid_constant__ CUtensorMap xmap)
 {
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;     // swizzled tiles want 1024-byte alignment
     const uint32_t xbytes = (uint32_t)a.npad * 128u;                 // npad rows x 128 bytes
-    const uint32_t abuf0 = base;
-    const uint32_t xbuf0 = base + (uint32_t)a.stages * kMmaTileBytes;
-    const uint32_t ring0 = xbuf0 + (uint32_t)a.stages * xbytes;
+    const uint32_t recv0 = base + (uint32_t)kMmaStages * xbytes;
+    const uint32_t ring0 = recv0 + (uint32_t)mma_recv_bytes(a.npad, a.shares);
     MmaShared* sh = (MmaShared*)(smem_raw + (ring0 - smem_u32(smem_raw)) + (size_t)a.n_slots * a.slot_bytes);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const long long b0 = a.NB * (long long)blockIdx.x / gridDim.x;
-    const long long b1 = a.NB * (long long)(blockIdx.x + 1) / gridDim.x;
-    const int nblk = (int)(b1 - b0);
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, tid >> 5, 0);
+    const int rank = (int)blockIdx.x % a.shares, panel = (int)blockIdx.x / a.shares;
+    const int kb0 = (int)((long long)a.KB * rank / a.shares);
+    const int nblk = (int)((long long)a.KB * (rank + 1) / a.shares) - kb0;      // at least one
     const WaitCtx wc = {&sh->abort_flag, a.budget};
+    const WaitCtx wx = {&sh->never_flag, a.budget};
 
     pdl_let_next_start();
-    if (tid == 0) {
-        for (int i = 0; i < kMmaSlots; ++i) {
-            mbar_init(smem_u32(&sh->full[i]), 1);
-            mbar_init(smem_u32(&sh->empty[i]), (uint32_t)a.batch * kMmaSides);
+    if (tid < kMmaMaxSlots) {
+        mbar_init(smem_u32(&sh->full[tid]), 1);
+        mbar_init(smem_u32(&sh->empty[tid]), kMmaQuads);
+        if (tid < kMmaStages) {
+            mbar_init(smem_u32(&sh->xfull[tid]), 1);
+            mbar_init(smem_u32(&sh->afull[tid]), kMmaQuads);
+            mbar_init(smem_u32(&sh->aempty[tid]), 1);
         }
-        for (int g = 0; g < kMmaPairs; ++g) {
-            // per block of the pair: one arrival from each warp of its team, one from the X copy's expect-tx
-            mbar_init(smem_u32(&sh->a_full[g]), 2u * (kMmaSides + (a.x_tma ? 1u : 0u)));
-            mbar_init(smem_u32(&sh->st_empty[g]), 1);
+        if (tid == 0) {
+            mbar_init(smem_u32(&sh->done), kMmaTeams);
+            mbar_init(smem_u32(&sh->rfull), 1);
+            sh->abort_flag = 0;
+            sh->never_flag = 0;
         }
-        for (int s = 0; s < 2; ++s) {
-            mbar_init(smem_u32(&sh->acc_full[s]), 1);
-            mbar_init(smem_u32(&sh->acc_empty[s]), kMmaEpiWarps);
-        }
-        mbar_init(smem_u32(&sh->drain), 1);
-        sh->abort_flag = 0;
-        sh->issued = 0u;
-        sh->last_flag = 0;
-        sh->never_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (!a.x_tma)   // rows of the X tiles beyond N are never fetched by the groups: they stay zero for the whole launch
-        for (uint32_t o = (uint32_t)tid * 16u; o < (uint32_t)a.stages * xbytes; o += kMmaThreads * 16u) sts_zero16(xbuf0 + o);
     if (warp == kMmaIssueWarp) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh->tmem_base)), "r"(kMmaTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -209,310 +279,193 @@ __global__ void __launch_bounds__(kMmaThreads, 1) mma_kernel(const MmaArgs a, co
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *(volatile uint32_t*)&sh->tmem_base;
+    // waited for before the first store to another CTA of the cluster (which has to run by then)
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
 
-    if (warp != kMmaProducerWarp) pdl_wait();    // (the producer streams block records already)
-    if (warp == kMmaProducerWarp) {
-        // ---------------------------------------------------------------- producer: block records, a batch per copy
-        int issued = 0;                                      // batches
+    if (warp != kMmaWeightWarp) pdl_wait();      // (weights are on their way already)
+    if (warp == kMmaWeightWarp) {
+        // ---------------------------------------------------------------- weights
+        const uint32_t full0 = smem_u32(&sh->full[0]), empty0 = smem_u32(&sh->empty[0]);
+        const uint32_t NS = (uint32_t)a.n_slots;
+        const uint32_t* off = a.off + ((size_t)panel * a.KB + kb0) * kMmaQuads;
+        uint32_t o0 = 0, o1 = 0;                 // the lane's block: its place and its end
+        int i = 0;
         bool ok = true;
-        for (int i0 = 0; i0 < nblk && ok; i0 += 32) {
-            // 33 directory words per round, one load per lane (clamped at the CTA's last block)
-            const uint32_t mine = __ldg(a.dir + b0 + min(i0 + lane, nblk));
-            const uint32_t end32 = __ldg(a.dir + b0 + min(i0 + 32, nblk));
-            for (int j = 0; j < 32 && i0 + j < nblk && ok; j += a.batch) {
-                const uint32_t o0 = __shfl_sync(0xFFFFFFFFu, mine, j);
-                const uint32_t o1 = j + a.batch >= 32 ? end32 : __shfl_sync(0xFFFFFFFFu, mine, (j + a.batch) & 31);
-                const int q = (i0 + j) / a.batch;
-                const int slot = q % a.n_slots;
-                if (q == a.n_slots) pdl_wait();              // (slots are given back by warps that have waited, too)
-                if (lane == 0 && !wait_phase(smem_u32(&sh->empty[slot]), ((uint32_t)(q / a.n_slots) & 1u) ^ 1u, wc)) ok = false;
-                ok = __shfl_sync(0xFFFFFFFFu, ok ? 1 : 0, 0) != 0;
+        // the first blocks, as many as there are slots, are asked for at once, a lane each; then four at a time
+        while (i < nblk) {
+            if ((i & 31) == 0) {
+                const int b = min(i + lane, nblk - 1);
+                o0 = __ldg(off + (size_t)b * kMmaQuads);
+                o1 = __ldg(off + (size_t)(b + 1) * kMmaQuads);
+            }
+            const int n = min(i == 0 ? (int)NS : kMmaTeams, nblk - i);
+            if (i > 0) {
+                if (i == (int)NS) pdl_wait();    // (slots are given back by warps that have waited, which the budget is not meant for)
+                for (int k = 0; k < n && ok; ++k) ok = wait_phase_warp(empty0 + 8u * ((uint32_t)(i + k) % NS), ((uint32_t)(i + k) / NS & 1u) ^ 1u, wc);
                 if (!ok) break;
-                if (lane >= j && lane < j + a.batch) sh->boff[slot][lane - j] = (mine - o0) * 16u;
-                __syncwarp();
-                if (lane == 0) {
-                    const uint32_t bytes = (o1 - o0) * 16u;
-                    const uint32_t fb = smem_u32(&sh->full[slot]);
-                    mbar_expect_tx(fb, bytes);
-                    bulk_g2s(ring0 + (uint32_t)slot * (uint32_t)a.slot_bytes, a.recs + (size_t)o0 * 16, bytes, fb);
-                    *(volatile uint32_t*)&sh->issued = (uint32_t)q + 1u;
-                }
-                issued = q + 1;
             }
+            const int k = lane - (i & 31);
+            if (k >= 0 && k < n) {
+                const uint32_t slot = (uint32_t)(i + k) % NS, bytes = (o1 - o0) * 32u;
+                mbar_expect_tx(full0 + 8u * slot, bytes);
+                bulk_g2s(ring0 + slot * (uint32_t)a.slot_bytes, a.cells + (size_t)o0 * 32, bytes, full0 + 8u * slot);
+            }
+            __syncwarp();
+            i += n;
         }
-        if (lane == 0 && sh->abort_flag) {
-            // leave nothing in flight: every copy issued into a slot's latest round must have landed
-            const WaitCtx wx = {&sh->never_flag, a.budget};
-            for (int q = issued > a.n_slots ? issued - a.n_slots : 0; q < issued; ++q)
-                wait_phase(smem_u32(&sh->full[q % a.n_slots]), (uint32_t)(q / a.n_slots) & 1u, wx);
-        }
+        // (teams that gave up have left blocks on their way; where they did not, these have landed)
+        for (int k = max(0, i - (int)NS); k < i; ++k) wait_landed(full0 + 8u * ((uint32_t)k % NS), (uint32_t)k / NS & 1u, a.budget);
     } else if (warp == kMmaXWarp) {
-        // ---------------------------------------------------------------- producer: X columns
+        // ---------------------------------------------------------------- activations
         if (lane == 0 && a.x_tma) {
-            int kc = (int)(b0 % a.KC);
-            int done_i = 0;
-            for (int i = 0; i < nblk; ++i) {
-                const int st = i % a.stages, pq = st >> 1;
-                if (!(i & 1) && !wait_phase(smem_u32(&sh->st_empty[pq]), ((uint32_t)(i / a.stages) & 1u) ^ 1u, wc)) break;
-                const uint32_t xb = smem_u32(&sh->a_full[pq]);
+            int i = 0;
+            for (; i < nblk; ++i) {
+                const int st = i % kMmaStages;
+                if (i >= kMmaStages && !wait_phase(smem_u32(&sh->aempty[st]), ((uint32_t)(i / kMmaStages) & 1u) ^ 1u, wc)) break;
+                const uint32_t xb = smem_u32(&sh->xfull[st]);
                 mbar_expect_tx(xb, xbytes);
-                tma_load_2d(xbuf0 + (uint32_t)st * xbytes, &xmap, kc * kMmaBlockCols, 0, xb);
-                done_i = i + 1;
-                if (++kc == a.KC) kc = 0;
+                tma_load_2d(base + (uint32_t)st * xbytes, &xmap, (kb0 + i) * kMmaBlockCols, 0, xb);
             }
-            if (sh->abort_flag) {
-                // the copies of the last stages may still be landing: give them the time they need
-                (void)done_i;
-                const long long t0 = clock64();
-                while (clock64() - t0 < 20000) {}
-            }
+            for (int k = max(0, i - kMmaStages); k < i; ++k) wait_phase(smem_u32(&sh->xfull[k % kMmaStages]), (uint32_t)(k / kMmaStages) & 1u, wx);
         }
-    } else if (warp == kMmaIssueWarp) {
-        // ---------------------------------------------------------------- MMA issue
+    } else if (warp >= kMmaIssueWarp) {
+        // ---------------------------------------------------------------- products
         if (lane == 0) {
             // instruction descriptor: fp32 accumulator, bf16 A and B, both K-major, N = npad, M = 128
             const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(a.npad >> 3) << 17) | ((128u >> 4) << 24);
-            const uint64_t adesc0 = umma_desc_sw128(abuf0), xdesc0 = umma_desc_sw128(xbuf0);
-            int seg = 0, pq = 0, kc = (int)(b0 % a.KC);
-            uint32_t par = 0u;                               // parity of the stage pair's current use
-            bool first = true;                               // the next block opens a row panel's run
-            for (int i = 0; i < nblk; i += 2) {
-                const int nb = min(2, nblk - i);
-                const uint32_t fb = smem_u32(&sh->a_full[pq]);
-                if (nb == 1)                                 // an odd tail: nobody fills the pair's second half
-                    for (int k = 0; k < kMmaSides + (a.x_tma ? 1 : 0); ++k) mbar_arrive(fb);
-                if (!wait_phase(fb, par, wc)) break;
+            const uint64_t xdesc0 = umma_desc_sw128(base);
+            const int team = warp - kMmaIssueWarp;
+            const uint32_t d = tmem + (uint32_t)(kMmaSumCols + team * a.npad);
+            for (int i = team; i < nblk; i += kMmaTeams) {
+                const int st = i % kMmaStages;
+                const uint32_t par = (uint32_t)(i / kMmaStages) & 1u;
+                if (a.x_tma && !wait_phase(smem_u32(&sh->xfull[st]), par, wc)) break;
+                if (!wait_phase(smem_u32(&sh->afull[st]), par, wc)) break;
                 tc_fence_after();
-                bool ok = true;
-                for (int h = 0; h < nb; ++h) {
-                    const int st = 2 * pq + h;
-                    const bool last = i + h == nblk - 1 || kc == a.KC - 1;
-                    const int stage = seg & 1;
-                    if (first && !wait_phase(smem_u32(&sh->acc_empty[stage]), (((uint32_t)seg >> 1) & 1u) ^ 1u, wc)) { ok = false; break; }
-                    // descriptors differ in their start address only (16-byte units in the low bits)
-                    const uint64_t ad = adesc0 + (uint64_t)((uint32_t)st * (kMmaTileBytes >> 4));
-                    const uint64_t xd = xdesc0 + (uint64_t)((uint32_t)st * (xbytes >> 4));
-                    const uint32_t d = tmem + (uint32_t)stage * kMmaMaxRows;
+                // descriptors differ in their start address only (16-byte units in the low bits)
+                const uint64_t xd = xdesc0 + (uint64_t)((uint32_t)st * (xbytes >> 4));
+                const uint32_t at = tmem + (uint32_t)(st * kMmaStageCols);
 #pragma unroll
-                    for (int kk = 0; kk < kMmaBlockCols / 16; ++kk)
-                        umma_bf16(d, ad + (uint64_t)(2 * kk), xd + (uint64_t)(2 * kk), idesc, (first && kk == 0) ? 0u : 1u);
-                    first = false;
-                    if (last) {
-                        umma_commit(smem_u32(&sh->acc_full[stage]));
-                        ++seg;
-                        first = true;
-                    }
-                    if (++kc == a.KC) kc = 0;
-                }
-                if (!ok) break;
-                umma_commit(smem_u32(&sh->st_empty[pq]));
-                if (++pq == (a.stages >> 1)) { pq = 0; par ^= 1u; }
+                for (int kk = 0; kk < kMmaBlockCols / 16; ++kk)
+                    umma_bf16_ts(d, at + 8u * kk, xd + (uint64_t)(2 * kk), idesc, (i < kMmaTeams && kk == 0) ? 0u : 1u);
+                umma_commit(smem_u32(&sh->aempty[st]));
             }
-        }
-    } else if (warp < kMmaEpiWarps) {
-        // ---------------------------------------------------------------- epilogue
-        const int et = tid;                                  // 0..127: row of the panel
-        const size_t mpad = (size_t)a.P * kMmaBlockRows;
-        int seg = 0;
-        bool dead = false;   // a wait ran out: no more work, but every named barrier below is still attended
-        for (int i = 0; i < nblk;) {
-            const long long b = b0 + i;
-            const int p = (int)(b / a.KC), kc = (int)(b % a.KC);
-            const int nseg = min(nblk - i, a.KC - kc);
-            const int stage = seg & 1;
-            const int row = p * kMmaBlockRows + et;
-            const bool whole = nseg == a.KC;                 // this CTA had the panel's whole K range
-            if (!dead && !wait_phase(smem_u32(&sh->acc_full[stage]), ((uint32_t)seg >> 1) & 1u, wc)) dead = true;
-            dead = __any_sync(0xFFFFFFFFu, dead);            // the warp stays together: tcgen05.ld is warp-wide
-            if (!dead) {
-                tc_fence_after();
-                const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)stage * kMmaMaxRows;
-                for (int c0 = 0; c0 < a.npad; c0 += 16) {
-                    uint32_t r[16];
-                    tmem_ld16(taddr + (uint32_t)c0, r);
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const int n = c0 + j;
-                        if (n < a.N && row < a.M) {
-                            const float v = __uint_as_float(r[j]);
-                            if (!whole) atomicAdd(a.partial + (size_t)n * mpad + row, v);
-                            else if (a.y_f32) ((float*)a.Y)[(size_t)n * a.M + row] = v;
-                            else ((uint16_t*)a.Y)[(size_t)n * a.M + row] = f32_to_bf16_rne(v);
-                        }
-                    }
-                }
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&sh->acc_empty[stage]));
-            }
-            if (!whole) {
-                __threadfence();
-                named_bar_sync(1, 32 * kMmaEpiWarps);
-                if (et == 0) {
-                    int lastone = 0;
-                    if (!dead) {
-                        const unsigned int old = atomicAdd(a.done + p, (unsigned int)nseg);
-                        lastone = (old + (unsigned int)nseg == (unsigned int)a.KC) ? 1 : 0;
-                    }
-                    sh->last_flag = lastone;
-                }
-                named_bar_sync(1, 32 * kMmaEpiWarps);
-                if (sh->last_flag) {
-                    // every part of the panel is in: round, write Y, leave the buffer clean (loads in batches of 8)
-                    __threadfence();
-                    if (row < a.M) {
-                        for (int n0 = 0; n0 < a.N; n0 += 8) {
-                            float v[8];
-#pragma unroll
-                            for (int j = 0; j < 8; ++j) v[j] = (n0 + j < a.N) ? __ldcg(a.partial + (size_t)(n0 + j) * mpad + row) : 0.f;
-#pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                const int n = n0 + j;
-                                if (n < a.N) {
-                                    a.partial[(size_t)n * mpad + row] = 0.f;
-                                    if (a.y_f32) ((float*)a.Y)[(size_t)n * a.M + row] = v[j];
-                                    else ((uint16_t*)a.Y)[(size_t)n * a.M + row] = f32_to_bf16_rne(v[j]);
-                                }
-                            }
-                        }
-                    }
-                    if (et == 0) a.done[p] = 0u;
-                }
-                named_bar_sync(1, 32 * kMmaEpiWarps);        // last_flag is rewritten by the next segment
-            }
-            ++seg;
-            i += nseg;
+            // (nothing of this CTA is left in the tensor pipe when this has been waited for)
+            umma_commit(smem_u32(&sh->done));
+            wait_phase(smem_u32(&sh->done), 0u, wx);
         }
     } else {
         // ---------------------------------------------------------------- expanding teams
-        const int tm = (warp - kMmaFirstGroupWarp) >> 1, side = (warp - kMmaFirstGroupWarp) & 1;
-        const int tt = side * 32 + lane;                     // thread of the team
-        const uint32_t lt = (1u << lane) - 1u;
-        bool dead = false;   // a wait ran out: no more work, but the team's barrier is still attended
-        // block i goes to team i % stages and to stage i % stages: a stage is always refilled by the team that
-        // filled it before, so its barrier is never looked at more than one phase early (teams beyond the stage
-        // count stay idle)
-        for (int i = tm; tm < a.stages && i < nblk; i += a.stages) {
-            const int st = i % a.stages, pq = st >> 1;
-            const uint32_t at = abuf0 + (uint32_t)st * kMmaTileBytes, xt = xbuf0 + (uint32_t)st * xbytes;
-            if (!dead && !wait_phase(smem_u32(&sh->st_empty[pq]), ((uint32_t)(i / a.stages) & 1u) ^ 1u, wc)) dead = true;
-            dead = __any_sync(0xFFFFFFFFu, dead);            // the warp stays together
-            if (dead) {
-                named_bar_sync(2 + tm, 64);
-                continue;
-            }
-            if (!a.x_tma) {
-                // the block's 64 columns of X, rows < N, into the swizzled B tile
-                const int k0 = (int)((b0 + i) % a.KC) * kMmaBlockCols;
-                if (a.x_vec) {
-                    for (int q = tt; q < a.N * 8; q += 64) {
-                        const int n = q >> 3, ch = q & 7;
-                        const uint32_t dst = xt + (uint32_t)n * 128u + (uint32_t)((ch ^ (n & 7)) << 4);
-                        if (k0 + ch * 8 < a.K) cp_async16(dst, a.X + (size_t)n * a.K + k0 + ch * 8, 16u);   // K % 8 == 0
-                        else sts_zero16(dst);
-                    }
-                } else {
-                    for (int q = tt; q < a.N * kMmaBlockCols; q += 64) {
-                        const int n = q >> 6, c = q & 63;
-                        const uint32_t v = (k0 + c < a.K) ? (uint32_t)a.X[(size_t)n * a.K + k0 + c] : 0u;
-                        sts_u16(xt + (uint32_t)n * 128u + (uint32_t)((((c >> 3) ^ (n & 7)) << 4) | ((c & 7) << 1)), v);
-                    }
-                }
-            }
-            // a clean tile: kept entries are scattered into zeros (each warp clears half of the rows)
+        const int q = warp % kMmaQuads, team = warp / kMmaQuads;
+        const uint32_t full0 = smem_u32(&sh->full[0]), empty0 = smem_u32(&sh->empty[0]);
+        const uint32_t NS = (uint32_t)a.n_slots;
+        bool ok = true;
+        uint32_t slot = (uint32_t)team, par = 0u;
+        for (int i = team; i < nblk; i += kMmaTeams) {
+            const int st = i % kMmaStages;
+            if (!(ok = wait_phase_warp(full0 + 8u * slot, par, wc))) break;
+            uint32_t w[32];
+#ifdef SD2_CHECKED
+            // checked build: the cells of a block must lie inside its slot, a lane's words inside its cell; a violation is recorded in the
+            // error word (value 2) and the block skipped
+            if (!block_fits(ring0 + slot * (uint32_t)a.slot_bytes, (uint32_t)a.slot_bytes, q, lane)) {
+                if (lane == 0 && a.err) atomicExch(a.err, 2);
 #pragma unroll
-            for (int j = 0; j < kMmaTileBytes / (16 * 64); ++j) sts_zero16(at + (uint32_t)(j * 64 + tt) * 16u);
-            named_bar_sync(2 + tm, 64);
-
-            const int q = i / a.batch, slot = q % a.n_slots;
-            {
-                // not before the batch's copy is on its way (the slot's earlier phases are then over)
-                const long long t0 = clock64();
-                uint32_t it = 0;
-                while (*(volatile uint32_t*)&sh->issued <= (uint32_t)q) {
-                    if ((++it & 63u) == 0u && (sh->abort_flag || clock64() - t0 > a.budget)) {
-                        sh->abort_flag = 1;
-                        dead = true;
-                        break;
-                    }
-                }
-            }
-            if (!dead && !wait_phase(smem_u32(&sh->full[slot]), (uint32_t)(q / a.n_slots) & 1u, wc)) dead = true;
-            dead = __any_sync(0xFFFFFFFFu, dead);
-            if (dead) continue;
-            const uint32_t rec = ring0 + (uint32_t)slot * (uint32_t)a.slot_bytes + sh->boff[slot][i % a.batch];
-            const int steps = (int)lds_u16(rec + 8u + 2u * (uint32_t)side);
-            const int cnt = (int)((lds_u32(rec + 16u + 32u * (uint32_t)side + ((uint32_t)lane & ~3u)) >> (8 * (lane & 3))) & 0xFFu);
-            uint32_t w = rec + (side ? lds_u32(rec + 12u) : (uint32_t)kMmaBlockHeaderBytes);
-            uint32_t cur = at + 4u * (uint32_t)lane + 2u * (uint32_t)side;       // row 0 of this lane's piece
-#ifdef SD2_CHECKED
-            // checked build: what the record says must stay inside its ring slot, and every store inside the tile;
-            // a violation is recorded in the error word (value 2) and the access is skipped
-            const uint32_t slot_end = ring0 + (uint32_t)(slot + 1) * (uint32_t)a.slot_bytes;
-            bool bad = steps > 2 * kMmaBlockRows / 8 || cnt > steps || w < rec || w > slot_end;
+                for (int k = 0; k < 32; ++k) w[k] = 0u;
+            } else
 #endif
-            for (int j = 0; j < steps; ++j) {
-                const bool active = cnt > j;
-                const uint32_t m = __ballot_sync(0xFFFFFFFFu, active);
-                const uint32_t nj = (uint32_t)__popc(m);
-#ifdef SD2_CHECKED
-                bad = bad || w + ((4u * nj + 15u) & ~15u) + 16u * nj > slot_end;
-                bad = __any_sync(0xFFFFFFFFu, bad);
-                if (bad) {
-                    if (lane == 0 && a.err) atomicExch(a.err, 2);
-                    break;
-                }
-#endif
-                if (active) {
-                    const uint32_t idx = (uint32_t)__popc(m & lt);
-                    const uint32_t code = lds_u32(w + 4u * idx);
-                    const uint4 v = lds_v4(w + ((4u * nj + 15u) & ~15u) + 16u * idx);
-                    const uint32_t lo = code & 0x0F0F0F0Fu, hi = (code >> 4) & 0x0F0F0F0Fu;
-                    const uint32_t po = (lo + hi) * 0x01010101u;        // byte k: gaps summed through entry 2k + 1
-                    const uint32_t pe = po - hi;                       // byte k: ... through entry 2k
-                    const uint32_t a0 = byte_times_128_plus<0>(pe, cur), a1 = byte_times_128_plus<0>(po, cur);
-                    const uint32_t a2 = byte_times_128_plus<1>(pe, cur), a3 = byte_times_128_plus<1>(po, cur);
-                    const uint32_t a4 = byte_times_128_plus<2>(pe, cur), a5 = byte_times_128_plus<2>(po, cur);
-                    const uint32_t a6 = byte_times_128_plus<3>(pe, cur), a7 = byte_times_128_plus<3>(po, cur);
-#ifdef SD2_CHECKED
-                    if (a0 < at || a7 >= at + (uint32_t)kMmaTileBytes) {
-                        if (a.err) atomicExch(a.err, 2);
-                    } else
-#endif
-                    {
-                        sts_u16(a0, v.x); sts_u16(a1, v.x >> 16);
-                        sts_u16(a2, v.y); sts_u16(a3, v.y >> 16);
-                        sts_u16(a4, v.z); sts_u16(a5, v.z >> 16);
-                        sts_u16(a6, v.w); sts_u16(a7, v.w >> 16);
-                        cur = a7;
-                    }
-                }
-                w += ((4u * nj + 15u) & ~15u) + 16u * nj;
-            }
+            expand_row(ring0 + slot * (uint32_t)a.slot_bytes, q, lane, w);
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&sh->empty[slot]));
-            if (!a.x_tma) cp_async_wait_all();
-            fence_async_smem();
+            mbar_arrive_n(empty0 + 8u * slot, 1u, lane == 0);
+            if ((slot += kMmaTeams) >= NS) { slot = (uint32_t)team; par ^= 1u; }
+            if (i >= kMmaStages && !(ok = wait_phase_warp(smem_u32(&sh->aempty[st]), ((uint32_t)(i / kMmaStages) & 1u) ^ 1u, wc))) break;
+            tc_fence_after();
+            tmem_st32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(st * kMmaStageCols), w);
+            if (!a.x_tma) {
+                fetch_x(a, (kb0 + i) * kMmaBlockCols, base + (uint32_t)st * xbytes, 32 * q + lane);
+                fence_async_smem();
+            }
+            tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(smem_u32(&sh->a_full[pq]));
+            mbar_arrive_n(smem_u32(&sh->afull[st]), 1u, lane == 0);
         }
-        cp_async_wait_all();
+        if (ok) ok = wait_phase_warp(smem_u32(&sh->done), 0u, wc);
+        tc_fence_after();
+        // A team has a quarter of the activation rows, four at a time: rows 4 f .. 4 f + 3 (f = team * fours + k) of weight row
+        // 32 q + lane.  They belong to CTA f % C of the cluster.  (Loops, not runs of code: what is gone through once comes from L2,
+        // and 500 instructions of it took 2 us.)
+        const int teams = min(nblk, kMmaTeams), fours = a.npad / (4 * kMmaTeams), C = a.shares;
+        const uint32_t lane_at = (uint32_t)((32 * q + lane) * 16);
+        const uint32_t four_bytes = kMmaBlockRows * 16, cta_bytes = (uint32_t)mma_own_fours(a.npad, C) * four_bytes;
+        if (C > 1) {
+            // (all CTAs of the cluster run, and their mbarriers are there)
+            asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+            if (warp == 0 && lane == 0) mbar_expect_tx(smem_u32(&sh->rfull), (uint32_t)((C - 1) * ((a.npad / 4 - rank + C - 1) / C)) * four_bytes);
+        }
+#pragma unroll 1
+        for (int k = 0; k < fours && ok; ++k) {
+            const int f = team * fours + k, owner = f % C;
+            const uint32_t t = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(kMmaSumCols + 4 * f);
+            float s[kMmaTeams][4];
+#pragma unroll
+            for (int g = 0; g < kMmaTeams; ++g) {
+                if (g < teams) tmem_ld4(t + (uint32_t)(g * a.npad), s[g]);
+                else s[g][0] = s[g][1] = s[g][2] = s[g][3] = 0.f;
+            }
+            tmem_ld_wait();
+            float v[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) v[j] = (s[0][j] + s[1][j]) + (s[2][j] + s[3][j]);
+            const uint32_t at = recv0 + (uint32_t)rank * cta_bytes + (uint32_t)(f / C) * four_bytes + lane_at;
+            if (C == 1) {
+                store_four(a, 4 * f, panel * kMmaBlockRows + 32 * q + lane, v);
+            } else if (owner == rank) {
+                sts_v4(at, make_uint4(__float_as_uint(v[0]), __float_as_uint(v[1]), __float_as_uint(v[2]), __float_as_uint(v[3])));
+            } else {
+                uint32_t to, bar;
+                asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(to) : "r"(at), "r"(owner));
+                asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(bar) : "r"(smem_u32(&sh->rfull)), "r"(owner));
+                st_async(to, v, bar);
+            }
+        }
+        tc_fence_before();
+        if (C > 1) {
+            named_bar_sync(1, 32 * kMmaExpandWarps);                             // the sums that this CTA keeps
+            if (ok) ok = wait_phase_warp(smem_u32(&sh->rfull), 0u, wc);          // ... and gets
+#pragma unroll 1
+            for (int f = rank + C * team; f < a.npad / 4 && ok; f += C * kMmaTeams) {
+                const uint32_t at = recv0 + (uint32_t)(f / C) * four_bytes + lane_at;
+                float v[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 2
+                for (int r = 0; r < C; ++r) {                                    // in the order of the columns, whatever came first
+                    const uint4 o = lds_v4(at + (uint32_t)r * cta_bytes);
+                    v[0] += __uint_as_float(o.x);
+                    v[1] += __uint_as_float(o.y);
+                    v[2] += __uint_as_float(o.z);
+                    v[3] += __uint_as_float(o.w);
+                }
+                store_four(a, 4 * f, panel * kMmaBlockRows + 32 * q + lane, v);
+            }
+        }
     }
 
     // ---------------------------------------------------------------- exit
+    // Nobody leaves while another CTA may still write to its memory: a CTA that has got its sums may go (threads that are gone count
+    // as arrived), one that gave up waits for the others.
+    __syncwarp();
+    if (a.shares == 1 || warp >= kMmaExpandWarps) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     tc_fence_before();
     __syncthreads();
     if (warp == kMmaIssueWarp) {
-        if (sh->abort_flag && lane == 0) {
-            // MMAs may still be running on tiles and columns that are about to go away
-            umma_commit(smem_u32(&sh->drain));
-            wait_phase(smem_u32(&sh->drain), 0u, WaitCtx{&sh->never_flag, a.budget});
-        }
-        __syncwarp();
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kMmaTmemCols) : "memory");
     }
-    if (tid == 0 && sh->abort_flag && a.err) atomicExch(a.err, 1);
+    if (*(volatile int*)&sh->abort_flag) {
+        if (tid == 0 && a.err) atomicExch(a.err, 1);
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
 }
 
 }  // namespace sd2
