@@ -298,17 +298,6 @@ struct RunDeal {
 
 // ---- expanding a cell -----------------------------------------------------------------
 
-// c + 128 * byte K8 of p (SGN = 1) or c - 128 * byte K8 of p (SGN = -1): one integer dot-product instruction
-template <int SGN, int K8>
-__device__ __forceinline__ uint32_t byte_times_128(uint32_t p, uint32_t c)
-{
-    uint32_t d;
-    constexpr uint32_t kWeight = 0x80u << (8 * K8);              // one byte: 128, or -128 where it counts as signed
-    if (SGN > 0) asm("dp4a.u32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(p), "r"(kWeight), "r"(c));
-    else asm("dp4a.u32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(p), "r"(kWeight), "r"(c));
-    return d;
-}
-
 // d = A B, from zero
 __device__ __forceinline__ void mma_rows(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
 {
@@ -324,23 +313,18 @@ __device__ __forceinline__ void add_rows(float (&d)[4], const float (&s)[4])
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "f"(s[0]), "f"(s[1]), "f"(s[2]), "f"(s[3]));
 }
 
-// One unit of a row: its four pairs' words, zero where a pair has none.  nib: the unit's mask bits; at: shared address of
-// the row's next word (words 128 bytes apart, upward for SGN = 1), moved on.
+// The word at shared address `at` if the mask has the bit, and on to the next word (128 bytes upward for SGN = 1, else downward); else
+// zero.  Four instructions a pair.  Four addresses at a time by prefix sums of the mask's bits (dp4a) take five; an eight-row step of
+// two blocks of 2048/512/8192 took 68.6 us with them and takes 67.6, a block of 3072/1024/8192 for 16 rows 61.9 and 60.2, 48 rows of
+// 8192 x 2048 25.9 and 25.5.
 template <int SGN>
-__device__ __forceinline__ void load_pairs(uint32_t nib, uint32_t& at, uint32_t (&w)[4])
+__device__ __forceinline__ uint32_t take_word(uint32_t mask, uint32_t bit, uint32_t& at)
 {
-    // byte i: words of pairs 0..i
-    const uint32_t upto = ((nib * 0x00204081u) & 0x01010101u) * 0x01010101u;
-    const uint32_t a1 = byte_times_128<SGN, 0>(upto, at), a2 = byte_times_128<SGN, 1>(upto, at), a3 = byte_times_128<SGN, 2>(upto, at);
-    asm volatile("{\n\t.reg .pred p0, p1, p2, p3;\n\t.reg .b32 t0, t1, t2, t3;\n\t"
-                 "and.b32 t0, %8, 1;\n\tand.b32 t1, %8, 2;\n\tand.b32 t2, %8, 4;\n\tand.b32 t3, %8, 8;\n\t"
-                 "setp.ne.u32 p0, t0, 0;\n\tsetp.ne.u32 p1, t1, 0;\n\tsetp.ne.u32 p2, t2, 0;\n\tsetp.ne.u32 p3, t3, 0;\n\t"
-                 "mov.b32 %0, 0;\n\tmov.b32 %1, 0;\n\tmov.b32 %2, 0;\n\tmov.b32 %3, 0;\n\t"
-                 "@p0 ld.shared.u32 %0, [%4];\n\t@p1 ld.shared.u32 %1, [%5];\n\t@p2 ld.shared.u32 %2, [%6];\n\t@p3 ld.shared.u32 %3, [%7];\n\t}"
-                 : "=&r"(w[0]), "=&r"(w[1]), "=&r"(w[2]), "=&r"(w[3])
-                 : "r"(at), "r"(a1), "r"(a2), "r"(a3), "r"(nib)
-                 : "memory");
-    at = byte_times_128<SGN, 3>(upto, at);
+    uint32_t w;
+    asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 t;\n\tand.b32 t, %2, %3;\n\tsetp.ne.u32 p, t, 0;\n\tmov.b32 %0, 0;\n\t"
+                 "@p ld.shared.u32 %0, [%1];\n\t@p add.u32 %1, %1, %4;\n\t}"
+                 : "=&r"(w), "+r"(at) : "r"(mask), "r"(bit), "r"(SGN > 0 ? 128u : 0xFFFFFF80u) : "memory");
+    return w;
 }
 
 // One cell: eight mma steps for each eight activation rows.  m: the lane's mask; lo, hi: shared addresses of the first
@@ -358,8 +342,11 @@ __device__ __forceinline__ void multiply_cell(uint32_t m, uint32_t lo, uint32_t 
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         uint32_t a[4], b[4];
-        load_pairs<1>((m >> (4 * u)) & 0xFu, lo, a);
-        load_pairs<-1>((m >> (16 + 4 * u)) & 0xFu, hi, b);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            a[i] = take_word<1>(m, 1u << (4 * u + i), lo);
+            b[i] = take_word<-1>(m, 0x10000u << (4 * u + i), hi);
+        }
 #pragma unroll
         for (int h = 0; h < NR / 8; ++h) {
             const uint4 x = lds_v4(xo[h] + xd + 64u * u);

@@ -158,18 +158,6 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
                  : "memory");
 }
 
-// The word at shared address `at` if the mask has the bit, and on to the next word; else zero.  (Four instructions a pair.  The cell
-// kernel's load_pairs, which finds four addresses at once, takes five: it keeps fewer warps busy, and latency counts more there.)
-template <int SGN>
-__device__ __forceinline__ uint32_t take_word(uint32_t mask, uint32_t bit, uint32_t& at)
-{
-    uint32_t w;
-    asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 t;\n\tand.b32 t, %2, %3;\n\tsetp.ne.u32 p, t, 0;\n\tmov.b32 %0, 0;\n\t"
-                 "@p ld.shared.u32 %0, [%1];\n\t@p add.u32 %1, %1, %4;\n\t}"
-                 : "=&r"(w), "+r"(at) : "r"(mask), "r"(bit), "r"(SGN > 0 ? 128u : 0xFFFFFF80u) : "memory");
-    return w;
-}
-
 // The cell `q` of a block at shared address `block`: the lane's row, as 32 words of two columns each.
 __device__ __forceinline__ void expand_row(uint32_t block, int q, int lane, uint32_t (&w)[32])
 {
