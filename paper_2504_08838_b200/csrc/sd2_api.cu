@@ -1695,7 +1695,8 @@ sd2_status sd2_embedding(const int32_t* tokens, const void* table, void* x, int6
     if (!tokens || !table || !x) return SD2_ERR_INVALID_ARG;
     if (N < 0 || V < 1 || H < 1 || N > 0x7FFFFFFF || V > 0x7FFFFFFF || H > 0x7FFFFFFF) return SD2_ERR_SHAPE;
     if (N == 0) return SD2_OK;
-    launch_pdl(embedding_kernel, (unsigned)N, kGlueThreads, 0, (cudaStream_t)cuda_stream, tokens, (const uint16_t*)table, (uint16_t*)x, (int)H, (int)V);
+    const int vec = ((H & 7) == 0 && ((((uintptr_t)table) | ((uintptr_t)x)) & 15) == 0) ? 1 : 0;
+    launch_pdl(embedding_kernel, (unsigned)N, kGlueThreads, 0, (cudaStream_t)cuda_stream, tokens, (const uint16_t*)table, (uint16_t*)x, (int)H, (int)V, vec);
     return cudaGetLastError() == cudaSuccess ? SD2_OK : SD2_ERR_CUDA;
 }
 

@@ -481,20 +481,26 @@ __global__ void __launch_bounds__(kGlueThreads) add_kernel(const uint16_t* a, co
 }
 
 // x[n, :] = table[token[n], :]
-__global__ void __launch_bounds__(kGlueThreads) embedding_kernel(const int32_t* tokens, const uint16_t* table, uint16_t* x, int H, int V)
+__global__ void __launch_bounds__(kGlueThreads) embedding_kernel(const int32_t* tokens, const uint16_t* table, uint16_t* x, int H, int V, int vec)
 {
     pdl_let_next_start();
     pdl_wait();
     const int tok = tokens[blockIdx.x];
-    for (int i = threadIdx.x; i < H; i += blockDim.x)
-        x[(size_t)blockIdx.x * H + i] = (tok >= 0 && tok < V) ? table[(size_t)tok * H + i] : (uint16_t)0;
+    const bool there = tok >= 0 && tok < V;
+    if (vec) {                               // H is a multiple of 8, x and table are 16-byte aligned
+        for (int i = threadIdx.x; i < H / 8; i += blockDim.x)
+            ((uint4*)(x + (size_t)blockIdx.x * H))[i] = there ? ((const uint4*)(table + (size_t)tok * H))[i] : make_uint4(0u, 0u, 0u, 0u);
+        return;
+    }
+    for (int i = threadIdx.x; i < H; i += blockDim.x) x[(size_t)blockIdx.x * H + i] = there ? table[(size_t)tok * H + i] : (uint16_t)0;
 }
 
 // logits[n, v] = sum_h W[v, h] x[n, h]: a warp takes kHeadRowsPerWarp vocabulary rows at a time (as many independent
 // 128-bit loads in flight per lane and column step) of its share of the table, the activation rows sit in shared memory as
 // bf16.  HBM bounds it: 128256 x 2048 takes 80 us for one and two rows (6.5 TB/s), from 102.  What that took:
 //   - even shares of rows per warp; steps of four rows dealt out in turn, 3.4 of them per warp, left warps idle: 94 us;
-//   - 256-byte requests that pass L1 by and four column steps in flight, on three CTAs per SM: 80 us;
+//   - 256-byte requests that pass L1 by and four column steps in flight, on three CTAs per SM: 80 us (asking for the first rows to
+//     be brought to L2 while the launches before still run slowed these down by more than it gave);
 //   - four rows that share what is read of the activations, and fma.rn.f32x2 (the same fp32 sums, even and odd columns
 //     apart): with one row per step every activation row took as long as a pass of its own, four of them 520 us.
 constexpr int kHeadRowsPerWarp = 4;
@@ -519,7 +525,11 @@ __global__ void __launch_bounds__(kGlueThreads, head_ctas(NT)) lm_head_kernel(co
     pdl_wait();
     extern __shared__ uint4 head_x[];        // [NT][H / 8]: zero beyond row N
     const int groups = H / 8;
-    for (int i = threadIdx.x; i < NT * H; i += blockDim.x) ((uint16_t*)head_x)[i] = i < N * H ? x[i] : (uint16_t)0;
+    if ((((uintptr_t)x) & 15) == 0) {
+        for (int i = threadIdx.x; i < NT * groups; i += blockDim.x) head_x[i] = i < N * groups ? ((const uint4*)x)[i] : make_uint4(0u, 0u, 0u, 0u);
+    } else {
+        for (int i = threadIdx.x; i < NT * H; i += blockDim.x) ((uint16_t*)head_x)[i] = i < N * H ? x[i] : (uint16_t)0;
+    }
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const long long warps = (gridDim.x * blockDim.x) >> 5, gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;

@@ -53,6 +53,12 @@ __device__ __forceinline__ uint32_t silu_mul_pair(uint32_t gpair, uint32_t upair
     return d;
 }
 
+// sums of two pairs of bf16 values, each rounded
+__device__ __forceinline__ uint32_t add_bf16_pairs(uint32_t a, uint32_t b)
+{
+    return (uint32_t)f32_to_bf16_rne(bf16_lo(a) + bf16_lo(b)) | (uint32_t)f32_to_bf16_rne(bf16_hi(a) + bf16_hi(b)) << 16;
+}
+
 __device__ __forceinline__ float warp_sum(float v)
 {
 #pragma unroll
@@ -564,6 +570,62 @@ __device__ __forceinline__ void publish_t_slice(int K, int N, const uint32_t* g,
     }
 }
 
+// xl[r] = rmsnorm(x[r] [+ res]) * norm_w for `rows` <= R rows, a thread eight columns (K <= 8 x the consumer threads, everything on
+// 16 bytes).  at: of the first row in res, sum_out and norm_out.  The rows are there for all after the caller's barrier.
+template <int R>
+__device__ __forceinline__ void stage_norm(int K, int rows, const uint16_t* x, const SFold& f, size_t at, uint16_t* xl, int xl_row,
+                                           float (*red)[kConsumerWarps], int ctid)
+{
+    const bool mine = ctid < (K >> 3), pub = blockIdx.x == 0;
+    uint4 v[R];
+    uint4 w = make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        v[r] = make_uint4(0u, 0u, 0u, 0u);
+        if (mine && r < rows) v[r] = __ldcg((const uint4*)(x + (size_t)r * K) + ctid);
+    }
+    if (mine) w = __ldg((const uint4*)f.norm_w + ctid);
+    if (f.res) {
+        uint4 q[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            q[r] = make_uint4(0u, 0u, 0u, 0u);
+            if (mine && r < rows) q[r] = __ldcg((const uint4*)(f.res + at + (size_t)r * K) + ctid);
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            v[r] = make_uint4(add_bf16_pairs(v[r].x, q[r].x), add_bf16_pairs(v[r].y, q[r].y), add_bf16_pairs(v[r].z, q[r].z), add_bf16_pairs(v[r].w, q[r].w));
+            if (mine && pub && f.sum_out && r < rows) ((uint4*)(f.sum_out + at + (size_t)r * K))[ctid] = v[r];
+        }
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const uint32_t u[4] = {v[r].x, v[r].y, v[r].z, v[r].w};
+        float ss = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) ss += bf16_lo(u[j]) * bf16_lo(u[j]) + bf16_hi(u[j]) * bf16_hi(u[j]);
+        ss = warp_sum(ss);
+        if ((ctid & 31) == 0) red[r][ctid >> 5] = ss;
+    }
+    named_bar_sync(1, kConsumerThreads);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        if (!mine || r >= rows) continue;
+        float tot = 0.f;
+#pragma unroll
+        for (int k = 0; k < kConsumerWarps; ++k) tot += red[r][k];
+        const float rs = rsqrtf(tot / (float)K + f.eps);
+        const uint32_t u[4] = {v[r].x, v[r].y, v[r].z, v[r].w}, g[4] = {w.x, w.y, w.z, w.w};
+        uint32_t o[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            o[j] = (uint32_t)f32_to_bf16_rne(bf16_lo(u[j]) * rs * bf16_lo(g[j])) | (uint32_t)f32_to_bf16_rne(bf16_hi(u[j]) * rs * bf16_hi(g[j])) << 16;
+        const uint4 ov = make_uint4(o[0], o[1], o[2], o[3]);
+        ((uint4*)(xl + (size_t)r * xl_row))[ctid] = ov;
+        if (pub && f.norm_out) ((uint4*)(f.norm_out + at + (size_t)r * K))[ctid] = ov;
+    }
+}
+
 // Stages the activations of one stage: xs[plane][window row c][group][W words], a word holding one
 // bf16 (NT = 1, high half) or the bf16 values of two panel rows, with the value of column
 // strip * B - V + c where strip = plane * groups + group % S (for S <= groups the strips repeat
@@ -595,7 +657,13 @@ __device__ __forceinline__ void stage_x(const SStage& st, int N, const uint16_t*
     const int tail_pad = S * B - K + st.V + 48;
     const bool vec = (K % 8 == 0) && ((((uintptr_t)x_src | (uintptr_t)g | (uintptr_t)u | (uintptr_t)t_out) & 15) == 0);
     const bool pub = glue && t_out && blockIdx.x == 0;
+    // Residual and norm where a thread can hold its eight columns of a row from the first load to the last store: input, residual and
+    // gains are asked for together.  (Through shared memory, with two-byte accesses and the loads one after the other, a row of 2048
+    // took 3.4 us from the barrier to the scatter.)
+    const bool held = FOLD && fold && fold->norm_w && vec && !glue && tag == 0u && K <= 8 * kConsumerThreads &&
+                      ((((uintptr_t)fold->res | (uintptr_t)fold->norm_w | (uintptr_t)fold->sum_out | (uintptr_t)fold->norm_out) & 15) == 0);
     for (int n0 = 0; n0 < NT; n0 += kRowsPerPass) {
+        if (held) stage_norm<kRowsPerPass>(K, min(kRowsPerPass, N - n0), x_src + (size_t)n0 * K, *fold, (size_t)(row0 + n0) * K, xlin + st.V, xlin_row, red, ctid);
 #pragma unroll
         for (int r = 0; r < kRowsPerPass; ++r) {
             const int n = n0 + r;
@@ -606,6 +674,7 @@ __device__ __forceinline__ void stage_x(const SStage& st, int N, const uint16_t*
             uint16_t* xl = xb + st.V;
             for (int i = ctid; i < st.V; i += kConsumerThreads) xb[i] = 0;
             for (int i = ctid; i < tail_pad; i += kConsumerThreads) xl[K + i] = 0;
+            if (held) continue;
             if (tag != 0u) {
                 stage_linear_tagged(K, x_src ? (const uint32_t*)x_src + (size_t)n * K : nullptr,
                                     g ? (const uint32_t*)g + (size_t)n * K : nullptr, u ? (const uint32_t*)u + (size_t)n * K : nullptr,
@@ -640,7 +709,7 @@ __device__ __forceinline__ void stage_x(const SStage& st, int N, const uint16_t*
                 }
             }
         }
-        if (FOLD && fold && fold->norm_w) {
+        if (FOLD && !held && fold && fold->norm_w) {
             const SFold& f = *fold;
             // residual and norm on the linear row(s), each thread on the elements it revisits in the second loop
             named_bar_sync(1, kConsumerThreads);

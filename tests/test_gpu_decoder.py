@@ -363,3 +363,32 @@ def test_decoder_block_step_rejects_inconsistent_heads():
     assert e.value.status == sd2.SD2_ERR_SHAPE
     for h in hs:
         sd2.sd2_free(h)
+
+
+@pytest.mark.parametrize("hidden,N", [(256, 1), (512, 2), (512, 3), (4096, 1), (4608, 1)])     # (4608: more than the threads hold)
+def test_folded_norm_is_the_same_through_registers_and_through_shared_memory(hidden, N):
+    # gains that are not on 16 bytes take the row through shared memory; sums are exact, norms differ by the order of one sum
+    shape = synth.DrafterShape("fold", hidden, 128, 256, 1)
+    hs = [sd2.sd2_compress(W, m) for W, m in synth.make_block(3, 0, shape, 0.1)]
+    x = dev(synth.normal_bf16(5, (N, hidden), 1.0))
+    gains = [dev(synth.normal_bf16(6 + i, (hidden,), 1.0)) for i in range(2)]
+    seen = []
+    for shift in (0, 1):
+        store = torch.zeros((2, hidden + 8), dtype=torch.bfloat16, device="cuda")
+        for i in range(2):
+            store[i, shift:shift + hidden] = gains[i]
+        kc, vc = (torch.zeros((N, 5, shape.kv), dtype=torch.bfloat16, device="cuda") for _ in range(2))
+        ws = torch.zeros(sd2.sd2_decoder_workspace_bytes(hs, N) // 2, dtype=torch.bfloat16, device="cuda")
+        y = torch.zeros((N, hidden), dtype=torch.bfloat16, device="cuda")
+        sd2.sd2_decoder_block_step(hs, store[0, shift:shift + hidden], store[1, shift:shift + hidden], x, y, kc, vc, hidden // 64, 2, 4, 1e-5, 1e4, ws)
+        sd2.sd2_stream_check()
+        at, row = sd2.sd2_block_workspace_bytes(hs, N) // 2, (2 * N * hidden + 255) // 256 * 128
+        q = ws[:N * hidden].float()
+        seen.append((q, ws[at:at + N * hidden].float(), ws[at + row:at + row + N * hidden].float()))
+    assert seen[0][1].abs().max() > 0 and seen[0][2].abs().max() > 0
+    # q: 0.1 * hidden terms of 0.02, each off by one bf16 step of its norm at most; norms: one step
+    assert (seen[0][0] - seen[1][0]).abs().max() <= 2.0 ** -7 * (0.02 * 4 * hidden ** 0.5) + 2.0 ** -7 * seen[0][0].abs().max()
+    for k in (1, 2):
+        assert ((seen[0][k] - seen[1][k]).abs() <= 2.0 ** -6 * seen[0][k].abs() + 1e-2).all()
+    for h in hs:
+        sd2.sd2_free(h)
