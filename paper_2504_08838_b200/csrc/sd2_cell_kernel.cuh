@@ -129,7 +129,7 @@ struct CellShared {
     uint2 gate[kPairSlots][NR / 8][32];         // bf16 results of gate tiles, as the finisher's lanes hold them
     float4 recv[kRecvSlots][NR / 8][32];
     int abort_flag;                                     // any warp: a bounded wait ran out
-    float red[2][kCellWarps];                           // FOLD: per-warp partial sums of squares of two rows
+    float red[4][kCellWarps];                           // FOLD: per-warp partial sums of squares of some rows
     CStage stage[2];                                    // descriptors of the current and the next stage
 };
 
@@ -490,6 +490,63 @@ __device__ __noinline__ bool fold_norm(const XRows& r, const SFold& f, const uin
                                        ConsumerSync& sync, const WaitCtx& wc, int ctid)
 {
     const int lane = ctid & 31;
+    // Eight columns of four rows to a thread, from the first load to the last store (input, residual and gains asked for together),
+    // where the rows are on 16 bytes and short enough; the staged copies are written over.
+    constexpr int kHeld = 4;
+    if ((r.ld & 7) == 0 && (c0 & 7) == 0 && (r.K & 7) == 0 && r.ld <= 8 * kCellConsumers &&
+        ((((uintptr_t)xg | (uintptr_t)f.res | (uintptr_t)f.norm_w | (uintptr_t)f.sum_out | (uintptr_t)f.norm_out) & 15) == 0)) {
+        const bool mine = ctid < (r.ld >> 3), own = mine && 8 * ctid >= c0 && 8 * ctid < c0 + r.K;
+        const uint4 w = own ? __ldg((const uint4*)f.norm_w + ctid) : make_uint4(0u, 0u, 0u, 0u);
+        for (int n0 = 0; n0 < r.N; n0 += kHeld) {
+            uint4 v[kHeld];
+#pragma unroll
+            for (int q = 0; q < kHeld; ++q) {
+                const bool there = mine && n0 + q < r.N;
+                v[q] = there ? __ldcg((const uint4*)(xg + (size_t)(n0 + q) * r.ld) + ctid) : make_uint4(0u, 0u, 0u, 0u);
+            }
+            if (f.res) {
+                uint4 a[kHeld];
+#pragma unroll
+                for (int q = 0; q < kHeld; ++q) {
+                    const bool there = mine && n0 + q < r.N;
+                    a[q] = there ? __ldcg((const uint4*)(f.res + (size_t)(row0 + n0 + q) * r.ld) + ctid) : make_uint4(0u, 0u, 0u, 0u);
+                }
+#pragma unroll
+                for (int q = 0; q < kHeld; ++q) {
+                    v[q] = make_uint4(add_bf16_pairs(v[q].x, a[q].x), add_bf16_pairs(v[q].y, a[q].y), add_bf16_pairs(v[q].z, a[q].z), add_bf16_pairs(v[q].w, a[q].w));
+                    if (own && pub && f.sum_out && n0 + q < r.N) ((uint4*)(f.sum_out + (size_t)(row0 + n0 + q) * r.ld))[ctid] = v[q];
+                }
+            }
+            if (!sync(wc, lane)) return false;     // red is free (and the rows are staged)
+#pragma unroll
+            for (int q = 0; q < kHeld; ++q) {
+                const uint32_t u[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
+                float ss = 0.f;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) ss += bf16_lo(u[j]) * bf16_lo(u[j]) + bf16_hi(u[j]) * bf16_hi(u[j]);
+                ss = warp_sum(ss);
+                if (lane == 0) red[q][ctid >> 5] = ss;
+            }
+            if (!sync(wc, lane)) return false;
+#pragma unroll
+            for (int q = 0; q < kHeld; ++q) {
+                if (!own || n0 + q >= r.N) continue;
+                float tot = 0.f;
+#pragma unroll
+                for (int k = 0; k < kCellWarps; ++k) tot += red[q][k];
+                const float rs = rsqrtf(tot / (float)r.ld + f.eps);
+                const uint32_t u[4] = {v[q].x, v[q].y, v[q].z, v[q].w}, g[4] = {w.x, w.y, w.z, w.w};
+                uint32_t o[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    o[j] = (uint32_t)f32_to_bf16_rne(bf16_lo(u[j]) * rs * bf16_lo(g[j])) | (uint32_t)f32_to_bf16_rne(bf16_hi(u[j]) * rs * bf16_hi(g[j])) << 16;
+                const uint4 ov = make_uint4(o[0], o[1], o[2], o[3]);
+                *(uint4*)(r.buf + (size_t)(n0 + q) * r.pitch + 2 * (8 * ctid - c0)) = ov;
+                if (pub && f.norm_out) ((uint4*)(f.norm_out + (size_t)(row0 + n0 + q) * r.ld))[ctid] = ov;
+            }
+        }
+        return true;
+    }
     for (int n0 = 0; n0 < r.N; n0 += 2) {
         if (!sync(wc, lane)) return false;     // the rows are staged; red is free
 #pragma unroll

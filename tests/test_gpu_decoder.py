@@ -365,7 +365,8 @@ def test_decoder_block_step_rejects_inconsistent_heads():
         sd2.sd2_free(h)
 
 
-@pytest.mark.parametrize("hidden,N", [(256, 1), (512, 2), (512, 3), (4096, 1), (4608, 1)])     # (4608: more than the threads hold)
+@pytest.mark.parametrize("hidden,N", [(256, 1), (512, 2), (512, 3), (4096, 1), (4608, 1),      # (4608: more than the threads hold)
+                                      (128, 4), (512, 4), (1024, 6), (3072, 5), (3328, 4)])     # over cells; (3328: the same)
 def test_folded_norm_is_the_same_through_registers_and_through_shared_memory(hidden, N):
     # gains that are not on 16 bytes take the row through shared memory; sums are exact, norms differ by the order of one sum
     shape = synth.DrafterShape("fold", hidden, 128, 256, 1)
