@@ -55,7 +55,9 @@ __device__ __forceinline__ float block_max(float v, float* red)
 }
 
 // y[n, :] = x[n, :] / sqrt(mean(x[n, :]^2) + eps) * w;  one CTA per row.  vec: H is a multiple of 8 and x, w, y are
-// 16-byte aligned, so a thread moves eight values per load (the second pass finds the row in L1)
+// 16-byte aligned, so a thread moves eight values per load; up to H = 8192 it holds its share of row and gains from one round of
+// loads to the stores
+constexpr int kNormHeld = 4;
 __global__ void __launch_bounds__(kGlueThreads) rmsnorm_kernel(const uint16_t* x, const uint16_t* w, uint16_t* y, int H, float eps, int vec)
 {
     pdl_let_next_start();
@@ -64,36 +66,40 @@ __global__ void __launch_bounds__(kGlueThreads) rmsnorm_kernel(const uint16_t* x
     const uint16_t* xr = x + (size_t)blockIdx.x * H;
     uint16_t* yr = y + (size_t)blockIdx.x * H;
     float ss = 0.f;
-    if (vec) {
-        const uint4* x4 = (const uint4*)xr;
-        for (int i = threadIdx.x; i < H / 8; i += blockDim.x) {
-            const uint4 v = x4[i];
-            const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+    if (vec && H <= 8 * kNormHeld * kGlueThreads) {
+        uint4 v[kNormHeld], g[kNormHeld];
+#pragma unroll
+        for (int k = 0; k < kNormHeld; ++k) {
+            const int i = threadIdx.x + k * kGlueThreads;
+            v[k] = i < H / 8 ? ((const uint4*)xr)[i] : make_uint4(0u, 0u, 0u, 0u);
+            g[k] = i < H / 8 ? ((const uint4*)w)[i] : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int k = 0; k < kNormHeld; ++k) {
+            const uint32_t u[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
 #pragma unroll
             for (int j = 0; j < 4; ++j) ss += bf16_lo(u[j]) * bf16_lo(u[j]) + bf16_hi(u[j]) * bf16_hi(u[j]);
         }
-    } else {
-        for (int i = threadIdx.x; i < H; i += blockDim.x) {
-            const float v = bf16_to_f32(xr[i]);
-            ss += v * v;
-        }
-    }
-    const float r = rsqrtf(block_sum(ss, red) / (float)H + eps);
-    if (vec) {
-        const uint4* x4 = (const uint4*)xr;
-        const uint4* w4 = (const uint4*)w;
-        for (int i = threadIdx.x; i < H / 8; i += blockDim.x) {
-            const uint4 v = x4[i], g = w4[i];
-            const uint32_t u[4] = {v.x, v.y, v.z, v.w}, q[4] = {g.x, g.y, g.z, g.w};
+        const float r = rsqrtf(block_sum(ss, red) / (float)H + eps);
+#pragma unroll
+        for (int k = 0; k < kNormHeld; ++k) {
+            const int i = threadIdx.x + k * kGlueThreads;
+            if (i >= H / 8) break;
+            const uint32_t u[4] = {v[k].x, v[k].y, v[k].z, v[k].w}, q[4] = {g[k].x, g[k].y, g[k].z, g[k].w};
             uint32_t o[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j)
                 o[j] = (uint32_t)f32_to_bf16_rne(bf16_lo(u[j]) * r * bf16_lo(q[j])) | ((uint32_t)f32_to_bf16_rne(bf16_hi(u[j]) * r * bf16_hi(q[j])) << 16);
             ((uint4*)yr)[i] = make_uint4(o[0], o[1], o[2], o[3]);
         }
-    } else {
-        for (int i = threadIdx.x; i < H; i += blockDim.x) yr[i] = f32_to_bf16_rne(bf16_to_f32(xr[i]) * r * bf16_to_f32(w[i]));
+        return;
     }
+    for (int i = threadIdx.x; i < H; i += blockDim.x) {
+        const float v = bf16_to_f32(xr[i]);
+        ss += v * v;
+    }
+    const float r = rsqrtf(block_sum(ss, red) / (float)H + eps);
+    for (int i = threadIdx.x; i < H; i += blockDim.x) yr[i] = f32_to_bf16_rne(bf16_to_f32(xr[i]) * r * bf16_to_f32(w[i]));
 }
 
 // s = a + b (rounded to bf16 and stored), y = rmsnorm(s) * w: the residual connection and the norm that follows it in

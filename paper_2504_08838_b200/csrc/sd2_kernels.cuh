@@ -1021,7 +1021,6 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const __grid_
                         if (clock64() - t0 > wc.budget) { sh->abort_flag = 1; break; }
                     }
                 }
-                __threadfence();
             }
             sh->stage_dead = sh->abort_flag;
         }
@@ -1203,12 +1202,11 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const __grid_
             q_mine = __shfl_sync(0xFFFFFFFFu, q_next, 0);
         }
         qbase += (uint32_t)n_cta;
-        // everything this CTA wrote in the stage is visible before it arrives at the barrier
+        // everything this CTA wrote in the stage is visible before it arrives at the barrier: the release covers what the other threads
+        // stored before the named barrier, as the acquire above covers what they load behind it.  (With two fences of their own and a
+        // returning add a block step of four stages took 37.0 us, not 35.2.)
         named_bar_sync(1, kConsumerThreads);
-        if (s + 1 < a.n_stages && ctid == 0 && !a.tagged) {
-            __threadfence();
-            atomicAdd(a.gbar, 1u);
-        }
+        if (s + 1 < a.n_stages && ctid == 0 && !a.tagged) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(a.gbar) : "memory");
     }
     if (s < a.n_stages || sh->abort_flag) {   // a bounded wait ran out somewhere in this CTA
         if (ctid == 0 && a.err) atomicExch(a.err, 1);
