@@ -313,18 +313,20 @@ __device__ __forceinline__ void add_rows(float (&d)[4], const float (&s)[4])
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "f"(s[0]), "f"(s[1]), "f"(s[2]), "f"(s[3]));
 }
 
-// The word at shared address `at` if the mask has the bit, and on to the next word (128 bytes upward for SGN = 1, else downward); else
-// zero.  Four instructions a pair.  Four addresses at a time by prefix sums of the mask's bits (dp4a) take five; an eight-row step of
-// two blocks of 2048/512/8192 took 68.6 us with them and takes 67.6, a block of 3072/1024/8192 for 16 rows 61.9 and 60.2, 48 rows of
-// 8192 x 2048 25.9 and 25.5.
-template <int SGN>
-__device__ __forceinline__ uint32_t take_word(uint32_t mask, uint32_t bit, uint32_t& at)
+// Two words from shared address `lo` upward and two from `hi` downward, 128 bytes apart, where the mask has the bits `bit` and the next,
+// and those 16 above; zero and no step where it has not.  Four instructions a pair.  Four addresses at a time by prefix sums of
+// the mask's bits (dp4a) take five; an eight-row step of two blocks of 2048/512/8192 took 68.6 us with them and takes 67.6, a block
+// of 3072/1024/8192 for 16 rows 61.9 and 60.2, 48 rows of 8192 x 2048 25.9 and 25.5.
+__device__ __forceinline__ void take_words(uint32_t mask, uint32_t bit, uint32_t& lo, uint32_t& hi, uint32_t& a, uint32_t& b, uint32_t& c, uint32_t& d)
 {
-    uint32_t w;
-    asm volatile("{\n\t.reg .pred p;\n\t.reg .b32 t;\n\tand.b32 t, %2, %3;\n\tsetp.ne.u32 p, t, 0;\n\tmov.b32 %0, 0;\n\t"
-                 "@p ld.shared.u32 %0, [%1];\n\t@p add.u32 %1, %1, %4;\n\t}"
-                 : "=&r"(w), "+r"(at) : "r"(mask), "r"(bit), "r"(SGN > 0 ? 128u : 0xFFFFFF80u) : "memory");
-    return w;
+    asm volatile("{\n\t.reg .pred p, q, r, s;\n\t.reg .b32 t, u, v, w;\n\t"
+                 "and.b32 t, %6, %7;\n\tand.b32 u, %6, %8;\n\tand.b32 v, %6, %9;\n\tand.b32 w, %6, %10;\n\t"
+                 "setp.ne.u32 p, t, 0;\n\tsetp.ne.u32 q, u, 0;\n\tsetp.ne.u32 r, v, 0;\n\tsetp.ne.u32 s, w, 0;\n\t"
+                 "mov.b32 %0, 0;\n\tmov.b32 %1, 0;\n\tmov.b32 %2, 0;\n\tmov.b32 %3, 0;\n\t"
+                 "@p ld.shared.u32 %0, [%4];\n\t@q ld.shared.u32 %1, [%5];\n\t@p add.u32 %4, %4, 128;\n\t@q sub.u32 %5, %5, 128;\n\t"
+                 "@r ld.shared.u32 %2, [%4];\n\t@s ld.shared.u32 %3, [%5];\n\t@r add.u32 %4, %4, 128;\n\t@s sub.u32 %5, %5, 128;\n\t}"
+                 : "=&r"(a), "=&r"(b), "=&r"(c), "=&r"(d), "+r"(lo), "+r"(hi)
+                 : "r"(mask), "r"(bit), "r"(bit << 16), "r"(bit << 1), "r"(bit << 17) : "memory");
 }
 
 // One cell: eight mma steps for each eight activation rows.  m: the lane's mask; lo, hi: shared addresses of the first
@@ -343,10 +345,7 @@ __device__ __forceinline__ void multiply_cell(uint32_t m, uint32_t lo, uint32_t 
     for (int u = 0; u < 4; ++u) {
         uint32_t a[4], b[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            a[i] = take_word<1>(m, 1u << (4 * u + i), lo);
-            b[i] = take_word<-1>(m, 0x10000u << (4 * u + i), hi);
-        }
+        for (int i = 0; i < 4; i += 2) take_words(m, 1u << (4 * u + i), lo, hi, a[i], b[i], a[i + 1], b[i + 1]);
 #pragma unroll
         for (int h = 0; h < NR / 8; ++h) {
             const uint4 x = lds_v4(xo[h] + xd + 64u * u);
@@ -486,63 +485,65 @@ struct ConsumerSync {
 // rows[n] = rmsnorm(rows[n] [+ res]) * norm_w on the staged columns, two rows at a time.  The sum of squares is over the
 // whole row: the columns that the other CTA of the cluster stages are read from global memory.  xg: the rows in global
 // memory, from the first column on; c0: first staged column.
+// scratch: shared memory that nobody else uses now.
 __device__ __noinline__ bool fold_norm(const XRows& r, const SFold& f, const uint16_t* xg, int row0, int c0, bool pub, float (*red)[kCellWarps],
+                                       uint16_t* scratch, int scratch_bytes,
                                        ConsumerSync& sync, const WaitCtx& wc, int ctid)
 {
     const int lane = ctid & 31;
-    // Eight columns of four rows to a thread, from the first load to the last store (input, residual and gains asked for together),
-    // where the rows are on 16 bytes and short enough; the staged copies are written over.
+    // Eight columns of up to four rows to a thread, from the first load to the last store (input, residual and gains asked for together,
+    // 16 bytes at a time), where the rows are on 16 bytes and short enough.  Whole rows stand in `scratch` while their squares are added
+    // up, in the order of the loop below; the staged copies are written over.
     constexpr int kHeld = 4;
-    if ((r.ld & 7) == 0 && (c0 & 7) == 0 && (r.K & 7) == 0 && r.ld <= 8 * kCellConsumers &&
+    const int fit = min(kHeld, scratch_bytes / (2 * r.ld));
+    if (fit > 0 && (r.ld & 7) == 0 && r.ld <= 8 * kCellConsumers &&
         ((((uintptr_t)xg | (uintptr_t)f.res | (uintptr_t)f.norm_w | (uintptr_t)f.sum_out | (uintptr_t)f.norm_out) & 15) == 0)) {
         const bool mine = ctid < (r.ld >> 3), own = mine && 8 * ctid >= c0 && 8 * ctid < c0 + r.K;
         const uint4 w = own ? __ldg((const uint4*)f.norm_w + ctid) : make_uint4(0u, 0u, 0u, 0u);
-        for (int n0 = 0; n0 < r.N; n0 += kHeld) {
+        for (int n0 = 0; n0 < r.N; n0 += fit) {
+            const int rows = min(fit, r.N - n0);
+            const size_t at = (size_t)(row0 + n0) * r.ld;
             uint4 v[kHeld];
 #pragma unroll
-            for (int q = 0; q < kHeld; ++q) {
-                const bool there = mine && n0 + q < r.N;
-                v[q] = there ? __ldcg((const uint4*)(xg + (size_t)(n0 + q) * r.ld) + ctid) : make_uint4(0u, 0u, 0u, 0u);
-            }
+            for (int q = 0; q < kHeld; ++q)
+                v[q] = mine && q < rows ? __ldcg((const uint4*)(xg + (size_t)(n0 + q) * r.ld) + ctid) : make_uint4(0u, 0u, 0u, 0u);
             if (f.res) {
                 uint4 a[kHeld];
 #pragma unroll
-                for (int q = 0; q < kHeld; ++q) {
-                    const bool there = mine && n0 + q < r.N;
-                    a[q] = there ? __ldcg((const uint4*)(f.res + (size_t)(row0 + n0 + q) * r.ld) + ctid) : make_uint4(0u, 0u, 0u, 0u);
-                }
+                for (int q = 0; q < kHeld; ++q)
+                    a[q] = mine && q < rows ? __ldcg((const uint4*)(f.res + at + (size_t)q * r.ld) + ctid) : make_uint4(0u, 0u, 0u, 0u);
 #pragma unroll
                 for (int q = 0; q < kHeld; ++q) {
-                    v[q] = make_uint4(add_bf16_pairs(v[q].x, a[q].x), add_bf16_pairs(v[q].y, a[q].y), add_bf16_pairs(v[q].z, a[q].z), add_bf16_pairs(v[q].w, a[q].w));
-                    if (own && pub && f.sum_out && n0 + q < r.N) ((uint4*)(f.sum_out + (size_t)(row0 + n0 + q) * r.ld))[ctid] = v[q];
+                    v[q] = add_bf16_rows(v[q], a[q]);
+                    if (own && pub && f.sum_out && q < rows) ((uint4*)(f.sum_out + at + (size_t)q * r.ld))[ctid] = v[q];
                 }
             }
-            if (!sync(wc, lane)) return false;     // red is free (and the rows are staged)
+#pragma unroll
+            for (int q = 0; q < kHeld; ++q)
+                if (mine && q < rows) ((uint4*)(scratch + (size_t)q * r.ld))[ctid] = v[q];
+            if (!sync(wc, lane)) return false;
 #pragma unroll
             for (int q = 0; q < kHeld; ++q) {
-                const uint32_t u[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
+                if (q >= rows) continue;
                 float ss = 0.f;
-#pragma unroll
-                for (int j = 0; j < 4; ++j) ss += bf16_lo(u[j]) * bf16_lo(u[j]) + bf16_hi(u[j]) * bf16_hi(u[j]);
+                for (int i = ctid; i < r.ld; i += kCellConsumers) {
+                    const float e = bf16_to_f32(scratch[(size_t)q * r.ld + i]);
+                    ss += e * e;
+                }
+                __syncwarp();
                 ss = warp_sum(ss);
                 if (lane == 0) red[q][ctid >> 5] = ss;
             }
             if (!sync(wc, lane)) return false;
 #pragma unroll
             for (int q = 0; q < kHeld; ++q) {
-                if (!own || n0 + q >= r.N) continue;
+                if (!own || q >= rows) continue;
                 float tot = 0.f;
 #pragma unroll
                 for (int k = 0; k < kCellWarps; ++k) tot += red[q][k];
-                const float rs = rsqrtf(tot / (float)r.ld + f.eps);
-                const uint32_t u[4] = {v[q].x, v[q].y, v[q].z, v[q].w}, g[4] = {w.x, w.y, w.z, w.w};
-                uint32_t o[4];
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                    o[j] = (uint32_t)f32_to_bf16_rne(bf16_lo(u[j]) * rs * bf16_lo(g[j])) | (uint32_t)f32_to_bf16_rne(bf16_hi(u[j]) * rs * bf16_hi(g[j])) << 16;
-                const uint4 ov = make_uint4(o[0], o[1], o[2], o[3]);
-                *(uint4*)(r.buf + (size_t)(n0 + q) * r.pitch + 2 * (8 * ctid - c0)) = ov;
-                if (pub && f.norm_out) ((uint4*)(f.norm_out + (size_t)(row0 + n0 + q) * r.ld))[ctid] = ov;
+                const uint4 o = scale_bf16_row(v[q], rsqrtf(tot / (float)r.ld + f.eps), w);
+                *(uint4*)(r.buf + (size_t)(n0 + q) * r.pitch + 2 * (8 * ctid - c0)) = o;
+                if (pub && f.norm_out) ((uint4*)(f.norm_out + at + (size_t)q * r.ld))[ctid] = o;
             }
         }
         return true;
@@ -1110,7 +1111,9 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                 for (int n = 0; n < N && (bulk || !x); ++n)
                     for (int i = Kr + ctid; i < Kp; i += kCellConsumers) *(uint16_t*)(xr.buf + (size_t)n * pitch + 2 * i) = 0;
                 if constexpr (FOLD) {
-                    if (norm && !fold_norm(xr, a.fold[MAXS == 1 ? 0 : s], x + (size_t)a.n0 * K, a.n0, xb, pub, sh->red, sync, wc, ctid)) break;
+                    // (scratch: the places for partial sums; all those of the stage before have been read before the grid barrier let this one begin)
+                    if (norm && !fold_norm(xr, a.fold[MAXS == 1 ? 0 : s], x + (size_t)a.n0 * K, a.n0, xb, pub, sh->red, (uint16_t*)(smem + kPartOff),
+                                           2 * (a.part_mask + 1) * (int)kSlotBytes, sync, wc, ctid)) break;
                 }
                 // (the next stage's rows come here by bulk copies, which do not see these stores in the order of `left` alone)
                 fence_async_smem();

@@ -53,10 +53,24 @@ __device__ __forceinline__ uint32_t silu_mul_pair(uint32_t gpair, uint32_t upair
     return d;
 }
 
-// sums of two pairs of bf16 values, each rounded
+// eight bf16 sums, each rounded
 __device__ __forceinline__ uint32_t add_bf16_pairs(uint32_t a, uint32_t b)
 {
     return (uint32_t)f32_to_bf16_rne(bf16_lo(a) + bf16_lo(b)) | (uint32_t)f32_to_bf16_rne(bf16_hi(a) + bf16_hi(b)) << 16;
+}
+__device__ __forceinline__ uint4 add_bf16_rows(uint4 a, uint4 b)
+{
+    return make_uint4(add_bf16_pairs(a.x, b.x), add_bf16_pairs(a.y, b.y), add_bf16_pairs(a.z, b.z), add_bf16_pairs(a.w, b.w));
+}
+// v * r * g for eight bf16 values and gains
+__device__ __forceinline__ uint4 scale_bf16_row(uint4 v, float r, uint4 g)
+{
+    const uint32_t u[4] = {v.x, v.y, v.z, v.w}, q[4] = {g.x, g.y, g.z, g.w};
+    uint32_t o[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        o[j] = (uint32_t)f32_to_bf16_rne(bf16_lo(u[j]) * r * bf16_lo(q[j])) | (uint32_t)f32_to_bf16_rne(bf16_hi(u[j]) * r * bf16_hi(q[j])) << 16;
+    return make_uint4(o[0], o[1], o[2], o[3]);
 }
 
 __device__ __forceinline__ float warp_sum(float v)
@@ -571,7 +585,8 @@ __device__ __forceinline__ void publish_t_slice(int K, int N, const uint32_t* g,
 }
 
 // xl[r] = rmsnorm(x[r] [+ res]) * norm_w for `rows` <= R rows, a thread eight columns (K <= 8 x the consumer threads, everything on
-// 16 bytes).  at: of the first row in res, sum_out and norm_out.  The rows are there for all after the caller's barrier.
+// 16 bytes).  at: of the first row in res, sum_out and norm_out.  The squares are added up from xl, in the order that the path with
+// two-byte accesses has.  The rows are there for all after the caller's barrier.
 template <int R>
 __device__ __forceinline__ void stage_norm(int K, int rows, const uint16_t* x, const SFold& f, size_t at, uint16_t* xl, int xl_row,
                                            float (*red)[kConsumerWarps], int ctid)
@@ -594,16 +609,22 @@ __device__ __forceinline__ void stage_norm(int K, int rows, const uint16_t* x, c
         }
 #pragma unroll
         for (int r = 0; r < R; ++r) {
-            v[r] = make_uint4(add_bf16_pairs(v[r].x, q[r].x), add_bf16_pairs(v[r].y, q[r].y), add_bf16_pairs(v[r].z, q[r].z), add_bf16_pairs(v[r].w, q[r].w));
+            v[r] = add_bf16_rows(v[r], q[r]);
             if (mine && pub && f.sum_out && r < rows) ((uint4*)(f.sum_out + at + (size_t)r * K))[ctid] = v[r];
         }
     }
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-        const uint32_t u[4] = {v[r].x, v[r].y, v[r].z, v[r].w};
-        float ss = 0.f;
+    for (int r = 0; r < R; ++r)
+        if (mine && r < rows) ((uint4*)(xl + (size_t)r * xl_row))[ctid] = v[r];
+    named_bar_sync(1, kConsumerThreads);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) ss += bf16_lo(u[j]) * bf16_lo(u[j]) + bf16_hi(u[j]) * bf16_hi(u[j]);
+    for (int r = 0; r < R; ++r) {
+        if (r >= rows) continue;
+        float ss = 0.f;
+        for (int i = ctid; i < K; i += kConsumerThreads) {
+            const float e = bf16_to_f32(xl[(size_t)r * xl_row + i]);
+            ss += e * e;
+        }
         ss = warp_sum(ss);
         if ((ctid & 31) == 0) red[r][ctid >> 5] = ss;
     }
@@ -614,15 +635,9 @@ __device__ __forceinline__ void stage_norm(int K, int rows, const uint16_t* x, c
         float tot = 0.f;
 #pragma unroll
         for (int k = 0; k < kConsumerWarps; ++k) tot += red[r][k];
-        const float rs = rsqrtf(tot / (float)K + f.eps);
-        const uint32_t u[4] = {v[r].x, v[r].y, v[r].z, v[r].w}, g[4] = {w.x, w.y, w.z, w.w};
-        uint32_t o[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-            o[j] = (uint32_t)f32_to_bf16_rne(bf16_lo(u[j]) * rs * bf16_lo(g[j])) | (uint32_t)f32_to_bf16_rne(bf16_hi(u[j]) * rs * bf16_hi(g[j])) << 16;
-        const uint4 ov = make_uint4(o[0], o[1], o[2], o[3]);
-        ((uint4*)(xl + (size_t)r * xl_row))[ctid] = ov;
-        if (pub && f.norm_out) ((uint4*)(f.norm_out + at + (size_t)r * K))[ctid] = ov;
+        const uint4 o = scale_bf16_row(v[r], rsqrtf(tot / (float)K + f.eps), w);
+        ((uint4*)(xl + (size_t)r * xl_row))[ctid] = o;
+        if (pub && f.norm_out) ((uint4*)(f.norm_out + at + (size_t)r * K))[ctid] = o;
     }
 }
 
@@ -657,9 +672,8 @@ __device__ __forceinline__ void stage_x(const SStage& st, int N, const uint16_t*
     const int tail_pad = S * B - K + st.V + 48;
     const bool vec = (K % 8 == 0) && ((((uintptr_t)x_src | (uintptr_t)g | (uintptr_t)u | (uintptr_t)t_out) & 15) == 0);
     const bool pub = glue && t_out && blockIdx.x == 0;
-    // Residual and norm where a thread can hold its eight columns of a row from the first load to the last store: input, residual and
-    // gains are asked for together.  (Through shared memory, with two-byte accesses and the loads one after the other, a row of 2048
-    // took 3.4 us from the barrier to the scatter.)
+    // Residual and norm where a thread can hold its eight columns of a row: input, residual and gains are asked for together, 16 bytes
+    // at a time.  (With two-byte accesses and the loads one after the other a row of 2048 took 3.4 us from the barrier to the scatter.)
     const bool held = FOLD && fold && fold->norm_w && vec && !glue && tag == 0u && K <= 8 * kConsumerThreads &&
                       ((((uintptr_t)fold->res | (uintptr_t)fold->norm_w | (uintptr_t)fold->sum_out | (uintptr_t)fold->norm_out) & 15) == 0);
     for (int n0 = 0; n0 < NT; n0 += kRowsPerPass) {

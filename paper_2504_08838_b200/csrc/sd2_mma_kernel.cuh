@@ -172,10 +172,7 @@ __device__ __forceinline__ void expand_row(uint32_t block, int q, int lane, uint
     const uint32_t pi = lds_u8(cell + 128u + lane) & 0x7Fu;
     uint32_t lo = v0 + 4u * lane, hi = v0 + (H - 1u) * 128u + pi;
 #pragma unroll
-    for (int e = 0; e < 16; ++e) {
-        w[e] = take_word<1>(m, 1u << e, lo);
-        w[16 + e] = take_word<-1>(m, 0x10000u << e, hi);
-    }
+    for (int e = 0; e < 16; e += 2) take_words(m, 1u << e, lo, hi, w[e], w[16 + e], w[e + 1], w[17 + e]);
 }
 
 #ifdef SD2_CHECKED
