@@ -137,6 +137,7 @@ constexpr int kMaxDevices = 64;
 constexpr int kBarrierPool = 64;             // grid-barrier word pairs handed out round-robin
 constexpr int kBarrierStrideWords = 64;      // 256 bytes apart
 constexpr int kSmemMax = 227 * 1024;         // dynamic shared memory a CTA may opt in to
+constexpr int kProgramInline = 2;            // a program in device memory for few rows: an instance apart from that of one stage
 constexpr int kMaxBlockRows = 1 << 16;       // activation rows a block step accepts (taken in panels)
 constexpr int kDrafterWordsBytes = 512;      // a drafter's device words: barrier (two lines), then 64 production counts
 
@@ -212,7 +213,7 @@ sd2_status ensure_device(int* dev_out)
         constexpr int kMany = kMaxStagesInline;
         if (set_smem_attr<1, 1>() != cudaSuccess || set_smem_attr<1, 2>() != cudaSuccess || set_smem_attr<1, 4>() != cudaSuccess ||
             set_smem_attr<kMany, 1>() != cudaSuccess || set_smem_attr<kMany, 2>() != cudaSuccess || set_smem_attr<kMany, 4>() != cudaSuccess ||
-            set_cell_attr<1, 8>() != cudaSuccess || set_cell_attr<1, 16>() != cudaSuccess ||
+            set_cell_attr<1, 8>() != cudaSuccess || set_cell_attr<kProgramInline, 8>() != cudaSuccess || set_cell_attr<1, 16>() != cudaSuccess ||
             set_cell_attr<kMany, 8>() != cudaSuccess || set_cell_attr<kMany, 16>() != cudaSuccess ||
             cudaFuncSetAttribute(cell_kernel<1, kWidePanelRows, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
             cudaFuncSetAttribute(mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
@@ -840,9 +841,10 @@ sd2_status run_cell_panels(CArgs<kMaxStagesInline>& a, int64_t N, const CellNeed
     const int64_t panels = (N + cap - 1) / cap;
     const int64_t rows = (N + panels - 1) / panels;
     CArgs<1> one;
+    CArgs<kProgramInline> program = {};
     const bool small = a.n_stages == 1 || a.ext;             // one inline stage is all that the launch reads
     if (small) {
-        one.inl[0] = a.inl[0];
+        program.inl[0] = one.inl[0] = a.inl[0];
         one.fold[0] = a.fold[0];
     }
     for (int64_t n0 = 0; n0 < N; n0 += rows) {
@@ -858,7 +860,8 @@ sd2_status run_cell_panels(CArgs<kMaxStagesInline>& a, int64_t N, const CellNeed
         sd2_status st;
         if (small) {
             static_cast<CArgsBase&>(one) = a;
-            st = a.N > 16 ? launch_wide_cells(one, grid, smem, s) : a.N > 8 ? launch_cells<1, 16>(one, grid, smem, s) : launch_cells<1, 8>(one, grid, smem, s);
+            static_cast<CArgsBase&>(program) = a;
+            st = a.ext && a.N <= 8 ? launch_cells<kProgramInline, 8>(program, grid, smem, s) : a.N > 16 ? launch_wide_cells(one, grid, smem, s) : a.N > 8 ? launch_cells<1, 16>(one, grid, smem, s) : launch_cells<1, 8>(one, grid, smem, s);
         } else {
             st = a.N > 8 ? launch_cells<kMaxStagesInline, 16>(a, grid, smem, s) : launch_cells<kMaxStagesInline, 8>(a, grid, smem, s);
         }
