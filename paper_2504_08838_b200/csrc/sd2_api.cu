@@ -1585,8 +1585,11 @@ sd2_status sd2_rmsnorm(const void* x, const void* w, void* y, int64_t N, int64_t
     if (!x || !w || !y) return SD2_ERR_INVALID_ARG;
     if (N < 0 || H < 1 || N > 0x7FFFFFFF || H > 0x7FFFFFFF) return SD2_ERR_SHAPE;
     if (N == 0) return SD2_OK;
-    const int vec = ((H & 7) == 0 && ((((uintptr_t)x) | ((uintptr_t)w) | ((uintptr_t)y)) & 15) == 0) ? 1 : 0;
-    launch_pdl(rmsnorm_kernel, (unsigned)N, kGlueThreads, 0, (cudaStream_t)cuda_stream, (const uint16_t*)x, (const uint16_t*)w, (uint16_t*)y, (int)H, eps, vec);
+    const bool vec = (H & 7) == 0 && ((((uintptr_t)x) | ((uintptr_t)w) | ((uintptr_t)y)) & 15) == 0;
+    const int64_t loads = (H / 8 + kGlueThreads - 1) / kGlueThreads;       // 16-byte loads of a thread
+    auto* const kernel = !vec ? rmsnorm_kernel<kNormPlain> : loads <= 1 ? rmsnorm_kernel<1> : loads <= 2 ? rmsnorm_kernel<2>
+                       : loads <= 4 ? rmsnorm_kernel<4> : rmsnorm_kernel<kNormLoop>;
+    launch_pdl(kernel, (unsigned)N, kGlueThreads, 0, (cudaStream_t)cuda_stream, (const uint16_t*)x, (const uint16_t*)w, (uint16_t*)y, (int)H, eps);
     return cudaGetLastError() == cudaSuccess ? SD2_OK : SD2_ERR_CUDA;
 }
 

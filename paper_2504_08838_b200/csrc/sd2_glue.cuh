@@ -54,11 +54,23 @@ __device__ __forceinline__ float block_max(float v, float* red)
     return t;
 }
 
-// y[n, :] = x[n, :] / sqrt(mean(x[n, :]^2) + eps) * w;  one CTA per row.  vec: H is a multiple of 8 and x, w, y are
-// 16-byte aligned, so a thread moves eight values per load; up to H = 8192 it holds its share of row and gains from one round of
-// loads to the stores
-constexpr int kNormHeld = 4;
-__global__ void __launch_bounds__(kGlueThreads) rmsnorm_kernel(const uint16_t* x, const uint16_t* w, uint16_t* y, int H, float eps, int vec)
+// the squares of eight values, added to `ss` in the order that every instance below has
+__device__ __forceinline__ float add_squares(float ss, uint4 v)
+{
+    const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) ss += bf16_lo(u[j]) * bf16_lo(u[j]) + bf16_hi(u[j]) * bf16_hi(u[j]);
+    return ss;
+}
+
+// y[n, :] = x[n, :] / sqrt(mean(x[n, :]^2) + eps) * w;  one CTA per row.
+// HELD > 0: H is a multiple of 8 and x, w, y are 16-byte aligned, so a thread moves eight values per load, and holds its share of row
+// and gains, up to HELD such loads of each, from one round of loads to the stores.  kNormLoop: the same for any H; the second pass finds
+// the row in L1.  kNormPlain: two bytes at a time.  What bounds it is the latency of the loads for a few rows and HBM for many, where
+// registers that a narrow row has no use for keep CTAs off the SM: hence an instance for every number of loads.
+constexpr int kNormLoop = 0, kNormPlain = -1;
+template <int HELD>
+__global__ void __launch_bounds__(kGlueThreads) rmsnorm_kernel(const uint16_t* x, const uint16_t* w, uint16_t* y, int H, float eps)
 {
     pdl_let_next_start();
     pdl_wait();
@@ -66,40 +78,34 @@ __global__ void __launch_bounds__(kGlueThreads) rmsnorm_kernel(const uint16_t* x
     const uint16_t* xr = x + (size_t)blockIdx.x * H;
     uint16_t* yr = y + (size_t)blockIdx.x * H;
     float ss = 0.f;
-    if (vec && H <= 8 * kNormHeld * kGlueThreads) {
-        uint4 v[kNormHeld], g[kNormHeld];
+    if constexpr (HELD > 0) {
+        uint4 v[HELD], g[HELD];
 #pragma unroll
-        for (int k = 0; k < kNormHeld; ++k) {
+        for (int k = 0; k < HELD; ++k) {
             const int i = threadIdx.x + k * kGlueThreads;
             v[k] = i < H / 8 ? ((const uint4*)xr)[i] : make_uint4(0u, 0u, 0u, 0u);
             g[k] = i < H / 8 ? ((const uint4*)w)[i] : make_uint4(0u, 0u, 0u, 0u);
         }
 #pragma unroll
-        for (int k = 0; k < kNormHeld; ++k) {
-            const uint32_t u[4] = {v[k].x, v[k].y, v[k].z, v[k].w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) ss += bf16_lo(u[j]) * bf16_lo(u[j]) + bf16_hi(u[j]) * bf16_hi(u[j]);
-        }
+        for (int k = 0; k < HELD; ++k) ss = add_squares(ss, v[k]);
         const float r = rsqrtf(block_sum(ss, red) / (float)H + eps);
 #pragma unroll
-        for (int k = 0; k < kNormHeld; ++k) {
+        for (int k = 0; k < HELD; ++k) {
             const int i = threadIdx.x + k * kGlueThreads;
-            if (i >= H / 8) break;
-            const uint32_t u[4] = {v[k].x, v[k].y, v[k].z, v[k].w}, q[4] = {g[k].x, g[k].y, g[k].z, g[k].w};
-            uint32_t o[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                o[j] = (uint32_t)f32_to_bf16_rne(bf16_lo(u[j]) * r * bf16_lo(q[j])) | ((uint32_t)f32_to_bf16_rne(bf16_hi(u[j]) * r * bf16_hi(q[j])) << 16);
-            ((uint4*)yr)[i] = make_uint4(o[0], o[1], o[2], o[3]);
+            if (i < H / 8) ((uint4*)yr)[i] = scale_bf16_row(v[k], r, g[k]);
         }
-        return;
+    } else if constexpr (HELD == kNormLoop) {
+        for (int i = threadIdx.x; i < H / 8; i += kGlueThreads) ss = add_squares(ss, ((const uint4*)xr)[i]);
+        const float r = rsqrtf(block_sum(ss, red) / (float)H + eps);
+        for (int i = threadIdx.x; i < H / 8; i += kGlueThreads) ((uint4*)yr)[i] = scale_bf16_row(((const uint4*)xr)[i], r, ((const uint4*)w)[i]);
+    } else {
+        for (int i = threadIdx.x; i < H; i += kGlueThreads) {
+            const float v = bf16_to_f32(xr[i]);
+            ss += v * v;
+        }
+        const float r = rsqrtf(block_sum(ss, red) / (float)H + eps);
+        for (int i = threadIdx.x; i < H; i += kGlueThreads) yr[i] = f32_to_bf16_rne(bf16_to_f32(xr[i]) * r * bf16_to_f32(w[i]));
     }
-    for (int i = threadIdx.x; i < H; i += blockDim.x) {
-        const float v = bf16_to_f32(xr[i]);
-        ss += v * v;
-    }
-    const float r = rsqrtf(block_sum(ss, red) / (float)H + eps);
-    for (int i = threadIdx.x; i < H; i += blockDim.x) yr[i] = f32_to_bf16_rne(bf16_to_f32(xr[i]) * r * bf16_to_f32(w[i]));
 }
 
 // s = a + b (rounded to bf16 and stored), y = rmsnorm(s) * w: the residual connection and the norm that follows it in

@@ -52,6 +52,28 @@ def test_rmsnorm(N, H):
     close_bf16(bits_of(y), do.rmsnorm(f64(x), f64(w), EPS), 1e-5)
 
 
+@pytest.mark.parametrize("H", [8224, 16384, 32768])
+def test_rmsnorm_of_wide_rows(H):
+    # rows that threads do not hold in registers; the squares add up in the order that narrower rows have: a row that is zero from a
+    # quarter on has a quarter of the mean, exactly, and twice the values.  (Columns 0..7, 2048..2055 and so on add up in one thread,
+    # next to 65536 they get lost there, pair by pair, and would not in another order.)
+    N, part = 64, H // 4
+    x = synth.normal_bf16(120 + H, (N, H), 1.0)
+    w = synth.normal_bf16(121 + H, (H,), 0.5)
+    y = torch.zeros((N, H), dtype=torch.bfloat16, device="cuda")
+    sd2.sd2_rmsnorm(dev(x), dev(w), y, EPS)
+    torch.cuda.synchronize()
+    close_bf16(bits_of(y), do.rmsnorm(f64(x), f64(w), EPS), 1e-5)
+    x[:, part:] = 0
+    x[:, [c for c in range(part) if c % 2048 < 8]] = 0x3D31              # 0.0432: two squares are 0.48 of a step of 65536
+    x[:, 0] = 0x4380                                                     # 256
+    narrow = torch.zeros((N, part), dtype=torch.bfloat16, device="cuda")
+    sd2.sd2_rmsnorm(dev(x), dev(w), y, 0.0)
+    sd2.sd2_rmsnorm(dev(x[:, :part]), dev(w[:part]), narrow, 0.0)
+    torch.cuda.synchronize()
+    assert torch.equal(y[:, :part], 2 * narrow) and not y[:, part:].any()
+
+
 def test_add_rmsnorm_is_the_two_operations_in_a_row():
     N, H = 4, 2048
     a = synth.normal_bf16(150, (N, H), 1.0)
