@@ -137,7 +137,6 @@ constexpr int kMaxDevices = 64;
 constexpr int kBarrierPool = 64;             // grid-barrier word pairs handed out round-robin
 constexpr int kBarrierStrideWords = 64;      // 256 bytes apart
 constexpr int kSmemMax = 227 * 1024;         // dynamic shared memory a CTA may opt in to
-constexpr int kProgramInline = 2;            // a program in device memory for few rows: an instance apart from that of one stage
 constexpr int kMaxBlockRows = 1 << 16;       // activation rows a block step accepts (taken in panels)
 constexpr int kDrafterWordsBytes = 512;      // a drafter's device words: barrier (two lines), then 64 production counts
 
@@ -213,7 +212,7 @@ sd2_status ensure_device(int* dev_out)
         constexpr int kMany = kMaxStagesInline;
         if (set_smem_attr<1, 1>() != cudaSuccess || set_smem_attr<1, 2>() != cudaSuccess || set_smem_attr<1, 4>() != cudaSuccess ||
             set_smem_attr<kMany, 1>() != cudaSuccess || set_smem_attr<kMany, 2>() != cudaSuccess || set_smem_attr<kMany, 4>() != cudaSuccess ||
-            set_cell_attr<1, 8>() != cudaSuccess || set_cell_attr<kProgramInline, 8>() != cudaSuccess || set_cell_attr<1, 16>() != cudaSuccess ||
+            set_cell_attr<1, 8>() != cudaSuccess || set_cell_attr<1, 16>() != cudaSuccess ||
             set_cell_attr<kMany, 8>() != cudaSuccess || set_cell_attr<kMany, 16>() != cudaSuccess ||
             cudaFuncSetAttribute(cell_kernel<1, kWidePanelRows, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
             cudaFuncSetAttribute(mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess ||
@@ -836,15 +835,15 @@ struct CellBuilder {
 // Launches a program over all N rows, in panels of equal size (rows are independent).
 sd2_status run_cell_panels(CArgs<kMaxStagesInline>& a, int64_t N, const CellNeeds& needs, int grid, cudaStream_t s)
 {
+    if (a.ext && a.fold_any) return SD2_ERR_UNSUPPORTED;     // stages in device memory carry no norms
     const int cap = widest_cell_panel(needs, a.n_stages == 1 && !a.fold_any ? kWidePanelRows : kPanelRows);
     if (cap == 0) return SD2_ERR_UNSUPPORTED;
     const int64_t panels = (N + cap - 1) / cap;
     const int64_t rows = (N + panels - 1) / panels;
     CArgs<1> one;
-    CArgs<kProgramInline> program = {};
     const bool small = a.n_stages == 1 || a.ext;             // one inline stage is all that the launch reads
     if (small) {
-        program.inl[0] = one.inl[0] = a.inl[0];
+        one.inl[0] = a.inl[0];
         one.fold[0] = a.fold[0];
     }
     for (int64_t n0 = 0; n0 < N; n0 += rows) {
@@ -860,8 +859,7 @@ sd2_status run_cell_panels(CArgs<kMaxStagesInline>& a, int64_t N, const CellNeed
         sd2_status st;
         if (small) {
             static_cast<CArgsBase&>(one) = a;
-            static_cast<CArgsBase&>(program) = a;
-            st = a.ext && a.N <= 8 ? launch_cells<kProgramInline, 8>(program, grid, smem, s) : a.N > 16 ? launch_wide_cells(one, grid, smem, s) : a.N > 8 ? launch_cells<1, 16>(one, grid, smem, s) : launch_cells<1, 8>(one, grid, smem, s);
+            st = a.N > 16 ? launch_wide_cells(one, grid, smem, s) : a.N > 8 ? launch_cells<1, 16>(one, grid, smem, s) : launch_cells<1, 8>(one, grid, smem, s);
         } else {
             st = a.N > 8 ? launch_cells<kMaxStagesInline, 16>(a, grid, smem, s) : launch_cells<kMaxStagesInline, 8>(a, grid, smem, s);
         }

@@ -298,17 +298,6 @@ struct RunDeal {
 
 // ---- expanding a cell -----------------------------------------------------------------
 
-// c + 128 * byte K8 of p (SGN = 1) or c - 128 * byte K8 of p (SGN = -1): one integer dot-product instruction
-template <int SGN, int K8>
-__device__ __forceinline__ uint32_t byte_times_128(uint32_t p, uint32_t c)
-{
-    uint32_t d;
-    constexpr uint32_t kWeight = 0x80u << (8 * K8);              // one byte: 128, or -128 where it counts as signed
-    if (SGN > 0) asm("dp4a.u32.u32 %0, %1, %2, %3;" : "=r"(d) : "r"(p), "r"(kWeight), "r"(c));
-    else asm("dp4a.u32.s32 %0, %1, %2, %3;" : "=r"(d) : "r"(p), "r"(kWeight), "r"(c));
-    return d;
-}
-
 // d = A B, from zero
 __device__ __forceinline__ void mma_rows(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
 {
@@ -324,30 +313,11 @@ __device__ __forceinline__ void add_rows(float (&d)[4], const float (&s)[4])
         : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "f"(s[0]), "f"(s[1]), "f"(s[2]), "f"(s[3]));
 }
 
-// One unit of a row: its four pairs' words, zero where a pair has none.  nib: the unit's mask bits; at: shared address of
-// the row's next word (words 128 bytes apart, upward for SGN = 1), moved on.
-template <int SGN>
-__device__ __forceinline__ void load_pairs(uint32_t nib, uint32_t& at, uint32_t (&w)[4])
-{
-    // byte i: words of pairs 0..i
-    const uint32_t upto = ((nib * 0x00204081u) & 0x01010101u) * 0x01010101u;
-    const uint32_t a1 = byte_times_128<SGN, 0>(upto, at), a2 = byte_times_128<SGN, 1>(upto, at), a3 = byte_times_128<SGN, 2>(upto, at);
-    asm volatile("{\n\t.reg .pred p0, p1, p2, p3;\n\t.reg .b32 t0, t1, t2, t3;\n\t"
-                 "and.b32 t0, %8, 1;\n\tand.b32 t1, %8, 2;\n\tand.b32 t2, %8, 4;\n\tand.b32 t3, %8, 8;\n\t"
-                 "setp.ne.u32 p0, t0, 0;\n\tsetp.ne.u32 p1, t1, 0;\n\tsetp.ne.u32 p2, t2, 0;\n\tsetp.ne.u32 p3, t3, 0;\n\t"
-                 "mov.b32 %0, 0;\n\tmov.b32 %1, 0;\n\tmov.b32 %2, 0;\n\tmov.b32 %3, 0;\n\t"
-                 "@p0 ld.shared.u32 %0, [%4];\n\t@p1 ld.shared.u32 %1, [%5];\n\t@p2 ld.shared.u32 %2, [%6];\n\t@p3 ld.shared.u32 %3, [%7];\n\t}"
-                 : "=&r"(w[0]), "=&r"(w[1]), "=&r"(w[2]), "=&r"(w[3])
-                 : "r"(at), "r"(a1), "r"(a2), "r"(a3), "r"(nib)
-                 : "memory");
-    at = byte_times_128<SGN, 3>(upto, at);
-}
-
-// The same by steps: two words from shared address `lo` upward and two from `hi` downward, 128 bytes apart, where the mask has the bits
-// `bit` and the next, and those 16 above; zero and no step where it has not.  Four instructions a pair; load_pairs takes five, but
-// finds four addresses at once.  Where warps have cell after cell the number of instructions counts (an eight-row step of two blocks
-// of 2048/512/8192 68.6 -> 67.6 us, a block of 3072/1024/8192 for 16 rows 61.9 -> 60.2, 48 rows of 8192 x 2048 25.9 -> 25.5), in a
-// launch of one stage for few rows, where a warp has one cell or two, the latency of one (five rows of 1531 x 3001 8.63, by steps 8.72).
+// The words of four pairs of a lane, by steps: two from shared address `lo` upward and two from `hi` downward, 128 bytes apart, where the
+// mask has the bits `bit` and the next, and those 16 above; zero and no step where it has not.  Four instructions a pair.  (Four
+// addresses at once, from prefix sums of the mask's bits, take five and no less time even where a warp has a single cell.  us, prefix sums
+// and steps, calls back to back: 512 x 512 for eight rows 4.83 and 4.70, 2048 x 8192 8.89 and 8.58, 8192 x 8192 21.4 and 21.2, steps of
+// two blocks of 256/64/1024 for four rows 32.1 and 31.9, of 2048/512/8192 for eight 67.2 and 65.7.)
 __device__ __forceinline__ void take_words(uint32_t mask, uint32_t bit, uint32_t& lo, uint32_t& hi, uint32_t& a, uint32_t& b, uint32_t& c, uint32_t& d)
 {
     asm volatile("{\n\t.reg .pred p, q, r, s;\n\t.reg .b32 t, u, v, w;\n\t"
@@ -367,7 +337,7 @@ __device__ __forceinline__ void take_words(uint32_t mask, uint32_t bit, uint32_t
 // a warp's cells 9.4e-8 (of one set of sums for 32 activation rows 15.2e-8), chains of a cell 7.5e-8, single steps 6.8e-8, which
 // is what the strips' fused multiply-adds have; at 11008 columns 14.9e-8, 8.7e-8, 8.2e-8 (strips 8.9e-8).  The order of the
 // sums is that of every instance, so a row has the same sums in every panel.
-template <int NR, bool FEW>
+template <int NR>
 __device__ __forceinline__ void multiply_cell(uint32_t m, uint32_t lo, uint32_t hi, const uint32_t (&xo)[NR / 8], uint32_t xd,
                                               float (&c)[NR / 8][4])
 {
@@ -375,13 +345,8 @@ __device__ __forceinline__ void multiply_cell(uint32_t m, uint32_t lo, uint32_t 
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         uint32_t a[4], b[4];
-        if (FEW) {
-            load_pairs<1>((m >> (4 * u)) & 0xFu, lo, a);
-            load_pairs<-1>((m >> (16 + 4 * u)) & 0xFu, hi, b);
-        } else {
 #pragma unroll
-            for (int i = 0; i < 4; i += 2) take_words(m, 1u << (4 * u + i), lo, hi, a[i], b[i], a[i + 1], b[i + 1]);
-        }
+        for (int i = 0; i < 4; i += 2) take_words(m, 1u << (4 * u + i), lo, hi, a[i], b[i], a[i + 1], b[i + 1]);
 #pragma unroll
         for (int h = 0; h < NR / 8; ++h) {
             const uint4 x = lds_v4(xo[h] + xd + 64u * u);
@@ -1191,7 +1156,7 @@ __global__ void __launch_bounds__(kCellThreads, 1) cell_kernel(const __grid_cons
                         const uint32_t m = lds_u32(cell + 4 * lane), v0 = cell + kCellHeaderBytes;
                         const uint32_t pi = lds_u8(cell + 128u + lane) & 0x7Fu;
                         const uint32_t xd = (uint32_t)d * (2 * kCellCols);
-                        multiply_cell<NR, MAXS == 1 && NR == 8>(m, v0 + 4u * lane, v0 + (H - 1u) * 128u + pi, xl, xd, acc);
+                        multiply_cell<NR>(m, v0 + 4u * lane, v0 + (H - 1u) * 128u + pi, xl, xd, acc);
                     }
                     __syncwarp();
                     mbar_arrive_n(empty0 + 8 * slot, 1u, lane == 0);
