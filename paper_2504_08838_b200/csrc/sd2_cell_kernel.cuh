@@ -495,10 +495,15 @@ __device__ __noinline__ bool fold_norm(const XRows& r, const SFold& f, const uin
     // Eight columns of up to four rows to a thread, from the first load to the last store (input, residual and gains asked for together,
     // 16 bytes at a time), where the rows are on 16 bytes and short enough.  Whole rows stand in `scratch` while their squares are added
     // up, in the order of the loop below; the staged copies are written over.
+    // From kHeldMin values on.  Below, few threads have a column, and code that is gone through once comes from L2: us of a decode block
+    // by the loop and through registers: hidden 256, four and twelve rows 36.2 and 39.1, 57.0 and 57.1; 512, two and six 34.9 and 37.5,
+    // 47.4 and 46.7; 768, two, four and eight 39.5 and 42.1, 46.0 and 46.1, 58.5 and 53.7; 1024, two and three 42.0 and 42.3, 47.1 and 44.2;
+    // 2048, eight 105 and 66.
+    constexpr int kHeldMin = 3072;
     constexpr int kHeld = 4;
-    const int fit = min(kHeld, scratch_bytes / (2 * r.ld));
-    if (fit > 0 && (r.ld & 7) == 0 && r.ld <= 8 * kCellConsumers &&
+    if (r.N * r.ld >= kHeldMin && (r.ld & 7) == 0 && r.ld <= 8 * kCellConsumers && 2 * r.ld <= scratch_bytes &&
         ((((uintptr_t)xg | (uintptr_t)f.res | (uintptr_t)f.norm_w | (uintptr_t)f.sum_out | (uintptr_t)f.norm_out) & 15) == 0)) {
+        const int fit = min(kHeld, scratch_bytes / (2 * r.ld));
         const bool mine = ctid < (r.ld >> 3), own = mine && 8 * ctid >= c0 && 8 * ctid < c0 + r.K;
         const uint4 w = own ? __ldg((const uint4*)f.norm_w + ctid) : make_uint4(0u, 0u, 0u, 0u);
         for (int n0 = 0; n0 < r.N; n0 += fit) {
