@@ -182,9 +182,11 @@ constexpr int kFoldStaticBytes = 256;   // static shared memory of the kernel in
 template <int MAXS, int NT>
 cudaError_t set_smem_attr()
 {
-    cudaError_t e = cudaFuncSetAttribute(stream_kernel<MAXS, NT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
+    cudaError_t e = cudaFuncSetAttribute(stream_kernel<MAXS, NT, kNoFold>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(stream_kernel<MAXS, NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - kFoldStaticBytes);
+    e = cudaFuncSetAttribute(stream_kernel<MAXS, NT, kFoldShared>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - kFoldStaticBytes);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(stream_kernel<MAXS, NT, kFoldHeld>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - kFoldStaticBytes);
 }
 
 template <int MAXS, int NR>
@@ -558,7 +560,9 @@ sd2_status launch_stream_nt(const SArgsT<MAXS>& a, int grid, int smem, bool coop
     if (!cooperative) attr[0] = pdl_attribute();
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = a.fold_any ? cudaLaunchKernelEx(&cfg, stream_kernel<MAXS, NT, true>, a) : cudaLaunchKernelEx(&cfg, stream_kernel<MAXS, NT, false>, a);
+    auto* const kernel = a.fold_any == kNoFold ? stream_kernel<MAXS, NT, kNoFold> : a.fold_any == kFoldHeld ? stream_kernel<MAXS, NT, kFoldHeld>
+                       : stream_kernel<MAXS, NT, kFoldShared>;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, a);
     if (e != cudaSuccess) { cudaGetLastError(); return SD2_ERR_CUDA; }
     if (cudaGetLastError() != cudaSuccess) return SD2_ERR_CUDA;
     return SD2_OK;
@@ -700,6 +704,22 @@ sd2_status run_panels(SArgs& a, int64_t N, const int xs_need[3], int K_max, int 
     return SD2_OK;
 }
 
+// How a program of inline stages takes its norms.  Threads hold rows that are on 16 bytes and no longer than eight columns of each, from 768
+// columns on: us of a decode block of one row by shared memory and held, hidden 512 28.4 and 29.1, 768 30.7 and 30.5, 1024 31.9 and 31.8,
+// 1536 37.0 and 36.3, 2048 46.0 and 44.5, 4096 71.4 and 62.3; of 256 for three rows 41.6 and 43.8.
+int fold_of(const SArgs& a)
+{
+    for (int i = 0; i < a.n_stages; ++i) {
+        const SFold& f = a.fold[i];
+        if (!f.norm_w) continue;
+        const SStage& st = a.inl[i];
+        if (!st.x || st.K % 8 || st.K < 768 || st.K > 8 * kConsumerThreads ||
+            (((uintptr_t)st.x | (uintptr_t)f.res | (uintptr_t)f.norm_w | (uintptr_t)f.sum_out | (uintptr_t)f.norm_out) & 15))
+            return kFoldShared;
+    }
+    return kFoldHeld;
+}
+
 // Runs a program of inline stages.
 sd2_status run_program(SArgs& a, int dev, int64_t N, const ProgramNeeds& needs, cudaStream_t s)
 {
@@ -710,6 +730,7 @@ sd2_status run_program(SArgs& a, int dev, int64_t N, const ProgramNeeds& needs, 
     a.err = g_dev[dev].err_word;
     a.wait_cycles = wait_budget(dev);
     a.free_tiles = needs.free_tiles(grid);
+    if (a.fold_any) a.fold_any = fold_of(a);
     a.gbar = coop ? g_dev[dev].barriers + (size_t)(g_next_barrier.fetch_add(1) % kBarrierPool) * kBarrierStrideWords : nullptr;
     return run_panels(a, N, needs.xs_need, needs.K_max, needs.max_tile, grid, s);
 }

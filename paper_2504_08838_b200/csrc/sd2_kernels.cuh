@@ -159,12 +159,17 @@ struct SStage {
 };
 static_assert(sizeof(SStage) % 16 == 0, "stage descriptors are copied in 16-byte pieces");
 
-// Decoder glue folded into a stage's staging pass (kernel instances with FOLD only; all NULL / 0: a plain linear).
+// Decoder glue folded into a stage's staging pass (kernel instances with a FOLD only; all NULL / 0: a plain linear).
 // With norm_w set, every CTA turns the activation row it has just fetched into  rmsnorm(row [+ res]) * norm_w
 // before scattering it into the lane windows: the residual connection and the norm in front of a block's linears
 // cost no launch and no hand-off of their own.  CTA 0 also stores the bf16 sum (sum_out) and the normalised row
 // (norm_out).  Kept out of SStage and out of the plain kernel instances: the drafter step's time is sensitive to
 // the size of the stage descriptors and of the CTA's bookkeeping (1.3 % when these fields sat in SStage).
+// kFoldShared: through shared memory with two-byte accesses, any row.  kFoldHeld: a thread holds eight columns of a row from the first load
+// to the last store (stage_norm), where all of a program's norms can be taken so (fold_of).  Instances apart, since either is slower
+// with the other's code beside it: a decode block of hidden 4608, which no thread can hold, took 83.3 us in an instance that had both and
+// takes 81.0.
+constexpr int kNoFold = 0, kFoldShared = 1, kFoldHeld = 2;
 struct SFold {
     const uint16_t* res;       // [N * K] added to the row first (rounded to bf16), or NULL
     const uint16_t* norm_w;    // [K] gains of the norm, or NULL: no norm
@@ -193,7 +198,7 @@ struct SArgsBase {
     int free_tiles;                 // 1: a consumer warp that is done draws the next tile from a shared counter;
                                     // 0: tile k of a stage goes to warp k % 16 (see the consumer loop)
     long long* reserved_ptr;
-    int fold_any;                   // host side: launch the FOLD instance
+    int fold_any;                   // host side: launch an instance with a FOLD
 };
 
 // MAXS: inline stages the argument block has room for.  A launch of one stage, or of stages in device memory, passes 0.5 KB
@@ -655,7 +660,7 @@ __device__ __forceinline__ void stage_norm(int K, int rows, const uint16_t* x, c
 // buffer (xlin holds two, `xlin_row` elements apart), then one scatter writes the packed words.
 // (Panels of two keep one buffer and take a pass per row: the second buffer would come out of the
 // weight ring, which costs them more than the extra pass.)
-template <int NT, bool FOLD = false>
+template <int NT, int FOLD = kNoFold>
 __device__ __forceinline__ void stage_x(const SStage& st, int N, const uint16_t* x_src, const uint16_t* g,
                                         const uint16_t* u, uint16_t* t_out, float* xs, uint16_t* xlin, int xlin_row, int ctid,
                                         uint32_t tag, const unsigned int* tagb, const WaitCtx& wc, int row0 = 0,
@@ -674,8 +679,7 @@ __device__ __forceinline__ void stage_x(const SStage& st, int N, const uint16_t*
     const bool pub = glue && t_out && blockIdx.x == 0;
     // Residual and norm where a thread can hold its eight columns of a row: input, residual and gains are asked for together, 16 bytes
     // at a time.  (With two-byte accesses and the loads one after the other a row of 2048 took 3.4 us from the barrier to the scatter.)
-    const bool held = FOLD && fold && fold->norm_w && vec && !glue && tag == 0u && K <= 8 * kConsumerThreads &&
-                      ((((uintptr_t)fold->res | (uintptr_t)fold->norm_w | (uintptr_t)fold->sum_out | (uintptr_t)fold->norm_out) & 15) == 0);
+    const bool held = FOLD == kFoldHeld && fold && fold->norm_w;
     for (int n0 = 0; n0 < NT; n0 += kRowsPerPass) {
         if (held) stage_norm<kRowsPerPass>(K, min(kRowsPerPass, N - n0), x_src + (size_t)n0 * K, *fold, (size_t)(row0 + n0) * K, xlin + st.V, xlin_row, red, ctid);
 #pragma unroll
@@ -723,7 +727,7 @@ __device__ __forceinline__ void stage_x(const SStage& st, int N, const uint16_t*
                 }
             }
         }
-        if (FOLD && !held && fold && fold->norm_w) {
+        if (FOLD == kFoldShared && fold && fold->norm_w) {
             const SFold& f = *fold;
             // residual and norm on the linear row(s), each thread on the elements it revisits in the second loop
             named_bar_sync(1, kConsumerThreads);
@@ -812,7 +816,7 @@ __device__ __forceinline__ void stage_x(const SStage& st, int N, const uint16_t*
     }
 }
 
-template <int MAXS, int NT, bool FOLD>
+template <int MAXS, int NT, int FOLD>
 __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const __grid_constant__ SArgsT<MAXS> a)
 {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -1059,9 +1063,9 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const __grid_
         } else if (st.paired) {   // g, u, t_out are this stage's outputs
             stage_x<NT>(st, N, x_src + xw, nullptr, nullptr, nullptr, xs, xlin, xlin_row, ctid, tag_in, tagb, wc);
         } else {
-            if constexpr (FOLD) {
+            if constexpr (FOLD != kNoFold) {
                 __shared__ float fold_red[2][kConsumerWarps];   // per-warp partial sums of squares of the rows being normalised
-                stage_x<NT, true>(st, N, x_src ? x_src + xw : nullptr, st.g ? st.g + xw : nullptr, st.u ? st.u + xw : nullptr,
+                stage_x<NT, FOLD>(st, N, x_src ? x_src + xw : nullptr, st.g ? st.g + xw : nullptr, st.u ? st.u + xw : nullptr,
                                   st.t_out ? st.t_out + xoff : nullptr, xs, xlin, xlin_row, ctid, tag_in, tagb, wc, a.n0, fold_red,
                                   (!a.ext && s < MAXS) ? &a.fold[MAXS == 1 ? 0 : s] : nullptr);
             } else {
