@@ -2166,8 +2166,14 @@ sd2_status sd2_drafter_create(const sd2_handle* h, int32_t L, int64_t n_max, sd2
     std::vector<SStage> stages((size_t)L * 7);
     ProgramNeeds needs;
     bool ok = dev_malloc((void**)&d->d_ws, (size_t)o) == cudaSuccess && cudaMemset(d->d_ws, 0, (size_t)o) == cudaSuccess;
-    // Tagged hand-off (stage tags are 8 bits wide): per block q, hdn, g, u, out as 32-bit words
-    const bool tagged = 7 * L <= 254;
+    // Tagged hand-off (stage tags are 8 bits wide): per block q, hdn, g, u, out as 32-bit words.  A stage waits for the tag of the one before
+    // it, so weights that share an input must share a stage, which they do not where they are cut into strips differently (q of 4096 x
+    // 4096 and k of 1024 x 4096: 16 and 32): such a drafter's stages meet at grid barriers.
+    bool tagged = 7 * L <= 254;
+    for (int i = 0; i < L; ++i) {
+        const sd2_handle* b = h + 7 * i;
+        if (b[1]->S != b[0]->S || b[2]->S != b[0]->S || b[5]->S != b[4]->S) tagged = false;
+    }
     std::vector<int64_t> tag_off((size_t)L * 6 + 1, 0);
     d->d_tags = nullptr;
     d->tags_bytes = 0;

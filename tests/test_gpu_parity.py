@@ -553,6 +553,34 @@ def test_drafter_step_in_several_panels_with_k_8192():
             sd2.sd2_free(h)
 
 
+@pytest.mark.parametrize("fmt,N", [(sd2.SD2_FORMAT_GAP4, 1), (sd2.SD2_FORMAT_GAP4, 5), (sd2.SD2_FORMAT_GAP4_STRIPS, 5)])
+def test_drafter_whose_q_and_k_are_cut_into_strips_differently(fmt, N):
+    # q of 4096 x 4096 has 16 strips a row, k and v of 128 x 4096 have 32: they take a stage each, all with the same input
+    shape = synth.DrafterShape("wide", 4096, 128, 512, 2)
+    lins = [synth.make_block(2, b, shape, 0.2) for b in range(2)]
+    blocks = [[sd2.sd2_compress(W, m, fmt, sd2.SD2_DTYPE_F32 if (b == 1 and i == 6) else sd2.SD2_DTYPE_BF16) for i, (W, m) in enumerate(lin)]
+              for b, lin in enumerate(lins)]
+    d = sd2.sd2_drafter_create(blocks, n_max=N)
+    x = synth.make_activations(2, 0, 0, N, shape.hidden)
+    want = _block_chain(blocks, shape, dev_bf16(x))
+    for _ in range(2):                       # twice: the barrier words must come back clean
+        y = torch.full((N, shape.hidden), float("nan"), dtype=torch.float32, device="cuda")
+        sd2.sd2_drafter_step(d, dev_bf16(x), y)
+        sd2.sd2_stream_check()
+        assert torch.equal(y, want)
+    inp = x
+    for b in range(2):
+        ptrs = sd2.sd2_drafter_buffers(d, b)
+        for i, rows in ((0, 4096), (1, 128), (2, 128)):
+            Yr, S = oracle.masked_linear(*lins[b][i], inp)
+            check(synth.bf16_bits_to_f32(_read_u16(ptrs[i], N * rows).reshape(N, rows)).astype(np.float64), Yr, S, False)
+        inp = _read_u16(ptrs[7], N * 4096).reshape(N, 4096)
+    sd2.sd2_drafter_free(d)
+    for hs in blocks:
+        for h in hs:
+            sd2.sd2_free(h)
+
+
 # ---- GAP4_MMA: blocks expanded in shared memory, multiplied on the tensor cores ------------------
 
 def _mma_case(seed, M, K, d, N, f32):
