@@ -10,6 +10,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <functional>
 #include <mutex>
 #include <new>
 #include <unordered_set>
@@ -268,13 +269,19 @@ int resolve_format(const sd2_options* opt, int64_t M, int64_t K)
     return f == SD2_FORMAT_GAP4_STRIPS ? (int)SD2_FORMAT_GAP4 : f;
 }
 
+sd2_status check_pack(int64_t M, int64_t K, const sd2_options* opt)
+{
+    if (M < 1 || K < 1 || M > 0x7FFFFFF0ll || K > 0x7FFFFFF0ll || M * K > (1ll << 40)) return SD2_ERR_SHAPE;
+    return opt && opt->y_dtype != SD2_DTYPE_BF16 && opt->y_dtype != SD2_DTYPE_F32 ? SD2_ERR_INVALID_ARG : SD2_OK;
+}
+
 sd2_status pack_any(const uint16_t* W, const uint8_t* mask, int64_t M, int64_t K, const sd2_options* opt,
                     uint8_t** blob, int64_t* bytes)
 {
     if (!W || !blob || !bytes) return SD2_ERR_INVALID_ARG;
-    if (M < 1 || K < 1 || M > 0x7FFFFFF0ll || K > 0x7FFFFFF0ll || M * K > (1ll << 40)) return SD2_ERR_SHAPE;
+    const sd2_status checked = check_pack(M, K, opt);
+    if (checked != SD2_OK) return checked;
     const int y_dtype = opt ? opt->y_dtype : SD2_DTYPE_BF16;
-    if (y_dtype != SD2_DTYPE_BF16 && y_dtype != SD2_DTYPE_F32) return SD2_ERR_INVALID_ARG;
     const int f = resolve_format(opt, M, K);
     PackResult r;
     try {
@@ -299,6 +306,8 @@ int unpack_any(const BlobHeader& hd, const uint8_t* blob, uint16_t* dense)
     return unpack_gap4(hd, blob, dense);
 }
 
+// A handle with a blob's facts, and its sections on the GPU (GAP4_MMA: without, the GPU has no use for the records and they need not
+// be there).
 sd2_status upload(const uint8_t* blob, int64_t bytes, const BlobHeader& hd, sd2_handle* out)
 {
     int dev = 0;
@@ -312,7 +321,7 @@ sd2_status upload(const uint8_t* blob, int64_t bytes, const BlobHeader& hd, sd2_
     const bool mma = hd.format == (uint32_t)kFormatGap4Mma;
     const size_t heights = hd.format == (uint32_t)kFormatGap4 ? (size_t)cell_geometry(hd.M, hd.K).cells() * 4
                          : mma ? (size_t)panel_geometry(hd.M, hd.K).cells() * 4 : 0;
-    if (mma) bytes = 0;                       // (the GPU has no use for the records)
+    if (mma) bytes = 0;
     if (dev_malloc(&d, align256((size_t)bytes) + heights) != cudaSuccess) { cudaGetLastError(); delete h; return SD2_ERR_ALLOC; }
     if (bytes && cudaMemcpy(d, blob, (size_t)bytes, cudaMemcpyHostToDevice) != cudaSuccess) {
         cudaGetLastError();
@@ -327,9 +336,9 @@ sd2_status upload(const uint8_t* blob, int64_t bytes, const BlobHeader& hd, sd2_
     h->y_dtype = (int)hd.y_dtype;
     h->device = dev;
     h->d_blob = (uint8_t*)d;
-    h->d_sec0 = (const uint32_t*)(h->d_blob + hd.sec_off[0]);
-    h->d_sec1 = (const uint32_t*)(h->d_blob + hd.sec_off[1]);
-    h->d_sec2 = (const void*)(h->d_blob + hd.sec_off[2]);
+    h->d_sec0 = mma ? nullptr : (const uint32_t*)(h->d_blob + hd.sec_off[0]);
+    h->d_sec1 = mma ? nullptr : (const uint32_t*)(h->d_blob + hd.sec_off[1]);
+    h->d_sec2 = mma ? nullptr : (const void*)(h->d_blob + hd.sec_off[2]);
     h->S = (int)hd.strips;
     h->B = (int)hd.strip_cols;
     h->T = (int)hd.n_tiles;
@@ -367,23 +376,49 @@ bool kernel_reads(const void* p, size_t size, int device)
     return readable_in_place(place, owner, device, p, size);
 }
 
-// Gives a fresh handle its cells (GAP4_MMA: panel cells), from dense weights (and a mask, or NULL: see pack_cells_kernel) in device
-// memory.
-sd2_status pack_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask, uint32_t nonzero)
+// Where a fresh handle's dense weights come from while its cells are packed: `fetch` puts the rows row0 .. row0 + rows - 1 of the weights and
+// of the mask (NULL: see pack_cells_kernel) in reach of a kernel.  It is asked for `step` rows at a time, in order, and twice for each of
+// them where step is less than all rows.
+struct CellSource {
+    int64_t step;
+    uint32_t nonzero;
+    std::function<sd2_status(int64_t row0, int64_t rows, const uint16_t** W, const uint8_t** mask)> fetch;
+};
+
+// Gives a fresh handle its cells (GAP4_MMA: panel cells).
+sd2_status pack_cells(sd2_handle h, const CellSource& src)
 {
     const bool panel = h->format == SD2_FORMAT_GAP4_MMA;
     const CellGeom g = panel ? panel_geometry(h->M, h->K) : cell_geometry(h->M, h->K);
     const int64_t n_cells = g.cells();
-    auto* const kernel = panel ? pack_cells_kernel<true> : pack_cells_kernel<false>;
     if (n_cells > 0x3FFFFFFF) return SD2_ERR_UNSUPPORTED;
     const size_t dir_bytes = align256((size_t)(n_cells + 1) * 4);
     std::vector<uint32_t> off((size_t)n_cells + 1);          // first the cells' heights, then their places
     uint32_t* d_height = (uint32_t*)(h->d_blob + align256((size_t)h->blob_bytes));
-    const unsigned grid = (unsigned)((n_cells + kPackWarps - 1) / kPackWarps);
-    kernel<<<grid, 32 * kPackWarps>>>(W, mask, nonzero, h->M, h->K, (int)g.T, g.D, d_height, nullptr, nullptr);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpy(off.data(), d_height, (size_t)n_cells * 4, cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return SD2_ERR_CUDA;
+    uint8_t* image = nullptr;
+    const uint16_t* W = nullptr;
+    const uint8_t* mask = nullptr;
+    // one pass over the weights: heights, or, once there is an image, the cells
+    auto pass = [&]() {
+        for (int64_t row0 = 0; row0 < h->M; row0 += src.step) {
+            const int64_t rows = std::min(src.step, h->M - row0);
+            if (!image || src.step < h->M) {
+                const sd2_status st = src.fetch(row0, rows, &W, &mask);
+                if (st != SD2_OK) return st;
+            }
+            const CellGeom part = panel ? panel_geometry(rows, h->K) : g;
+            const int64_t first = panel ? row0 / kPanelRowsOfBlock * g.D * g.per : 0;
+            const unsigned grid = (unsigned)((part.cells() + kPackWarps - 1) / kPackWarps);
+            auto* const kernel = panel ? pack_cells_kernel<true> : pack_cells_kernel<false>;
+            kernel<<<grid, 32 * kPackWarps>>>(W, mask, src.nonzero, rows, h->K, (int)part.T, g.D, image ? nullptr : d_height + first,
+                                              image ? (const uint32_t*)image + first : nullptr, image ? image + dir_bytes : nullptr);
+            if (cudaGetLastError() != cudaSuccess) return SD2_ERR_CUDA;
+        }
+        return SD2_OK;
+    };
+    sd2_status st = pass();
+    if (st != SD2_OK) return st;
+    if (cudaMemcpy(off.data(), d_height, (size_t)n_cells * 4, cudaMemcpyDeviceToHost) != cudaSuccess) return SD2_ERR_CUDA;
     uint64_t units = 0;
     uint32_t max_run = 0;
     for (int64_t c = 0; c < n_cells; ++c) {
@@ -395,19 +430,15 @@ sd2_status pack_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask, uint
     }
     if (units > 0xFFFFFFF0ull) return SD2_ERR_UNSUPPORTED;
     off[(size_t)n_cells] = (uint32_t)units;
-    uint8_t* image = nullptr;
     const size_t bytes = dir_bytes + (size_t)units * 32;
     if (dev_malloc(&image, bytes) != cudaSuccess) return SD2_ERR_ALLOC;
     h->d_image = image;                                       // (sd2_free has it from here on)
     h->d_cells = image + dir_bytes;
-    e = cudaMemset(image, 0, bytes);
+    cudaError_t e = cudaMemset(image, 0, bytes);
     if (e == cudaSuccess) e = cudaMemcpy(image, off.data(), off.size() * 4, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) {
-        kernel<<<grid, 32 * kPackWarps>>>(W, mask, nonzero, h->M, h->K, (int)g.T, g.D, nullptr, (const uint32_t*)image, image + dir_bytes);
-        e = cudaGetLastError();
-    }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(0);       // W and mask may go away now
     if (e != cudaSuccess) return SD2_ERR_CUDA;
+    if ((st = pass()) != SD2_OK) return st;
+    if (cudaStreamSynchronize(0) != cudaSuccess) return SD2_ERR_CUDA;       // the weights may go away now
     h->device_bytes += (int64_t)bytes;
     h->cell_bytes = (n_cells + 1) * 4 + (int64_t)units * 32;
     h->cell_T = (int)g.T;
@@ -416,30 +447,46 @@ sd2_status pack_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask, uint
     return SD2_OK;
 }
 
-// The same from weights and mask in host memory or where the handle's GPU can read them.  The cells of a GAP4 handle are a second
-// image of the weights: where there is no memory for them, or for the dense weights that they are made from, the handle goes without,
-// and calls of several rows read its strips.  On any other failure the handle is freed.
-sd2_status add_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask, uint32_t nonzero = 0x7FFFu)
+// The same from weights and a mask that lie in host memory or where the handle's GPU can read them, or from the records of a GAP4_MMA blob
+// (which have been checked).  The cells of a GAP4 handle are a second image of the weights: where there is no memory for them, or for the
+// dense weights that they are made from, the handle goes without, and calls of several rows read its strips.  Panel cells are all that
+// a GAP4_MMA handle has: they are made kPanelScratch weights at a time, so that little memory is needed beside them.  On any other
+// failure the handle is freed.
+constexpr int64_t kPanelScratch = 1 << 24;
+sd2_status add_cells(sd2_handle h, const uint16_t* W, const uint8_t* mask, uint32_t nonzero = 0x7FFFu, const BlobHeader* hd = nullptr,
+                     const uint8_t* blob = nullptr)
 {
-    const size_t n = (size_t)(h->M * h->K);
-    uint16_t* w_dev = nullptr;
+    const bool w_here = W && kernel_reads(W, sizeof *W, h->device), m_here = !mask || kernel_reads(mask, sizeof *mask, h->device);
+    CellSource src;
+    src.nonzero = nonzero;
+    src.step = h->M;
+    if (h->format == SD2_FORMAT_GAP4_MMA && !(w_here && m_here))
+        src.step = std::min(h->M, std::max<int64_t>(kPanelScratch / h->K / kPanelRowsOfBlock, 1) * kPanelRowsOfBlock);
+    const size_t n = (size_t)(src.step * h->K);
+    uint16_t *w_dev = nullptr, *rows_host = nullptr;
     uint8_t* m_dev = nullptr;
     sd2_status st = SD2_OK;
-    if (!kernel_reads(W, sizeof *W, h->device)) {
-        if (dev_malloc(&w_dev, n * 2) != cudaSuccess) st = SD2_ERR_ALLOC;
-        else if (cudaMemcpy(w_dev, W, n * 2, cudaMemcpyHostToDevice) != cudaSuccess) st = SD2_ERR_CUDA;
-    }
-    if (st == SD2_OK && mask && !kernel_reads(mask, sizeof *mask, h->device)) {
-        if (dev_malloc(&m_dev, n) != cudaSuccess) st = SD2_ERR_ALLOC;
-        else if (cudaMemcpy(m_dev, mask, n, cudaMemcpyHostToDevice) != cudaSuccess) st = SD2_ERR_CUDA;
-    }
+    if (!w_here && dev_malloc(&w_dev, n * 2) != cudaSuccess) st = SD2_ERR_ALLOC;
+    if (st == SD2_OK && !m_here && dev_malloc(&m_dev, n) != cudaSuccess) st = SD2_ERR_ALLOC;
+    if (st == SD2_OK && blob && !(rows_host = (uint16_t*)lib_malloc(n * 2))) st = SD2_ERR_ALLOC;
+    auto fetch = [&](int64_t row0, int64_t rows, const uint16_t** w, const uint8_t** m) {
+        const size_t at = (size_t)(row0 * h->K), count = (size_t)(rows * h->K);
+        if (blob) unpack_mma_panels(*hd, blob, row0 / kMmaBlockRows, (row0 + rows + kMmaBlockRows - 1) / kMmaBlockRows, rows_host);
+        *w = w_here ? W + at : w_dev;
+        *m = m_here ? (mask ? mask + at : nullptr) : m_dev;
+        if (!w_here && cudaMemcpy(w_dev, blob ? rows_host : W + at, count * 2, cudaMemcpyHostToDevice) != cudaSuccess) return SD2_ERR_CUDA;
+        if (!m_here && cudaMemcpy(m_dev, mask + at, count, cudaMemcpyHostToDevice) != cudaSuccess) return SD2_ERR_CUDA;
+        return SD2_OK;
+    };
     try {
-        if (st == SD2_OK) st = pack_cells(h, w_dev ? w_dev : W, m_dev ? m_dev : mask, nonzero);
+        src.fetch = std::ref(fetch);
+        if (st == SD2_OK) st = pack_cells(h, src);
     } catch (const std::bad_alloc&) {
         st = SD2_ERR_ALLOC;
     }
     cudaFree(w_dev);
     cudaFree(m_dev);
+    std::free(rows_host);
     if (st == SD2_OK) return st;
     cudaGetLastError();
     if (h->format == SD2_FORMAT_GAP4 && (st == SD2_ERR_ALLOC || st == SD2_ERR_UNSUPPORTED)) return SD2_OK;
@@ -1453,10 +1500,15 @@ sd2_status sd2_compress(const void* weight_bf16, const uint8_t* mask, int64_t M,
     }
     uint8_t* blob = nullptr;
     int64_t bytes = 0;
-    if (st == SD2_OK) st = pack_any(W, mask, M, K, opt, &blob, &bytes);
+    BlobHeader hd;
+    if (st == SD2_OK && resolve_format(opt, M, K) == SD2_FORMAT_GAP4_MMA) {       // (its handles keep no records)
+        st = check_pack(M, K, opt);
+        if (st == SD2_OK) st = from_pack(size_gap4_mma(W, mask, M, K, opt->y_dtype, &hd));
+    } else if (st == SD2_OK) {
+        st = pack_any(W, mask, M, K, opt, &blob, &bytes);
+        if (st == SD2_OK) std::memcpy(&hd, blob, sizeof hd);
+    }
     if (st == SD2_OK) {
-        BlobHeader hd;
-        std::memcpy(&hd, blob, sizeof hd);
         sd2_handle h = nullptr;
         st = upload(blob, bytes, hd, &h);
         std::free(blob);
@@ -1482,15 +1534,11 @@ sd2_status sd2_load_blob(const void* blob, int64_t blob_bytes, sd2_handle* out)
     if (hd.format == (uint32_t)kFormatGap4) {
         if (check_gap4(hd, (const uint8_t*)blob) != 0) return SD2_ERR_CORRUPT;
         dense = (uint16_t*)lib_malloc((size_t)(hd.M * hd.K) * 2);     // for the cells; NULL: the handle goes without
-    } else if (hd.format == (uint32_t)kFormatGap4Mma) {
-        if (unpack_any(hd, (const uint8_t*)blob, nullptr) != 0) return SD2_ERR_CORRUPT;
-        dense = (uint16_t*)lib_malloc((size_t)(hd.M * hd.K) * 2);
-        if (!dense) return SD2_ERR_ALLOC;
     }
     int rc;
     try {
         rc = unpack_any(hd, (const uint8_t*)blob, dense);
-        if (rc != 0 && dense && hd.format == (uint32_t)kFormatGap4) {   // a column that two lanes share has a sum in strips, but no dense form
+        if (rc != 0 && dense) {              // a column that two lanes share has a sum in strips, but no dense form
             std::free(dense);
             dense = nullptr;
             rc = unpack_any(hd, (const uint8_t*)blob, nullptr);
@@ -1503,7 +1551,8 @@ sd2_status sd2_load_blob(const void* blob, int64_t blob_bytes, sd2_handle* out)
     sd2_status st = rc != 0 ? SD2_ERR_CORRUPT : upload((const uint8_t*)blob, blob_bytes, hd, &h);
     // for the cells what decoded to +0 or -0 was masked out, or was a kept zero, which adds nothing (panel cells are what a handle
     // is decompressed from: they keep a -0)
-    if (st == SD2_OK && dense) st = add_cells(h, dense, nullptr, hd.format == (uint32_t)kFormatGap4 ? 0x7FFFu : 0xFFFFu);
+    if (st == SD2_OK && dense) st = add_cells(h, dense, nullptr);
+    else if (st == SD2_OK && h->format == SD2_FORMAT_GAP4_MMA) st = add_cells(h, nullptr, nullptr, 0xFFFFu, &hd, (const uint8_t*)blob);
     std::free(dense);
     if (st == SD2_OK) *out = h;
     return st;

@@ -58,6 +58,54 @@ def test_panels(M, K, N, density, shift):
     sd2.sd2_free(h)
 
 
+@pytest.mark.parametrize("M,K,density", [(130, 264, 0.5), (257, 129, 1.0), (300, 1000, 0.02), (64, 4099, 0.1), (1, 1, 1.0), (129, 65, 0.0)])
+def test_the_facts_of_a_panel_handle_are_those_of_its_blob(M, K, density):
+    W = synth.normal_bf16(M + K, (M, K), 0.02)
+    mask = synth.bernoulli_mask(M + K + 1, (M, K), density) if 0.0 < density < 1.0 else np.full((M, K), int(density), np.uint8)
+    for m in (mask, None):
+        want = sd2.sd2_unpack_host(sd2.sd2_pack_host(W, m, sd2.SD2_FORMAT_GAP4_MMA), want_dense=False)[1]
+        h = sd2.sd2_compress(W, m, sd2.SD2_FORMAT_GAP4_MMA)
+        assert {k: v for k, v in sd2.sd2_info(h).items() if k in want} == want
+        sd2.sd2_free(h)
+
+
+def test_panel_handles_are_made_in_little_memory():
+    # 8200 rows are made in five parts, the last of eight rows, in the 48 MiB beside the handle that a part of the weights and its mask
+    # take (all of them take 201 MB)
+    M = K = 8192
+    M += 8
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(5)
+    w = torch.empty((M, K), dtype=torch.bfloat16, device="cuda").normal_(0.0, 0.02, generator=gen)
+    w.masked_fill_(w == 0, 0.02)                                          # (a loaded handle has no words for kept zeros)
+    m = (torch.rand((M, K), device="cuda", generator=gen) < 0.25).to(torch.uint8)
+    x = torch.empty((16, K), dtype=torch.bfloat16, device="cuda").normal_(0.0, 1.0, generator=gen)
+    h = sd2.sd2_compress(w, m, sd2.SD2_FORMAT_GAP4_MMA)                   # in place: in one part
+    want = torch.zeros((16, M), dtype=torch.bfloat16, device="cuda")
+    sd2.sd2_spmm(h, x, want)
+    sd2.sd2_stream_check()
+    need = sd2.sd2_spmm_query(h, 16)["device_bytes"]
+    W, mask = bits_of(w), m.cpu().numpy()
+    dense = sd2.sd2_decompress(h)
+    assert np.array_equal(dense, oracle.roundtrip_ref(W, mask))
+    sd2.sd2_free(h)
+    blob = sd2.sd2_pack_host(W, mask, sd2.SD2_FORMAT_GAP4_MMA)
+    y = torch.zeros_like(want)
+    del w, m
+    torch.cuda.empty_cache()
+    hog = torch.empty(torch.cuda.mem_get_info()[0] - need - (72 << 20), dtype=torch.uint8, device="cuda")
+    assert need + (48 << 20) < torch.cuda.mem_get_info()[0] < need + (96 << 20)
+    for make in (lambda: sd2.sd2_load_blob(blob), lambda: sd2.sd2_compress(W, mask, sd2.SD2_FORMAT_GAP4_MMA)):
+        h = make()
+        assert sd2.sd2_spmm_query(h, 16)["device_bytes"] == need and np.array_equal(sd2.sd2_decompress(h), dense)
+        sd2.sd2_spmm(h, x, y.zero_())
+        sd2.sd2_stream_check()
+        assert torch.equal(y, want)
+        sd2.sd2_free(h)
+    del hog
+    torch.cuda.empty_cache()
+
+
 def test_a_loaded_panel_handle_decompresses_bit_for_bit():
     M, K = 130, 200
     W = synth.normal_bf16(51, (M, K), 0.02)
