@@ -355,7 +355,6 @@ def test_wait_budgets_do_not_count_the_kernel_before(fmt, N, monkeypatch):
     sd2.sd2_spmm(slow, xs, ys)
     sd2.sd2_spmm(h, x, y)
     sd2.sd2_stream_check()
-    close = {"rtol": 0.01, "atol": 0.01} if fmt == sd2.SD2_FORMAT_GAP4_MMA else {"rtol": 0.0, "atol": 0.0}   # (that one's order of sums varies)
-    torch.testing.assert_close(y, want, **close)
+    assert torch.isfinite(want).all() and torch.equal(y, want)                                       # (every format adds up in one order)
     for hh in (slow, h):
         sd2.sd2_free(hh)

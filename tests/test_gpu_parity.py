@@ -581,7 +581,7 @@ def test_drafter_whose_q_and_k_are_cut_into_strips_differently(fmt, N):
             sd2.sd2_free(h)
 
 
-# ---- GAP4_MMA: blocks expanded in shared memory, multiplied on the tensor cores ------------------
+# ---- GAP4_MMA: blocks expanded in registers, multiplied on the tensor cores from tensor memory ------------------
 
 def _mma_case(seed, M, K, d, N, f32):
     W, mask, X = case(seed, M, K, d, N)
@@ -596,7 +596,7 @@ def _mma_case(seed, M, K, d, N, f32):
 @pytest.mark.parametrize("M,K,d,N", [(128, 128, 0.5, 16), (128, 256, 0.5, 64), (130, 264, 0.5, 16), (300, 1000, 0.1, 17),
                                      (256, 2048, 0.5, 32), (1000, 520, 0.9, 48), (64, 4099, 0.5, 16), (257, 129, 1.0, 5),
                                      (2048, 512, 0.5, 1), (40, 24, 0.02, 64),
-                                     # many blocks per CTA: every stage, ring slot and accumulator is reused several times
+                                     # many blocks per CTA: every stage and ring slot is reused several times
                                      (2048, 8192, 0.5, 16), (1024, 16384, 0.7, 64), (3072, 4160, 0.3, 33)])
 @pytest.mark.parametrize("f32", [True, False])
 def test_mma_path_matches_oracle(M, K, d, N, f32):
@@ -606,13 +606,15 @@ def test_mma_path_matches_oracle(M, K, d, N, f32):
 
 
 def test_mma_path_more_than_64_rows_and_repeated_calls():
-    # 150 rows: three launches of at most 64; a second call must find the partial sums clean
+    # 150 rows: three launches of at most 64; every call adds up in the same order
     M, K, N = 384, 1024, 150
     W, mask, X = case(9100, M, K, 0.5, N)
     h = sd2.sd2_compress(W, mask, sd2.SD2_FORMAT_GAP4_MMA, sd2.SD2_DTYPE_F32)
     Yr, S = oracle.masked_linear(W, mask, X)
-    for _ in range(3):
-        check(run_spmm(h, X, True), Yr, S, True)
+    first = run_spmm(h, X, True)
+    check(first, Yr, S, True)
+    for _ in range(2):
+        assert np.array_equal(run_spmm(h, X, True), first)
     sd2.sd2_free(h)
 
 
