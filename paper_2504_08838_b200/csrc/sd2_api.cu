@@ -73,6 +73,7 @@ struct sd2_drafter_s {
     std::vector<sd2_handle> owned;      // paired gate|up stacks the drafter built for itself
     std::vector<int> pair_block;        // the block each of them belongs to
     std::vector<int64_t> ws_off;        // per block: offsets of q,k,v,hdn,g,u,t and the block output inside d_ws
+    int64_t x_off;             // a copy of the step's input inside d_ws, or -1 (see sd2_drafter_create)
     uint8_t* d_ws;
     SStage* d_stages;
     unsigned int* d_gbar;
@@ -2211,6 +2212,13 @@ sd2_status sd2_drafter_create(const sd2_handle* h, int32_t L, int64_t n_max, sd2
         d->ws_off[(size_t)b * 8 + 7] = o + off[7];
         o = a256(o + off[7] + 2 * n_max * dims[(size_t)b].out);
     }
+    // A launch replaces the input of its first stage.  Where q, k and v of the first block are cut into strips differently they take a
+    // stage each, and read a copy.  (A condition in the kernel, for which stages to replace it, cost every single launch 0.04 us of 4.84.)
+    d->x_off = -1;
+    if (h[1]->S != h[0]->S || h[2]->S != h[0]->S) {
+        d->x_off = o;
+        o = a256(o + 2 * n_max * d->hidden);
+    }
     d->ws_off[(size_t)L * 8] = o;
     std::vector<SStage> stages((size_t)L * 7);
     ProgramNeeds needs;
@@ -2258,7 +2266,8 @@ sd2_status sd2_drafter_create(const sd2_handle* h, int32_t L, int64_t n_max, sd2
         for (int b = 0; b < L; ++b) {
             uint8_t* base = d->d_ws;
             const int64_t* wo = &d->ws_off[(size_t)b * 8];
-            const uint16_t* xin = b == 0 ? nullptr : (const uint16_t*)(base + d->ws_off[(size_t)(b - 1) * 8 + 7]);
+            const int64_t x_off = b == 0 ? d->x_off : d->ws_off[(size_t)(b - 1) * 8 + 7];
+            const uint16_t* xin = x_off < 0 ? nullptr : (const uint16_t*)(base + x_off);
             void* yout = base + wo[7];
             BlockTags tg;
             if (tagged) {
@@ -2375,6 +2384,13 @@ sd2_status sd2_drafter_step(sd2_drafter d, const void* x, void* y, int64_t N, vo
     a.inl[0] = d->first_stage;
     a.n_stages = d->n_stages;
     a.x_in = (const uint16_t*)x;
+    if (d->x_off >= 0) {
+        a.x_in = nullptr;
+        if (cudaMemcpyAsync(d->d_ws + d->x_off, x, (size_t)(2 * N * d->hidden), cudaMemcpyDefault, (cudaStream_t)cuda_stream) != cudaSuccess) {
+            cudaGetLastError();
+            return SD2_ERR_CUDA;
+        }
+    }
     a.y_out = y;
     a.gbar = d->d_gbar;
     a.free_tiles = d->free_tiles;

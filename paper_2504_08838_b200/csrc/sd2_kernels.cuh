@@ -181,7 +181,7 @@ struct SFold {
 
 struct SArgsBase {
     const SStage* ext;              // device array of stages (programs longer than four stages)
-    const uint16_t* x_in;           // input of the stages that name none (a drafter's q|k|v of its first block: one stage, or three)
+    const uint16_t* x_in;           // replaces stage 0's x when not NULL
     void* y_out;                    // replaces the last stage's mat[0].y when not NULL
     unsigned int* gbar;             // grid barrier: [0] arrivals, [32] exits (two cache lines)
     int* err;                       // device error word
@@ -1047,10 +1047,10 @@ __global__ void __launch_bounds__(kStreamThreads, 1) stream_kernel(const __grid_
         const SStage& st = sh->stage[s & 1];
 
         const int K = st.K;
-        const uint16_t* x_src = st.x || st.g ? st.x : a.x_in;
+        const uint16_t* x_src = (s == 0 && a.x_in) ? a.x_in : st.x;
         const size_t xoff = (size_t)a.n0 * K;
         // tagged inputs are 32-bit words: twice the stride of bf16; stage s reads what stage s - 1 tagged
-        const bool tin = a.tagged && st.tagged_in;
+        const bool tin = a.tagged && st.tagged_in && !(s == 0 && a.x_in);
         const size_t xw = tin ? 2 * xoff : xoff;
         const uint32_t tag_in = tin ? (uint32_t)s : 0u;      // the stage part of a tag; the row part is tag_base[n]
         const uint32_t tag_out = (uint32_t)(s + 1);
