@@ -754,7 +754,8 @@ def run_sweep(args):
                     continue
                 blob = sd2.sd2_pack_host(W, mask, fmt, sd2.SD2_DTYPE_BF16)
                 h0 = sd2.sd2_load_blob(blob)
-                R = max(2, int(np.ceil(4.0 * l2 / h0.compressed_bytes)))
+                read = sd2.sd2_spmm_query(h0, min(ns) if name == "gap4" else max(ns))["streamed_bytes"]
+                R = max(2, int(np.ceil(4.0 * l2 / read)))
                 loaded[name] = [h0] + [sd2.sd2_load_blob(blob) for _ in range(R - 1)]
             Wd0 = torch.from_numpy(np.where(mask != 0, W, np.uint16(0)).view(np.int16)).cuda().view(torch.bfloat16)
             Rd = max(2, int(np.ceil(4.0 * l2 / (2 * M * K))))
