@@ -94,7 +94,8 @@ typedef struct {
 
 /* ---- format builder on the host (no device needed) ----------------------------------- */
 
-/* Encode W.*mask into a self-describing byte blob (the exact image sd2_compress uploads).
+/* Encode W.*mask into a self-describing byte blob (its sections are what sd2_compress uploads; of
+ * GAP4_MMA weights the GPU gets panel cells instead, about 1.25 times the records at 50 %).
  *   weight_bf16 : host, [M*K] bf16 patterns.
  *   mask        : host, [M*K] bytes, non-zero = kept; NULL = keep every weight that is
  *                 not +0/-0.  The mask is authoritative: a kept weight may be zero, NaN or
@@ -118,18 +119,22 @@ sd2_status sd2_blob_free(void* blob);
 /* ---- handles ------------------------------------------------------------------------- */
 
 /* Compress once per weight (the topology is static), copy to the current device.
- * weight_bf16 and mask may each be host or device memory. */
+ * weight_bf16 and mask may each be host or device memory.  GAP4 (for its cells, which it can do
+ * without) takes a copy of what the GPU cannot read in place, GAP4_MMA at most 48 MiB for a while
+ * (more where 128 rows are more than 16 million weights). */
 sd2_status sd2_compress(const void* weight_bf16, const uint8_t* mask, int64_t M, int64_t K,
                         const sd2_options* opt, sd2_handle* out);
 
-/* Make a handle from a blob produced by sd2_pack_host (host memory). */
+/* Make a handle from a blob produced by sd2_pack_host (host memory).  The same memory for a while, on
+ * the host too. */
 sd2_status sd2_load_blob(const void* blob, int64_t blob_bytes, sd2_handle* out);
 
 /* Read the device copy back and decode it: dense_bf16_out ([M*K], host or device)
  * receives W.*mask bit-exactly (masked-out entries +0). */
 sd2_status sd2_decompress(sd2_handle h, void* dense_bf16_out);
 
-/* Any out pointer may be NULL. */
+/* Any out pointer may be NULL.  compressed_bytes: of the blob's sections, which for GAP4_MMA are not what
+ * the handle keeps (sd2_spmm_query tells what it owns and what a launch reads). */
 sd2_status sd2_info(sd2_handle h, int64_t* M, int64_t* K, int64_t* nnz,
                     int64_t* compressed_bytes, int32_t* format);
 

@@ -32,8 +32,8 @@
 // What bounds it: HBM for large matrices (15 slots per clock and SM at 50 % density against 33 that twelve warps expanded, 29
 // for sixteen rows, before the sums were added up in fp32); between stages some 2.8 us: from the last output to the barrier's release 1.2, to the activations 0.6, to
 // the first cell 0.9.  One launch with its start and its last sums is 8 us at least, and launches of a stream overlap there.
-// Against the strips, which gather row by row (us): 5 rows of 1531 x 3001 18.5 -> 8.6, 48 rows of 8192 x 2048 111 -> 26, two
-// blocks of 2048/512/8192 for 8 rows 230 -> 68, a block of 3072/1024/8192 for 16 rows 342 -> 61.
+// Against the strips, which gather row by row (us): 5 rows of 1531 x 3001 18.5 -> 8.7, 48 rows of 8192 x 2048 111 -> 25.5, two
+// blocks of 2048/512/8192 for 8 rows 230 -> 67.5, a block of 3072/1024/8192 for 16 rows 342 -> 60.
 //
 // Every wait (ring barriers, counters, grid barrier) is bounded by a cycle budget: when it runs out the CTA raises the
 // error word and winds down instead of hanging.

@@ -24,12 +24,13 @@
 // The sums of a cluster meet by stores into the shared memory of the CTA that writes the activation row, in one order: results
 // do not depend on timing, and a handle has no state that launches share.
 //
-// What bounds it: HBM while blocks are expanded (24 of them in 6.4 us on each of 128 CTAs, 6.5 TB/s), then what stands between
-// launches: the last products, reading and exchanging the sums 2 us, the next start and its first block 2 us.  3072 x 8192 at 50 %
-// for 16 rows takes 11.5 us in a row of launches, 8192 x 3072 for 64 rows 13.1.  Before, 16-bit values were scattered into operand
-// tiles in shared memory (eight dependent steps of 340 cycles a block) and shares added up by red.add: 20.0 and 35.3.  Half-size
-// CTAs, two to an SM, whose successors fetch weights early: 11.2 for 16 rows, but 5.2 to 5.5 for 2048 x 2048 instead of 5.0, and sums
-// twice as far from 64 bits; not taken.
+// What bounds it: both 3072 x 8192 (24 panels, five shares each, 120 CTAs of 25 or 26 blocks) and 8192 x 3072 (64 panels, two shares,
+// 128 CTAs of 24 blocks) have 41.5 MB of panel cells at 50 %, 6.4 us at HBM's rate; in a row of launches the first takes 11.5 us for 16
+// rows, the second 13.1 for 64 (11.7 and 13.2 in a graph on cold weights).  The rest stands between launches: the last products, reading
+// and exchanging the sums, the next start and its first block.  Before, 16-bit values were scattered into operand tiles in shared
+// memory (eight dependent steps of 340 cycles a block) and shares added up by red.add: 20.0 and 35.3.  Half-size CTAs, two to an SM,
+// whose successors fetch weights early: 11.2 for 16 rows, but 5.2 to 5.5 for 2048 x 2048 instead of 5.0, and sums twice as far from
+// 64 bits; not taken.
 //
 // Every wait is bounded; a wait that runs out sets the error word and the CTA leaves in order (copies drained, tensor memory
 // returned).
